@@ -57,7 +57,10 @@ typedef enum {
 
 typedef enum { LEM_BC_DIRICHLET0 = 0, LEM_BC_PERIODIC = 1 } lem_bc;
 typedef enum { LEM_MODE_PHI = 0, LEM_MODE_EXP = 1 } lem_mode;
-/* LEM_PREC_FP64: propagators, residual and apply in IEEE binary64.
+/* LEM_PREC_FP64: propagators, residual and apply in IEEE binary64, or closer to the exact sums:
+ * where tiles share propagators (LEM_APPLY_FP64_GEMM) each output of the apply is an exact sum of
+ * digit products of the FP64 operands on the tensor cores, rounded once (operands cut 2^-56 below
+ * the largest value of their row or window).
  * Propagators of the split tiers are built with tensor-core products (every Pade product,
  * squaring and elimination update an exact sum of FP16 slice products, about 2^-45 of the
  * operands' scale; the environment variable LEM_BUILD_PRODUCTS=fp64 forces FP64 products).
@@ -89,7 +92,9 @@ typedef enum { LEM_SCHEME_EULER = 0, LEM_SCHEME_RB3 = 1 } lem_scheme;
 
 /* How lem_step applies the propagators (lem_info.apply_path). */
 typedef enum {
-  LEM_APPLY_FP64_GEMM = 0,   /* FP64, one gathered GEMM per class of tiles */
+  LEM_APPLY_FP64_GEMM = 0,   /* FP64, gathered products of windows and shared propagators (digit
+                                products on the tensor cores; lem_step_fp64_noalloc: one FP64 GEMM
+                                per class) */
   LEM_APPLY_FP64_GEMV = 1,   /* FP64, one batched GEMV over all tiles (many classes) */
   LEM_APPLY_F32_GEMV = 2,    /* FP32 propagators, float-float accumulation (complex: of FP32
                                 FMA sums over 16-byte chunks of a row) */
@@ -235,7 +240,8 @@ lem_status lem_set_timing(lem_ctx* ctx, int enable);
 lem_status lem_get_timing(lem_ctx* ctx, double* total_ms, int64_t* launches);
 
 /* Allocation-free FP64 step (the paper has no counterpart; this is a service to callers).
- * Same result as lem_step on an LEM_PREC_FP64 context, for callers that must not allocate
+ * Same result as lem_step on an LEM_PREC_FP64 context (on the GEMM apply path to FP64 rounding,
+ * on the batched GEMV bit for bit per step), for callers that must not allocate
  * device memory while they step: runtimes that own all device memory through their own
  * pool and forbid later driver allocations, and loops that cannot take cudaMalloc's
  * implicit synchronisation. Its per-step scratch comes from one static 8 MiB device array

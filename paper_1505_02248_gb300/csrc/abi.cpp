@@ -97,6 +97,7 @@ void free_ctx(lem_ctx* c) {
   if (!c) return;
   split_destroy(c);
   band_destroy(c);
+  oz_destroy(c);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   cudaFreeAsync(c->d_coef, c->stream);
   cudaFreeAsync(c->d_tiles, c->stream);
@@ -160,6 +161,7 @@ lem_status adopt_propagators(lem_ctx* dst, lem_ctx* src, cudaEvent_t built) {
   LEM_CUDA_TRY(cudaStreamWaitEvent(dst->stream, built, 0));
   LEM_CUDA_TRY(cudaMemcpyAsync(dst->d_P, src->d_P, sizeof(double) * dst->n_int * dst->n_loc,
                                cudaMemcpyDeviceToDevice, dst->stream));
+  LEM_TRY(oz_pack(dst));
   dst->squarings = src->squarings;
   dst->built = true;
   dst->build_gen++;
@@ -279,6 +281,14 @@ lem_status lem_create(const lem_problem_desc* desc, int device, void* cuda_strea
   } else {
     c->apply_path = many_classes ? LEM_APPLY_FP64_GEMV : LEM_APPLY_FP64_GEMM;
   }
+  if (c->apply_path == LEM_APPLY_FP64_GEMM) {
+    s = oz_prepare(c);
+    if (s == LEM_ENOMEM) {  // no room for the digits: the FP64 GEMM needs fewer bytes
+      oz_destroy(c);
+      s = LEM_OK;
+    }
+    if (s != LEM_OK) { free_ctx(c); return s; }
+  }
   if (c->apply_path == LEM_APPLY_F32_GEMV || c->apply_path == LEM_APPLY_FP64_GEMV) {
     s = gemv_set_smem(c);
     if (s != LEM_OK) { free_ctx(c); return s; }
@@ -330,7 +340,8 @@ static lem_status step_impl(lem_ctx* ctx, double* d_state, int nsteps, bool devi
   for (int k = 0; k < nsteps; ++k) {
     if (ctx->desc.reaction && ctx->desc.refresh > 0 && ctx->steps_since_build >= ctx->desc.refresh)
       LEM_TRY(build_propagators(ctx, d_state));
-    if (ctx->apply_path == LEM_APPLY_FP64_GEMM) LEM_TRY(step_fp64(ctx, d_state));
+    if (ctx->oz) LEM_TRY(step_oz(ctx, d_state));
+    else if (ctx->apply_path == LEM_APPLY_FP64_GEMM) LEM_TRY(step_fp64(ctx, d_state));
     else LEM_TRY(step_gemv(ctx, d_state, ctx->apply_path == LEM_APPLY_F32_GEMV));
     ctx->steps_since_build++;
   }
@@ -396,6 +407,8 @@ lem_status lem_set_propagators(lem_ctx* ctx, const double* h_P, const int* h_squ
   LEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
   LEM_CUDA_TRY(cudaMemcpy(ctx->d_P, h_P, sizeof(double) * n, cudaMemcpyHostToDevice));
   for (size_t c = 0; c < ctx->classes.size(); ++c) ctx->squarings[c] = h_squarings ? h_squarings[c] : -1;
+  LEM_TRY(oz_pack(ctx));
+  if (ctx->oz) LEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
   ctx->built = true;
   ctx->build_gen++;
   ctx->steps_since_build = 0;

@@ -941,6 +941,8 @@ lem_status build_propagators_impl(lem_ctx* ctx, const double* d_state) {
   if (rb3 && ctx->desc.reaction)
     LEM_CUDA_TRY(cudaMemcpyAsync(ctx->d_um, d_state, sizeof(double) * ctx->npts, cudaMemcpyDeviceToDevice,
                                  ctx->stream));
+  LEM_TRY(oz_pack(ctx));
+  if (ctx->oz) LEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
   ctx->built = true;
   ctx->build_gen++;
   ctx->steps_since_build = 0;

@@ -71,6 +71,7 @@ struct Stencil {
 
 struct SplitPlan;  // tcgen05 split-precision state (step_split.cu)
 struct BandPlan;   // truncated propagators (step_band.cu)
+struct OzPlan;     // FP64 step on the tensor cores (step_oz.cu)
 
 }  // namespace lem
 
@@ -113,6 +114,7 @@ struct lem_ctx {
   int* d_status = nullptr;             // device error word
   int64_t device_bytes = 0;
   lem::SplitPlan* split = nullptr;
+  lem::OzPlan* oz = nullptr;           // FP64 GEMM apply path: digit products on the tensor cores
   // truncated propagators (lem_set_truncation): off while band_tol < 0
   double band_tol = -1.0;
   int band_gen = -1;                   // build_gen the packed boxes were made from
@@ -139,6 +141,13 @@ lem_status build_propagators(lem_ctx* ctx, const double* d_state);
 lem_status step_fp64(lem_ctx* ctx, double* d_u);
 // step_fp64.cu: dt F(u) (or its complex / porous variants) into r on the context stream
 cudaError_t launch_residual_fp64(const lem_ctx* ctx, double* r, const double* u);
+// step_oz.cu: the FP64 step of contexts with shared propagators. oz_pack follows every change of
+// the propagators.
+lem_status oz_prepare(lem_ctx* ctx);
+lem_status oz_pack(lem_ctx* ctx);
+lem_status step_oz(lem_ctx* ctx, double* d_u);
+lem_status oz_check_error(lem_ctx* ctx);
+void oz_destroy(lem_ctx* ctx);
 // step_gemv.cu
 lem_status step_gemv(lem_ctx* ctx, double* d_u, bool f32);
 // blocks per tile of a batched GEMV launch with `threads` threads per block

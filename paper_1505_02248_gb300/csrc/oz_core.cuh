@@ -1,0 +1,286 @@
+// FP64 products on the tcgen05 tensor cores: exact sums of FP16 digit products (an Ozaki-type
+// splitting), used by the FP64 step (step_oz.cu) and the propagator build (builder_tc.cu).
+//
+// Each row i of A is scaled by 2^-e_i (max |A_i,:| < 2^e_i) and cut into S = 7 balanced base-256
+// digits (|d| <= 128, exact in FP16; 55 bits and a sign below 2^e_i), each column j of B likewise
+// with 2^-f_j. Level L = s + t collects the products of digit s of A with digit t of B. Every
+// partial sum of a level is an integer below 2^24 over a bounded stretch of K, which FP32
+// accumulation holds exactly: levels 4..6 (at most 7 pairs) over 128 K, levels 0..3 (at most 4)
+// over 256 K. After each stretch the level sums are drained from TMEM into 64-bit integers, so
+//   C_ij = 2^(e_i + f_j - 62) (hi 2^24 + lo)
+// is exact but for the dropped levels (L > 6, below 2^-58 of 2^(e_i + f_j) a term) and the one
+// rounding to FP64: closer to the true sum than K FP64 multiply-adds. The FP64 pipe (2
+// multiply-adds per clock and SM) does not take part.
+//
+// What bounds it: 28 digit products per K. An MMA of N columns takes N / 2 clk but not less than
+// its shared-memory operand reads (A 32 clk, B N / 4), 48 clk at N = 64. So one MMA takes digit s
+// of A against up to four consecutive digits of B as one operand of 4 x 64 rows: consecutive
+// digits of B lie back to back in shared memory, and their products belong to consecutive
+// levels, whose accumulators lie back to back in TMEM. Eleven MMAs then do a K step of 16 in 896
+// clk (28 of N = 64 take 1344). Operands stream from L2 at 43 KB per K step of 16.
+#pragma once
+#include <cuda_fp16.h>
+#include <stdint.h>
+
+#include "oz_convert.h"
+#include "tc_ptx.cuh"
+
+namespace lem {
+namespace oz {
+
+constexpr int S = 7;      // digits per operand, levels kept
+constexpr int BM = 128;   // output rows per CTA (TMEM lanes)
+constexpr int BN = 64;    // output columns per CTA
+constexpr int KB = 16;    // K elements per block (one MMA K step)
+constexpr int A_SLICE = BM * KB;          // halves of one digit's tile
+constexpr int B_SLICE = BN * KB;
+constexpr int A_BLOCK = S * A_SLICE;      // halves of one K block, all digits
+constexpr int B_BLOCK = S * B_SLICE;
+constexpr int A_BYTES = A_BLOCK * 2;      // 28 KB
+constexpr int B_BYTES = B_BLOCK * 2;      // 14 KB
+constexpr int STAGE = A_BYTES + B_BYTES;
+constexpr int STAGES = 5;                 // 215 KB of the SM's 227
+constexpr int STRETCH_LO = 8;             // K blocks per exact stretch of levels 4..6 (128 K)
+constexpr int STRETCH_HI = 16;            // of levels 0..3 (256 K)
+constexpr int EPI_WARPS = 8;              // two per TMEM lane quarter, 32 columns each
+constexpr int THREADS = 64 + 32 * EPI_WARPS;
+constexpr int SMEM = STAGES * STAGE + 1024 + 256;
+constexpr uint64_t WAIT_NS = 2000000000ull;
+constexpr int SUM_PITCH = BM + 1;         // staged sums: column pitch in 16-byte (hi, lo) pairs
+
+static_assert(BN * SUM_PITCH * 16 <= STAGES * STAGE, "staged sums reuse the operand stages");
+
+// Operand tiles: for each block of 128 (A) or 64 (B) rows and each K block of 16, the seven
+// digits' tiles back to back. A tile is in the tcgen05 K-major layout without swizzle: 8-row x
+// 8-element core matrices of 128 contiguous bytes, two along K (128 B apart), 8-row groups 256 B
+// apart. So element (r, k) of a tile sits at half offset (r / 8) 128 + (k / 8) 64 + (r % 8) 8 + k % 8.
+__device__ __forceinline__ int tile_off(int r, int k8) {  // k8: first of 8 consecutive K elements
+  return (r / 8) * 128 + (k8 / 8) * 64 + (r % 8) * 8;
+}
+
+// The seven digits of 8 consecutive K elements (as N + kBias) into their tiles: `dst` is the
+// element's place in digit 0's tile, tiles lie `slice` halves apart.
+__device__ __forceinline__ void store_digits(__half* dst, int slice, const unsigned long long (&N)[8]) {
+  uint32_t lo[8], hi[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    lo[u] = uint32_t(N[u]);
+    hi[u] = uint32_t(N[u] >> 32);
+  }
+  const __half2 bias = __half2half2(__ushort_as_half(0x6480));  // 1024 + 128
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t t;
+      if (s == 0) {  // the top field has nine bits (0 .. 256)
+        t = ((hi[2 * q] >> 16) & 0x1FFu) + ((hi[2 * q + 1] & 0x1FF0000u)) + 0x64006400u;
+      } else {
+        const int byte = 6 - s;  // place of digit s in N
+        const uint32_t a = byte >= 4 ? hi[2 * q] : lo[2 * q], b = byte >= 4 ? hi[2 * q + 1] : lo[2 * q + 1];
+        const uint32_t sel = uint32_t(byte & 3) | (uint32_t(4 + (byte & 3)) << 8);
+        t = __byte_perm(a, b, (sel & 0xF) | ((sel >> 8) << 8));
+        t = (t & 0x00FF00FFu) | 0x64006400u;
+      }
+      // 1024 + (digit + 128) as a half, minus 1152: the digit, exactly
+      const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&t), bias);
+      w[q] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    *reinterpret_cast<uint4*>(dst + s * slice) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// Shared-memory layout of a CTA, and its barriers.
+struct Shared {
+  uint8_t* stage;   // STAGES x STAGE bytes, then the staged sums
+  uint64_t* full;   // [STAGES] stage loaded
+  uint64_t* empty;  // [STAGES] stage consumed by the MMAs
+  uint64_t* accf;   // [2] levels 0..3 / 4..6 complete for a stretch
+  uint64_t* acce;   // [2] drained
+  uint32_t* tslot;
+};
+
+__device__ __forceinline__ Shared carve(uint8_t* raw) {
+  Shared sh;
+  // (offset arithmetic on the shared array keeps the pointers in the shared address space)
+  sh.stage = raw + ((1024u - (ptx::smem_u32(raw) & 1023u)) & 1023u);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sh.stage + STAGES * STAGE);
+  sh.full = bars;
+  sh.empty = bars + STAGES;
+  sh.accf = bars + 2 * STAGES;
+  sh.acce = sh.accf + 2;
+  sh.tslot = reinterpret_cast<uint32_t*>(sh.acce + 2);
+  return sh;
+}
+
+// Barriers and TMEM (all 512 columns: 448 hold the levels); every thread of the CTA calls it.
+__device__ __forceinline__ uint32_t setup(const Shared& sh, volatile int* s_abort) {
+  if (threadIdx.x == 0) {
+    *s_abort = 0;
+    for (int q = 0; q < STAGES; ++q) {
+      ptx::mbar_init(&sh.full[q], 1);
+      ptx::mbar_init(&sh.empty[q], 1);
+    }
+    for (int h = 0; h < 2; ++h) {
+      ptx::mbar_init(&sh.accf[h], 1);
+      ptx::mbar_init(&sh.acce[h], EPI_WARPS);
+    }
+    ptx::fence_barrier_init();
+  }
+  if (threadIdx.x / 32 == 1) {
+    ptx::tmem_alloc(sh.tslot, 512);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  return *sh.tslot;
+}
+
+__device__ __forceinline__ void release(uint32_t tmem) {
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x / 32 == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, 512);
+  }
+}
+
+// acc += weight x one level's sums (32 columns of this thread's row)
+__device__ __forceinline__ void drain(uint32_t taddr, int weight, long long (&acc)[32]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float r[16];
+    ptx::tmem_ld_32x32b_x16(taddr + uint32_t(16 * h), r);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) acc[16 * h + j] += (long long)(__float2int_rn(r[j])) * weight;
+  }
+}
+
+// The digit products of `nkb` K blocks (nkb >= 1) of one 128 x 64 output tile; tA and tB point at
+// the tile's first K block. Warp 0 loads, warp 1 issues the MMAs, warps 2..9 drain: thread =
+// output row (TMEM lane), 32 of its 64 columns. The drained sums end up in shared memory (over
+// the operand stages), pair (hi, lo) of element (row, col) at [col * SUM_PITCH + row]. Every
+// thread of the CTA calls it; a barrier ends it. A wait that runs out records `err`, sets s_abort
+// and lets the CTA finish (with meaningless sums).
+__device__ __forceinline__ void products(const Shared& sh, uint32_t tmem, const __half* __restrict__ tA,
+                                         const __half* __restrict__ tB, int nkb, int* err, volatile int* s_abort) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  if (warp == 0) {
+    if (lane == 0) {
+      int issued = 0, q = 0;
+      uint32_t par = 0;
+      for (int kb = 0; kb < nkb && !*s_abort; ++kb) {
+        if (kb >= STAGES && !ptx::mbar_wait(&sh.empty[q], par ^ 1u, WAIT_NS)) {
+          atomicExch(err, 1);
+          *s_abort = 1;
+          break;
+        }
+        uint8_t* st = sh.stage + q * STAGE;
+        ptx::mbar_arrive_expect_tx(&sh.full[q], STAGE);
+        ptx::bulk_load(st, tA + size_t(kb) * A_BLOCK, A_BYTES, &sh.full[q]);
+        ptx::bulk_load(st + A_BYTES, tB + size_t(kb) * B_BLOCK, B_BYTES, &sh.full[q]);
+        issued = kb + 1;
+        if (++q == STAGES) {
+          q = 0;
+          par ^= 1u;
+        }
+      }
+      // every copy issued has landed before the CTA reuses the stages or exits
+      for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
+        ptx::mbar_wait(&sh.full[kb % STAGES], (kb / STAGES) & 1, WAIT_NS);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      bool ok = true;
+      int q = 0;
+      uint32_t par = 0;
+      for (int kb = 0; kb < nkb; ++kb) {
+        if (!ptx::mbar_wait(&sh.full[q], par, WAIT_NS)) { ok = false; break; }
+        ptx::tc_fence_after();
+        const uint32_t a0 = ptx::smem_u32(sh.stage + q * STAGE);
+        const uint64_t dA = ptx::plain_kmajor_desc(a0, 128, 256);
+        const uint64_t dB = ptx::plain_kmajor_desc(a0 + A_BYTES, 128, 256);
+        constexpr uint64_t SA = A_SLICE * 2 / 16, SB = B_SLICE * 2 / 16;  // descriptor steps per digit
+        // levels 0..3: digit s of A against digits 0 .. 3 - s of B
+        const bool hi0 = kb % STRETCH_HI == 0, lo0 = kb % STRETCH_LO == 0;
+        if (hi0 && kb > 0) {
+          if (!ptx::mbar_wait(&sh.acce[0], (kb / STRETCH_HI - 1) & 1, WAIT_NS)) { ok = false; break; }
+          ptx::tc_fence_after();
+        }
+        ptx::mma_f16(tmem, dA, dB, ptx::idesc_f16_f32(BM, 4 * BN), hi0 ? 0u : 1u);
+        ptx::mma_f16(tmem + BN, dA + SA, dB, ptx::idesc_f16_f32(BM, 3 * BN), 1u);
+        ptx::mma_f16(tmem + 2 * BN, dA + 2 * SA, dB, ptx::idesc_f16_f32(BM, 2 * BN), 1u);
+        ptx::mma_f16(tmem + 3 * BN, dA + 3 * SA, dB, ptx::idesc_f16_f32(BM, BN), 1u);
+        if (kb % STRETCH_HI == STRETCH_HI - 1 || kb == nkb - 1) ptx::mma_commit(&sh.accf[0]);
+        // levels 4..6: digit s of A against digits max(4 - s, 0) .. 6 - s of B
+        if (lo0 && kb > 0) {
+          if (!ptx::mbar_wait(&sh.acce[1], (kb / STRETCH_LO - 1) & 1, WAIT_NS)) { ok = false; break; }
+          ptx::tc_fence_after();
+        }
+        ptx::mma_f16(tmem + 4 * BN, dA, dB + 4 * SB, ptx::idesc_f16_f32(BM, 3 * BN), lo0 ? 0u : 1u);
+#pragma unroll
+        for (int s = 1; s < 5; ++s)
+          ptx::mma_f16(tmem + 4 * BN, dA + s * SA, dB + (4 - s) * SB, ptx::idesc_f16_f32(BM, 3 * BN), 1u);
+        ptx::mma_f16(tmem + 5 * BN, dA + 5 * SA, dB, ptx::idesc_f16_f32(BM, 2 * BN), 1u);
+        ptx::mma_f16(tmem + 6 * BN, dA + 6 * SA, dB, ptx::idesc_f16_f32(BM, BN), 1u);
+        ptx::mma_commit(&sh.empty[q]);
+        if (kb % STRETCH_LO == STRETCH_LO - 1 || kb == nkb - 1) ptx::mma_commit(&sh.accf[1]);
+        if (++q == STAGES) {
+          q = 0;
+          par ^= 1u;
+        }
+      }
+      if (!ok) {
+        atomicExch(err, 2);
+        *s_abort = 1;
+      }
+    }
+  } else {
+    const int e = warp - 2, quarter = warp & 3, half = e >> 2;
+    const uint32_t base = tmem + (uint32_t(32 * quarter) << 16) + uint32_t(32 * half);
+    long long hi[32], lo[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
+    bool ok = true;
+    const int nlo = (nkb + STRETCH_LO - 1) / STRETCH_LO;
+    int chi = 0;
+    for (int c = 0; c < nlo; ++c) {
+      if ((c & 1) || c == nlo - 1) {  // levels 0..3 end with every second stretch of the others
+        if (*s_abort || !ptx::mbar_wait(&sh.accf[0], chi & 1, WAIT_NS)) { ok = false; break; }
+        ++chi;
+        ptx::tc_fence_after();
+#pragma unroll
+        for (int L = 0; L < 4; ++L) drain(base + uint32_t(L * BN), 1 << (8 * (3 - L)), hi);
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&sh.acce[0]);
+      }
+      if (*s_abort || !ptx::mbar_wait(&sh.accf[1], c & 1, WAIT_NS)) { ok = false; break; }
+      ptx::tc_fence_after();
+#pragma unroll
+      for (int L = 4; L < 7; ++L) drain(base + uint32_t(L * BN), 1 << (8 * (6 - L)), lo);
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&sh.acce[1]);
+    }
+    if (!ok) {
+      if (lane == 0) {
+        atomicExch(err, 3);
+        *s_abort = 1;
+      }
+    } else {
+      // the last accf phase: every MMA of the tile, hence every load, has completed, so the
+      // stages are free for the sums
+      longlong2* sums = reinterpret_cast<longlong2*>(sh.stage);
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        sums[(32 * half + j) * SUM_PITCH + 32 * quarter + lane] = make_longlong2(hi[j], lo[j]);
+    }
+  }
+  __syncthreads();
+}
+
+}  // namespace oz
+}  // namespace lem

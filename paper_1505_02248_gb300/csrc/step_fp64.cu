@@ -1,4 +1,5 @@
-// Plain FP64 LEM step (Sec. 3 steps 1-3, Eq. lem): the reference GPU path.
+// Plain FP64 LEM step (Sec. 3 steps 1-3, Eq. lem) on the FP64 pipe: the allocation-free step, and
+// lem_step where the digits of the tensor-core FP64 step (step_oz.cu) do not fit in memory.
 //   PHI:  r = dt F(u^n) (stencil residual, Eq. spacedisc with g = 0, plus dt(u - u^3), or the
 //         stencil applied to |u|^(m-1) u for the porous-medium equation);
 //         U_i = r|_{M_i} (halo gather); Y_i = P_{c(i)} U_i; u_D += Y_i (owner scatter).

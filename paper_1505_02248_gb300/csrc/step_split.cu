@@ -1617,6 +1617,7 @@ lem_status split_batch_check_error(SplitBatch* b) {
 }
 
 lem_status split_check_error(lem_ctx* ctx) {
+  LEM_TRY(oz_check_error(ctx));
   if (!ctx->split) return LEM_OK;
   int e = 0;
   LEM_CUDA_TRY(cudaMemcpy(&e, ctx->split->d_err, sizeof(int), cudaMemcpyDeviceToHost));
