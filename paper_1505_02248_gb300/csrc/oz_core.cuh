@@ -17,7 +17,9 @@
 // of A against up to four consecutive digits of B as one operand of 4 x 64 rows: consecutive
 // digits of B lie back to back in shared memory, and their products belong to consecutive
 // levels, whose accumulators lie back to back in TMEM. Eleven MMAs then do a K step of 16 in 896
-// clk (28 of N = 64 take 1344). Operands stream from L2 at 43 KB per K step of 16.
+// clk (28 of N = 64 take 1344). Measured 1130 clk a K step: shared memory serves 352 clk of A reads,
+// 448 of B reads and 336 of the 43 KB that stream in (without the loads 950, without the drains
+// 1050, loads alone 720).
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -42,12 +44,14 @@ constexpr int STAGE = A_BYTES + B_BYTES;
 constexpr int STAGES = 5;                 // 215 KB of the SM's 227
 constexpr int STRETCH_LO = 8;             // K blocks per exact stretch of levels 4..6 (128 K)
 constexpr int STRETCH_HI = 16;            // of levels 0..3 (256 K)
+constexpr int GROUP = 4;                  // K blocks whose levels 0..3 go before their levels 4..6
 constexpr int EPI_WARPS = 8;              // two per TMEM lane quarter, 32 columns each
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
 constexpr int SMEM = STAGES * STAGE + 1024 + 256;
 constexpr uint64_t WAIT_NS = 2000000000ull;
 constexpr int SUM_PITCH = BM + 1;         // staged sums: column pitch in 16-byte (hi, lo) pairs
 
+static_assert(STRETCH_LO % GROUP == 0 && STRETCH_HI % STRETCH_LO == 0 && GROUP < STAGES, "groups end stretches");
 static_assert(BN * SUM_PITCH * 16 <= STAGES * STAGE, "staged sums reuse the operand stages");
 
 // Operand tiles: for each block of 128 (A) or 64 (B) rows and each K block of 16, the seven
@@ -193,44 +197,53 @@ __device__ __forceinline__ void products(const Shared& sh, uint32_t tmem, const 
     }
   } else if (warp == 1) {
     if (lane == 0) {
+      // K blocks are taken four at a time, first their products of levels 0..3, then those of
+      // levels 4..6: while one group of levels is drained the MMAs of the other group run (one K
+      // block at a time, the drains held the MMAs up: 1360 clk a K block).
+      constexpr uint64_t SA = A_SLICE * 2 / 16, SB = B_SLICE * 2 / 16;  // descriptor steps per digit
+      const uint32_t s0 = ptx::smem_u32(sh.stage);
+      const uint64_t dA0 = ptx::plain_kmajor_desc(s0, 128, 256), dB0 = ptx::plain_kmajor_desc(s0 + A_BYTES, 128, 256);
       bool ok = true;
-      int q = 0;
+      int qa = 0, qb = 0;
       uint32_t par = 0;
-      for (int kb = 0; kb < nkb; ++kb) {
-        if (!ptx::mbar_wait(&sh.full[q], par, WAIT_NS)) { ok = false; break; }
-        ptx::tc_fence_after();
-        const uint32_t a0 = ptx::smem_u32(sh.stage + q * STAGE);
-        const uint64_t dA = ptx::plain_kmajor_desc(a0, 128, 256);
-        const uint64_t dB = ptx::plain_kmajor_desc(a0 + A_BYTES, 128, 256);
-        constexpr uint64_t SA = A_SLICE * 2 / 16, SB = B_SLICE * 2 / 16;  // descriptor steps per digit
-        // levels 0..3: digit s of A against digits 0 .. 3 - s of B
-        const bool hi0 = kb % STRETCH_HI == 0, lo0 = kb % STRETCH_LO == 0;
-        if (hi0 && kb > 0) {
-          if (!ptx::mbar_wait(&sh.acce[0], (kb / STRETCH_HI - 1) & 1, WAIT_NS)) { ok = false; break; }
+      for (int k0 = 0; k0 < nkb && ok; k0 += GROUP) {
+        const int k1 = k0 + GROUP < nkb ? k0 + GROUP : nkb;
+        if (k0 % STRETCH_HI == 0 && k0 > 0) {
+          if (!ptx::mbar_wait(&sh.acce[0], (k0 / STRETCH_HI - 1) & 1, WAIT_NS)) { ok = false; break; }
+        }
+        for (int kb = k0; kb < k1; ++kb) {
+          if (!ptx::mbar_wait(&sh.full[qa], par, WAIT_NS)) { ok = false; break; }
+          ptx::tc_fence_after();
+          const uint64_t dA = dA0 + uint64_t(qa * (STAGE >> 4)), dB = dB0 + uint64_t(qa * (STAGE >> 4));
+          // digit s of A against digits 0 .. 3 - s of B
+          ptx::mma_f16(tmem, dA, dB, ptx::idesc_f16_f32(BM, 4 * BN), kb % STRETCH_HI == 0 ? 0u : 1u);
+          ptx::mma_f16(tmem + BN, dA + SA, dB, ptx::idesc_f16_f32(BM, 3 * BN), 1u);
+          ptx::mma_f16(tmem + 2 * BN, dA + 2 * SA, dB, ptx::idesc_f16_f32(BM, 2 * BN), 1u);
+          ptx::mma_f16(tmem + 3 * BN, dA + 3 * SA, dB, ptx::idesc_f16_f32(BM, BN), 1u);
+          if (++qa == STAGES) {
+            qa = 0;
+            par ^= 1u;
+          }
+        }
+        if (!ok) break;
+        if (k1 % STRETCH_HI == 0 || k1 == nkb) ptx::mma_commit(&sh.accf[0]);
+        if (k0 % STRETCH_LO == 0 && k0 > 0) {
+          if (!ptx::mbar_wait(&sh.acce[1], (k0 / STRETCH_LO - 1) & 1, WAIT_NS)) { ok = false; break; }
           ptx::tc_fence_after();
         }
-        ptx::mma_f16(tmem, dA, dB, ptx::idesc_f16_f32(BM, 4 * BN), hi0 ? 0u : 1u);
-        ptx::mma_f16(tmem + BN, dA + SA, dB, ptx::idesc_f16_f32(BM, 3 * BN), 1u);
-        ptx::mma_f16(tmem + 2 * BN, dA + 2 * SA, dB, ptx::idesc_f16_f32(BM, 2 * BN), 1u);
-        ptx::mma_f16(tmem + 3 * BN, dA + 3 * SA, dB, ptx::idesc_f16_f32(BM, BN), 1u);
-        if (kb % STRETCH_HI == STRETCH_HI - 1 || kb == nkb - 1) ptx::mma_commit(&sh.accf[0]);
-        // levels 4..6: digit s of A against digits max(4 - s, 0) .. 6 - s of B
-        if (lo0 && kb > 0) {
-          if (!ptx::mbar_wait(&sh.acce[1], (kb / STRETCH_LO - 1) & 1, WAIT_NS)) { ok = false; break; }
-          ptx::tc_fence_after();
-        }
-        ptx::mma_f16(tmem + 4 * BN, dA, dB + 4 * SB, ptx::idesc_f16_f32(BM, 3 * BN), lo0 ? 0u : 1u);
+        for (int kb = k0; kb < k1; ++kb) {
+          const uint64_t dA = dA0 + uint64_t(qb * (STAGE >> 4)), dB = dB0 + uint64_t(qb * (STAGE >> 4));
+          // digit s of A against digits max(4 - s, 0) .. 6 - s of B
+          ptx::mma_f16(tmem + 4 * BN, dA, dB + 4 * SB, ptx::idesc_f16_f32(BM, 3 * BN), kb % STRETCH_LO == 0 ? 0u : 1u);
 #pragma unroll
-        for (int s = 1; s < 5; ++s)
-          ptx::mma_f16(tmem + 4 * BN, dA + s * SA, dB + (4 - s) * SB, ptx::idesc_f16_f32(BM, 3 * BN), 1u);
-        ptx::mma_f16(tmem + 5 * BN, dA + 5 * SA, dB, ptx::idesc_f16_f32(BM, 2 * BN), 1u);
-        ptx::mma_f16(tmem + 6 * BN, dA + 6 * SA, dB, ptx::idesc_f16_f32(BM, BN), 1u);
-        ptx::mma_commit(&sh.empty[q]);
-        if (kb % STRETCH_LO == STRETCH_LO - 1 || kb == nkb - 1) ptx::mma_commit(&sh.accf[1]);
-        if (++q == STAGES) {
-          q = 0;
-          par ^= 1u;
+          for (int s = 1; s < 5; ++s)
+            ptx::mma_f16(tmem + 4 * BN, dA + s * SA, dB + (4 - s) * SB, ptx::idesc_f16_f32(BM, 3 * BN), 1u);
+          ptx::mma_f16(tmem + 5 * BN, dA + 5 * SA, dB, ptx::idesc_f16_f32(BM, 2 * BN), 1u);
+          ptx::mma_f16(tmem + 6 * BN, dA + 6 * SA, dB, ptx::idesc_f16_f32(BM, BN), 1u);
+          ptx::mma_commit(&sh.empty[qb]);
+          if (++qb == STAGES) qb = 0;
         }
+        if (k1 % STRETCH_LO == 0 || k1 == nkb) ptx::mma_commit(&sh.accf[1]);
       }
       if (!ok) {
         atomicExch(err, 2);

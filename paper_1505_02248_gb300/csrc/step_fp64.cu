@@ -16,15 +16,18 @@ namespace {
 // r[p] = sum of the dt-scaled stencil around p (+ dt (u - u^3)); walls drop neighbours.
 // NL (the reaction kind) 2, porous medium (Eq. porous): the stencil acts on
 // phi(u) = |u|^(m-1) u.
+// One thread per column x and row of a block (64 x 4, 1D 256 x 1): a flat index split by 64-bit
+// division took 14.9 us on 1024^2, against 9 us of FP64 multiply-adds.
 template <int NL>
 __global__ void residual_fp64_kernel(double* __restrict__ r, const double* __restrict__ u,
                                      const double* __restrict__ coef, int64_t cstride,
                                      int64_t ny, int64_t nx, int ndim, int pery, int perx,
                                      double dt, double pm) {
   const int64_t npts = ny * nx;
-  for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < npts;
-       p += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t y = p / nx, x = p % nx;
+  const int64_t x = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (x >= nx) return;
+  for (int64_t y = int64_t(blockIdx.y) * blockDim.y + threadIdx.y; y < ny; y += int64_t(gridDim.y) * blockDim.y) {
+    const int64_t p = y * nx + x;
     // coefficient `w` (0..4 = C, W, E, S, N) at node p
     auto cf = [&](int w) { return cstride ? coef[int64_t(w) * npts + p] : coef[w]; };
     auto val = [&](int64_t q) {
@@ -130,14 +133,17 @@ cudaError_t launch_residual_fp64(const lem_ctx* ctx, double* r, const double* u)
     return cudaGetLastError();
   }
   const int py = ctx->bcy == LEM_BC_PERIODIC, px = ctx->bcx == LEM_BC_PERIODIC;
+  const dim3 block = ctx->ny == 1 ? dim3(256, 1) : dim3(64, 4);
+  const dim3 grid(unsigned((ctx->nx + block.x - 1) / block.x),
+                  unsigned(std::min<int64_t>((ctx->ny + block.y - 1) / block.y, 32768)));
   if (d.reaction == 2)
-    residual_fp64_kernel<2><<<blocks, 256, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
+    residual_fp64_kernel<2><<<grid, block, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
                                                              d.ndim, py, px, d.dt, d.porous_m);
   else if (d.reaction == 1)
-    residual_fp64_kernel<1><<<blocks, 256, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
+    residual_fp64_kernel<1><<<grid, block, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
                                                              d.ndim, py, px, d.dt, d.porous_m);
   else
-    residual_fp64_kernel<0><<<blocks, 256, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
+    residual_fp64_kernel<0><<<grid, block, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
                                                              d.ndim, py, px, d.dt, d.porous_m);
   return cudaGetLastError();
 }

@@ -7,8 +7,9 @@
 //
 // GB300's FP64 pipe runs 1.1 TFLOP/s, its FP16 tensor cores 1900. The 1024^2 periodic problem
 // (1024 windows of 2304 nodes, 1024 x 2304 propagator) took 4.67 ms a step as one FP64 GEMM, at
-// the FP64 pipe's rate, and takes 0.19 ms here; a walled 389 x 517 mesh with 16 classes, their
-// GEMMs one after another, 29.2 ms a step, and 0.14 ms here.
+// the FP64 pipe's rate, and takes 0.145 ms here (products 113 us, window digits 20, residual 15); a
+// walled 389 x 517 mesh with 16 classes, their GEMMs one after another, 29.2 ms a step, and 0.112
+// ms here.
 //
 // Layout: windows are the rows of A (128 windows of one class form a block), owner rows of the
 // class's propagator the columns of B. The propagators are cut once per build. One launch covers
@@ -56,59 +57,74 @@ struct PropRows {   // 64 owner rows of one class
   int64_t b_off;
 };
 
-// Window digits: a CTA cuts 8 windows (one core-matrix row group, so the 16-byte stores of 8
-// lanes fill 128 bytes). One warp per window finds the largest exponent; then each thread cuts 8
-// consecutive nodes of one window. Bound by the 14 bytes written per node (and about 40 integer
-// operations); the two reads of the window come from L2.
-__global__ void __launch_bounds__(256) oz_windows_kernel(const double* __restrict__ src,
-                                                         const TileDesc* __restrict__ tiles,
-                                                         const int32_t* __restrict__ order,
-                                                         const WinBlock* __restrict__ blocks, int wb0, int64_t ny,
-                                                         int64_t nx, int* __restrict__ e, __half* __restrict__ out) {
-  const WinBlock b = blocks[wb0 + blockIdx.x / 16];
-  const int r0 = (blockIdx.x % 16) * 8;
+// k / d for 0 <= k < 2^16 and 1 < d < 2^16 by one multiply (inv = div_inv(d)); d = 1: inv = 0.
+__host__ __device__ __forceinline__ uint32_t div_inv(uint32_t d) { return d > 1 ? 0xFFFFFFFFu / d + 1u : 0u; }
+__device__ __forceinline__ int div_by(int k, uint32_t inv) { return inv ? int(__umulhi(uint32_t(k), inv)) : k; }
+
+// Window digits: a CTA cuts R windows of one block (8: one core-matrix row group, so the 16-byte
+// stores of 8 lanes fill 128 bytes; fewer where 8 a CTA would leave SMs idle). Its warps find each
+// window's largest exponent, then each thread cuts 8 consecutive nodes of one window. Bound by
+// the 14 bytes written per node and about 40 integer operations; the two reads of the window come
+// from L2. (Eight windows per 256-thread CTA and 64-bit node arithmetic: 43 us for 1024 windows
+// of 2304 nodes.)
+constexpr int WIN_THREADS = 512;
+template <int R>
+__global__ void __launch_bounds__(WIN_THREADS) oz_windows_kernel(const double* __restrict__ src,
+                                                                 const TileDesc* __restrict__ tiles,
+                                                                 const int32_t* __restrict__ order,
+                                                                 const WinBlock* __restrict__ blocks, int wb0, int ny,
+                                                                 int nx, int* __restrict__ e, __half* __restrict__ out) {
+  constexpr int PER = oz::BM / R;  // CTAs per block
+  const WinBlock b = blocks[wb0 + blockIdx.x / PER];
+  const int r0 = (blockIdx.x % PER) * R;
   if (r0 >= b.count) return;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  __shared__ TileDesc td[8];
-  __shared__ int ex[8];
-  if (threadIdx.x < 8) td[threadIdx.x] = tiles[order[b.first + min(r0 + int(threadIdx.x), b.count - 1)]];
-  __syncthreads();
-  const int wx = td[0].wext[1], wn = td[0].wext[0] * wx;  // one class: one window shape
-  auto node = [&](const TileDesc& t, int a, int c) {
-    int64_t gy = int64_t(t.org[0]) + a, gx = int64_t(t.org[1]) + c;
-    gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
-    gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
-    return gy * nx + gx;
-  };
-  {
-    int E = 0;
-    int a = lane / wx, c = lane % wx;
-    const int da = 32 / wx, dc = 32 % wx;
-    for (int k = lane; k < wn; k += 32) {
-      E = max(E, oz::exp_field(static_cast<unsigned long long>(__double_as_longlong(src[node(td[warp], a, c)]))));
-      a += da;
-      c += dc;
-      if (c >= wx) {
-        c -= wx;
-        ++a;
-      }
-    }
-    for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
-    if (lane == 0) {
-      ex[warp] = oz::scale_exp(E);
-      e[b.e_off + r0 + warp] = ex[warp];
+  __shared__ int2 org[R];
+  __shared__ int ex[R], wext[2];
+  if (threadIdx.x < R) {
+    const TileDesc& t = tiles[order[b.first + min(r0 + int(threadIdx.x), b.count - 1)]];
+    org[threadIdx.x] = make_int2(t.org[0], t.org[1]);
+    ex[threadIdx.x] = 0;
+    if (threadIdx.x == 0) {  // one class: one window shape
+      wext[0] = t.wext[0];
+      wext[1] = t.wext[1];
     }
   }
   __syncthreads();
-  const int r = threadIdx.x % 8;
-  const int er = ex[r] == oz::kNonFinite ? 4096 : ex[r];  // (non-finite: every digit 0)
+  const int wx = wext[1], wn = wext[0] * wx;
+  const uint32_t inv = div_inv(uint32_t(wx));
+  auto at = [&](int2 o, int a, int c) {  // (meshes hold at most 2^31 nodes)
+    int gy = o.x + a, gx = o.y + c;
+    gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
+    gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
+    return src[uint32_t(gy) * uint32_t(nx) + uint32_t(gx)];
+  };
+  {
+    constexpr int WPR = WIN_THREADS / 32 / R;  // warps per window
+    const int r = warp / WPR;
+    const int2 o = org[r];
+    int E = 0;
+#pragma unroll 4
+    for (int k = (warp % WPR) * 32 + lane; k < wn; k += 32 * WPR) {
+      const int a = div_by(k, inv);
+      E = max(E, oz::exp_field(static_cast<unsigned long long>(__double_as_longlong(at(o, a, k - a * wx)))));
+    }
+    for (int q = 16; q > 0; q >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, q));
+    if (lane == 0) atomicMax(&ex[r], E);
+  }
+  __syncthreads();
+  const int r = threadIdx.x % R;
+  const int sc = oz::scale_exp(ex[r]);
+  if (threadIdx.x < R) e[b.e_off + r0 + r] = sc;
+  const int er = sc == oz::kNonFinite ? 4096 : sc;  // (non-finite: every digit 0)
+  const int2 o = org[r];
   __half* dst0 = out + b.a_off;
-  for (int k8 = (threadIdx.x / 8) * 8; k8 < b.nkb * oz::KB; k8 += 256) {
+  for (int k8 = (threadIdx.x / R) * 8; k8 < b.nkb * oz::KB; k8 += WIN_THREADS / R * 8) {
     unsigned long long N[8];
-    int a = k8 / wx, c = k8 - a * wx;
+    int a = div_by(k8, inv), c = k8 - a * wx;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const double v = k8 + u < wn ? src[node(td[r], a, c)] : 0.0;
+      const double v = k8 + u < wn ? at(o, a, c) : 0.0;
       N[u] = oz::biased_digits(static_cast<unsigned long long>(__double_as_longlong(v)), er);
       if (++c >= wx) {
         c = 0;
@@ -222,29 +238,42 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_kernel(const __grid_co
   const int lcw = 6 - (31 - __clz(ks)), cw = 1 << lcw, c0 = rank * cw;  // this CTA's columns
   if (!s_abort && c0 < un.ncol) {
     const int ix = s_ix;
-    // i / ix for i < 2^14 by one multiply (exact: i ix < 2^28)
-    const uint32_t inv = ix > 1 ? 0xFFFFFFFFu / uint32_t(ix) + 1u : 0u;
-#pragma unroll 4
-    for (int q = threadIdx.x; q < wb.count * cw; q += oz::THREADS) {
-      const int col = c0 + (q & (cw - 1)), row = q >> lcw;
-      if (col >= un.ncol) continue;
-      longlong2 v = make_longlong2(0, 0);
-      if (ks == 1) {
-        v = sums[col * oz::SUM_PITCH + row];
-      } else {
-        for (int j = 0; j < ks; ++j) {
-          const longlong2 o = *cl.map_shared_rank(sums + col * oz::SUM_PITCH + row, j);
-          v.x += o.x;
-          v.y += o.y;
+    const uint32_t inv = div_inv(uint32_t(ix));
+    constexpr int U = 8;  // elements per thread in flight (the state is read before any is written)
+    const int total = wb.count * cw;
+    for (int q0 = threadIdx.x; q0 < total; q0 += U * oz::THREADS) {
+      int64_t node[U];
+      double old[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        const int q = q0 + k * oz::THREADS, col = c0 + (q & (cw - 1)), row = q >> lcw;
+        node[k] = -1;
+        if (q < total && col < un.ncol) {
+          const int i = un.col0 + col, iy = div_by(i, inv);
+          node[k] = s_node[row] + int64_t(iy) * p.nx + (i - iy * ix);
         }
+        old[k] = p.accumulate && node[k] >= 0 ? p.u[node[k]] : 0.0;
       }
-      const int er = s_e[row], fc = s_f[col], i = un.col0 + col;
-      const double y = er == oz::kNonFinite || fc == oz::kNonFinite
-                           ? plain_dot(p, p.tiles[p.order[wb.first + row]], i)
-                           : oz::sums_to_double(v.x, v.y, er + fc - 62);
-      const int iy = ix > 1 ? int(__umulhi(uint32_t(i), inv)) : i;
-      const int64_t node = s_node[row] + int64_t(iy) * p.nx + (i - iy * ix);
-      p.u[node] = p.accumulate ? p.u[node] + y : y;
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        if (node[k] < 0) continue;
+        const int q = q0 + k * oz::THREADS, col = c0 + (q & (cw - 1)), row = q >> lcw;
+        longlong2 v = make_longlong2(0, 0);
+        if (ks == 1) {
+          v = sums[col * oz::SUM_PITCH + row];
+        } else {
+          for (int j = 0; j < ks; ++j) {
+            const longlong2 o = *cl.map_shared_rank(sums + col * oz::SUM_PITCH + row, j);
+            v.x += o.x;
+            v.y += o.y;
+          }
+        }
+        const int er = s_e[row], fc = s_f[col];
+        const double y = er == oz::kNonFinite || fc == oz::kNonFinite
+                             ? plain_dot(p, p.tiles[p.order[wb.first + row]], un.col0 + col)
+                             : oz::sums_to_double(v.x, v.y, er + fc - 62);
+        p.u[node[k]] = p.accumulate ? old[k] + y : y;
+      }
     }
   }
   if (ks > 1) cl.sync();  // the sums stay until every CTA of the cluster has read them
@@ -439,8 +468,10 @@ lem_status step_oz(lem_ctx* ctx, double* d_u) {
   cudaEvent_t stop;
   LEM_CUDA_TRY(ctx->timing_begin(&stop));
   for (const OzPlan::Group& g : z->groups) {
-    oz_windows_kernel<<<unsigned(g.nwb) * 16, 256, 0, st>>>(src, ctx->d_tiles, ctx->d_class_order, z->d_blocks, g.wb0,
-                                                            ctx->ny, ctx->nx, z->d_e, z->d_a);
+    auto cut = g.nwb >= 24 ? oz_windows_kernel<8> : g.nwb >= 12 ? oz_windows_kernel<4> : oz_windows_kernel<2>;
+    const int per = g.nwb >= 24 ? 16 : g.nwb >= 12 ? 32 : 64;
+    cut<<<unsigned(g.nwb * per), WIN_THREADS, 0, st>>>(src, ctx->d_tiles, ctx->d_class_order, z->d_blocks, g.wb0,
+                                                       int(ctx->ny), int(ctx->nx), z->d_e, z->d_a);
     LEM_CUDA_TRY(cudaGetLastError());
     StepParams p{z->d_blocks, z->d_units, ctx->d_tiles, ctx->d_class_order, z->d_a, z->d_b, z->d_e, z->d_f, ctx->d_P,
                  src, d_u, ctx->n_int, ctx->n_loc, ctx->ny, ctx->nx, g.unit0, g.ks, phi ? 1 : 0, z->d_err};
