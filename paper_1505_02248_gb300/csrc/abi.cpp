@@ -281,7 +281,7 @@ lem_status lem_create(const lem_problem_desc* desc, int device, void* cuda_strea
   } else {
     c->apply_path = many_classes ? LEM_APPLY_FP64_GEMV : LEM_APPLY_FP64_GEMM;
   }
-  if (c->apply_path == LEM_APPLY_FP64_GEMM) {
+  if (c->apply_path == LEM_APPLY_FP64_GEMM && c->n_loc <= 8000) {  // (oz::kMaxK)
     s = oz_prepare(c);
     if (s == LEM_ENOMEM) {  // no room for the digits: the FP64 GEMM needs fewer bytes
       oz_destroy(c);

@@ -1,8 +1,8 @@
 // Local propagator builder (Sec. 3 step 2; Pade approximation with scaling and squaring
-// as named in Sec. 1 and Sec. 4), batched over propagator classes, in FP64. For the
-// split-precision tiers the matrix products run on the tensor cores as exact sums of FP16
-// slice products (builder_tc.cu, about 2^-45 relative to the operands' scale); the Pade
-// denominator solve stays in FP64 either way.
+// as named in Sec. 1 and Sec. 4), batched over propagator classes, in FP64. The matrix
+// products of the split-precision tiers run on the tensor cores as sums of digit products
+// (builder_tc.cu, about 2^-45 relative to the operands' scale), those of the FP64 tier on the FP64
+// pipe; the pivots of the Pade denominator solve are FP64 either way.
 //
 // For each class the local matrix X = dt A_M (principal submatrix on the window, i.e.
 // Dirichlet data at the artificial boundary; plus dt diag(1 - 3u^2) with the reaction, or
@@ -22,6 +22,7 @@
 #include <string>
 #include <vector>
 
+#include <cooperative_groups.h>
 #include <nvtx3/nvToolsExt.h>
 
 #include "dgemm.cuh"
@@ -46,7 +47,7 @@ struct BatchClass {
 };
 
 // ---------------------------------------------------------------- assembly
-// nonlin 1: + dt diag(1 - 3u^2); nonlin 2 (porous medium): X diag(phi'(u)) with
+// X is zero on entry. nonlin 1: + dt diag(1 - 3u^2); nonlin 2 (porous medium): X diag(phi'(u)) with
 // phi'(u) = m |u|^(m-1), each entry scaled by phi' at its column's node.
 __global__ void assemble_local_kernel(double* X, int n, const BatchClass* bc, int nb,
                                       const double* coef, int64_t cstride, int64_t ny,
@@ -56,7 +57,6 @@ __global__ void assemble_local_kernel(double* X, int n, const BatchClass* bc, in
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nb || k >= n) return;
   double* row = X + (int64_t(b) * n + k) * n;
-  for (int j = 0; j < n; ++j) row[j] = 0.0;
   const BatchClass c = bc[b];
   const int wy = c.rep.wext[0], wx = c.rep.wext[1];
   if (k >= wy * wx) return;  // padding row
@@ -70,7 +70,7 @@ __global__ void assemble_local_kernel(double* X, int n, const BatchClass* bc, in
   auto cf = [&](int which) { return coef[which * (cstride ? npts : 1) + (cstride ? p : 0)]; };
   const bool porous = u && nonlin == 2;
   // phi'(u) at global node q (1 unless porous)
-  auto dphi = [&](int64_t q) { return porous ? pm * pow(fabs(u[q]), pm - 1.0) : 1.0; };
+  auto dphi = [&](int64_t q) { return porous ? pm * abs_pow(u[q], pm - 1.0) : 1.0; };
   // the four neighbours' global nodes (wrapped; a window never holds a node beyond a wall)
   const int64_t qw = gy * nx + (gx + nx - 1) % nx, qe = gy * nx + (gx + 1) % nx;
   const int64_t qs = ((gy + ny - 1) % ny) * nx + gx, qn = ((gy + 1) % ny) * nx + gx;
@@ -101,7 +101,6 @@ __global__ void assemble_local_complex_kernel(double* X, int n, const BatchClass
   if (b >= nb || k >= h) return;
   double* rr = X + (int64_t(b) * n + k) * n;
   double* ri = X + (int64_t(b) * n + h + k) * n;
-  for (int j = 0; j < n; ++j) rr[j] = ri[j] = 0.0;
   const BatchClass c = bc[b];
   const int wy = c.rep.wext[0], wx = c.rep.wext[1];
   if (k >= wy * wx) return;  // padding node
@@ -133,15 +132,83 @@ __global__ void assemble_local_complex_kernel(double* X, int n, const BatchClass
   }
 }
 
-// column 1-norms -> per-matrix max (non-negative doubles order like their bit patterns)
-__global__ void norm1_kernel(const double* X, int n, unsigned long long* out) {
+// column 1-norms -> per-matrix max (non-negative doubles order like their bit patterns); a block
+// takes 32 columns, 8 threads a column
+__global__ void __launch_bounds__(256) norm1_kernel(const double* X, int n, unsigned long long* out) {
   const int b = blockIdx.y;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
+  const int c = threadIdx.x % 32, g = threadIdx.x / 32, j = blockIdx.x * 32 + c;
+  __shared__ double part[8][32];
   const double* M = X + int64_t(b) * n * n;
   double s = 0.0;
-  for (int i = 0; i < n; ++i) s += fabs(M[int64_t(i) * n + j]);
-  atomicMax(out + b, (unsigned long long)__double_as_longlong(s));
+  if (j < n) {
+#pragma unroll 8
+    for (int i = g; i < n; i += 8) s += fabs(M[int64_t(i) * n + j]);
+  }
+  part[g][c] = s;
+  __syncthreads();
+  if (g == 0 && j < n) {
+    for (int q = 1; q < 8; ++q) s += part[q][c];
+    atomicMax(out + b, (unsigned long long)__double_as_longlong(s));
+  }
+}
+
+// X <- X c and B2 <- X c^2 (c = 2^-s per matrix; B2 null: not wanted)
+__global__ void scale_kernel(double* X, double* B2, int64_t nn, const double* c) {
+  const int b = blockIdx.y;
+  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (e >= nn) return;
+  const double v = X[b * nn + e] * c[b];
+  X[b * nn + e] = v;
+  if (B2) B2[b * nn + e] = v * c[b];
+}
+
+// The linear combinations of the Pade-13 evaluation in one pass over the powers:
+//   W = b13 Z6 + b11 Z4 + b9 Z2,  A3 = b7 Z6 + b5 Z4 + b3 Z2 (+ b1 I),
+//   V = b12 Z6 + b10 Z4 + b8 Z2,  VT = b6 Z6 + b4 Z4 + b2 Z2 (+ b0 I);
+// blockIdx.z 0: the T blocks (diagonal terms), 1: the B blocks (V's is not needed: it cancels in
+// the solve's right-hand side). Bound by the FP64 pipe (12
+// multiply-adds per element); one pass per combination read the powers four times over.
+struct PadeTerms {
+  const double* z2[2];
+  const double* z4[2];
+  const double* z6[2];
+  double* w[2];
+  double* a3[2];
+  double* v[1];
+  double* vt[1];
+  double b[14];
+};
+__global__ void pade_terms_kernel(const __grid_constant__ PadeTerms p, int n, int64_t total) {
+  const int h = blockIdx.z;
+  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (e >= total) return;
+  const double z2 = p.z2[h][e], z4 = p.z4[h][e], z6 = p.z6[h][e];
+  const int64_t nn = int64_t(n) * n;
+  const unsigned in = unsigned(e % nn);
+  const bool dg = h == 0 && in / unsigned(n) == in % unsigned(n);
+  p.w[h][e] = fma(p.b[9], z2, fma(p.b[11], z4, p.b[13] * z6));
+  double a = fma(p.b[3], z2, fma(p.b[5], z4, p.b[7] * z6));
+  if (dg) a += p.b[1];
+  p.a3[h][e] = a;
+  if (h) return;
+  p.v[0][e] = fma(p.b[8], z2, fma(p.b[10], z4, p.b[12] * z6));
+  double t = fma(p.b[2], z2, fma(p.b[4], z4, p.b[6] * z6));
+  if (dg) t += p.b[0];
+  p.vt[0][e] = t;
+}
+
+// G = [V_T - U_T | V_T + U_T | 2 U_B] (UB null: no third block)
+__global__ void solve_system_kernel(double* G, int n, int gjcols, const double* VT, const double* UT,
+                                    const double* UB) {
+  const int b = blockIdx.y;
+  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x, nn = int64_t(n) * n;
+  if (e >= nn) return;
+  const int i = int(e / n), j = int(e % n);
+  const double v = VT[b * nn + e], u = UT[b * nn + e];
+  double* row = G + (int64_t(b) * n + i) * gjcols + j;
+  row[0] = v - u;
+  row[n] = v + u;
+  if (UB) row[2 * n] = 2.0 * UB[b * nn + e];
 }
 
 // out[b] = sum_t w_t in_t[b] + diag * dscale[b] * I   (dscale may be null: 1)
@@ -170,85 +237,40 @@ __global__ void lincomb_kernel(double* out, int n, int64_t ld, int ncols, Lin L)
   out[off] = v;
 }
 
-// Gauss-Jordan elimination with partial pivoting on G = [Q | RHS] (n x (n + m), row-major).
-// Step k: pick the largest |G[i][k]|, i >= k; swap rows; normalise row k by the pivot.
-__global__ void gj_pivot_kernel(double* G, int n, int ncols, int k, int* status) {
-  const int b = blockIdx.x;
-  double* M = G + int64_t(b) * n * ncols;
-  __shared__ double sv[256];
-  __shared__ int si[256];
-  double best = -1.0;
-  int bi = k;
-  for (int i = k + threadIdx.x; i < n; i += blockDim.x) {
-    double v = fabs(M[int64_t(i) * ncols + k]);
-    if (v > best) { best = v; bi = i; }
-  }
-  sv[threadIdx.x] = best;
-  si[threadIdx.x] = bi;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      double o = sv[threadIdx.x + s];
-      int oi = si[threadIdx.x + s];
-      if (o > sv[threadIdx.x] || (o == sv[threadIdx.x] && oi < si[threadIdx.x])) {
-        sv[threadIdx.x] = o;
-        si[threadIdx.x] = oi;
-      }
-    }
-    __syncthreads();
-  }
-  const int p = si[0];
-  const double pv = M[int64_t(p) * ncols + k];
-  __syncthreads();  // every thread holds pv before row k / row p are rewritten
-  if (!(sv[0] > 0.0) || !isfinite(pv)) {
-    if (threadIdx.x == 0) atomicExch(status, int(LEM_ENUMERIC));
-    return;
-  }
-  for (int j = threadIdx.x; j < ncols; j += blockDim.x) {
-    double a = M[int64_t(k) * ncols + j];
-    double c = M[int64_t(p) * ncols + j];
-    if (p != k) M[int64_t(p) * ncols + j] = a;
-    M[int64_t(k) * ncols + j] = c / pv;
-  }
-}
-
-// eliminate column k from every row i != k:  G[i][j] -= G[i][k] * G[k][j], j > k
-__global__ void gj_update_kernel(double* G, int n, int ncols, int k) {
-  const int b = blockIdx.z;
-  double* M = G + int64_t(b) * n * ncols;
-  const int i = blockIdx.y;
-  if (i == k) return;
-  const double f = M[int64_t(i) * ncols + k];
-  if (f == 0.0) return;
-  for (int j = k + 1 + blockIdx.x * blockDim.x + threadIdx.x; j < ncols; j += gridDim.x * blockDim.x)
-    M[int64_t(i) * ncols + j] = fma(-f, M[int64_t(k) * ncols + j], M[int64_t(i) * ncols + j]);
-}
-
 // ---------------------------------------------------------------- blocked Gauss-Jordan
-// For the tensor-core build the elimination runs in panels of GJ_KB columns. The panel's
-// GJ_KB pivot steps (partial pivoting, FP64) are applied to the panel columns and to a tracker
+// Gauss-Jordan elimination with partial pivoting on G = [Q | RHS] (n x gjcols, row-major), in panels
+// of GJ_KB columns. The panel's GJ_KB pivot steps (partial pivoting, FP64) are applied to the panel columns and to a tracker
 // Y (n x GJ_KB): at step c, right after the row swap, Y[k0 + c][c] = 1 is injected, and every
 // later swap, scaling and elimination acts on Y too. At the end of the panel the composite row
 // operation is M = T Pi with T = I + W E_K^T (Pi: the panel's swaps, K: rows k0 .. k0 + kb),
-// and Y = T[:, K], so the trailing columns become
+// and Y = T[:, K], so any other column becomes
 //   rows K:      Y_K (Pi G)[K, :]
 //   other rows:  (Pi G)[i, :] + Y_i (Pi G)[K, :],
-// one rank-kb product C = Y B + D with B the permuted pivot rows and D the permuted trailing
-// columns with rows K taken as zero. The FP64 work drops from n^2 gjcols to about 2 n^2 GJ_KB.
-constexpr int GJ_KB = 64;
+// one rank-kb product C = Y B + D with B the permuted pivot rows and D the permuted columns with
+// rows K taken as zero, on the tensor cores or (FP64 tier) as an FP64 product; one pivot at a time
+// every pivot read and wrote all of G.
+//
+// With the tensor cores, panels may be gathered GJ_SB columns at a time: a panel's product is applied to the other columns
+// of its group only (to those still to be eliminated and, being the tracker of the group's earlier
+// panels, to those already eliminated), after which the group's n x GJ_SB block is the tracker of
+// all its pivots, and one rank-GJ_SB product updates the columns behind the group. A tile of a
+// rank-64 product costs little less than one of a rank-256 product (its sums are converted and
+// written all the same): one product per panel took 11 ms of a build of 25 matrices of 784.
+constexpr int GJ_KB = 64, GJ_SB = 256;
 
-__global__ void bgj_pivot_kernel(double* G, int n, int ld, int k0, int c, int kb, double* Y, int* piv,
-                                 int* status) {
+// One pivot step of a panel at columns k0 - s0 .. of the group block Y (n x GJ_SB, its first column
+// standing for matrix column s0), for matrices too large for bgj_panel_kernel. In place: the
+// pivot column becomes the tracker column.
+__global__ void bgj_pivot_kernel(double* Y, int n, int c0, int k0, int c, int kb, int* piv, int* status) {
   const int b = blockIdx.x;
-  double* M = G + int64_t(b) * n * ld;
-  double* Yb = Y + int64_t(b) * n * GJ_KB;
-  const int col = k0 + c, r = k0 + c;
+  double* M = Y + int64_t(b) * n * GJ_SB + c0;
+  const int r = k0 + c;
   __shared__ double sv[256];
   __shared__ int si[256];
   double best = -1.0;
   int bi = r;
   for (int i = r + threadIdx.x; i < n; i += blockDim.x) {
-    const double v = fabs(M[int64_t(i) * ld + col]);
+    const double v = fabs(M[int64_t(i) * GJ_SB + c]);
     if (v > best) { best = v; bi = i; }
   }
   sv[threadIdx.x] = best;
@@ -266,61 +288,266 @@ __global__ void bgj_pivot_kernel(double* G, int n, int ld, int k0, int c, int kb
     __syncthreads();
   }
   const int p = si[0];
-  const double pv = M[int64_t(p) * ld + col];
+  const double pv = M[int64_t(p) * GJ_SB + c];
   __syncthreads();  // every thread holds pv before rows r / p are rewritten
   if (!(sv[0] > 0.0) || !isfinite(pv)) {
-    if (threadIdx.x == 0) atomicExch(status, int(LEM_ENUMERIC));
+    if (threadIdx.x == 0) {
+      atomicExch(status, int(LEM_ENUMERIC));
+      piv[b * GJ_SB + c0 + c] = r;  // no swap
+    }
     return;
   }
-  if (threadIdx.x == 0) piv[b * GJ_KB + c] = p;
+  if (threadIdx.x == 0) piv[b * GJ_SB + c0 + c] = p;
   const double inv = 1.0 / pv;
-  // panel columns col .. k0 + kb - 1 of rows r and p, then the tracker rows
-  for (int j = col + threadIdx.x; j < k0 + kb; j += blockDim.x) {
-    const double a = M[int64_t(r) * ld + j], q = M[int64_t(p) * ld + j];
-    if (p != r) M[int64_t(p) * ld + j] = a;
-    M[int64_t(r) * ld + j] = q * inv;
-  }
   for (int j = threadIdx.x; j < kb; j += blockDim.x) {
-    const double a = Yb[int64_t(r) * GJ_KB + j], q = Yb[int64_t(p) * GJ_KB + j];
-    if (p != r) Yb[int64_t(p) * GJ_KB + j] = a;
-    Yb[int64_t(r) * GJ_KB + j] = (j == c ? 1.0 : q) * inv;  // inject the unit column, then scale
+    const double a = M[int64_t(r) * GJ_SB + j], q = M[int64_t(p) * GJ_SB + j];
+    if (p != r) M[int64_t(p) * GJ_SB + j] = a;
+    M[int64_t(r) * GJ_SB + j] = (j == c ? 1.0 : q) * inv;  // inject the unit column, then scale
   }
 }
 
-// Eliminate panel column k0 + c from every row but the pivot row: 4 rows per block, thread t
-// of a row updates panel column k0 + c + 1 + t and tracker column t.
-__global__ void bgj_elim_kernel(double* G, int n, int ld, int k0, int c, int kb, double* Y) {
+// Eliminate panel column c from every row but the pivot row: 4 rows per block, thread t of a row
+// updates panel column t.
+__global__ void bgj_elim_kernel(double* Y, int n, int c0, int k0, int c, int kb) {
   const int b = blockIdx.y;
   const int i = blockIdx.x * 4 + threadIdx.x / 64, t = threadIdx.x % 64;
-  const int r = k0 + c, col = k0 + c;
-  if (i >= n || i == r) return;
-  double* M = G + int64_t(b) * n * ld;
-  double* Yb = Y + int64_t(b) * n * GJ_KB;
-  const double f = M[int64_t(i) * ld + col];
-  if (f == 0.0) return;
-  const int j = col + 1 + t;
-  if (j < k0 + kb) M[int64_t(i) * ld + j] = fma(-f, M[int64_t(r) * ld + j], M[int64_t(i) * ld + j]);
-  if (t < kb) Yb[int64_t(i) * GJ_KB + t] = fma(-f, Yb[int64_t(r) * GJ_KB + t], Yb[int64_t(i) * GJ_KB + t]);
+  const int r = k0 + c;
+  double* M = Y + int64_t(b) * n * GJ_SB + c0;
+  const bool live = i < n && i != r;
+  const double f = live ? M[int64_t(i) * GJ_SB + c] : 0.0;
+  __syncthreads();  // column c is read before it is overwritten
+  if (!live || f == 0.0 || t >= kb) return;
+  double* m = M + int64_t(i) * GJ_SB + t;
+  *m = fma(-f, M[int64_t(r) * GJ_SB + t], t == c ? 0.0 : *m);
 }
 
-// The panel's row swaps, in order, on the trailing columns j >= k0 + kb.
-__global__ void bgj_swap_kernel(double* G, int n, int ld, int k0, int kb, const int* piv) {
-  const int b = blockIdx.y;
-  const int j = k0 + kb + blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= ld) return;
-  double* M = G + int64_t(b) * n * ld;
+// A whole panel in one launch, a cluster of CTAs per matrix, each holding a share of the panel's
+// rows in shared memory. The panel's columns are overwritten by the tracker as they are
+// eliminated (a pivot column is no longer needed once its tracker column begins), so each pivot
+// step is one update of the share: M[i][j] -= M[i][c] M[r][j], with column c taken as zero before
+// it. Per step every CTA writes its best pivot candidate with that candidate's row (and the holder
+// of row r that row) into every other's shared memory, one cluster barrier follows, and every CTA
+// picks the same winner from its own copy. Bound by the chain of a step (reduction, barrier,
+// reciprocal) and by the FP64 pipe for the update, 2 multiply-adds per clock and SM. Two launches
+// per pivot column (kept for matrices beyond PANEL_MAX_N) cost 17 us on 25 matrices of 784 nodes.
+// Updating the next pivot's column first, to search it during the update, gained nothing.
+constexpr int PANEL_THREADS = 256, PANEL_PITCH = GJ_KB + 1, PANEL_MAX_CLUSTER = 8, PANEL_MAX_ROWS = 360;
+constexpr int PANEL_MAX_N = PANEL_MAX_CLUSTER * PANEL_MAX_ROWS;
+
+struct PanelPub {
+  double cand[GJ_KB];  // the candidate's row
+  long long val;       // its magnitude (the bits)
+  int idx;
+  int pad;
+};
+struct PanelStep {
+  PanelPub from[PANEL_MAX_CLUSTER];
+  double rrow[GJ_KB];  // row r
+};
+
+// src: the panel's columns (leading dimension lds, matrices ss apart); Y: where the tracker goes
+// (column c0 of the group block; may be src).
+__global__ void __launch_bounds__(PANEL_THREADS) bgj_panel_kernel(const double* src, int64_t lds, int64_t ss, int n,
+                                                                  int c0, int k0, int kb, int csize, int rows_per,
+                                                                  double* Y, int* piv, int* status) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) double psm[];
+  PanelStep* steps = reinterpret_cast<PanelStep*>(psm);  // [2], by the step's parity
+  double* prow = psm + 2 * sizeof(PanelStep) / sizeof(double);  // [GJ_KB] the scaled pivot row
+  double* M = prow + GJ_KB;                           // [rows_per][PANEL_PITCH]
+  double* fcol = M + size_t(rows_per) * PANEL_PITCH;  // [rows_per] column c before the step
+  int* fzero = reinterpret_cast<int*>(fcol + rows_per);  // [rows_per] whether it is zero there (kept as it is:
+                                                         // an FP64 comparison costs as much as the update)
+  __shared__ long long wv[PANEL_THREADS / 32];
+  __shared__ int wi[PANEL_THREADS / 32];
+  const int b = blockIdx.x / csize, rank = blockIdx.x % csize;
+  const int lo = rank * rows_per, cnt = max(0, min(rows_per, n - lo));
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  const double* Sb = src + int64_t(b) * ss;
+  for (int e = tid; e < cnt * GJ_KB; e += PANEL_THREADS) {
+    const int i = e / GJ_KB, j = e % GJ_KB;
+    if (j < kb) M[i * PANEL_PITCH + j] = Sb[int64_t(lo + i) * lds + j];
+  }
+  cl.sync();  // every CTA of the cluster runs before its memory is written
+  const int j = tid % GJ_KB, grp = tid / GJ_KB;
   for (int c = 0; c < kb; ++c) {
-    const int p = piv[b * GJ_KB + c];
-    if (p == k0 + c) continue;
-    const double a = M[int64_t(k0 + c) * ld + j];
-    M[int64_t(k0 + c) * ld + j] = M[int64_t(p) * ld + j];
-    M[int64_t(p) * ld + j] = a;
+    const int r = k0 + c;
+    PanelStep& st = steps[c & 1];
+    // this CTA's largest |M[i][c]|, i >= r (the smallest row of equals); magnitudes compare as
+    // integers, a NaN never wins
+    long long best = -1;
+    int bi = n;
+    for (int i = tid; i < cnt; i += PANEL_THREADS) {
+      const double v = M[i * PANEL_PITCH + c];
+      fcol[i] = v;
+      const long long m = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll;
+      fzero[i] = m == 0;
+      if (lo + i >= r && m > best && m <= 0x7FF0000000000000ll) {
+        best = m;
+        bi = lo + i;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ov > best || (ov == best && oi < bi)) {
+        best = ov;
+        bi = oi;
+      }
+    }
+    if (lane == 0) {
+      wv[warp] = best;
+      wi[warp] = bi;
+    }
+    __syncthreads();
+    best = wv[0];
+    bi = wi[0];
+    const int nw = min(PANEL_THREADS / 32, (cnt + 31) / 32);  // warps that hold rows
+    for (int w = 1; w < nw; ++w)
+      if (wv[w] > best || (wv[w] == best && wi[w] < bi)) {
+        best = wv[w];
+        bi = wi[w];
+      }
+    if (tid < kb) {
+      if (bi < n) {
+        const double v = M[(bi - lo) * PANEL_PITCH + tid];
+        for (int q = 0; q < csize; ++q) cl.map_shared_rank(&st, q)->from[rank].cand[tid] = v;
+      }
+    } else if (tid >= 64 && tid < 64 + kb) {
+      if (r >= lo && r < lo + cnt) {
+        const double v = M[(r - lo) * PANEL_PITCH + tid - 64];
+        for (int q = 0; q < csize; ++q) cl.map_shared_rank(&st, q)->rrow[tid - 64] = v;
+      }
+    } else if (tid >= 128 && tid < 128 + csize) {
+      PanelPub* o = &cl.map_shared_rank(&st, tid - 128)->from[rank];
+      o->val = best;
+      o->idx = bi;
+    }
+    cl.sync();
+    int win = 0, p = n;
+    long long pval = -2;
+    for (int q = 0; q < csize; ++q) {
+      const long long v = st.from[q].val;
+      const int oi = st.from[q].idx;
+      if (v > pval || (v == pval && oi < p)) {
+        pval = v;
+        p = oi;
+        win = q;
+      }
+    }
+    if (pval <= 0 || pval >= 0x7FF0000000000000ll) {  // zero or non-finite pivot (the same in every CTA)
+      if (rank == 0) {
+        if (tid == 0) atomicExch(status, int(LEM_ENUMERIC));
+        for (int q = c + tid; q < kb; q += PANEL_THREADS) piv[b * GJ_SB + c0 + q] = k0 + q;  // no more swaps
+      }
+      break;
+    }
+    if (tid < kb) {
+      const double inv = 1.0 / st.from[win].cand[c];
+      prow[tid] = tid == c ? inv : st.from[win].cand[tid] * inv;
+    } else if (tid >= 64 && tid < 64 + kb && p != r && p >= lo && p < lo + cnt) {
+      const int q = tid - 64;
+      const double old = st.rrow[q];
+      M[(p - lo) * PANEL_PITCH + q] = old;
+      if (q == c) {
+        fcol[p - lo] = old;
+        fzero[p - lo] = (__double_as_longlong(old) & 0x7FFFFFFFFFFFFFFFll) == 0;
+      }
+    }
+    if (rank == 0 && tid == 128) piv[b * GJ_SB + c0 + c] = p;
+    __syncthreads();
+    if (j < kb) {
+      const double pj = prow[j];
+      constexpr int U = 4, ST = PANEL_THREADS / GJ_KB;  // rows in flight, row step
+      auto upd = [&](double f, int zero, double m, int i) {
+        const double v = fma(-f, pj, j == c ? 0.0 : m);
+        return lo + i == r ? pj : zero ? m : v;
+      };
+      int i = grp;
+      for (; i + (U - 1) * ST < cnt; i += U * ST) {
+        double f[U], m[U];
+        int z[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          f[u] = fcol[i + u * ST];
+          z[u] = fzero[i + u * ST];
+          m[u] = M[(i + u * ST) * PANEL_PITCH + j];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) m[u] = upd(f[u], z[u], m[u], i + u * ST);
+#pragma unroll
+        for (int u = 0; u < U; ++u) M[(i + u * ST) * PANEL_PITCH + j] = m[u];
+      }
+#pragma unroll 1
+      for (; i < cnt; i += ST) M[i * PANEL_PITCH + j] = upd(fcol[i], fzero[i], M[i * PANEL_PITCH + j], i);
+    }
+    __syncthreads();
+  }
+  cl.sync();  // no CTA leaves while another may write into its memory
+  double* Yb = Y + int64_t(b) * n * GJ_SB + c0;
+  for (int e = tid; e < cnt * GJ_KB; e += PANEL_THREADS) {
+    const int i = e / GJ_KB, q = e % GJ_KB;
+    if (q < kb) Yb[int64_t(lo + i) * GJ_SB + q] = M[i * PANEL_PITCH + q];
   }
 }
 
-// rows of the owner tile D inside the window, from the squared result R (n x ld, col0)
-__global__ void extract_rows_kernel(double* P, int64_t n_int, int64_t n_loc, const double* R,
-                                    int n, int64_t ld, int col0, const BatchClass* bc) {
+static cudaError_t launch_panel(const double* src, int64_t lds, int64_t ss, int n, int c0, int k0, int kb, double* Y,
+                                int* piv, int* status, int nb, cudaStream_t st) {
+  // 8 rows a CTA at least: panels of 64 rows took 167, 134 and 122 us on 2, 4 and 8 CTAs
+  const int csize = std::min(PANEL_MAX_CLUSTER, (n + 7) / 8);
+  const int rows_per = (n + csize - 1) / csize;
+  const size_t smem = 2 * sizeof(PanelStep) + sizeof(double) * (size_t(rows_per) * (PANEL_PITCH + 2) + GJ_KB);
+  cudaError_t e = cudaFuncSetAttribute(bgj_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(nb) * csize);
+  cfg.blockDim = dim3(PANEL_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = unsigned(csize);
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, bgj_panel_kernel, src, lds, ss, n, c0, k0, kb, csize, rows_per, Y, piv, status);
+}
+
+// Row swaps k0 + c <-> piv[c], c < kb, in order, on columns [0, cols) of a matrix but [x0, x1).
+// rows (not null): the pivot rows k0 .. k0 + kb - 1 then move there (kb x cols), leaving zeros.
+__global__ void bgj_swap_kernel(double* M, int64_t ld, int64_t stride, int cols, int x0, int x1, int k0, int kb,
+                                const int* piv, double* rows) {
+  const int b = blockIdx.y;
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= cols || (j >= x0 && j < x1)) return;
+  double* m = M + int64_t(b) * stride + j;
+  for (int c = 0; c < kb; ++c) {
+    const int p = piv[b * GJ_SB + c];
+    if (p == k0 + c) continue;
+    const double a = m[int64_t(k0 + c) * ld];
+    m[int64_t(k0 + c) * ld] = m[int64_t(p) * ld];
+    m[int64_t(p) * ld] = a;
+  }
+  if (!rows) return;
+  double* r = rows + int64_t(b) * kb * cols + j;
+  for (int c = 0; c < kb; c += 16) {  // sixteen loads in flight
+    double v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v[u] = c + u < kb ? m[int64_t(k0 + c + u) * ld] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (c + u < kb) {
+        r[int64_t(c + u) * cols] = v[u];
+        m[int64_t(k0 + c + u) * ld] = 0.0;
+      }
+  }
+}
+
+// rows of the owner tile D inside the window, from the squared result (n x n): R, or R1 for the
+// matrices that `odd` marks (they stopped squaring an odd number of steps early)
+__global__ void extract_rows_kernel(double* P, int64_t n_int, int64_t n_loc, const double* R0, const double* R1,
+                                    const int* odd, int n, const BatchClass* bc) {
   const int b = blockIdx.y;
   const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= n_int * n_loc) return;
@@ -331,7 +558,7 @@ __global__ void extract_rows_kernel(double* P, int64_t n_int, int64_t n_loc, con
   double v = 0.0;
   if (i < ie && k < wl && k < n) {
     const int row = (c.rep.iofs[0] + i / c.rep.iext[1]) * c.rep.wext[1] + c.rep.iofs[1] + i % c.rep.iext[1];
-    v = R[int64_t(b) * n * ld + int64_t(row) * ld + col0 + k];
+    v = (odd && odd[b] ? R1 : R0)[int64_t(b) * n * n + int64_t(row) * n + k];
   }
   P[int64_t(b) * n_int * n_loc + e] = v;
 }
@@ -339,8 +566,8 @@ __global__ void extract_rows_kernel(double* P, int64_t n_int, int64_t n_loc, con
 // Complex problems: owner rows of the embedded result R (n x n, n = 2 x window nodes) into P
 // (n_int x n_loc, both embedded sizes): rows [0, n_int/2) the real parts, [n_int/2, n_int) the
 // imaginary parts of the owner nodes; columns as in R (real parts, then imaginary parts).
-__global__ void extract_rows_complex_kernel(double* P, int64_t n_int, int64_t n_loc, const double* R, int n,
-                                            const BatchClass* bc) {
+__global__ void extract_rows_complex_kernel(double* P, int64_t n_int, int64_t n_loc, const double* R0,
+                                            const double* R1, const int* odd, int n, const BatchClass* bc) {
   const int b = blockIdx.y;
   const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= n_int * n_loc) return;
@@ -352,7 +579,7 @@ __global__ void extract_rows_complex_kernel(double* P, int64_t n_int, int64_t n_
   double v = 0.0;
   if (io < ie && k < n) {
     const int row = (c.rep.iofs[0] + io / c.rep.iext[1]) * c.rep.wext[1] + c.rep.iofs[1] + io % c.rep.iext[1];
-    v = R[int64_t(b) * n * n + int64_t(comp * hn + row) * n + k];
+    v = (odd && odd[b] ? R1 : R0)[int64_t(b) * n * n + int64_t(comp * hn + row) * n + k];
   }
   P[int64_t(b) * n_int * n_loc + e] = v;
 }
@@ -392,39 +619,76 @@ struct TcGuard {
 };
 }  // namespace
 
+// One A against a list of right factors, on the tensor cores (tcg not null) or in FP64.
+static lem_status mul_list(lem_ctx* ctx, TcGemm* tcg, int nbatch, const int* map, int M, int K, const double* A,
+                           int64_t lda, int64_t sA, const TcProduct* list, int np, int zr0, int zr1) {
+  if (tcg) return tc_gemm(tcg, nbatch, map, M, K, A, lda, sA, list, np, zr0, zr1, ctx->stream);
+  DgemmList g{};
+  g.M = M; g.K = K; g.np = np; g.A = A; g.lda = lda; g.sA = sA; g.map = map;
+  for (int t = 0; t < np; ++t) {
+    const TcProduct& p = list[t];
+    g.N[t] = p.N;
+    g.B[t] = p.B; g.ldb[t] = p.ldb; g.sB[t] = p.sB;
+    g.D[t] = p.D; g.ldd[t] = p.ldd; g.sD[t] = p.sD;
+    g.C[t] = p.C; g.ldc[t] = p.ldc; g.sC[t] = p.sC;
+    g.diag[t] = p.diag;
+  }
+  int nsm = 0;
+  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || nsm < 1) nsm = 152;
+  LEM_CUDA_TRY(dgemm_list(g, nbatch, nsm, ctx->stream));
+  return LEM_OK;
+}
+
 // Gauss-Jordan elimination of G = [Q | RHS] (nb matrices of n x gjcols): on exit the RHS
-// columns hold Q^{-1} RHS. With a tensor-core workspace the blocked form (FP64 panels,
-// rank-GJ_KB trailing products on tcgen05); otherwise one FP64 pivot step at a time.
-static lem_status solve_gj(lem_ctx* ctx, TcGemm* tcg, double* G, int n, int gjcols, int nb, Buf& ybuf, Buf& pivbuf) {
+// columns hold Q^{-1} RHS. Panels in FP64, the other columns by products (tcg: on tcgen05). The
+// split apply's propagators keep one product per panel: a group's product rounds otherwise, and
+// the FP16 pieces cut from the propagators would differ.
+static lem_status solve_gj(lem_ctx* ctx, TcGemm* tcg, double* G, int n, int gjcols, int nb, Buf& ybuf, Buf& pivbuf,
+                           Buf& rowbuf) {
   cudaStream_t st = ctx->stream;
-  if (tcg) {
-    LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&ybuf.p), sizeof(double) * nb * n * GJ_KB, st));
-    LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&pivbuf.p), sizeof(int) * nb * GJ_KB, st));
-    double* Y = ybuf.p;
-    int* piv = reinterpret_cast<int*>(pivbuf.p);
-    for (int k0 = 0; k0 < n; k0 += GJ_KB) {
-      const int kb = std::min(GJ_KB, n - k0);
-      LEM_CUDA_TRY(cudaMemsetAsync(Y, 0, sizeof(double) * nb * n * GJ_KB, st));
-      for (int c = 0; c < kb; ++c) {
-        bgj_pivot_kernel<<<nb, 256, 0, st>>>(G, n, gjcols, k0, c, kb, Y, piv, ctx->d_status);
-        bgj_elim_kernel<<<dim3((n + 3) / 4, nb), 256, 0, st>>>(G, n, gjcols, k0, c, kb, Y);
+  const int group = tcg && !ctx->split ? GJ_SB : GJ_KB;
+  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&ybuf.p), sizeof(double) * nb * n * GJ_SB, st));
+  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&pivbuf.p), sizeof(int) * nb * GJ_SB, st));
+  if (!tcg)  // FP64 products write over their right factor: the pivot rows move out first
+    LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&rowbuf.p), sizeof(double) * nb * GJ_KB * gjcols, st));
+  double* Y = ybuf.p;
+  int* piv = reinterpret_cast<int*>(pivbuf.p);
+  const int64_t sG = int64_t(n) * gjcols, sY = int64_t(n) * GJ_SB;
+  for (int s0 = 0; s0 < n; s0 += group) {  // a group of columns
+    const int sb = std::min(group, n - s0);
+    const bool one = sb <= GJ_KB && n <= PANEL_MAX_N;  // a single panel, read from G itself
+    if (!one) copy_cols_kernel<<<grid1(int64_t(n) * sb, nb), 256, 0, st>>>(Y, GJ_SB, 0, G, gjcols, s0, n, sb);
+    for (int c0 = 0; c0 < sb; c0 += GJ_KB) {
+      const int kb = std::min(GJ_KB, sb - c0), k0 = s0 + c0;
+      if (n <= PANEL_MAX_N) {
+        LEM_CUDA_TRY(one ? launch_panel(G + s0, gjcols, sG, n, c0, k0, kb, Y, piv, ctx->d_status, nb, st)
+                         : launch_panel(Y + c0, GJ_SB, sY, n, c0, k0, kb, Y, piv, ctx->d_status, nb, st));
+      } else {
+        for (int c = 0; c < kb; ++c) {
+          bgj_pivot_kernel<<<nb, 256, 0, st>>>(Y, n, c0, k0, c, kb, piv, ctx->d_status);
+          bgj_elim_kernel<<<dim3((n + 3) / 4, nb), 256, 0, st>>>(Y, n, c0, k0, c, kb);
+        }
       }
-      const int m_r = gjcols - (k0 + kb);
-      bgj_swap_kernel<<<dim3((m_r + 255) / 256, nb), 256, 0, st>>>(G, n, gjcols, k0, kb, piv);
+      if (kb == sb) continue;
+      // the group's other columns: C = Y_panel B + D with B the pivot rows, D without them
+      bgj_swap_kernel<<<dim3(1, nb), 256, 0, st>>>(Y, GJ_SB, sY, sb, c0, c0 + kb, k0, kb, piv + c0, nullptr);
       LEM_CUDA_TRY(cudaGetLastError());
-      double* T = G + (k0 + kb);  // trailing columns
-      const int64_t sG = int64_t(n) * gjcols;
-      LEM_TRY(tc_gemm_ex(tcg, nb, nullptr, n, m_r, kb, Y, GJ_KB, int64_t(n) * GJ_KB,  // A = Y
-                         T + int64_t(k0) * gjcols, gjcols, sG,                         // B = pivot rows
-                         T, gjcols, sG, k0, k0 + kb,                                   // D, rows K zero
-                         T, gjcols, sG, st));
+      TcProduct pr[2];
+      int np = 0;
+      for (int side = 0; side < 2; ++side) {
+        double* T = Y + (side ? c0 + kb : 0);
+        const int cols = side ? sb - c0 - kb : c0;
+        if (cols > 0) pr[np++] = TcProduct{cols, T + int64_t(k0) * GJ_SB, GJ_SB, sY, T, GJ_SB, sY, T, GJ_SB, sY, nullptr};
+      }
+      LEM_TRY(mul_list(ctx, tcg, nb, nullptr, n, kb, Y + c0, GJ_SB, sY, pr, np, k0, k0 + kb));
     }
-  } else {
-    for (int k = 0; k < n; ++k) {
-      gj_pivot_kernel<<<nb, 256, 0, st>>>(G, n, gjcols, k, ctx->d_status);
-      int bx = std::max(1, std::min(8, (gjcols - k - 1 + 255) / 256));
-      gj_update_kernel<<<dim3(bx, n, nb), 256, 0, st>>>(G, n, gjcols, k);
-    }
+    const int m_r = gjcols - (s0 + sb);
+    double* T = G + (s0 + sb);  // the columns behind the group
+    bgj_swap_kernel<<<dim3((m_r + 255) / 256, nb), 256, 0, st>>>(T, gjcols, sG, m_r, 0, 0, s0, sb, piv, rowbuf.p);
+    LEM_CUDA_TRY(cudaGetLastError());
+    const double* B = tcg ? T + int64_t(s0) * gjcols : rowbuf.p;
+    const TcProduct pr{m_r, B, tcg ? gjcols : m_r, tcg ? sG : int64_t(sb) * m_r, T, gjcols, sG, T, gjcols, sG, nullptr};
+    LEM_TRY(mul_list(ctx, tcg, nb, nullptr, n, sb, Y, GJ_SB, sY, &pr, 1, s0, s0 + sb));
   }
   LEM_CUDA_TRY(cudaGetLastError());
   return LEM_OK;
@@ -444,27 +708,27 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
     hbc[b].whole[1] = c.whole[1];
   }
   // device scratch for this batch (freed at return)
-  const int nmat = phi ? 16 : 9;
+  const int nmat = phi ? 15 : 9;
   const int gjcols = phi ? 3 * n : 2 * n;
-  Buf scratch, bcbuf, normbuf, scalebuf;
+  Buf scratch, bcbuf, normbuf, scalebuf, ybuf, pivbuf, rowbuf, mapbuf;
   size_t bytes = sizeof(double) * (size_t(nmat) * nn + size_t(n) * gjcols) * nb;
   LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&scratch.p), bytes, st));
   LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&bcbuf.p), sizeof(BatchClass) * nb, st));
   LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&normbuf.p), sizeof(double) * nb, st));
   LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&scalebuf.p), sizeof(double) * 2 * nb, st));
+  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&mapbuf.p), sizeof(int) * 2 * nb, st));
   BatchClass* d_bc = reinterpret_cast<BatchClass*>(bcbuf.p);
   LEM_CUDA_TRY(cudaMemcpyAsync(d_bc, hbc.data(), sizeof(BatchClass) * nb, cudaMemcpyHostToDevice, st));
   double* S = scratch.p;
   auto M = [&](int i) { return S + size_t(i) * nn * nb; };
-  double* Xs = M(0); double* T2 = M(1); double* T4 = M(2); double* T6 = M(3);
-  double* TW = M(4); double* T3 = M(5); double* UT = M(6); double* VT = M(7); double* RT2 = M(8);
-  double *B2 = nullptr, *B4 = nullptr, *B6 = nullptr, *BW = nullptr, *B3 = nullptr, *UB = nullptr,
-         *VB = nullptr;
-  if (phi) { B2 = M(9); B4 = M(10); B6 = M(11); BW = M(12); B3 = M(13); UB = M(14); VB = M(15); }
+  double *Xs = M(0), *T2 = M(1), *T4 = M(2), *T6 = M(3), *TW = M(4), *TV = M(5), *T3 = M(6), *VT = M(7), *UT = M(8);
+  double *B2 = nullptr, *B4 = nullptr, *B6 = nullptr, *BW = nullptr, *B3 = nullptr, *UB = nullptr;
+  if (phi) { B2 = M(9); B4 = M(10); B6 = M(11); BW = M(12); B3 = M(13); UB = M(14); }
   double* G = S + size_t(nmat) * nn * nb;  // n x gjcols per batch entry
 
   // X = dt A_M (+ reaction Jacobian)
   const double* u = ctx->desc.reaction ? d_state : nullptr;
+  LEM_CUDA_TRY(cudaMemsetAsync(Xs, 0, sizeof(double) * nn * nb, st));
   if (ctx->cplx)  // the real embedding of the complex window matrix
     assemble_local_complex_kernel<<<dim3((n / 2 + 127) / 128, nb), 128, 0, st>>>(
         Xs, n, d_bc, nb, ctx->d_coef, ctx->desc.coef_stride, ctx->ny, ctx->nx, ctx->desc.ndim);
@@ -475,7 +739,7 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
   LEM_CUDA_TRY(cudaGetLastError());
   // exact 1-norms -> s per class (host decides, same rule as theta_13 scaling)
   LEM_CUDA_TRY(cudaMemsetAsync(normbuf.p, 0, sizeof(double) * nb, st));
-  norm1_kernel<<<dim3((n + 127) / 128, nb), 128, 0, st>>>(
+  norm1_kernel<<<dim3((n + 31) / 32, nb), 256, 0, st>>>(
       Xs, n, reinterpret_cast<unsigned long long*>(normbuf.p));
   LEM_CUDA_TRY(cudaGetLastError());
   std::vector<double> norms(nb), scales(2 * nb);
@@ -496,158 +760,89 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
   double* d_c = scalebuf.p;
   double* d_cb1 = scalebuf.p + nb;
   LEM_CUDA_TRY(cudaMemcpyAsync(d_c, scales.data(), sizeof(double) * 2 * nb, cudaMemcpyHostToDevice, st));
+  // Classes sorted by s, descending: at squaring q the classes still squaring (s > q) are a
+  // prefix of the order, so one index map serves every squaring. A class that stops an odd
+  // number of squarings early has its result in the other buffer of the pair.
+  std::vector<int> order(2 * nb);
+  std::iota(order.begin(), order.begin() + nb, 0);
+  std::stable_sort(order.begin(), order.begin() + nb, [&](int a, int b) { return s[a] > s[b]; });
+  for (int b = 0; b < nb; ++b) order[nb + b] = (smax - s[b]) & 1;
+  const int* d_map = reinterpret_cast<const int*>(mapbuf.p);
+  const int* d_odd = d_map + nb;
+  LEM_CUDA_TRY(cudaMemcpyAsync(mapbuf.p, order.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
 
-  double bj[14];
-  for (int j = 0; j < 14; ++j) bj[j] = kPadeInt[j] / kPadeInt[0];
+  PadeTerms pt{};
+  for (int j = 0; j < 14; ++j) pt.b[j] = kPadeInt[j] / kPadeInt[0];
   const dim3 gsq = grid1(nn, nb);
-  auto lin = [&](double* out, std::initializer_list<std::pair<const double*, double>> terms,
-                 double diag, const double* dscale, const double* wscale0) -> lem_status {
-    Lin L{};
-    L.nin = 0;
-    for (auto& t : terms) { L.in[L.nin] = t.first; L.w[L.nin] = t.second; ++L.nin; }
-    L.diag = diag; L.dscale = dscale; L.wscale0 = wscale0;
-    lincomb_kernel<<<gsq, 256, 0, st>>>(out, n, n, n, L);
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? LEM_OK : cuda_fail(e, "lincomb_kernel");
-  };
   TcGuard tc;
   tc.st = st;
-  if (ctx->build_tc) LEM_TRY(tc_gemm_create(n, nb, gjcols, st, &tc.g));
-  // C = A B + beta C for every class of the batch
-  auto mm = [&](const double* A, const double* B, double* C, double beta) -> lem_status {
-    if (tc.g) return tc_gemm(tc.g, n, nb, nullptr, A, B, beta != 0.0 ? C : nullptr, C, st);
-    LEM_CUDA_TRY(dgemm_sq(n, nb, A, B, C, 1.0, beta, st));
-    return LEM_OK;
+  if (ctx->build_tc) LEM_TRY(tc_gemm_create(n, nb, gjcols, phi ? 4 : 2, st, &tc.g));
+  // C = A B (+ D, which may be C) (+ diag I) for every product of the list, on the first nact
+  // classes of the order (nact == nb: all)
+  struct Term { const double* B; const double* D; double* C; const double* diag; };
+  auto mul = [&](int nact, const double* A, std::initializer_list<Term> list) -> lem_status {
+    TcProduct pr[4];
+    int np = 0;
+    for (const Term& t : list) pr[np++] = TcProduct{n, t.B, n, nn, t.D, n, nn, t.C, n, nn, t.diag};
+    return mul_list(ctx, tc.g, nact, nact == nb ? nullptr : d_map, n, n, A, n, nn, pr, np, 0, 0);
   };
-  // Xs = X / 2^s   (per class)
-  LEM_TRY(lin(Xs, {{Xs, 1.0}}, 0.0, nullptr, d_c));
-  LEM_TRY(mm(Xs, Xs, T2, 0.0));
-  LEM_TRY(mm(T2, T2, T4, 0.0));
-  LEM_TRY(mm(T4, T2, T6, 0.0));
+  // Xs = X / 2^s (per class), Z^2's top-right c Xs; then the powers
+  scale_kernel<<<gsq, 256, 0, st>>>(Xs, B2, nn, d_c);
+  LEM_CUDA_TRY(cudaGetLastError());
+  LEM_TRY(mul(nb, Xs, {{Xs, nullptr, T2, nullptr}}));
   if (phi) {
-    LEM_TRY(lin(B2, {{Xs, 1.0}}, 0.0, nullptr, d_c));  // Z^2 top-right = c Xs
-    LEM_TRY(mm(T2, B2, B4, 0.0));
-    LEM_TRY(mm(T4, B2, B6, 0.0));
+    LEM_TRY(mul(nb, T2, {{T2, nullptr, T4, nullptr}, {B2, nullptr, B4, nullptr}}));
+    LEM_TRY(mul(nb, T4, {{T2, nullptr, T6, nullptr}, {B2, nullptr, B6, nullptr}}));
+  } else {
+    LEM_TRY(mul(nb, T2, {{T2, nullptr, T4, nullptr}}));
+    LEM_TRY(mul(nb, T4, {{T2, nullptr, T6, nullptr}}));
   }
   // W1 = b13 Z6 + b11 Z4 + b9 Z2 ;  W3 = Z6 W1 + b7 Z6 + b5 Z4 + b3 Z2 + b1 I ; U = Z W3
-  LEM_TRY(lin(TW, {{T6, bj[13]}, {T4, bj[11]}, {T2, bj[9]}}, 0.0, nullptr, nullptr));
-  LEM_TRY(lin(T3, {{T6, bj[7]}, {T4, bj[5]}, {T2, bj[3]}}, bj[1], nullptr, nullptr));
-  LEM_TRY(mm(T6, TW, T3, 1.0));
-  LEM_TRY(mm(Xs, T3, UT, 0.0));
-  if (phi) {
-    LEM_TRY(lin(BW, {{B6, bj[13]}, {B4, bj[11]}, {B2, bj[9]}}, 0.0, nullptr, nullptr));
-    LEM_TRY(lin(B3, {{B6, bj[7]}, {B4, bj[5]}, {B2, bj[3]}}, 0.0, nullptr, nullptr));
-    LEM_TRY(mm(T6, BW, B3, 1.0));
-    LEM_TRY(lin(UB, {}, 1.0, d_cb1, nullptr));  // c b1 I (from Z's top-right c I times b1)
-    LEM_TRY(mm(Xs, B3, UB, 1.0));
-  }
   // V = Z6 (b12 Z6 + b10 Z4 + b8 Z2) + b6 Z6 + b4 Z4 + b2 Z2 + b0 I
-  LEM_TRY(lin(TW, {{T6, bj[12]}, {T4, bj[10]}, {T2, bj[8]}}, 0.0, nullptr, nullptr));
-  LEM_TRY(lin(VT, {{T6, bj[6]}, {T4, bj[4]}, {T2, bj[2]}}, bj[0], nullptr, nullptr));
-  LEM_TRY(mm(T6, TW, VT, 1.0));
+  pt.z2[0] = T2; pt.z4[0] = T4; pt.z6[0] = T6; pt.w[0] = TW; pt.v[0] = TV; pt.a3[0] = T3; pt.vt[0] = VT;
+  pt.z2[1] = B2; pt.z4[1] = B4; pt.z6[1] = B6; pt.w[1] = BW; pt.a3[1] = B3;
+  pade_terms_kernel<<<dim3(unsigned((nn * nb + 255) / 256), 1, phi ? 2 : 1), 256, 0, st>>>(pt, n, nn * nb);
+  LEM_CUDA_TRY(cudaGetLastError());
   if (phi) {
-    LEM_TRY(lin(BW, {{B6, bj[12]}, {B4, bj[10]}, {B2, bj[8]}}, 0.0, nullptr, nullptr));
-    LEM_TRY(lin(VB, {{B6, bj[6]}, {B4, bj[4]}, {B2, bj[2]}}, 0.0, nullptr, nullptr));
-    LEM_TRY(mm(T6, BW, VB, 1.0));
+    LEM_TRY(mul(nb, T6, {{TW, T3, T3, nullptr}, {BW, B3, B3, nullptr}, {TV, VT, VT, nullptr}}));
+    // UB = X B3 + c b1 I (Z's top-right c I times b1); V_B + U_B - (V_B - U_B) = 2 U_B: V_B drops out
+    LEM_TRY(mul(nb, Xs, {{T3, nullptr, UT, nullptr}, {B3, nullptr, UB, d_cb1}}));
+  } else {
+    LEM_TRY(mul(nb, T6, {{TW, T3, T3, nullptr}, {TV, VT, VT, nullptr}}));
+    LEM_TRY(mul(nb, Xs, {{T3, nullptr, UT, nullptr}}));
   }
   // G = [V_T - U_T | V_T + U_T | (V_B + U_B) - (V_B - U_B) = 2 U_B]
-  {
-    Lin L{};
-    L.nin = 2; L.in[0] = VT; L.in[1] = UT; L.w[0] = 1.0; L.w[1] = -1.0;
-    lincomb_kernel<<<gsq, 256, 0, st>>>(T2, n, n, n, L);  // T2 reused as scratch
-    L.w[1] = 1.0;
-    lincomb_kernel<<<gsq, 256, 0, st>>>(T4, n, n, n, L);
-    LEM_CUDA_TRY(cudaGetLastError());
-    copy_cols_kernel<<<gsq, 256, 0, st>>>(G, gjcols, 0, T2, n, 0, n, n);
-    copy_cols_kernel<<<gsq, 256, 0, st>>>(G, gjcols, n, T4, n, 0, n, n);
-    if (phi) {
-      Lin L2{};
-      L2.nin = 1; L2.in[0] = UB; L2.w[0] = 2.0;
-      lincomb_kernel<<<gsq, 256, 0, st>>>(T6, n, n, n, L2);
-      copy_cols_kernel<<<gsq, 256, 0, st>>>(G, gjcols, 2 * n, T6, n, 0, n, n);
-    }
-    LEM_CUDA_TRY(cudaGetLastError());
-  }
+  solve_system_kernel<<<gsq, 256, 0, st>>>(G, n, gjcols, VT, UT, UB);
+  LEM_CUDA_TRY(cudaGetLastError());
   LEM_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
-  Buf ybuf, pivbuf;  // freed after the final synchronisation
-  LEM_TRY(solve_gj(ctx, tc.g, G, n, gjcols, nb, ybuf, pivbuf));
+  LEM_TRY(solve_gj(ctx, tc.g, G, n, gjcols, nb, ybuf, pivbuf, rowbuf));
   LEM_CUDA_TRY(cudaGetLastError());
-  // R_T -> RT2 (ping) ; R_B -> B2 (ping) ; squarings per class (s differs per class:
-  // classes that need fewer squarings are squared by a masked update; simplest: square each
-  // batch entry separately when the counts differ).
-  copy_cols_kernel<<<gsq, 256, 0, st>>>(RT2, n, 0, G, gjcols, n, n, n);
-  if (phi) copy_cols_kernel<<<gsq, 256, 0, st>>>(B2, n, 0, G, gjcols, 2 * n, n, n);
+  // R_T and R_B, then the squarings (R_T, R_B)^2 = (R_T^2, R_T R_B + R_B)
+  double *RT = T2, *RTn = T4, *RB = B2, *RBn = B4;
+  copy_cols_kernel<<<gsq, 256, 0, st>>>(RT, n, 0, G, gjcols, n, n, n);
+  if (phi) copy_cols_kernel<<<gsq, 256, 0, st>>>(RB, n, 0, G, gjcols, 2 * n, n, n);
   LEM_CUDA_TRY(cudaGetLastError());
-  double* RT = RT2; double* RTn = T4;
-  double* RB = B2;  double* RBn = B4;
-  bool uniform = true;
-  for (int b = 0; b < nb; ++b) uniform = uniform && (s[b] == s[0]);
-  Buf mapbuf;
-  if (tc.g && !uniform) {
-    // Classes sorted by s, descending: at squaring q the classes still squaring (s > q) are a
-    // prefix of the order, so one index map serves every squaring.
-    std::vector<int> order(nb);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return s[a] > s[b]; });
-    LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&mapbuf.p), sizeof(int) * nb, st));
-    const int* d_map = reinterpret_cast<const int*>(mapbuf.p);
-    LEM_CUDA_TRY(cudaMemcpyAsync(mapbuf.p, order.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, st));
-    for (int q = 0; q < smax; ++q) {
-      int nact = 0;
-      while (nact < nb && s[order[nact]] > q) ++nact;
-      if (phi) LEM_TRY(tc_gemm(tc.g, n, nact, d_map, RT, RB, RB, RBn, st));  // R_T R_B + R_B
-      LEM_TRY(tc_gemm(tc.g, n, nact, d_map, RT, RT, nullptr, RTn, st));
-      std::swap(RT, RTn);
-      if (phi) std::swap(RB, RBn);
-    }
-    // a class that stopped squaring an odd number of steps early holds its result in the
-    // other buffer of the pair
-    for (int b = 0; b < nb; ++b) {
-      if ((smax - s[b]) % 2 == 0) continue;
-      LEM_CUDA_TRY(cudaMemcpyAsync(RT + b * nn, RTn + b * nn, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
-      if (phi)
-        LEM_CUDA_TRY(cudaMemcpyAsync(RB + b * nn, RBn + b * nn, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
-    }
-  } else if (uniform) {
-    for (int q = 0; q < s[0]; ++q) {
-      if (phi) {  // (R_T, R_B)^2 = (R_T^2, R_T R_B + R_B)
-        if (tc.g) {
-          LEM_TRY(tc_gemm(tc.g, n, nb, nullptr, RT, RB, RB, RBn, st));
-        } else {
-          LEM_CUDA_TRY(cudaMemcpyAsync(RBn, RB, sizeof(double) * nn * nb, cudaMemcpyDeviceToDevice, st));
-          LEM_TRY(mm(RT, RB, RBn, 1.0));
-        }
-        std::swap(RB, RBn);
-      }
-      LEM_TRY(mm(RT, RT, RTn, 0.0));
-      std::swap(RT, RTn);
-    }
-  } else {
-    for (int b = 0; b < nb; ++b) {
-      double* rt = RT + b * nn; double* rtn = RTn + b * nn;
-      double* rb = phi ? RB + b * nn : nullptr; double* rbn = phi ? RBn + b * nn : nullptr;
-      for (int q = 0; q < s[b]; ++q) {
-        if (phi) {
-          LEM_CUDA_TRY(cudaMemcpyAsync(rbn, rb, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
-          LEM_CUDA_TRY(dgemm_sq(n, 1, rt, rb, rbn, 1.0, 1.0, st));
-          std::swap(rb, rbn);
-        }
-        LEM_CUDA_TRY(dgemm_sq(n, 1, rt, rt, rtn, 1.0, 0.0, st));
-        std::swap(rt, rtn);
-      }
-      // move the result into the batch-uniform buffer position of RT/RB
-      if (rt != RT + b * nn) LEM_CUDA_TRY(cudaMemcpyAsync(RT + b * nn, rt, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
-      if (phi && rb != RB + b * nn) LEM_CUDA_TRY(cudaMemcpyAsync(RB + b * nn, rb, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
-    }
+  for (int q = 0; q < smax; ++q) {
+    int nact = 0;
+    while (nact < nb && s[order[nact]] > q) ++nact;
+    if (!phi)
+      LEM_TRY(mul(nact, RT, {{RT, nullptr, RTn, nullptr}}));
+    else if (q == smax - 1)  // phi_1 is R_B: the last R_T^2 is not needed
+      LEM_TRY(mul(nact, RT, {{RB, RB, RBn, nullptr}}));
+    else
+      LEM_TRY(mul(nact, RT, {{RB, RB, RBn, nullptr}, {RT, nullptr, RTn, nullptr}}));
+    std::swap(RT, RTn);
+    if (phi) std::swap(RB, RBn);
   }
   const double* R = phi ? RB : RT;
+  const double* R1 = phi ? RBn : RTn;
   double* Pout = ctx->d_P + size_t(c0) * ctx->n_int * ctx->n_loc;
   if (ctx->cplx)
     extract_rows_complex_kernel<<<grid1(ctx->n_int * ctx->n_loc, nb), 256, 0, st>>>(Pout, ctx->n_int, ctx->n_loc, R,
-                                                                                    n, d_bc);
+                                                                                    R1, d_odd, n, d_bc);
   else
-    extract_rows_kernel<<<grid1(ctx->n_int * ctx->n_loc, nb), 256, 0, st>>>(
-        Pout, ctx->n_int, ctx->n_loc, R, n, n, 0, d_bc);
+    extract_rows_kernel<<<grid1(ctx->n_int * ctx->n_loc, nb), 256, 0, st>>>(Pout, ctx->n_int, ctx->n_loc, R, R1, d_odd,
+                                                                            n, d_bc);
   LEM_CUDA_TRY(cudaGetLastError());
   int status = 0;
   LEM_CUDA_TRY(cudaMemcpyAsync(&status, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -689,7 +884,7 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   }
   constexpr int NAUG = 10;  // Z, Z2, Z4, Z6, W, W3, U, V, R, Rn
   const int gjcols = 5 * n;
-  Buf scratch, bcbuf, normbuf, scalebuf, ybuf, pivbuf, mapbuf;
+  Buf scratch, bcbuf, normbuf, scalebuf, ybuf, pivbuf, rowbuf, mapbuf;
   const size_t bytes = sizeof(double) * (size_t(NAUG) * 4 * nn + size_t(n) * gjcols) * nb;
   LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&scratch.p), bytes, st));
   LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&bcbuf.p), sizeof(BatchClass) * nb, st));
@@ -710,11 +905,12 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
 
   // X = dt J_M, the 1-norms, s per class
   const double* u = ctx->desc.reaction ? d_state : nullptr;
+  LEM_CUDA_TRY(cudaMemsetAsync(Z.m[0], 0, sizeof(double) * nn * nb, st));
   assemble_local_kernel<<<dim3((n + 127) / 128, nb), 128, 0, st>>>(
       Z.m[0], n, d_bc, nb, ctx->d_coef, ctx->desc.coef_stride, ctx->ny, ctx->nx, ctx->desc.ndim, u, ctx->desc.dt,
       ctx->desc.reaction, ctx->desc.porous_m);
   LEM_CUDA_TRY(cudaMemsetAsync(normbuf.p, 0, sizeof(double) * nb, st));
-  norm1_kernel<<<dim3((n + 127) / 128, nb), 128, 0, st>>>(Z.m[0], n,
+  norm1_kernel<<<dim3((n + 31) / 32, nb), 256, 0, st>>>(Z.m[0], n,
                                                            reinterpret_cast<unsigned long long*>(normbuf.p));
   LEM_CUDA_TRY(cudaGetLastError());
   std::vector<double> norms(nb), scales(nb);
@@ -753,18 +949,18 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   };
   TcGuard tc;
   tc.st = st;
-  if (ctx->build_tc) LEM_TRY(tc_gemm_create(n, nb, gjcols, st, &tc.g));
-  auto mm = [&](const double* A, const double* B, double* C, const double* D) -> lem_status {
-    if (tc.g) return tc_gemm(tc.g, n, nb, nullptr, A, B, D, C, st);
-    if (D && D != C) LEM_CUDA_TRY(cudaMemcpyAsync(C, D, sizeof(double) * nn * nb, cudaMemcpyDeviceToDevice, st));
-    LEM_CUDA_TRY(dgemm_sq(n, nb, A, B, C, 1.0, D ? 1.0 : 0.0, st));
-    return LEM_OK;
+  if (ctx->build_tc) LEM_TRY(tc_gemm_create(n, nb, gjcols, 4, st, &tc.g));
+  // one A against four B
+  auto mul4 = [&](int nact, const int* map, const double* A, const double* const (&B)[4], const double* const (&D)[4],
+                  double* const (&C)[4]) -> lem_status {
+    TcProduct pr[4];
+    for (int t = 0; t < 4; ++t) pr[t] = TcProduct{n, B[t], n, nn, D[t], n, nn, C[t], n, nn, nullptr};
+    return mul_list(ctx, tc.g, nact, map, n, n, A, n, nn, pr, 4, 0, 0);
   };
   // C = A * B (C distinct from A and B)
   auto amul = [&](const Aug& A, const Aug& B, Aug& C) -> lem_status {
-    LEM_TRY(mm(A.m[0], B.m[0], C.m[0], nullptr));
+    LEM_TRY(mul4(nb, nullptr, A.m[0], {B.m[0], B.m[1], B.m[2], B.m[3]}, {}, C.m));
     for (int j = 0; j < 3; ++j) {
-      LEM_TRY(mm(A.m[0], B.m[1 + j], C.m[1 + j], nullptr));
       const double w0 = B.b[j], w1 = j >= 1 ? B.b[j - 1] : 0.0, w2 = j >= 2 ? B.b[j - 2] : 0.0;
       if (w0 != 0.0 || w1 != 0.0 || w2 != 0.0)  // + sum_{a <= j} B.b[j - a] A.B_a
         LEM_TRY(lin(C.m[1 + j], {{C.m[1 + j], 1.0}, {A.m[1], w0}, {A.m[2], w1}, {A.m[3], w2}}, 0.0, nullptr));
@@ -833,7 +1029,7 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   for (int q = 0; q < 4; ++q) copy_cols_kernel<<<gsq, 256, 0, st>>>(G, gjcols, (1 + q) * n, W3.m[q], n, 0, n, n);
   LEM_CUDA_TRY(cudaGetLastError());
   LEM_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
-  LEM_TRY(solve_gj(ctx, tc.g, G, n, gjcols, nb, ybuf, pivbuf));
+  LEM_TRY(solve_gj(ctx, tc.g, G, n, gjcols, nb, ybuf, pivbuf, rowbuf));
   for (int q = 0; q < 4; ++q) copy_cols_kernel<<<gsq, 256, 0, st>>>(R.m[q], n, 0, G, gjcols, (1 + q) * n, n, n);
   LEM_CUDA_TRY(cudaGetLastError());
 
@@ -852,57 +1048,25 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   std::vector<int> order(nb);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return s[a] > s[b]; });
-  const bool uniform = s[order.front()] == s[order.back()];
-  if (tc.g) {
-    const int* d_map = nullptr;
-    if (!uniform) {
-      LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&mapbuf.p), sizeof(int) * nb, st));
-      LEM_CUDA_TRY(cudaMemcpyAsync(mapbuf.p, order.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, st));
-      d_map = reinterpret_cast<const int*>(mapbuf.p);
-    }
-    for (int q = 0; q < smax; ++q) {
-      int nact = 0;
-      while (nact < nb && s[order[nact]] > q) ++nact;
-      LEM_TRY(prep(R));
-      LEM_TRY(tc_gemm(tc.g, n, nact, d_map, R.m[0], H1, H1, Rn.m[1], st));
-      LEM_TRY(tc_gemm(tc.g, n, nact, d_map, R.m[0], H2, D2, Rn.m[2], st));
-      LEM_TRY(tc_gemm(tc.g, n, nact, d_map, R.m[0], H3, D3, Rn.m[3], st));
-      LEM_TRY(tc_gemm(tc.g, n, nact, d_map, R.m[0], R.m[0], nullptr, Rn.m[0], st));
-      std::swap(R, Rn);
-    }
-    for (int b = 0; b < nb; ++b) {  // classes that stopped an odd number of steps early
-      if ((smax - s[b]) % 2 == 0) continue;
-      for (int q = 0; q < 4; ++q)
-        LEM_CUDA_TRY(cudaMemcpyAsync(R.m[q] + b * nn, Rn.m[q] + b * nn, sizeof(double) * nn,
-                                     cudaMemcpyDeviceToDevice, st));
-    }
-  } else {
-    for (int q = 0; q < smax; ++q) {
-      LEM_TRY(prep(R));
-      for (int b = 0; b < nb; ++b) {
-        if (s[b] <= q) {  // finished: carry it into the other buffer
-          for (int k = 0; k < 4; ++k)
-            LEM_CUDA_TRY(cudaMemcpyAsync(Rn.m[k] + b * nn, R.m[k] + b * nn, sizeof(double) * nn,
-                                         cudaMemcpyDeviceToDevice, st));
-          continue;
-        }
-        const int64_t o = b * nn;
-        LEM_CUDA_TRY(cudaMemcpyAsync(Rn.m[1] + o, H1 + o, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
-        LEM_CUDA_TRY(cudaMemcpyAsync(Rn.m[2] + o, D2 + o, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
-        LEM_CUDA_TRY(cudaMemcpyAsync(Rn.m[3] + o, D3 + o, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
-        LEM_CUDA_TRY(dgemm_sq(n, 1, R.m[0] + o, H1 + o, Rn.m[1] + o, 1.0, 1.0, st));
-        LEM_CUDA_TRY(dgemm_sq(n, 1, R.m[0] + o, H2 + o, Rn.m[2] + o, 1.0, 1.0, st));
-        LEM_CUDA_TRY(dgemm_sq(n, 1, R.m[0] + o, H3 + o, Rn.m[3] + o, 1.0, 1.0, st));
-        LEM_CUDA_TRY(dgemm_sq(n, 1, R.m[0] + o, R.m[0] + o, Rn.m[0] + o, 1.0, 0.0, st));
-      }
-      std::swap(R, Rn);
-    }
+  // classes that stop squaring an odd number of steps early have their result in the other buffer
+  order.resize(2 * nb);
+  for (int b = 0; b < nb; ++b) order[nb + b] = (smax - s[b]) & 1;
+  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&mapbuf.p), sizeof(int) * 2 * nb, st));
+  LEM_CUDA_TRY(cudaMemcpyAsync(mapbuf.p, order.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
+  const int* d_map = reinterpret_cast<const int*>(mapbuf.p);
+  const int* d_odd = d_map + nb;
+  for (int q = 0; q < smax; ++q) {
+    int nact = 0;
+    while (nact < nb && s[order[nact]] > q) ++nact;
+    LEM_TRY(prep(R));
+    LEM_TRY(mul4(nact, nact == nb ? nullptr : d_map, R.m[0], {R.m[0], H1, H2, H3}, {nullptr, H1, D2, D3}, Rn.m));
+    std::swap(R, Rn);
   }
   const size_t pc = size_t(ctx->n_int) * ctx->n_loc;
   extract_rows_kernel<<<grid1(ctx->n_int * ctx->n_loc, nb), 256, 0, st>>>(ctx->d_P + size_t(c0) * pc, ctx->n_int,
-                                                                         ctx->n_loc, R.m[1], n, n, 0, d_bc);
+                                                                         ctx->n_loc, R.m[1], Rn.m[1], d_odd, n, d_bc);
   extract_rows_kernel<<<grid1(ctx->n_int * ctx->n_loc, nb), 256, 0, st>>>(ctx->d_P3 + size_t(c0) * pc, ctx->n_int,
-                                                                         ctx->n_loc, R.m[3], n, n, 0, d_bc);
+                                                                         ctx->n_loc, R.m[3], Rn.m[3], d_odd, n, d_bc);
   LEM_CUDA_TRY(cudaGetLastError());
   int status = 0;
   LEM_CUDA_TRY(cudaMemcpyAsync(&status, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -926,11 +1090,11 @@ lem_status build_propagators_impl(lem_ctx* ctx, const double* d_state) {
   const int64_t nc = int64_t(ctx->classes.size());
   const int64_t n = ctx->n_loc;
   const bool rb3 = ctx->desc.scheme == LEM_SCHEME_RB3;
-  const int nmat = rb3 ? 45 : ctx->desc.mode == LEM_MODE_PHI ? 19 : 11;
+  const int nmat = rb3 ? 45 : ctx->desc.mode == LEM_MODE_PHI ? 18 : 11;
   // batch size from a scratch budget of 8 GiB
   const int gjc = rb3 ? 5 * int(n) : ctx->desc.mode == LEM_MODE_PHI ? 3 * int(n) : 2 * int(n);
   const double per = double(nmat) * n * n * sizeof(double) +
-                     (ctx->build_tc ? double(tc_gemm_bytes(int(n), 1, gjc)) + sizeof(double) * n * GJ_KB : 0.0);
+                     (ctx->build_tc ? double(tc_gemm_bytes(int(n), 1, gjc, ctx->desc.mode == LEM_MODE_PHI ? 4 : 2)) + sizeof(double) * n * GJ_SB : sizeof(double) * (double(n) * GJ_SB + double(gjc) * GJ_KB));
   int64_t bmax = std::max<int64_t>(1, int64_t((8.0 * (1ull << 30)) / per));
   bmax = std::min<int64_t>(bmax, 65535);
   for (int64_t c0 = 0; c0 < nc; c0 += bmax) {

@@ -192,21 +192,41 @@ lem_status split_batch_step(SplitBatch* b, int nsteps, cudaStream_t st, cudaEven
 double split_batch_gemm_flops(const SplitBatch* b, lem_ctx* const* ctxs);
 lem_status split_batch_check_error(SplitBatch* b);
 void split_batch_destroy(SplitBatch* b);
-// builder_tc.cu: FP64 products of the propagator build as exact sums of FP16 slice products
-// on the tensor cores (split-precision tiers)
+// builder_tc.cu: FP64 products of the split tiers' propagator build as sums of digit products on
+// the tensor cores
 struct TcGemm;
-// workspace for products of nb matrices of n x n and rank-64 updates of n x gjcols ones
-size_t tc_gemm_bytes(int n, int nb, int gjcols);
-lem_status tc_gemm_create(int n, int nb, int gjcols, cudaStream_t st, TcGemm** out);
+// One right factor of a product batch: C = A B + D (D null: none) + diag[matrix] I (null: none).
+struct TcProduct {
+  int N;               // columns of B, D and C
+  const double* B;
+  int64_t ldb, sB;
+  const double* D;
+  int64_t ldd, sD;
+  double* C;
+  int64_t ldc, sC;
+  const double* diag;
+};
+// workspace for products of nb matrices of n x n with up to np right factors at once, and for
+// rank-256 updates of n x gjcols ones
+size_t tc_gemm_bytes(int n, int nb, int gjcols, int np);
+lem_status tc_gemm_create(int n, int nb, int gjcols, int np, cudaStream_t st, TcGemm** out);
 void tc_gemm_destroy(TcGemm* g, cudaStream_t st);
-// C = A B + D (D optional) on strided batches of row-major FP64 matrices (A M x K, B K x N)
-lem_status tc_gemm_ex(TcGemm* g, int nbatch, const int* map, int M, int N, int K, const double* A, int64_t lda,
-                      int64_t sA, const double* B, int64_t ldb, int64_t sB, const double* D, int64_t ldd,
-                      int64_t sD, int zr0, int zr1, double* C, int64_t ldc, int64_t sC, cudaStream_t st);
-// the same for square n x n matrices stored back to back
-lem_status tc_gemm(TcGemm* g, int n, int nbatch, const int* map, const double* A, const double* B, const double* D,
-                   double* C, cudaStream_t st);
+// the products of one A with every right factor of the list, on strided batches of row-major
+// FP64 matrices (A M x K, B K x N)
+lem_status tc_gemm(TcGemm* g, int nbatch, const int* map, int M, int K, const double* A, int64_t lda,
+                   int64_t sA, const TcProduct* list, int np, int zr0, int zr1, cudaStream_t st);
 lem_status tc_gemm_check(TcGemm* g, cudaStream_t st);
+// |x|^e for the porous medium: small whole exponents by multiplication (pow costs hundreds of
+// instructions on the FP64 pipe: 20 us for a mesh of 400 nodes)
+#ifdef __CUDACC__
+__device__ __forceinline__ double abs_pow(double x, double e) {
+  const double a = fabs(x);
+  if (e == 1.0) return a;
+  if (e == 2.0) return a * a;
+  if (e == 3.0) return a * a * a;
+  return pow(a, e);
+}
+#endif
 // builder.cu: whether propagators of a precision tier are built with the tensor-core products
 bool builder_uses_tc(int prec);
 // abi.cpp: take a built single-class propagator from a context with the same local operator

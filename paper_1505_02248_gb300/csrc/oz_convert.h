@@ -45,71 +45,27 @@ LEM_HD unsigned long long biased_digits(unsigned long long bits, int e) {
   return N + kBias;
 }
 
-// (hi 2^24 + lo) 2^(s) as a double, rounded to nearest even: hi and lo hold the level sums
-// sum_{L <= 3} S_L 2^(8 (3 - L)) and sum_{L = 4..6} S_L 2^(8 (6 - L)); |hi| < 2^62, |lo| < 2^62.
-LEM_HD double sums_to_double(long long hi, long long lo, int s) {
-  long long H = hi + (lo >> 24);
-  unsigned int R = (unsigned int)(lo & 0xFFFFFF);  // value = H 2^24 + R
-  unsigned long long sign = 0;
-  if (H < 0) {  // magnitude
-    sign = 1ull << 63;
-    H = ~H + (R == 0 ? 1 : 0);
-    R = (0x1000000u - R) & 0xFFFFFFu;
+// Coarse digits: N = round(x 2^(49 - e)), |N| <= 2^49, as seven balanced base-128 digits, each
+// rounded to nearest from the top (|d_0| <= 128, the others at most 64 in magnitude).
+LEM_HD void coarse_digits(unsigned long long bits, int e, int (&d)[7]) {
+  const int E = exp_field(bits);
+  const int sh = 1026 + e - E;  // >= 4
+  long long N = 0;
+  if (E != 0 && sh < 54) {
+    const long long m = (long long)((bits & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull);
+    N = (m + (1ll << (sh - 1))) >> sh;
+    if (bits >> 63) N = -N;
   }
-  unsigned long long m;  // the magnitude's 64 leading bits
-  int ex;                // value = m 2^ex (+ sticky)
-  unsigned int sticky = 0;
-  if (H == 0) {
-    if (R == 0) return 0.0;
-#ifdef __CUDA_ARCH__
-    const int z = __clz(int(R));
-#else
-    const int z = __builtin_clz(R);
-#endif
-    m = (unsigned long long)R << (32 + z);
-    ex = -(32 + z);
-  } else {
-#ifdef __CUDA_ARCH__
-    const int z = __clzll(H);
-#else
-    const int z = __builtin_clzll((unsigned long long)H);
-#endif
-    m = (unsigned long long)H << z;
-    if (z <= 24) {
-      m |= R >> (24 - z);
-      sticky = R & ((1u << (24 - z)) - 1u);
-    } else {
-      m |= (unsigned long long)R << (z - 24);
-    }
-    ex = 24 - z;
+  for (int s = 0; s < 6; ++s) {
+    const int p = 7 * (6 - s);
+    const long long q = (N + (1ll << (p - 1))) >> p;  // arithmetic shift: floor
+    N -= q << p;
+    d[s] = (int)q;
   }
-  const unsigned int low = (unsigned int)(m & 0x7FF);
-  unsigned long long q = m >> 11;  // 53 bits
-  const int be = ex + 63 + s + 1023;  // biased exponent of the leading bit
-  if (be >= 1) {
-    if (low > 0x400u || (low == 0x400u && (sticky != 0 || (q & 1)))) ++q;  // (2^53 carries over)
-    unsigned long long b = ((unsigned long long)(unsigned int)(be - 1) << 52) + q;
-    if (be >= 2047 || b >= 0x7FF0000000000000ull) b = 0x7FF0000000000000ull;
-    b |= sign;
-#ifdef __CUDA_ARCH__
-    return __longlong_as_double((long long)b);
-#else
-    double d;
-    __builtin_memcpy(&d, &b, 8);
-    return d;
-#endif
-  }
-  // subnormal result: drop 1 - be more bits, rounding once
-  const int drop = 12 - be;  // bits of m below the subnormal's unit
-  unsigned long long b = 0;
-  if (drop <= 64) {
-    const unsigned long long top = drop == 64 ? 0ull : m >> drop;
-    const unsigned long long half = 1ull << (drop - 1);
-    const unsigned long long rest = drop == 64 ? m : m & ((half << 1) - 1);
-    b = top;
-    if (rest > half || (rest == half && (sticky != 0 || (top & 1)))) ++b;
-  }
-  b |= sign;
+  d[6] = (int)N;
+}
+
+LEM_HD double bits_double(unsigned long long b) {
 #ifdef __CUDA_ARCH__
   return __longlong_as_double((long long)b);
 #else
@@ -117,6 +73,51 @@ LEM_HD double sums_to_double(long long hi, long long lo, int s) {
   __builtin_memcpy(&d, &b, 8);
   return d;
 #endif
+}
+LEM_HD unsigned long long double_bits(double d) {
+#ifdef __CUDA_ARCH__
+  return (unsigned long long)__double_as_longlong(d);
+#else
+  unsigned long long b;
+  __builtin_memcpy(&b, &d, 8);
+  return b;
+#endif
+}
+
+// Largest K of a product: the level sums stay below 2^51 2^24.
+constexpr int kMaxK = 8000;
+
+// (hi 2^24 + lo) 2^s as a double, rounded to nearest even (twice if it is subnormal): hi and lo
+// hold the level sums sum_{L <= 3} S_L 2^(8 (3 - L)) and sum_{L = 4..6} S_L 2^(8 (6 - L));
+// |hi + (lo >> 24)| < 2^51. Two FP64 additions, the first exact: H = hi + (lo >> 24) enters as
+// the low mantissa bits of 1.5 2^52, the 24 bits below it as 1 + R 2^-24, and the integers need no
+// conversion instructions. (All in integers it took about 80 instructions an element, and the
+// epilogue of a tile 22 us.)
+LEM_HD double sums_unscaled(long long hi, long long lo) {  // (hi 2^24 + lo) 2^-24
+  const long long H = hi + (lo >> 24);
+  const unsigned long long R = (unsigned long long)lo & 0xFFFFFFull;
+  const double h = bits_double((unsigned long long)H + 0x4338000000000000ull) - 6755399441055745.0;  // H - 1
+  return h + bits_double(0x3FF0000000000000ull | (R << 28));
+}
+// v 2^t where v and the result are normal numbers or v is zero; *far is set where they are not.
+// No branches, so that several elements' instructions interleave.
+LEM_HD double scale_near(double v, int t, bool* far) {
+  const unsigned long long b = double_bits(v);
+  const unsigned int e = (unsigned int)((b >> 52) & 0x7FF);
+  const bool zero = e == 0;  // (an FP64 comparison would cost as much as an addition)
+  *far = *far || (!zero && (unsigned int)((int)e + t - 1) >= 2046u);
+  return bits_double(zero ? b : b + ((unsigned long long)(unsigned int)t << 52));
+}
+LEM_HD double scale_far(double v, int t) {  // in three steps, of which the last one rounds
+  const int q = t / 3;
+  const double f = bits_double((unsigned long long)(1023 + q) << 52);
+  return v * f * f * bits_double((unsigned long long)(1023 + t - 2 * q) << 52);
+}
+LEM_HD double sums_to_double(long long hi, long long lo, int s) {
+  const double v = sums_unscaled(hi, lo);
+  bool far = false;
+  const double y = scale_near(v, s + 24, &far);
+  return far ? scale_far(v, s + 24) : y;
 }
 
 }  // namespace oz

@@ -32,7 +32,7 @@ __global__ void residual_fp64_kernel(double* __restrict__ r, const double* __res
     auto cf = [&](int w) { return cstride ? coef[int64_t(w) * npts + p] : coef[w]; };
     auto val = [&](int64_t q) {
       const double v = u[q];
-      if constexpr (NL == 2) return pow(fabs(v), pm - 1.0) * v;
+      if constexpr (NL == 2) return abs_pow(v, pm - 1.0) * v;
       return v;
     };
     const double uc = u[p];

@@ -135,9 +135,16 @@ __global__ void __launch_bounds__(WIN_THREADS) oz_windows_kernel(const double* _
   }
 }
 
+// Owner rows with at most SPARSE nonzero entries (selections, shifts) are formed as FP64
+// multiply-adds over those entries, in order: exact where the product with the whole row is,
+// whatever the range of the window's values, and cheaper. Their entries are kept with the digits.
+constexpr int SPARSE = 8;
+constexpr int kSparseRow = 1 << 21;  // in place of the scale exponent
+
 // Propagator digits, once per build: a CTA cuts 8 owner rows.
 __global__ void __launch_bounds__(256) oz_prop_kernel(const double* __restrict__ P, int64_t n_int, int64_t n_loc,
                                                       const PropRows* __restrict__ rows, int* __restrict__ f,
+                                                      double* __restrict__ sv, int* __restrict__ sk,
                                                       __half* __restrict__ out) {
   const PropRows p = rows[blockIdx.x / 8];
   const int r0 = (blockIdx.x % 8) * 8;
@@ -145,14 +152,26 @@ __global__ void __launch_bounds__(256) oz_prop_kernel(const double* __restrict__
   __shared__ int ex[8];
   auto row = [&](int i) { return P + (int64_t(p.cls) * n_int + p.row0 + i) * n_loc; };
   {
-    int E = 0;
+    int E = 0, cnt = 0;
+    const int fr = p.f_off + r0 + warp;
     if (r0 + warp < p.rows)
-      for (int k = lane; k < p.cols; k += 32)
-        E = max(E, oz::exp_field(static_cast<unsigned long long>(__double_as_longlong(row(r0 + warp)[k]))));
+      for (int k0 = 0; k0 < p.cols; k0 += 32) {
+        const int k = k0 + lane;
+        const double v = k < p.cols ? row(r0 + warp)[k] : 0.0;
+        E = max(E, oz::exp_field(static_cast<unsigned long long>(__double_as_longlong(v))));
+        const unsigned nz = __ballot_sync(0xffffffffu, v != 0.0);
+        const int at = cnt + __popc(nz & ((1u << lane) - 1u));
+        if (v != 0.0 && at < SPARSE) {
+          sv[size_t(fr) * SPARSE + at] = v;
+          sk[size_t(fr) * SPARSE + at] = k;
+        }
+        cnt += __popc(nz);
+      }
     for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+    if (lane < SPARSE && lane >= cnt) sk[size_t(fr) * SPARSE + lane] = -1;
     if (lane == 0) {
       ex[warp] = oz::scale_exp(E);
-      f[p.f_off + r0 + warp] = ex[warp];
+      f[fr] = ex[warp] != oz::kNonFinite && cnt > 0 && cnt <= SPARSE ? kSparseRow : ex[warp];
     }
   }
   __syncthreads();
@@ -180,11 +199,13 @@ struct StepParams {
   const __half* b;
   const int* e;
   const int* f;
+  const double* sv;    // entries of sparse owner rows
+  const int* sk;
   const double* P;     // (rows with infinities or NaN are formed in FP64)
   const double* src;
   double* u;
   int64_t n_int, n_loc, ny, nx;
-  int unit0, ks, accumulate;
+  int unit0, nunits, ks, accumulate;
   int* err;
 };
 
@@ -202,81 +223,185 @@ __device__ __noinline__ double plain_dot(const StepParams& p, const TileDesc& t,
   return s;
 }
 
-// One unit per cluster of ks CTAs (ks = 1: no cluster). The scatter adds each owner's increment
-// to the state (PHI) or stores it (EXP); thread = column first, so a row's owners are written in
-// runs of the tile width.
+// The same over the few entries of a sparse owner row.
+__device__ __noinline__ double sparse_dot(const StepParams& p, const TileDesc& t, int fr) {
+  double s = 0.0;
+  for (int q = 0; q < SPARSE; ++q) {
+    const int k = p.sk[size_t(fr) * SPARSE + q];
+    if (k < 0) break;
+    int64_t gy = int64_t(t.org[0]) + k / t.wext[1], gx = int64_t(t.org[1]) + k % t.wext[1];
+    gy = gy < 0 ? gy + p.ny : (gy >= p.ny ? gy - p.ny : gy);
+    gx = gx < 0 ? gx + p.nx : (gx >= p.nx ? gx - p.nx : gx);
+    s = fma(p.sv[size_t(fr) * SPARSE + q], p.src[gy * p.nx + gx], s);
+  }
+  return s;
+}
+
+// Where a unit's outputs go: window by window and owner by owner.
+struct StepUnit {
+  const StepParams& p;
+  Unit un;
+  WinBlock wb;
+  const int64_t* node0;  // first owner node and scale exponent of each window
+  const int* e;
+  const int* f;          // scale exponents of the 64 owner rows
+  int ix;                // owners per tile row
+  uint32_t inv;
+  // (rows and columns formed otherwise lie outside for the digit sums: formed() writes them)
+  __device__ int scale(int row, int col) const { return e[row] + f[col] - 62; }
+  __device__ double value(int, int, double v) const { return v; }
+  __device__ int64_t row_at(int row) const { return row < wb.count && e[row] != oz::kNonFinite ? node0[row] : -1; }
+  __device__ int64_t off(int col) const {
+    const int i = un.col0 + col, iy = div_by(i, inv);
+    return int64_t(iy) * p.nx + (i - iy * ix);
+  }
+  __device__ int64_t col_at(int col) const {
+    return col < un.ncol && f[col] != oz::kNonFinite && f[col] != kSparseRow ? off(col) : INT64_MIN / 2;
+  }
+  // Elements of non-finite windows, non-finite owner rows and sparse owner rows, by this warp:
+  // rows r0 .. r0 + nr - 1, columns c0 .. c0 + nc - 1.
+  __device__ void formed(int r0, int nr, int c0, int nc, int lane) const {
+    bool any = false;
+    for (int r = r0 + lane; r < r0 + nr; r += 32) any |= e[r] == oz::kNonFinite;
+    for (int c = c0 + lane; c < c0 + nc; c += 32) any |= f[c] == oz::kNonFinite || f[c] == kSparseRow;
+    if (!__any_sync(0xffffffffu, any)) return;
+    for (int q = lane; q < nr * nc; q += 32) {
+      const int row = r0 + q / nc, col = c0 + q % nc;
+      if (row >= wb.count || col >= un.ncol) continue;
+      const bool plain = e[row] == oz::kNonFinite || f[col] == oz::kNonFinite;
+      if (!plain && f[col] != kSparseRow) continue;
+      const TileDesc& t = p.tiles[p.order[wb.first + row]];
+      const double y = plain ? plain_dot(p, t, un.col0 + col) : sparse_dot(p, t, un.f_off + col);
+      const int64_t w = node0[row] + off(col);
+      store(w, y, load(w, row));
+    }
+  }
+  __device__ double load(int64_t w, int) const { return p.accumulate ? p.u[w] : 0.0; }
+  __device__ void store(int64_t w, double y, double old) const { p.u[w] = p.accumulate ? old + y : y; }
+};
+
+// Per-unit tables of the epilogue.
+struct StepTables {
+  int64_t node0[oz::BM];
+  int e[oz::BM], f[oz::BN];
+  int ix;
+  __device__ void fill(const StepParams& p, const Unit& un, const WinBlock& wb, int t) {
+    if (t < oz::BM) {
+      const TileDesc& d = p.tiles[p.order[wb.first + min(t, wb.count - 1)]];
+      node0[t] = int64_t(d.t0[0]) * p.nx + d.t0[1];
+      e[t] = p.e[wb.e_off + t];
+      if (t == 0) ix = d.iext[1];
+    } else if (t < oz::BM + oz::BN) {
+      f[t - oz::BM] = p.f[un.f_off + t - oz::BM];
+    }
+  }
+};
+
+// The units of one CTA, every gridDim.x-th: increments are added to the state (PHI) or the owners
+// stored (EXP).
+struct StepWork {
+  const StepParams& p;
+  StepTables* tab;  // [2] by the unit's parity
+  __device__ int index(int k) const { return p.unit0 + int(blockIdx.x) + k * int(gridDim.x); }
+  __device__ int count() const { return (p.nunits - int(blockIdx.x) + int(gridDim.x) - 1) / int(gridDim.x); }
+  __device__ oz::Tile tile(int k) const {
+    const Unit& un = p.units[index(k)];
+    const WinBlock& wb = p.blocks[un.wb];
+    return {p.a + wb.a_off, p.b + un.b_off, wb.nkb};
+  }
+  __device__ void begin(int k) {
+    const Unit& un = p.units[index(k)];
+    tab[k & 1].fill(p, un, p.blocks[un.wb], int(threadIdx.x) - 64);
+    oz::epi_sync();
+  }
+  __device__ void finish(int k, int quarter, int half, int lane, double* out, const long long (&hi)[32],
+                         const long long (&lo)[32]) {
+    const Unit un = p.units[index(k)];
+    const StepTables& t = tab[k & 1];
+    StepUnit o{p, un, p.blocks[un.wb], t.node0, t.e, t.f, t.ix, div_inv(uint32_t(t.ix))};
+    oz::write_tile(o, quarter, half, lane, out, hi, lo);
+    o.formed(32 * quarter, 32, 32 * half, 32, lane);
+  }
+};
+
 __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_kernel(const __grid_constant__ StepParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ volatile int s_abort;
+  __shared__ StepTables tab[2];
+  const oz::Shared sh = oz::carve(smem_raw);
+  const uint32_t tmem = oz::setup(sh, &s_abort);
+  StepWork work{p, tab};
+  oz::run<oz::Fine>(sh, tmem, work, p.err, &s_abort);
+  oz::release(tmem);
+}
+
+// The share of one CTA of a cluster of ks: K blocks [k0, k1) of one unit.
+struct SplitWork {
+  const oz::Shared& sh;
+  oz::Tile t;
+  __device__ int count() const { return t.nkb > 0 ? 1 : 0; }
+  __device__ oz::Tile tile(int) const { return t; }
+  __device__ void begin(int) const {}
+  __device__ void finish(int, int quarter, int half, int lane, double*, const long long (&hi)[32],
+                         const long long (&lo)[32]) const {
+    oz::stage_sums(sh, quarter, half, lane, hi, lo);
+  }
+};
+
+// One unit per cluster of ks CTAs, its K blocks divided; each CTA then adds the others' sums for
+// its share of the columns and writes them.
+__global__ void __launch_bounds__(oz::THREADS, 1) oz_step_split_kernel(const __grid_constant__ StepParams p) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  __shared__ volatile int s_abort;
+  __shared__ StepTables tab;
   const oz::Shared sh = oz::carve(smem_raw);
   const int ks = p.ks, rank = int(blockIdx.x) % ks;
   const Unit un = p.units[p.unit0 + int(blockIdx.x) / ks];
   const WinBlock wb = p.blocks[un.wb];
-  __shared__ int64_t s_node[oz::BM];  // first owner node and scale exponent of each window
-  __shared__ int s_e[oz::BM], s_f[oz::BN], s_ix;
-  if (threadIdx.x < wb.count) {
-    const TileDesc& t = p.tiles[p.order[wb.first + threadIdx.x]];
-    s_node[threadIdx.x] = int64_t(t.t0[0]) * p.nx + t.t0[1];
-    s_e[threadIdx.x] = p.e[wb.e_off + threadIdx.x];
-    if (threadIdx.x == 0) s_ix = t.iext[1];
-  } else if (threadIdx.x >= oz::BM && threadIdx.x < oz::BM + oz::BN) {
-    s_f[threadIdx.x - oz::BM] = p.f[un.f_off + int(threadIdx.x) - oz::BM];
-  }
+  tab.fill(p, un, wb, int(threadIdx.x));
   const uint32_t tmem = oz::setup(sh, &s_abort);
   const int k0 = wb.nkb * rank / ks, k1 = wb.nkb * (rank + 1) / ks;
-  const bool any = k1 > k0;
-  if (any)
-    oz::products(sh, tmem, p.a + wb.a_off + size_t(k0) * oz::A_BLOCK, p.b + un.b_off + size_t(k0) * oz::B_BLOCK,
-                 k1 - k0, p.err, &s_abort);
+  SplitWork work{sh, {p.a + wb.a_off + size_t(k0) * oz::A_BLOCK, p.b + un.b_off + size_t(k0) * oz::B_BLOCK, k1 - k0}};
+  oz::run<oz::Fine>(sh, tmem, work, p.err, &s_abort);
   longlong2* sums = reinterpret_cast<longlong2*>(sh.stage);
   cg::cluster_group cl = cg::this_cluster();
-  if (ks > 1) {
-    if (!any)
-      for (int q = threadIdx.x; q < oz::BN * oz::SUM_PITCH; q += blockDim.x) sums[q] = make_longlong2(0, 0);
-    cl.sync();
-  }
+  if (k1 == k0)
+    for (int q = threadIdx.x; q < oz::BN * oz::SUM_PITCH; q += blockDim.x) sums[q] = make_longlong2(0, 0);
+  cl.sync();
   const int lcw = 6 - (31 - __clz(ks)), cw = 1 << lcw, c0 = rank * cw;  // this CTA's columns
   if (!s_abort && c0 < un.ncol) {
-    const int ix = s_ix;
-    const uint32_t inv = div_inv(uint32_t(ix));
-    constexpr int U = 8;  // elements per thread in flight (the state is read before any is written)
+    const StepUnit o{p, un, wb, tab.node0, tab.e, tab.f, tab.ix, div_inv(uint32_t(tab.ix))};
+    constexpr int U = 4;  // elements per thread in flight
     const int total = wb.count * cw;
     for (int q0 = threadIdx.x; q0 < total; q0 += U * oz::THREADS) {
-      int64_t node[U];
+      int64_t where[U];
       double old[U];
+      bool in[U];
 #pragma unroll
       for (int k = 0; k < U; ++k) {
-        const int q = q0 + k * oz::THREADS, col = c0 + (q & (cw - 1)), row = q >> lcw;
-        node[k] = -1;
-        if (q < total && col < un.ncol) {
-          const int i = un.col0 + col, iy = div_by(i, inv);
-          node[k] = s_node[row] + int64_t(iy) * p.nx + (i - iy * ix);
-        }
-        old[k] = p.accumulate && node[k] >= 0 ? p.u[node[k]] : 0.0;
+        const int q = q0 + k * oz::THREADS, row = min(q >> lcw, oz::BM - 1);
+        const int64_t ra = o.row_at(row), ca = o.col_at(c0 + (q & (cw - 1)));
+        in[k] = ra >= 0 && ca >= 0 && q < total;
+        where[k] = ra + ca;
+        old[k] = in[k] ? o.load(where[k], row) : 0.0;
       }
 #pragma unroll
       for (int k = 0; k < U; ++k) {
-        if (node[k] < 0) continue;
+        if (!in[k]) continue;
         const int q = q0 + k * oz::THREADS, col = c0 + (q & (cw - 1)), row = q >> lcw;
         longlong2 v = make_longlong2(0, 0);
-        if (ks == 1) {
-          v = sums[col * oz::SUM_PITCH + row];
-        } else {
-          for (int j = 0; j < ks; ++j) {
-            const longlong2 o = *cl.map_shared_rank(sums + col * oz::SUM_PITCH + row, j);
-            v.x += o.x;
-            v.y += o.y;
-          }
+        for (int j = 0; j < ks; ++j) {
+          const longlong2 s = *cl.map_shared_rank(sums + col * oz::SUM_PITCH + row, j);
+          v.x += s.x;
+          v.y += s.y;
         }
-        const int er = s_e[row], fc = s_f[col];
-        const double y = er == oz::kNonFinite || fc == oz::kNonFinite
-                             ? plain_dot(p, p.tiles[p.order[wb.first + row]], un.col0 + col)
-                             : oz::sums_to_double(v.x, v.y, er + fc - 62);
-        p.u[node[k]] = p.accumulate ? old[k] + y : y;
+        o.store(where[k], oz::sums_to_double(v.x, v.y, o.scale(row, col)), old[k]);
       }
     }
+    // (ten warps: 128 / 8 rows for the first eight)
+    if (threadIdx.x < 256) o.formed(int(threadIdx.x) / 32 * 16, 16, c0, cw, int(threadIdx.x) % 32);
   }
-  if (ks > 1) cl.sync();  // the sums stay until every CTA of the cluster has read them
+  cl.sync();  // the sums stay until every CTA of the cluster has read them
   oz::release(tmem);
 }
 
@@ -290,6 +415,7 @@ struct OzPlan {
   std::vector<PropRows> rows;
   struct Group { int wb0, nwb, unit0, nunits, ks; };
   std::vector<Group> groups;   // window blocks whose digits are held together
+  int nsm = 152;
   size_t a_halves = 0, b_halves = 0;
   int ne = 0, nf = 0;
   WinBlock* d_blocks = nullptr;
@@ -299,6 +425,8 @@ struct OzPlan {
   __half* d_b = nullptr;
   int* d_e = nullptr;
   int* d_f = nullptr;
+  double* d_sv = nullptr;
+  int* d_sk = nullptr;
   int* d_err = nullptr;
 };
 
@@ -352,35 +480,40 @@ void plan_oz(const lem_ctx* ctx, OzPlan* z) {
   close();
 }
 
-// CTAs per unit: the split whose estimated time is least, in clk: a K block takes about 1000, a
-// unit's set-up and scatter about 8000, a cluster's reduction about 4000 more; `slots` CTAs run
-// at once (with clusters, as many as fit beside each other).
-int pick_split(const OzPlan::Group& g, const OzPlan* z) {
+cudaLaunchConfig_t split_config(int ks, int units, cudaStream_t st, cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(units * ks));
+  cfg.blockDim = dim3(oz::THREADS);
+  cfg.dynamicSmemBytes = oz::SMEM;
+  cfg.stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = unsigned(ks);
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// CTAs per unit: the split whose estimated time is least, in clk. A K block takes about 1130; a
+// unit's share of the scatter that the next unit's MMAs do not cover 3000, set-up and the last
+// scatter 12000; with a cluster set-up, reduction and scatter 20000 a wave. As many clusters run
+// at once as fit beside each other.
+int pick_split(const OzPlan::Group& g, const OzPlan* z, int nsm) {
   double kblocks = 0.0;
   for (int q = 0; q < g.nunits; ++q) kblocks = std::max(kblocks, double(z->blocks[z->units[g.unit0 + q].wb].nkb));
   int best = 1;
-  double best_t = 0.0;
-  for (int ks : {1, 2, 4, 8}) {
-    if (ks > 1 && kblocks / ks < 4) break;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(ks);
-    cfg.blockDim = dim3(oz::THREADS);
-    cfg.dynamicSmemBytes = oz::SMEM;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = unsigned(ks);
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+  double best_t = std::ceil(double(g.nunits) / nsm) * (kblocks * 1130.0 + 3000.0) + 12000.0;
+  for (int ks : {2, 4, 8}) {
+    if (kblocks / ks < 4) break;
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = split_config(ks, 1, nullptr, &at);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, oz_step_kernel, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, oz_step_split_kernel, &cfg) != cudaSuccess || n < 1) {
       cudaGetLastError();
-      if (ks > 1) break;
-      n = 152;
+      break;
     }
-    const double waves = std::ceil(double(g.nunits) / n);
-    const double t = waves * (kblocks / ks * 1000.0 + 8000.0 + (ks > 1 ? 4000.0 : 0.0));
-    if (ks == 1 || t < 0.95 * best_t) {
+    const double t = std::ceil(double(g.nunits) / n) * (kblocks / ks * 1130.0 + 20000.0);
+    if (t < 0.95 * best_t) {
       best = ks;
       best_t = t;
     }
@@ -395,7 +528,8 @@ void oz_destroy(lem_ctx* ctx) {
   if (!z) return;
   for (void* p : {static_cast<void*>(z->d_blocks), static_cast<void*>(z->d_units), static_cast<void*>(z->d_rows),
                   static_cast<void*>(z->d_a), static_cast<void*>(z->d_b), static_cast<void*>(z->d_e),
-                  static_cast<void*>(z->d_f), static_cast<void*>(z->d_err)})
+                  static_cast<void*>(z->d_f), static_cast<void*>(z->d_sv), static_cast<void*>(z->d_sk),
+                  static_cast<void*>(z->d_err)})
     if (p) cudaFreeAsync(p, ctx->stream);
   delete z;
   ctx->oz = nullptr;
@@ -408,7 +542,9 @@ lem_status oz_prepare(lem_ctx* ctx) {
   ctx->oz = z;
   plan_oz(ctx, z);
   LEM_CUDA_TRY(cudaFuncSetAttribute(oz_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM));
-  for (auto& g : z->groups) g.ks = pick_split(g, z);
+  LEM_CUDA_TRY(cudaFuncSetAttribute(oz_step_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM));
+  if (cudaDeviceGetAttribute(&z->nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || z->nsm < 1) z->nsm = 152;
+  for (auto& g : z->groups) g.ks = pick_split(g, z, z->nsm);
   auto alloc = [&](auto** p, size_t n) { return dev_alloc(ctx, reinterpret_cast<void**>(p), sizeof(**p) * n); };
   LEM_TRY(alloc(&z->d_blocks, z->blocks.size()));
   LEM_TRY(alloc(&z->d_units, z->units.size()));
@@ -416,6 +552,8 @@ lem_status oz_prepare(lem_ctx* ctx) {
   LEM_TRY(alloc(&z->d_b, z->b_halves));
   LEM_TRY(alloc(&z->d_e, size_t(z->ne)));
   LEM_TRY(alloc(&z->d_f, size_t(z->nf)));
+  LEM_TRY(alloc(&z->d_sv, size_t(z->nf) * SPARSE));
+  LEM_TRY(alloc(&z->d_sk, size_t(z->nf) * SPARSE));
   LEM_TRY(alloc(&z->d_err, 1));
   cudaStream_t st = ctx->stream;
   LEM_CUDA_TRY(cudaMemcpyAsync(z->d_blocks, z->blocks.data(), sizeof(WinBlock) * z->blocks.size(),
@@ -432,7 +570,7 @@ lem_status oz_pack(lem_ctx* ctx) {
   OzPlan* z = ctx->oz;
   if (!z) return LEM_OK;
   oz_prop_kernel<<<unsigned(z->rows.size() * 8), 256, 0, ctx->stream>>>(ctx->d_P, ctx->n_int, ctx->n_loc, z->d_rows,
-                                                                        z->d_f, z->d_b);
+                                                                        z->d_f, z->d_sv, z->d_sk, z->d_b);
   LEM_CUDA_TRY(cudaGetLastError());
   return LEM_OK;
 }
@@ -473,20 +611,16 @@ lem_status step_oz(lem_ctx* ctx, double* d_u) {
     cut<<<unsigned(g.nwb * per), WIN_THREADS, 0, st>>>(src, ctx->d_tiles, ctx->d_class_order, z->d_blocks, g.wb0,
                                                        int(ctx->ny), int(ctx->nx), z->d_e, z->d_a);
     LEM_CUDA_TRY(cudaGetLastError());
-    StepParams p{z->d_blocks, z->d_units, ctx->d_tiles, ctx->d_class_order, z->d_a, z->d_b, z->d_e, z->d_f, ctx->d_P,
-                 src, d_u, ctx->n_int, ctx->n_loc, ctx->ny, ctx->nx, g.unit0, g.ks, phi ? 1 : 0, z->d_err};
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(unsigned(g.nunits * g.ks));
-    cfg.blockDim = dim3(oz::THREADS);
-    cfg.dynamicSmemBytes = oz::SMEM;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = unsigned(g.ks);
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_step_kernel, p));
+    StepParams p{z->d_blocks, z->d_units, ctx->d_tiles, ctx->d_class_order, z->d_a, z->d_b, z->d_e, z->d_f, z->d_sv, z->d_sk, ctx->d_P,
+                 src, d_u, ctx->n_int, ctx->n_loc, ctx->ny, ctx->nx, g.unit0, g.nunits, g.ks, phi ? 1 : 0, z->d_err};
+    if (g.ks == 1) {
+      oz_step_kernel<<<std::min(g.nunits, z->nsm), oz::THREADS, oz::SMEM, st>>>(p);
+      LEM_CUDA_TRY(cudaGetLastError());
+    } else {
+      cudaLaunchAttribute at;
+      const cudaLaunchConfig_t cfg = split_config(g.ks, g.nunits, st, &at);
+      LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_step_split_kernel, p));
+    }
   }
   ctx->timing_end(stop);
   return LEM_OK;
