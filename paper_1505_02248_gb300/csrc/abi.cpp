@@ -113,6 +113,7 @@ void free_ctx(lem_ctx* c) {
   cudaFreeAsync(c->d_Y, c->stream);
   cudaFreeAsync(c->d_state_tmp, c->stream);
   cudaFreeAsync(c->d_status, c->stream);
+  cudaFreeAsync(c->d_ws, c->stream);
   delete c;
 }
 

@@ -593,12 +593,43 @@ __global__ void copy_cols_kernel(double* dst, int64_t ldd, int dcol0, const doub
   dst[int64_t(b) * n * ldd + int64_t(i) * ldd + dcol0 + j] = src[int64_t(b) * n * lds + int64_t(i) * lds + scol0 + j];
 }
 
-// Builder scratch from cudaMallocAsync. It is freed after the build has synchronised its
-// stream, on the legacy stream: that waits for no non-blocking stream, where cudaFree would
-// wait for the whole device.
-struct Buf {
-  double* p = nullptr;
-  ~Buf() { if (p) cudaFreeAsync(p, 0); }
+// Device scratch of one build batch, released when the batch is done. A context that rebuilds
+// (refresh > 0) keeps one block of the size its builds took, up to kKeepBytes, and later batches
+// are laid out in it: taking and returning gigabytes at the stream-ordered pool cost 5 ms of a
+// 27 ms build, since the pool gives them back to the driver at every synchronisation. Otherwise
+// each piece comes from cudaMallocAsync and is freed after the build has synchronised its stream,
+// on the legacy stream: that waits for no non-blocking stream, where cudaFree would wait for the
+// whole device.
+constexpr size_t kKeepBytes = size_t(4) << 30;
+struct Scratch {
+  lem_ctx* ctx;
+  size_t used = 0;
+  std::vector<void*> own;
+  explicit Scratch(lem_ctx* c) : ctx(c) {}
+  Scratch(const Scratch&) = delete;
+  Scratch& operator=(const Scratch&) = delete;
+  lem_status get(void** p, size_t bytes) {
+    const size_t b = (bytes + 255) / 256 * 256, o = used;
+    used += b;
+    if (used <= ctx->ws_bytes) {
+      *p = static_cast<char*>(ctx->d_ws) + o;
+      return LEM_OK;
+    }
+    LEM_CUDA_TRY(cudaMallocAsync(p, b, ctx->stream));
+    own.push_back(*p);
+    return LEM_OK;
+  }
+  template <class T>
+  lem_status get(T** p, size_t count) { return get(reinterpret_cast<void**>(p), sizeof(T) * count); }
+  ~Scratch() {
+    for (void* p : own) cudaFreeAsync(p, 0);
+    if (own.empty() || ctx->desc.refresh <= 0 || !ctx->desc.reaction || used > kKeepBytes) return;
+    // (the batch is over: its stream was synchronised, or the build failed and this context stays unbuilt)
+    if (ctx->d_ws) cudaFreeAsync(ctx->d_ws, ctx->stream);
+    ctx->device_bytes -= int64_t(ctx->ws_bytes);
+    ctx->ws_bytes = 0;
+    if (dev_alloc(ctx, &ctx->d_ws, used) == LEM_OK) ctx->ws_bytes = used;
+  }
 };
 
 inline dim3 grid1(int64_t total, int by) { return dim3(unsigned((total + 255) / 256), by); }
@@ -614,8 +645,7 @@ bool builder_uses_tc(int prec) {
 namespace {
 struct TcGuard {
   TcGemm* g = nullptr;
-  cudaStream_t st = nullptr;
-  ~TcGuard() { tc_gemm_destroy(g, st); }
+  ~TcGuard() { tc_gemm_destroy(g); }
 };
 }  // namespace
 
@@ -643,16 +673,15 @@ static lem_status mul_list(lem_ctx* ctx, TcGemm* tcg, int nbatch, const int* map
 // columns hold Q^{-1} RHS. Panels in FP64, the other columns by products (tcg: on tcgen05). The
 // split apply's propagators keep one product per panel: a group's product rounds otherwise, and
 // the FP16 pieces cut from the propagators would differ.
-static lem_status solve_gj(lem_ctx* ctx, TcGemm* tcg, double* G, int n, int gjcols, int nb, Buf& ybuf, Buf& pivbuf,
-                           Buf& rowbuf) {
+static lem_status solve_gj(lem_ctx* ctx, TcGemm* tcg, double* G, int n, int gjcols, int nb, Scratch& ws) {
   cudaStream_t st = ctx->stream;
   const int group = tcg && !ctx->split ? GJ_SB : GJ_KB;
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&ybuf.p), sizeof(double) * nb * n * GJ_SB, st));
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&pivbuf.p), sizeof(int) * nb * GJ_SB, st));
-  if (!tcg)  // FP64 products write over their right factor: the pivot rows move out first
-    LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&rowbuf.p), sizeof(double) * nb * GJ_KB * gjcols, st));
-  double* Y = ybuf.p;
-  int* piv = reinterpret_cast<int*>(pivbuf.p);
+  double *Y = nullptr, *rows = nullptr;
+  int* piv = nullptr;
+  LEM_TRY(ws.get(&Y, size_t(nb) * n * GJ_SB));
+  LEM_TRY(ws.get(&piv, size_t(nb) * GJ_SB));
+  // FP64 products write over their right factor: the pivot rows move out first
+  if (!tcg) LEM_TRY(ws.get(&rows, size_t(nb) * GJ_KB * gjcols));
   const int64_t sG = int64_t(n) * gjcols, sY = int64_t(n) * GJ_SB;
   for (int s0 = 0; s0 < n; s0 += group) {  // a group of columns
     const int sb = std::min(group, n - s0);
@@ -684,9 +713,9 @@ static lem_status solve_gj(lem_ctx* ctx, TcGemm* tcg, double* G, int n, int gjco
     }
     const int m_r = gjcols - (s0 + sb);
     double* T = G + (s0 + sb);  // the columns behind the group
-    bgj_swap_kernel<<<dim3((m_r + 255) / 256, nb), 256, 0, st>>>(T, gjcols, sG, m_r, 0, 0, s0, sb, piv, rowbuf.p);
+    bgj_swap_kernel<<<dim3((m_r + 255) / 256, nb), 256, 0, st>>>(T, gjcols, sG, m_r, 0, 0, s0, sb, piv, rows);
     LEM_CUDA_TRY(cudaGetLastError());
-    const double* B = tcg ? T + int64_t(s0) * gjcols : rowbuf.p;
+    const double* B = tcg ? T + int64_t(s0) * gjcols : rows;
     const TcProduct pr{m_r, B, tcg ? gjcols : m_r, tcg ? sG : int64_t(sb) * m_r, T, gjcols, sG, T, gjcols, sG, nullptr};
     LEM_TRY(mul_list(ctx, tcg, nb, nullptr, n, sb, Y, GJ_SB, sY, &pr, 1, s0, s0 + sb));
   }
@@ -710,16 +739,16 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
   // device scratch for this batch (freed at return)
   const int nmat = phi ? 15 : 9;
   const int gjcols = phi ? 3 * n : 2 * n;
-  Buf scratch, bcbuf, normbuf, scalebuf, ybuf, pivbuf, rowbuf, mapbuf;
-  size_t bytes = sizeof(double) * (size_t(nmat) * nn + size_t(n) * gjcols) * nb;
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&scratch.p), bytes, st));
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&bcbuf.p), sizeof(BatchClass) * nb, st));
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&normbuf.p), sizeof(double) * nb, st));
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&scalebuf.p), sizeof(double) * 2 * nb, st));
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&mapbuf.p), sizeof(int) * 2 * nb, st));
-  BatchClass* d_bc = reinterpret_cast<BatchClass*>(bcbuf.p);
+  Scratch ws(ctx);
+  double *S = nullptr, *d_norm = nullptr, *d_c = nullptr;
+  BatchClass* d_bc = nullptr;
+  int* d_map = nullptr;
+  LEM_TRY(ws.get(&S, (size_t(nmat) * nn + size_t(n) * gjcols) * nb));
+  LEM_TRY(ws.get(&d_bc, size_t(nb)));
+  LEM_TRY(ws.get(&d_norm, size_t(nb)));
+  LEM_TRY(ws.get(&d_c, size_t(2) * nb));
+  LEM_TRY(ws.get(&d_map, size_t(2) * nb));
   LEM_CUDA_TRY(cudaMemcpyAsync(d_bc, hbc.data(), sizeof(BatchClass) * nb, cudaMemcpyHostToDevice, st));
-  double* S = scratch.p;
   auto M = [&](int i) { return S + size_t(i) * nn * nb; };
   double *Xs = M(0), *T2 = M(1), *T4 = M(2), *T6 = M(3), *TW = M(4), *TV = M(5), *T3 = M(6), *VT = M(7), *UT = M(8);
   double *B2 = nullptr, *B4 = nullptr, *B6 = nullptr, *BW = nullptr, *B3 = nullptr, *UB = nullptr;
@@ -738,12 +767,12 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
         ctx->desc.dt, ctx->desc.reaction, ctx->desc.porous_m);
   LEM_CUDA_TRY(cudaGetLastError());
   // exact 1-norms -> s per class (host decides, same rule as theta_13 scaling)
-  LEM_CUDA_TRY(cudaMemsetAsync(normbuf.p, 0, sizeof(double) * nb, st));
+  LEM_CUDA_TRY(cudaMemsetAsync(d_norm, 0, sizeof(double) * nb, st));
   norm1_kernel<<<dim3((n + 31) / 32, nb), 256, 0, st>>>(
-      Xs, n, reinterpret_cast<unsigned long long*>(normbuf.p));
+      Xs, n, reinterpret_cast<unsigned long long*>(d_norm));
   LEM_CUDA_TRY(cudaGetLastError());
   std::vector<double> norms(nb), scales(2 * nb);
-  LEM_CUDA_TRY(cudaMemcpyAsync(norms.data(), normbuf.p, sizeof(double) * nb, cudaMemcpyDeviceToHost, st));
+  LEM_CUDA_TRY(cudaMemcpyAsync(norms.data(), d_norm, sizeof(double) * nb, cudaMemcpyDeviceToHost, st));
   LEM_CUDA_TRY(cudaStreamSynchronize(st));
   std::vector<int> s(nb);
   int smax = 0;
@@ -757,8 +786,7 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
     scales[b] = std::ldexp(1.0, -sb);                       // c = 2^-s
     scales[nb + b] = std::ldexp(1.0, -sb) * (kPadeInt[1] / kPadeInt[0]);  // c * b1
   }
-  double* d_c = scalebuf.p;
-  double* d_cb1 = scalebuf.p + nb;
+  double* d_cb1 = d_c + nb;
   LEM_CUDA_TRY(cudaMemcpyAsync(d_c, scales.data(), sizeof(double) * 2 * nb, cudaMemcpyHostToDevice, st));
   // Classes sorted by s, descending: at squaring q the classes still squaring (s > q) are a
   // prefix of the order, so one index map serves every squaring. A class that stops an odd
@@ -767,16 +795,18 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
   std::iota(order.begin(), order.begin() + nb, 0);
   std::stable_sort(order.begin(), order.begin() + nb, [&](int a, int b) { return s[a] > s[b]; });
   for (int b = 0; b < nb; ++b) order[nb + b] = (smax - s[b]) & 1;
-  const int* d_map = reinterpret_cast<const int*>(mapbuf.p);
   const int* d_odd = d_map + nb;
-  LEM_CUDA_TRY(cudaMemcpyAsync(mapbuf.p, order.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
+  LEM_CUDA_TRY(cudaMemcpyAsync(d_map, order.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
 
   PadeTerms pt{};
   for (int j = 0; j < 14; ++j) pt.b[j] = kPadeInt[j] / kPadeInt[0];
   const dim3 gsq = grid1(nn, nb);
   TcGuard tc;
-  tc.st = st;
-  if (ctx->build_tc) LEM_TRY(tc_gemm_create(n, nb, gjcols, phi ? 4 : 2, st, &tc.g));
+  if (ctx->build_tc) {
+    char* mem = nullptr;
+    LEM_TRY(ws.get(&mem, tc_gemm_bytes(n, nb, gjcols, phi ? 4 : 2)));
+    LEM_TRY(tc_gemm_create(n, nb, gjcols, phi ? 4 : 2, mem, st, &tc.g));
+  }
   // C = A B (+ D, which may be C) (+ diag I) for every product of the list, on the first nact
   // classes of the order (nact == nb: all)
   struct Term { const double* B; const double* D; double* C; const double* diag; };
@@ -815,7 +845,7 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
   solve_system_kernel<<<gsq, 256, 0, st>>>(G, n, gjcols, VT, UT, UB);
   LEM_CUDA_TRY(cudaGetLastError());
   LEM_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
-  LEM_TRY(solve_gj(ctx, tc.g, G, n, gjcols, nb, ybuf, pivbuf, rowbuf));
+  LEM_TRY(solve_gj(ctx, tc.g, G, n, gjcols, nb, ws));
   LEM_CUDA_TRY(cudaGetLastError());
   // R_T and R_B, then the squarings (R_T, R_B)^2 = (R_T^2, R_T R_B + R_B)
   double *RT = T2, *RTn = T4, *RB = B2, *RBn = B4;
@@ -847,8 +877,6 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
   int status = 0;
   LEM_CUDA_TRY(cudaMemcpyAsync(&status, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
   LEM_CUDA_TRY(cudaStreamSynchronize(st));
-  // scratch is released by the Buf destructors (stream-ordered frees are unnecessary
-  // after the synchronisation above)
   if (status != 0) return fail(LEM_ENUMERIC, "singular Pade denominator (V - U) in the propagator build");
   if (tc.g) LEM_TRY(tc_gemm_check(tc.g, st));
   return LEM_OK;
@@ -884,15 +912,16 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   }
   constexpr int NAUG = 10;  // Z, Z2, Z4, Z6, W, W3, U, V, R, Rn
   const int gjcols = 5 * n;
-  Buf scratch, bcbuf, normbuf, scalebuf, ybuf, pivbuf, rowbuf, mapbuf;
-  const size_t bytes = sizeof(double) * (size_t(NAUG) * 4 * nn + size_t(n) * gjcols) * nb;
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&scratch.p), bytes, st));
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&bcbuf.p), sizeof(BatchClass) * nb, st));
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&normbuf.p), sizeof(double) * nb, st));
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&scalebuf.p), sizeof(double) * nb, st));
-  BatchClass* d_bc = reinterpret_cast<BatchClass*>(bcbuf.p);
+  Scratch ws(ctx);
+  double *S = nullptr, *d_norm = nullptr, *d_scale = nullptr;
+  BatchClass* d_bc = nullptr;
+  int* d_map = nullptr;
+  LEM_TRY(ws.get(&S, (size_t(NAUG) * 4 * nn + size_t(n) * gjcols) * nb));
+  LEM_TRY(ws.get(&d_bc, size_t(nb)));
+  LEM_TRY(ws.get(&d_norm, size_t(nb)));
+  LEM_TRY(ws.get(&d_scale, size_t(nb)));
+  LEM_TRY(ws.get(&d_map, size_t(2) * nb));
   LEM_CUDA_TRY(cudaMemcpyAsync(d_bc, hbc.data(), sizeof(BatchClass) * nb, cudaMemcpyHostToDevice, st));
-  double* S = scratch.p;
   auto aug = [&](int i) {
     Aug a;
     for (int q = 0; q < 4; ++q) a.m[q] = S + (size_t(i) * 4 + q) * nn * nb;
@@ -909,12 +938,12 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   assemble_local_kernel<<<dim3((n + 127) / 128, nb), 128, 0, st>>>(
       Z.m[0], n, d_bc, nb, ctx->d_coef, ctx->desc.coef_stride, ctx->ny, ctx->nx, ctx->desc.ndim, u, ctx->desc.dt,
       ctx->desc.reaction, ctx->desc.porous_m);
-  LEM_CUDA_TRY(cudaMemsetAsync(normbuf.p, 0, sizeof(double) * nb, st));
+  LEM_CUDA_TRY(cudaMemsetAsync(d_norm, 0, sizeof(double) * nb, st));
   norm1_kernel<<<dim3((n + 31) / 32, nb), 256, 0, st>>>(Z.m[0], n,
-                                                           reinterpret_cast<unsigned long long*>(normbuf.p));
+                                                           reinterpret_cast<unsigned long long*>(d_norm));
   LEM_CUDA_TRY(cudaGetLastError());
   std::vector<double> norms(nb), scales(nb);
-  LEM_CUDA_TRY(cudaMemcpyAsync(norms.data(), normbuf.p, sizeof(double) * nb, cudaMemcpyDeviceToHost, st));
+  LEM_CUDA_TRY(cudaMemcpyAsync(norms.data(), d_norm, sizeof(double) * nb, cudaMemcpyDeviceToHost, st));
   LEM_CUDA_TRY(cudaStreamSynchronize(st));
   std::vector<int> s(nb);
   int smax = 0;
@@ -927,7 +956,7 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
     ctx->squarings[c0 + b] = sb;
     scales[b] = std::ldexp(1.0, -sb);
   }
-  LEM_CUDA_TRY(cudaMemcpyAsync(scalebuf.p, scales.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, st));
+  LEM_CUDA_TRY(cudaMemcpyAsync(d_scale, scales.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, st));
 
   const dim3 gsq = grid1(nn, nb);
   auto lin = [&](double* out, std::initializer_list<std::pair<const double*, double>> terms, double diag,
@@ -948,8 +977,11 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
     return e == cudaSuccess ? LEM_OK : cuda_fail(e, "lincomb_kernel");
   };
   TcGuard tc;
-  tc.st = st;
-  if (ctx->build_tc) LEM_TRY(tc_gemm_create(n, nb, gjcols, 4, st, &tc.g));
+  if (ctx->build_tc) {
+    char* mem = nullptr;
+    LEM_TRY(ws.get(&mem, tc_gemm_bytes(n, nb, gjcols, 4)));
+    LEM_TRY(tc_gemm_create(n, nb, gjcols, 4, mem, st, &tc.g));
+  }
   // one A against four B
   auto mul4 = [&](int nact, const int* map, const double* A, const double* const (&B)[4], const double* const (&D)[4],
                   double* const (&C)[4]) -> lem_status {
@@ -994,7 +1026,7 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   };
 
   // Z(Xs): T = X / 2^s, B = (I, 0, 0), Toeplitz part N (b = (0, 1, 0))
-  LEM_TRY(lin(Z.m[0], {{Z.m[0], 1.0}}, 0.0, scalebuf.p));
+  LEM_TRY(lin(Z.m[0], {{Z.m[0], 1.0}}, 0.0, d_scale));
   LEM_TRY(lin(Z.m[1], {}, 1.0, nullptr));
   LEM_CUDA_TRY(cudaMemsetAsync(Z.m[2], 0, sizeof(double) * nn * nb, st));
   LEM_CUDA_TRY(cudaMemsetAsync(Z.m[3], 0, sizeof(double) * nn * nb, st));
@@ -1029,7 +1061,7 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   for (int q = 0; q < 4; ++q) copy_cols_kernel<<<gsq, 256, 0, st>>>(G, gjcols, (1 + q) * n, W3.m[q], n, 0, n, n);
   LEM_CUDA_TRY(cudaGetLastError());
   LEM_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
-  LEM_TRY(solve_gj(ctx, tc.g, G, n, gjcols, nb, ybuf, pivbuf, rowbuf));
+  LEM_TRY(solve_gj(ctx, tc.g, G, n, gjcols, nb, ws));
   for (int q = 0; q < 4; ++q) copy_cols_kernel<<<gsq, 256, 0, st>>>(R.m[q], n, 0, G, gjcols, (1 + q) * n, n, n);
   LEM_CUDA_TRY(cudaGetLastError());
 
@@ -1051,9 +1083,7 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   // classes that stop squaring an odd number of steps early have their result in the other buffer
   order.resize(2 * nb);
   for (int b = 0; b < nb; ++b) order[nb + b] = (smax - s[b]) & 1;
-  LEM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&mapbuf.p), sizeof(int) * 2 * nb, st));
-  LEM_CUDA_TRY(cudaMemcpyAsync(mapbuf.p, order.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
-  const int* d_map = reinterpret_cast<const int*>(mapbuf.p);
+  LEM_CUDA_TRY(cudaMemcpyAsync(d_map, order.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
   const int* d_odd = d_map + nb;
   for (int q = 0; q < smax; ++q) {
     int nact = 0;

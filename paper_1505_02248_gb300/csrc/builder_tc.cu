@@ -253,18 +253,13 @@ struct TcGemm {
 
 size_t tc_gemm_bytes(int n, int nb, int gjcols, int np) {
   const Caps c = caps_for(n, nb, gjcols, np);
-  return sizeof(__half) * (c.a + c.b) + sizeof(int) * (c.e + c.f) + 16;
+  return sizeof(__half) * (c.a + c.b) + sizeof(int) * (c.e + c.f) + 256;
 }
 
-void tc_gemm_destroy(TcGemm* g, cudaStream_t st) {
-  if (!g) return;
-  for (void* q : {static_cast<void*>(g->sa), static_cast<void*>(g->sb), static_cast<void*>(g->e),
-                  static_cast<void*>(g->f), static_cast<void*>(g->err)})
-    if (q) cudaFreeAsync(q, st);
-  delete g;
-}
+void tc_gemm_destroy(TcGemm* g) { delete g; }
 
-lem_status tc_gemm_create(int n, int nb, int gjcols, int np, cudaStream_t st, TcGemm** out) {
+// mem: tc_gemm_bytes of device memory (256-byte aligned) that outlives the workspace
+lem_status tc_gemm_create(int n, int nb, int gjcols, int np, void* mem, cudaStream_t st, TcGemm** out) {
   *out = nullptr;
   // the shared-memory attribute is per device (cheap to set again)
   if (cudaFuncSetAttribute(oz_mul_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM) != cudaSuccess)
@@ -278,17 +273,14 @@ lem_status tc_gemm_create(int n, int nb, int gjcols, int np, cudaStream_t st, Tc
   if (cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && nsm > 0)
     g->nsm = nsm;
-  auto alloc = [&](auto** p, size_t count) -> bool {
-    if (cudaMallocAsync(reinterpret_cast<void**>(p), sizeof(**p) * count, st) == cudaSuccess) return true;
-    cudaGetLastError();
-    return false;
-  };
-  if (!alloc(&g->sa, c.a) || !alloc(&g->sb, c.b) || !alloc(&g->e, c.e) || !alloc(&g->f, c.f) || !alloc(&g->err, 1)) {
-    tc_gemm_destroy(g, st);
-    return fail(LEM_ENOMEM, "tensor-core build workspace");
-  }
+  // (every part but the last is a whole number of digit blocks or of 64 integers)
+  g->sa = static_cast<__half*>(mem);
+  g->sb = g->sa + c.a;
+  g->e = reinterpret_cast<int*>(g->sb + c.b);
+  g->f = g->e + c.e;
+  g->err = g->f + c.f;
   if (cudaMemsetAsync(g->err, 0, sizeof(int), st) != cudaSuccess) {
-    tc_gemm_destroy(g, st);
+    tc_gemm_destroy(g);
     return cuda_fail(cudaGetLastError(), "tensor-core build workspace");
   }
   *out = g;

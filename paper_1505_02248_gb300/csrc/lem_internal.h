@@ -112,6 +112,8 @@ struct lem_ctx {
   double* d_Y = nullptr;               // ntiles * n_int (local results)
   double* d_state_tmp = nullptr;       // npts (host-state path)
   int* d_status = nullptr;             // device error word
+  void* d_ws = nullptr;                // builder scratch kept between refreshes (builder.cu)
+  size_t ws_bytes = 0;
   int64_t device_bytes = 0;
   lem::SplitPlan* split = nullptr;
   lem::OzPlan* oz = nullptr;           // FP64 GEMM apply path: digit products on the tensor cores
@@ -209,8 +211,8 @@ struct TcProduct {
 // workspace for products of nb matrices of n x n with up to np right factors at once, and for
 // rank-256 updates of n x gjcols ones
 size_t tc_gemm_bytes(int n, int nb, int gjcols, int np);
-lem_status tc_gemm_create(int n, int nb, int gjcols, int np, cudaStream_t st, TcGemm** out);
-void tc_gemm_destroy(TcGemm* g, cudaStream_t st);
+lem_status tc_gemm_create(int n, int nb, int gjcols, int np, void* mem, cudaStream_t st, TcGemm** out);
+void tc_gemm_destroy(TcGemm* g);
 // the products of one A with every right factor of the list, on strided batches of row-major
 // FP64 matrices (A M x K, B K x N)
 lem_status tc_gemm(TcGemm* g, int nbatch, const int* map, int M, int K, const double* A, int64_t lda,
