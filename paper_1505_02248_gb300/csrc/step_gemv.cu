@@ -269,14 +269,19 @@ lem_status gemv_prepare_f32(lem_ctx* ctx) {
 // propagator (four rows per warp) and writes the owner values of u^{n+1} into the other state
 // buffer; one grid barrier ends the step. Linear real problems on the GEMV path only (no
 // Jacobian refresh, one scheme stage).
-// SMEMP: one tile per block, its propagator kept in shared memory for all steps.
+// A tile's owner rows are shared out over rsplit blocks (each stages the tile's window), so that a
+// handful of tiles still uses the device: the FP64 pipe does 2 multiply-adds per clock and SM, and
+// one block per tile of 64 x 96 took most of a step (1024 nodes, 16 tiles: 5.6 us a step; with 8
+// blocks of 8 rows a tile 4.2, of which the grid barrier is the larger part).
+// SMEMP: one share of a tile per block, its propagator rows kept in shared memory for all steps.
+static int persist_threads(int rsplit) { return rsplit > 1 ? 128 : 256; }
 template <typename PT, bool SMEMP>
 __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restrict__ P, int64_t n_int, int64_t n_loc,
                                                               const TileDesc* __restrict__ tiles, int ntiles,
                                                               const double* __restrict__ coef, int64_t cstride,
                                                               int64_t ny, int64_t nx, int ndim, int pery, int perx,
                                                               int phi, double* __restrict__ src,
-                                                              double* __restrict__ u, int nsteps) {
+                                                              double* __restrict__ u, int nsteps, int rsplit) {
   namespace cg = cooperative_groups;
   cg::grid_group grid = cg::this_grid();
   extern __shared__ __align__(16) unsigned char wraw[];
@@ -287,9 +292,18 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
   using Acc = typename std::conditional<sizeof(PT) == 8, AccD, AccF>::type;
   // SMEMP: the block's tile propagator (n_int x n_loc) after the window buffer
   PT* Ps = reinterpret_cast<PT*>(wraw + ((sizeof(double) * size_t(n_loc) + 15) & ~size_t(15)));
+  // owner rows [*ib, *ie) of share `part` of a tile (shares are whole groups of 4 rows)
+  auto share = [&](const TileDesc& td, int part, int* ib, int* ie) {
+    const int owners = td.iext[0] * td.iext[1], per = ((owners + rsplit - 1) / rsplit + 3) / 4 * 4;
+    *ib = min(owners, part * per);
+    *ie = min(owners, *ib + per);
+  };
   if (SMEMP) {
-    const PT* src_p = P + int64_t(tiles[blockIdx.x].cls) * n_int * n_loc;
-    for (int64_t e = threadIdx.x; e < n_int * n_loc; e += blockDim.x) Ps[e] = src_p[e];
+    const TileDesc td = tiles[blockIdx.x / rsplit];
+    int ib, ie;
+    share(td, blockIdx.x % rsplit, &ib, &ie);
+    const PT* src_p = P + (int64_t(td.cls) * n_int + ib) * n_loc;
+    for (int64_t e = threadIdx.x; e < (ie - ib) * n_loc; e += blockDim.x) Ps[e] = src_p[e];
     __syncthreads();
   }
   // u^n and u^{n+1} alternate between u and src (every node has exactly one owner tile, so
@@ -297,9 +311,11 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
   double* cur = u;
   double* nxt = src;
   for (int step = 0; step < nsteps; ++step) {
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-      const TileDesc td = tiles[t];
+    for (int t = blockIdx.x; t < ntiles * rsplit; t += gridDim.x) {
+      const TileDesc td = tiles[t / rsplit];
       const int wl = td.wext[0] * td.wext[1];
+      int ib, ie;
+      share(td, t % rsplit, &ib, &ie);
       // the window's source from u^n: the residual dt A u^n at each window node (PHI), or u^n
       for (int k = threadIdx.x; k < wl; k += blockDim.x) {
         const int a = k / td.wext[1], b = k % td.wext[1];
@@ -326,14 +342,13 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
         w[k] = PT(v);
       }
       __syncthreads();
-      const PT* Pt = SMEMP ? Ps : P + int64_t(td.cls) * n_int * n_loc;
-      const int ie = td.iext[0] * td.iext[1];
+      const PT* Pt = SMEMP ? Ps - int64_t(ib) * n_loc : P + int64_t(td.cls) * n_int * n_loc;
       constexpr int V = 16 / sizeof(PT);
       const bool vec = (n_loc % V) == 0 && (wl % V) == 0;
-      for (int i0 = warp * 4; i0 < ie; i0 += nw * 4) {
+      for (int i0 = ib + warp * 4; i0 < ie; i0 += nw * 4) {
         const int i = i0 + grp;
         const bool live = i < ie;
-        const PT* row = Pt + int64_t(live ? i : 0) * n_loc;
+        const PT* row = Pt + int64_t(live ? i : ib) * n_loc;
         // the same partition of a row over the 8 lanes, and the same order, as gemv_tiles_kernel
         // (16-byte chunks j = lane, lane + 8, ... when rows allow them): bit-identical results
         Acc acc;
@@ -368,8 +383,10 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
       u[p] = cur[p];
 }
 
-// Whether lem_step may run its steps in one persistent launch, and with how many blocks.
-static int persistent_blocks(lem_ctx* ctx, bool f32, int nsteps) {
+// Whether lem_step may run its steps in one persistent launch, and with how many blocks; *rsplit:
+// blocks per tile (at most one block per SM then, of 8 rows at least).
+static int persistent_blocks(lem_ctx* ctx, bool f32, int nsteps, int* rsplit) {
+  *rsplit = 1;
   const lem_problem_desc& d = ctx->desc;
   if (nsteps < 2 || d.reaction || d.scheme != LEM_SCHEME_EULER || ctx->cplx) return 0;
   if (ctx->npts > (int64_t(1) << 20) || ctx->tiles.size() > 4096) return 0;
@@ -381,26 +398,31 @@ static int persistent_blocks(lem_ctx* ctx, bool f32, int nsteps) {
     return 0;
   }
   const size_t smem = sizeof(double) * size_t(ctx->n_loc);
-  cudaError_t e = f32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemv_persistent_kernel<float, false>, 256, smem)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemv_persistent_kernel<double, false>, 256, smem);
+  // one block per share of a tile, within what the device holds at once
+  const int64_t nt = int64_t(ctx->tiles.size());
+  *rsplit = int(std::max<int64_t>(1, std::min<int64_t>(nsm / nt, ctx->n_int / 8)));
+  const int threads = persist_threads(*rsplit);
+  cudaError_t e = f32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemv_persistent_kernel<float, false>, threads, smem)
+                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemv_persistent_kernel<double, false>, threads, smem);
   if (e != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     return 0;
   }
-  // one block per tile, within what the device holds at once
-  return int(std::min<int64_t>(int64_t(per_sm) * nsm, int64_t(ctx->tiles.size())));
+  return int(std::min<int64_t>(int64_t(per_sm) * nsm, nt * *rsplit));
 }
 
 lem_status step_gemv_multi(lem_ctx* ctx, double* d_u, int nsteps, bool f32, bool* done) {
   *done = false;
-  const int blocks = persistent_blocks(ctx, f32, nsteps);
+  int rsplit = 1;
+  const int blocks = persistent_blocks(ctx, f32, nsteps, &rsplit);
   if (blocks < 1) return LEM_OK;
   if (f32 && ctx->p32_gen != ctx->build_gen) LEM_TRY(gemv_prepare_f32(ctx));
   const lem_problem_desc& d = ctx->desc;
-  // one tile per block with a propagator small enough for shared memory: keep it there
+  // one share per block with propagator rows few enough for shared memory: keep them there
   const size_t wbytes = (sizeof(double) * size_t(ctx->n_loc) + 15) & ~size_t(15);
-  const size_t pbytes = (f32 ? sizeof(float) : sizeof(double)) * size_t(ctx->n_int) * size_t(ctx->n_loc);
-  bool smemp = blocks == int(ctx->tiles.size()) && wbytes + pbytes <= 200 * 1024 &&
+  const size_t rows = size_t((ctx->n_int + rsplit - 1) / rsplit + 3) / 4 * 4;
+  const size_t pbytes = (f32 ? sizeof(float) : sizeof(double)) * rows * size_t(ctx->n_loc);
+  bool smemp = int64_t(blocks) == int64_t(ctx->tiles.size()) * rsplit && wbytes + pbytes <= 200 * 1024 &&
                std::getenv("LEM_NO_SMEM_P") == nullptr;
   const void* fn_s = f32 ? reinterpret_cast<const void*>(gemv_persistent_kernel<float, true>)
                          : reinterpret_cast<const void*>(gemv_persistent_kernel<double, true>);
@@ -408,7 +430,7 @@ lem_status step_gemv_multi(lem_ctx* ctx, double* d_u, int nsteps, bool f32, bool
     int per_sm = 0, nsm = 0;
     if (cudaFuncSetAttribute(fn_s, cudaFuncAttributeMaxDynamicSharedMemorySize, int(wbytes + pbytes)) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_s, 256, wbytes + pbytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_s, persist_threads(rsplit), wbytes + pbytes) != cudaSuccess ||
         int64_t(per_sm) * nsm < blocks) {
       cudaGetLastError();
       smemp = false;
@@ -423,10 +445,10 @@ lem_status step_gemv_multi(lem_ctx* ctx, double* d_u, int nsteps, bool f32, bool
   int64_t n_int = ctx->n_int, n_loc = ctx->n_loc, cstride = d.coef_stride, ny = ctx->ny, nx = ctx->nx;
   const void* P = f32 ? static_cast<const void*>(ctx->d_P32) : static_cast<const void*>(ctx->d_P);
   void* args[] = {&P, &n_int, &n_loc, &ctx->d_tiles, &ntiles, &ctx->d_coef, &cstride, &ny, &nx,
-                  &ndim, &pery, &perx, &phi, &ctx->d_r, &d_u, &nsteps};
+                  &ndim, &pery, &perx, &phi, &ctx->d_r, &d_u, &nsteps, &rsplit};
   cudaEvent_t stop;
   LEM_CUDA_TRY(ctx->timing_begin(&stop));
-  LEM_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(256), args, smem, ctx->stream));
+  LEM_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(persist_threads(rsplit)), args, smem, ctx->stream));
   ctx->timing_end(stop);
   *done = true;
   return LEM_OK;
