@@ -24,6 +24,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "gemv_acc.cuh"
 #include "lem_internal.h"
 
 namespace lem {
@@ -154,24 +155,27 @@ __device__ __forceinline__ void box_origin(const BandClass& c, int d, int& py, i
   x0 = min(max(px - c.lx, 0), c.wx - c.bxc);
 }
 
-// grid (owner rows, classes): row d of class c as its stored box (FP64, and FP32 if Pb32)
+// grid (owner rows, classes): row d of class c as its stored box. interleaved: chunk q (16 bytes) of
+// rows 32 g .. 32 g + 31 lie back to back, so that a warp with one row per lane reads 512
+// consecutive bytes per chunk (row by row, each of its loads touched 32 lines).
+template <typename PT>
 __global__ void band_pack_kernel(const double* __restrict__ P, int64_t n_int, int64_t n_loc,
-                                 const BandClass* __restrict__ cls, double* __restrict__ Pb,
-                                 float* __restrict__ Pb32) {
+                                 const BandClass* __restrict__ cls, int interleaved, PT* __restrict__ Pb) {
+  constexpr int V = 16 / sizeof(PT);
   const BandClass c = cls[blockIdx.y];
   const int d = blockIdx.x;
   if (d >= c.iy * c.ix) return;
   int py, px, y0, x0;
   box_origin(c, d, py, px, y0, x0);
   const double* row = P + (int64_t(blockIdx.y) * n_int + d) * n_loc;
-  const int64_t o = c.off + int64_t(d) * c.L;
   for (int k = threadIdx.x; k < c.L; k += blockDim.x) {
     const int a = k / c.bxp, j = k % c.bxp;
     const int y = y0 + a, x = x0 + j;
     const bool keep = j < c.bxc && y - py >= -c.ly && y - py <= c.hy && x - px >= -c.lx && x - px <= c.hx;
     const double v = keep ? row[y * c.wx + x] : 0.0;
-    Pb[o + k] = v;
-    if (Pb32) Pb32[o + k] = float(v);
+    const int64_t at = interleaved ? c.off + int64_t(d / 32) * 32 * c.L + int64_t(k / V) * 32 * V + (d % 32) * V + k % V
+                                   : c.off + int64_t(d) * c.L + k;
+    Pb[at] = PT(v);
   }
 }
 
@@ -313,59 +317,78 @@ __global__ void __launch_bounds__(256) gemv_band_kernel(const PT* __restrict__ P
   }
 }
 
-// Short box rows (1D windows, small 2D boxes): one thread per owner row, no reduction. Each
-// thread walks its row's chunks in order with BU 16-byte loads ahead (read-only path, so the
-// other half of each 32-byte sector a warp touches is still in L1 when the next chunk needs
-// it), box coordinates (a, j) advanced incrementally. FP32 rows sum a chunk's products by FMA
-// and add the chunk sum into a float-float accumulator; FP64 rows use FMAs throughout.
+// What the one-thread-per-row kernel needs of a tile and its class, in one record (one load before
+// the row's chunks can start instead of two dependent ones).
+struct BandTile {
+  int org[2], t0[2];
+  int wy, wx, ix, oy, ox, ly, lx, byc, bxc, bxp, rows, L;
+  int64_t off;
+};
+
+// Short box rows (1D windows, small 2D boxes): one thread per owner row, no reduction. Each thread
+// walks its row's chunks in order, BU 16-byte loads ahead, its warp's rows interleaved chunk by
+// chunk; box coordinates (a, j) advance incrementally. FP32 rows sum a chunk's products by FMA and
+// add the chunk sum into a float-float accumulator; FP64 rows use FMAs throughout.
+// Bound by the latency of a block's chain of loads. 300 001 nodes, tiles of 64 + 2 x 16, boxes of about
+// 36 FP32 values (43 MB), a call of ten steps: 220 us with rows stored one after another and every
+// block's first load behind the residual; 159 us interleaved, kept in L2 and chained, so that the
+// first boxes are on their way while the residual runs (two chunks ahead 164, five 170, eight, with
+// fewer blocks resident, 193, and 204 passing through L2). Warps with shares of their own, and the
+// residual formed in the windows instead of its own launch, were slower (178 us and 198).
 template <typename PT>
 __global__ void __launch_bounds__(256) gemv_band_row_kernel(const PT* __restrict__ Pb,
-                                                            const BandClass* __restrict__ cls,
-                                                            const TileDesc* __restrict__ tiles,
+                                                            const BandTile* __restrict__ tiles,
                                                             const double* __restrict__ src, double* __restrict__ u,
-                                                            int64_t ny, int64_t nx, int accumulate, int rsplit) {
+                                                            int64_t ny, int64_t nx, int accumulate, int rsplit,
+                                                            int keep) {
   extern __shared__ __align__(16) unsigned char wraw[];
   PT* w = reinterpret_cast<PT*>(wraw);
   const int t = blockIdx.x / rsplit, part = blockIdx.x % rsplit;
-  const TileDesc td = tiles[t];
-  const BandClass c = cls[td.cls];
-  const int ien = td.iext[0] * td.iext[1];
-  const int rows_per = (ien + rsplit - 1) / rsplit;
-  const int ib = part * rows_per, ie = min(ien, ib + rows_per);
+  const BandTile c = tiles[t];
+  const int rows_per = ((c.rows + rsplit - 1) / rsplit + 31) / 32 * 32;
+  const int ib = part * rows_per, ie = min(c.rows, ib + rows_per);
+  if (ib >= ie) return;
   constexpr int V = 16 / sizeof(PT);
   const int cpr = c.bxp / V;
   const int nch = c.byc * cpr;
   int i = ib + int(threadIdx.x);
   int4 v[BU];
+  const unsigned long long policy = l2_policy(keep);
   auto load = [&](int row, int q0, int4 (&dst)[BU]) {
     const bool live = row < ie;
-    const int4* r4 = reinterpret_cast<const int4*>(Pb + c.off + int64_t(live ? row : ib) * c.L);
+    const int4* r4 = reinterpret_cast<const int4*>(Pb + c.off + int64_t((live ? row : ib) / 32) * 32 * c.L) +
+                     (live ? row : ib) % 32;
 #pragma unroll
-    for (int k = 0; k < BU; ++k) dst[k] = (live && q0 + k < nch) ? __ldg(r4 + q0 + k) : make_int4(0, 0, 0, 0);
+    for (int k = 0; k < BU; ++k)
+      dst[k] = (live && q0 + k < nch) ? load_policy(r4 + (q0 + k) * 32, policy) : make_int4(0, 0, 0, 0);
   };
   load(i, 0, v);  // in flight while the window is staged
-  const int wn = td.wext[0] * td.wext[1];
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (chained: the window's source is written from here on)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int wn = c.wy * c.wx;
   for (int k = threadIdx.x; k < wn + 4; k += blockDim.x) {
     if (k >= wn) {  // padding read by the last chunk of a box row (its P values are zero)
       w[k] = PT(0);
       continue;
     }
-    const int a = k / td.wext[1], b = k % td.wext[1];
-    int64_t gy = int64_t(td.org[0]) + a, gx = int64_t(td.org[1]) + b;
+    const int a = c.wy > 1 ? k / c.wx : 0, b = k - a * c.wx;
+    int64_t gy = int64_t(c.org[0]) + a, gx = int64_t(c.org[1]) + b;
     gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
     gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
-    w[k] = PT(src[gy * nx + gx]);
+    to_prec(src[gy * nx + gx], w[k]);
   }
   __syncthreads();
   for (; i < ie; i += blockDim.x) {
-    int py, px, y0, x0;
-    box_origin(c, i, py, px, y0, x0);
+    const int iy = i / c.ix, jx = i - iy * c.ix;
+    const int y0 = min(max(c.oy + iy - c.ly, 0), c.wy - c.byc), x0 = min(max(c.ox + jx - c.lx, 0), c.wx - c.bxc);
+    const int64_t p = int64_t(c.t0[0] + iy) * nx + c.t0[1] + jx;
+    const double before = accumulate ? u[p] : 0.0;
     double acc = 0.0;
     float hi = 0.0f, lo = 0.0f;
     int a = 0, j = 0;  // box row and chunk of chunk q
     for (int q0 = 0; q0 < nch; q0 += BU) {
       int4 nv[BU];
-      load(i, q0 + BU, nv);
+      if (q0 + BU < nch) load(i, q0 + BU, nv);
 #pragma unroll
       for (int k = 0; k < BU; ++k) {
         if (q0 + k < nch) {
@@ -392,9 +415,8 @@ __global__ void __launch_bounds__(256) gemv_band_row_kernel(const PT* __restrict
 #pragma unroll
       for (int k = 0; k < BU; ++k) v[k] = nv[k];
     }
-    const double y = sizeof(PT) == 8 ? acc : double(hi) + double(lo);
-    const int64_t p = int64_t(td.t0[0] + i / td.iext[1]) * nx + td.t0[1] + i % td.iext[1];
-    u[p] = accumulate ? u[p] + y : y;
+    const double y = sizeof(PT) == 8 ? acc : f32_to_f64(hi) + f32_to_f64(lo);
+    u[p] = accumulate ? before + y : y;
     load(i + int(blockDim.x), 0, v);
   }
 }
@@ -405,7 +427,6 @@ using BandKernel = void (*)(const PT*, const BandClass*, const TileDesc*, const 
 
 template <typename PT>
 BandKernel<PT> band_kernel_for(int lpr) {
-  if (lpr == 1) return gemv_band_row_kernel<PT>;
   if (lpr == 2) return gemv_band_kernel<PT, 2>;
   if (lpr == 4) return gemv_band_kernel<PT, 4>;
   return gemv_band_kernel<PT, 8>;
@@ -453,14 +474,15 @@ struct BandPlan {
   int64_t cap = 0;  // values the packed arrays hold
   int64_t used = 0;
   int wmax = 0;     // largest window (nodes) of any class, for the staged window
-  BandLaunch l64, l32;  // launch shapes for FP64 and FP32 boxes
+  BandLaunch launch;
+  BandTile* d_tiles = nullptr;  // one-thread-per-row kernels only
 };
 
 void band_destroy(lem_ctx* ctx) {
   BandPlan* b = ctx->band;
   if (!b) return;
   for (void* p : {static_cast<void*>(b->d_cls), static_cast<void*>(b->d_ext), static_cast<void*>(b->d_Pb),
-                  static_cast<void*>(b->d_Pb32)})
+                  static_cast<void*>(b->d_Pb32), static_cast<void*>(b->d_tiles)})
     if (p) cudaFreeAsync(p, ctx->stream);
   delete b;
   ctx->band = nullptr;
@@ -503,6 +525,7 @@ lem_status band_prepare(lem_ctx* ctx) {
   LEM_CUDA_TRY(cudaMemcpyAsync(ext.data(), b->d_ext, sizeof(int) * ext.size(), cudaMemcpyDeviceToHost, st));
   LEM_CUDA_TRY(cudaStreamSynchronize(st));
   int64_t total = 0;
+  b->used = 0;
   for (int k = 0; k < nc; ++k) {
     BandClass& c = b->cls[k];
     c.ly = ext[4 * k]; c.hy = ext[4 * k + 1]; c.lx = ext[4 * k + 2]; c.hx = ext[4 * k + 3];
@@ -510,32 +533,50 @@ lem_status band_prepare(lem_ctx* ctx) {
     c.bxc = std::min(c.lx + c.hx + 1, c.wx);
     c.bxp = (c.bxc + 3) / 4 * 4;
     c.L = c.byc * c.bxp;
-    c.off = total;
-    total += int64_t(c.iy) * c.ix * c.L;
+    b->used += int64_t(c.iy) * c.ix * c.L;
   }
   const bool f32 = ctx->apply_path == LEM_APPLY_F32_BAND;
+  b->launch = band_launch(ctx, b->cls, f32 ? 4 : 8);
+  const bool by_row = b->launch.lpr == 1;
+  for (BandClass& c : b->cls) {  // (interleaved rows come in groups of 32)
+    c.off = total;
+    const int64_t rows = int64_t(c.iy) * c.ix;
+    total += (by_row ? (rows + 31) / 32 * 32 : rows) * c.L;
+  }
   if (total > b->cap) {
     if (b->d_Pb) cudaFreeAsync(b->d_Pb, st);
     if (b->d_Pb32) cudaFreeAsync(b->d_Pb32, st);
     b->d_Pb = nullptr;
     b->d_Pb32 = nullptr;
     b->cap = 0;
-    LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&b->d_Pb), sizeof(double) * size_t(total)));
     if (f32) LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&b->d_Pb32), sizeof(float) * size_t(total)));
+    else LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&b->d_Pb), sizeof(double) * size_t(total)));
     b->cap = total;
-  } else if (f32 && !b->d_Pb32) {
-    LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&b->d_Pb32), sizeof(float) * size_t(b->cap)));
   }
-  b->used = total;
   LEM_CUDA_TRY(cudaMemcpyAsync(b->d_cls, b->cls.data(), sizeof(BandClass) * nc, cudaMemcpyHostToDevice, st));
-  band_pack_kernel<<<dim3(unsigned(ctx->n_int), unsigned(nc)), 128, 0, st>>>(ctx->d_P, ctx->n_int, ctx->n_loc, b->d_cls,
-                                                                           b->d_Pb, f32 ? b->d_Pb32 : nullptr);
+  const dim3 pgrid(unsigned(ctx->n_int), unsigned(nc));
+  if (f32)
+    band_pack_kernel<float><<<pgrid, 128, 0, st>>>(ctx->d_P, ctx->n_int, ctx->n_loc, b->d_cls, by_row, b->d_Pb32);
+  else
+    band_pack_kernel<double><<<pgrid, 128, 0, st>>>(ctx->d_P, ctx->n_int, ctx->n_loc, b->d_cls, by_row, b->d_Pb);
   LEM_CUDA_TRY(cudaGetLastError());
-  b->l64 = band_launch(ctx, b->cls, 8);
-  b->l32 = band_launch(ctx, b->cls, 4);
+  if (by_row) {
+    std::vector<BandTile> bt(ctx->tiles.size());
+    for (size_t k = 0; k < bt.size(); ++k) {
+      const TileDesc& t = ctx->tiles[k];
+      const BandClass& c = b->cls[t.cls];
+      bt[k] = BandTile{{t.org[0], t.org[1]}, {t.t0[0], t.t0[1]}, c.wy, c.wx, c.ix, c.oy, c.ox, c.ly, c.lx,
+                       c.byc, c.bxc, c.bxp, c.iy * c.ix, c.L, c.off};
+    }
+    if (!b->d_tiles) LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&b->d_tiles), sizeof(BandTile) * bt.size()));
+    // (pageable memory: the copy has left the vector when the call returns)
+    LEM_CUDA_TRY(cudaMemcpyAsync(b->d_tiles, bt.data(), sizeof(BandTile) * bt.size(), cudaMemcpyHostToDevice, st));
+  }
   const int bytes = int(sizeof(double) * size_t(b->wmax + 4));
   if (bytes > 48 * 1024) {
-    for (int lpr : {1, 2, 4, 8}) {
+    LEM_CUDA_TRY(cudaFuncSetAttribute(gemv_band_row_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    LEM_CUDA_TRY(cudaFuncSetAttribute(gemv_band_row_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    for (int lpr : {2, 4, 8}) {
       LEM_CUDA_TRY(cudaFuncSetAttribute(band_kernel_for<double>(lpr), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
       LEM_CUDA_TRY(cudaFuncSetAttribute(band_kernel_for<float>(lpr), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     }
@@ -564,28 +605,47 @@ lem_status band_step(lem_ctx* ctx, double* d_u) {
   if (ctx->band_gen != ctx->build_gen) LEM_TRY(band_prepare(ctx));
   BandPlan* b = ctx->band;
   cudaStream_t st = ctx->stream;
+  const bool f32 = ctx->apply_path == LEM_APPLY_F32_BAND;
   const bool phi = ctx->desc.mode == LEM_MODE_PHI;
+  const double* src = ctx->d_r;
   if (phi) {
     LEM_CUDA_TRY(launch_residual_fp64(ctx, ctx->d_r, d_u));
   } else {
     LEM_CUDA_TRY(cudaMemcpyAsync(ctx->d_r, d_u, sizeof(double) * ctx->npts, cudaMemcpyDeviceToDevice, st));
   }
-  const bool f32 = ctx->apply_path == LEM_APPLY_F32_BAND;
-  const unsigned nt = unsigned(ctx->tiles.size());
-  const BandLaunch& L = f32 ? b->l32 : b->l64;
+  const BandLaunch& L = b->launch;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(ctx->tiles.size()) * L.rsplit);
+  cfg.blockDim = dim3(L.threads);
+  cfg.dynamicSmemBytes = (f32 ? sizeof(float) : sizeof(double)) * size_t(b->wmax + 4);
+  cfg.stream = st;
   cudaEvent_t stop;
   LEM_CUDA_TRY(ctx->timing_begin(&stop));
-  if (f32) {
-    const size_t smem = sizeof(float) * size_t(b->wmax + 4);
-    band_kernel_for<float>(L.lpr)<<<nt * L.rsplit, L.threads, smem, st>>>(b->d_Pb32, b->d_cls, ctx->d_tiles, ctx->d_r,
-                                                                         d_u, ctx->ny, ctx->nx, phi ? 1 : 0, L.rsplit);
+  const int acc = phi ? 1 : 0;
+  const TileDesc* tiles = ctx->d_tiles;
+  const BandClass* cls = b->d_cls;
+  const float* P32 = b->d_Pb32;
+  const double* P64 = b->d_Pb;
+  if (L.lpr == 1) {
+    cfg.attrs = &at;  // (the kernel waits for the residual itself, its first boxes on the way)
+    cfg.numAttrs = phi ? 1 : 0;
+    const BandTile* bt = b->d_tiles;
+    // boxes that fit in L2 beside the state are kept there from step to step
+    const int keep = b->cap * (f32 ? 4 : 8) <= 64000000;
+    LEM_CUDA_TRY(f32 ? cudaLaunchKernelEx(&cfg, gemv_band_row_kernel<float>, P32, bt, src, d_u, ctx->ny, ctx->nx, acc,
+                                          L.rsplit, keep)
+                     : cudaLaunchKernelEx(&cfg, gemv_band_row_kernel<double>, P64, bt, src, d_u, ctx->ny, ctx->nx, acc,
+                                          L.rsplit, keep));
   } else {
-    const size_t smem = sizeof(double) * size_t(b->wmax + 4);
-    band_kernel_for<double>(L.lpr)<<<nt * L.rsplit, L.threads, smem, st>>>(b->d_Pb, b->d_cls, ctx->d_tiles, ctx->d_r,
-                                                                          d_u, ctx->ny, ctx->nx, phi ? 1 : 0, L.rsplit);
+    LEM_CUDA_TRY(f32 ? cudaLaunchKernelEx(&cfg, band_kernel_for<float>(L.lpr), P32, cls, tiles, src, d_u, ctx->ny, ctx->nx,
+                                          acc, L.rsplit)
+                     : cudaLaunchKernelEx(&cfg, band_kernel_for<double>(L.lpr), P64, cls, tiles, src, d_u, ctx->ny, ctx->nx,
+                                          acc, L.rsplit));
   }
   ctx->timing_end(stop);
-  LEM_CUDA_TRY(cudaGetLastError());
   return LEM_OK;
 }
 

@@ -23,6 +23,9 @@ __global__ void residual_fp64_kernel(double* __restrict__ r, const double* __res
                                      const double* __restrict__ coef, int64_t cstride,
                                      int64_t ny, int64_t nx, int ndim, int pery, int perx,
                                      double dt, double pm) {
+  // a launch chained to this one may begin its set-up (no-ops in an ordinary chain of launches)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t npts = ny * nx;
   const int64_t x = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (x >= nx) return;
@@ -57,10 +60,14 @@ __global__ void residual_fp64_kernel(double* __restrict__ r, const double* __res
 __global__ void residual_complex_kernel(double* __restrict__ r, const double* __restrict__ u,
                                         const double* __restrict__ coef, int64_t cstride, int64_t ny, int64_t nx,
                                         int ndim, int pery, int perx) {
+  // a launch chained to this one may begin its set-up (no-ops in an ordinary chain of launches)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t npts = ny * nx;
-  for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < npts;
-       p += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t y = p / nx, x = p % nx;
+  const int64_t x = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (x >= nx) return;
+  for (int64_t y = int64_t(blockIdx.y) * blockDim.y + threadIdx.y; y < ny; y += int64_t(gridDim.y) * blockDim.y) {
+    const int64_t p = y * nx + x;
     double ar = 0.0, ai = 0.0;
     auto mac = [&](int w, int64_t q) {
       const double a = cstride ? coef[int64_t(w) * npts + p] : coef[w];
@@ -123,29 +130,25 @@ __global__ void scatter_fp64_kernel(double* __restrict__ u, const double* __rest
 
 }  // namespace
 
+// The kernels wait for the launch ahead before they touch anything, so they may be placed early.
 cudaError_t launch_residual_fp64(const lem_ctx* ctx, double* r, const double* u) {
   const lem_problem_desc& d = ctx->desc;
-  int blocks = int(std::min<int64_t>((ctx->npts + 255) / 256, 152 * 16));
-  if (ctx->cplx) {
-    residual_complex_kernel<<<blocks, 256, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
-                                                             d.ndim, ctx->bcy == LEM_BC_PERIODIC,
-                                                             ctx->bcx == LEM_BC_PERIODIC);
-    return cudaGetLastError();
-  }
   const int py = ctx->bcy == LEM_BC_PERIODIC, px = ctx->bcx == LEM_BC_PERIODIC;
-  const dim3 block = ctx->ny == 1 ? dim3(256, 1) : dim3(64, 4);
-  const dim3 grid(unsigned((ctx->nx + block.x - 1) / block.x),
-                  unsigned(std::min<int64_t>((ctx->ny + block.y - 1) / block.y, 32768)));
-  if (d.reaction == 2)
-    residual_fp64_kernel<2><<<grid, block, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
-                                                             d.ndim, py, px, d.dt, d.porous_m);
-  else if (d.reaction == 1)
-    residual_fp64_kernel<1><<<grid, block, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
-                                                             d.ndim, py, px, d.dt, d.porous_m);
-  else
-    residual_fp64_kernel<0><<<grid, block, 0, ctx->stream>>>(r, u, ctx->d_coef, d.coef_stride, ctx->ny, ctx->nx,
-                                                             d.ndim, py, px, d.dt, d.porous_m);
-  return cudaGetLastError();
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.stream = ctx->stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  const double* coef = ctx->d_coef;
+  cfg.blockDim = ctx->ny == 1 ? dim3(256, 1) : dim3(64, 4);
+  cfg.gridDim = dim3(unsigned((ctx->nx + cfg.blockDim.x - 1) / cfg.blockDim.x),
+                     unsigned(std::min<int64_t>((ctx->ny + cfg.blockDim.y - 1) / cfg.blockDim.y, 32768)));
+  if (ctx->cplx)
+    return cudaLaunchKernelEx(&cfg, residual_complex_kernel, r, u, coef, d.coef_stride, ctx->ny, ctx->nx, d.ndim, py, px);
+  auto* kernel = d.reaction == 2 ? residual_fp64_kernel<2> : d.reaction == 1 ? residual_fp64_kernel<1> : residual_fp64_kernel<0>;
+  return cudaLaunchKernelEx(&cfg, kernel, r, u, coef, d.coef_stride, ctx->ny, ctx->nx, d.ndim, py, px, d.dt, d.porous_m);
 }
 
 lem_status step_fp64(lem_ctx* ctx, double* d_u) {

@@ -1,4 +1,4 @@
-"""The batched GEMVs (csrc/step_gemv.cu) with loaded propagators of small whole
+"""The batched GEMVs (csrc/step_gemv.cu, csrc/step_band.cu) with loaded propagators of small whole
 numbers: every residual, product and partial sum stays below 2^24, so FP32 and FP64 rows alike must
 give exactly P R in whole numbers, whatever the order of their sums. Windows whose values fill no whole
 16-byte chunk, clipped windows, ragged last tiles, owners that fill no group of rows, and one, two
@@ -71,6 +71,41 @@ def _propagators(ctx, wins, rng, cplx, reach):
             P[c, :ni, :nl] = A
     ctx.set_propagators(P)
     return of
+
+
+def _run(shape, bc, tile, H, prec, steps, path, cplx=False, trunc=False, seed=0):
+    rng = np.random.default_rng(seed)
+    coef = _coef(shape, rng, cplx)
+    ctx = L.Lem(shape, (bc,) * len(shape), coef, 1.0, tile, H, prec=prec)
+    if trunc:
+        ctx.set_truncation(0.0)
+    assert L.APPLY_PATHS[ctx.info()["apply_path"]] == path
+    wins = decompose(shape, (bc,) * len(shape), tile, H)
+    P = _propagators(ctx, wins, rng, cplx, 3 if trunc else None)
+    n = int(np.prod(shape))
+    u = rng.integers(-2, 3, n).astype(float)
+    if cplx:
+        u = u + 1j * rng.integers(-2, 3, n)
+    d_u = torch.tensor(u, device="cuda")
+    ctx.step(d_u, steps)
+    ctx.sync()
+    for _ in range(steps):
+        r, new = _residual(u, coef, shape, (bc,) * len(shape)), u.copy()
+        for t, w in enumerate(wins):
+            new[w.D] += P[ctx.tile_class(t)] @ r[w.M]
+        u = new
+    assert np.abs(u).max() < 2 ** 22
+    assert np.array_equal(d_u.cpu().numpy(), u)
+    ctx.close()
+
+
+@pytest.mark.parametrize("shape,bc,tile,H", [((130,), "dirichlet", (20,), (5,)), ((3000,), "dirichlet", (64,), (16,)),
+                                             ((900,), "periodic", (45,), (11,)), ((31, 45), "dirichlet", (7, 9), (4, 4)),
+                                             ((48, 96), "periodic", (24, 32), (4, 4))])
+@pytest.mark.parametrize("prec", ["fp64", "split_fast"])
+@pytest.mark.parametrize("steps", [1, 2, 3])
+def test_truncated_propagators(shape, bc, tile, H, prec, steps):
+    _run(shape, bc, tile, H, prec, steps, "f32_band" if prec == "split_fast" else "fp64_band", trunc=True)
 
 
 # one tile more than half the SMs (one block a tile), a few tiles (many blocks a tile), owners that are no
