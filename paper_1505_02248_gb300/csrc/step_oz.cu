@@ -7,9 +7,9 @@
 //
 // GB300's FP64 pipe runs 1.1 TFLOP/s, its FP16 tensor cores 1900. The 1024^2 periodic problem
 // (1024 windows of 2304 nodes, 1024 x 2304 propagator) took 4.67 ms a step as one FP64 GEMM, at
-// the FP64 pipe's rate, and takes 0.145 ms here (products 113 us, window digits 20, residual 15); a
-// walled 389 x 517 mesh with 16 classes, their GEMMs one after another, 29.2 ms a step, and 0.112
-// ms here.
+// the FP64 pipe's rate, and takes 0.134 ms here (products 104 us, window digits 20, residual 12, the
+// launches chained: 0.141 in a plain sequence); a walled 389 x 517 mesh with 16 classes, their GEMMs one
+// after another, 29.2 ms a step, and 0.103 ms here (0.109 unchained).
 //
 // Layout: windows are the rows of A (128 windows of one class form a block), owner rows of the
 // class's propagator the columns of B. The propagators are cut once per build. One launch covers
@@ -77,6 +77,9 @@ __global__ void __launch_bounds__(WIN_THREADS) oz_windows_kernel(const double* _
   constexpr int PER = oz::BM / R;  // CTAs per block
   const WinBlock b = blocks[wb0 + blockIdx.x / PER];
   const int r0 = (blockIdx.x % PER) * R;
+  // (chained: the set-up of the multiplying kernel may begin under this one, this one's under the residual)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (r0 >= b.count) return;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   __shared__ int2 org[R];
@@ -330,6 +333,7 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_kernel(const __grid_co
   __shared__ StepTables tab[2];
   const oz::Shared sh = oz::carve(smem_raw);
   const uint32_t tmem = oz::setup(sh, &s_abort);
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the window digits are written
   StepWork work{p, tab};
   oz::run<oz::Fine>(sh, tmem, work, p.err, &s_abort);
   oz::release(tmem);
@@ -358,8 +362,9 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_split_kernel(const __g
   const int ks = p.ks, rank = int(blockIdx.x) % ks;
   const Unit un = p.units[p.unit0 + int(blockIdx.x) / ks];
   const WinBlock wb = p.blocks[un.wb];
-  tab.fill(p, un, wb, int(threadIdx.x));
   const uint32_t tmem = oz::setup(sh, &s_abort);
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the window digits are written
+  tab.fill(p, un, wb, int(threadIdx.x));
   const int k0 = wb.nkb * rank / ks, k1 = wb.nkb * (rank + 1) / ks;
   SplitWork work{sh, {p.a + wb.a_off + size_t(k0) * oz::A_BLOCK, p.b + un.b_off + size_t(k0) * oz::B_BLOCK, k1 - k0}};
   oz::run<oz::Fine>(sh, tmem, work, p.err, &s_abort);
@@ -480,6 +485,15 @@ void plan_oz(const lem_ctx* ctx, OzPlan* z) {
   close();
 }
 
+// a launch chained to the one ahead of it: the kernel waits for that one itself
+cudaLaunchAttribute chained() {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  return at;
+}
+
+// at: room for two attributes
 cudaLaunchConfig_t split_config(int ks, int units, cudaStream_t st, cudaLaunchAttribute* at) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(units * ks));
@@ -489,8 +503,9 @@ cudaLaunchConfig_t split_config(int ks, int units, cudaStream_t st, cudaLaunchAt
   at->id = cudaLaunchAttributeClusterDimension;
   at->val.clusterDim.x = unsigned(ks);
   at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  at[1] = chained();
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cfg;
 }
 
@@ -505,8 +520,9 @@ int pick_split(const OzPlan::Group& g, const OzPlan* z, int nsm) {
   double best_t = std::ceil(double(g.nunits) / nsm) * (kblocks * 1130.0 + 3000.0) + 12000.0;
   for (int ks : {2, 4, 8}) {
     if (kblocks / ks < 4) break;
-    cudaLaunchAttribute at;
-    const cudaLaunchConfig_t cfg = split_config(ks, 1, nullptr, &at);
+    cudaLaunchAttribute at[2];
+    cudaLaunchConfig_t cfg = split_config(ks, 1, nullptr, at);
+    cfg.numAttrs = 1;
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, oz_step_split_kernel, &cfg) != cudaSuccess || n < 1) {
       cudaGetLastError();
@@ -608,17 +624,26 @@ lem_status step_oz(lem_ctx* ctx, double* d_u) {
   for (const OzPlan::Group& g : z->groups) {
     auto cut = g.nwb >= 24 ? oz_windows_kernel<8> : g.nwb >= 12 ? oz_windows_kernel<4> : oz_windows_kernel<2>;
     const int per = g.nwb >= 24 ? 16 : g.nwb >= 12 ? 32 : 64;
-    cut<<<unsigned(g.nwb * per), WIN_THREADS, 0, st>>>(src, ctx->d_tiles, ctx->d_class_order, z->d_blocks, g.wb0,
-                                                       int(ctx->ny), int(ctx->nx), z->d_e, z->d_a);
-    LEM_CUDA_TRY(cudaGetLastError());
+    cudaLaunchAttribute at[2] = {chained()};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(g.nwb * per));
+    cfg.blockDim = dim3(WIN_THREADS);
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, cut, src, static_cast<const TileDesc*>(ctx->d_tiles),
+                                    static_cast<const int32_t*>(ctx->d_class_order),
+                                    static_cast<const WinBlock*>(z->d_blocks), g.wb0, int(ctx->ny), int(ctx->nx), z->d_e,
+                                    z->d_a));
     StepParams p{z->d_blocks, z->d_units, ctx->d_tiles, ctx->d_class_order, z->d_a, z->d_b, z->d_e, z->d_f, z->d_sv, z->d_sk, ctx->d_P,
                  src, d_u, ctx->n_int, ctx->n_loc, ctx->ny, ctx->nx, g.unit0, g.nunits, g.ks, phi ? 1 : 0, z->d_err};
     if (g.ks == 1) {
-      oz_step_kernel<<<std::min(g.nunits, z->nsm), oz::THREADS, oz::SMEM, st>>>(p);
-      LEM_CUDA_TRY(cudaGetLastError());
+      cfg.gridDim = dim3(unsigned(std::min(g.nunits, z->nsm)));
+      cfg.blockDim = dim3(oz::THREADS);
+      cfg.dynamicSmemBytes = oz::SMEM;
+      LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_step_kernel, p));
     } else {
-      cudaLaunchAttribute at;
-      const cudaLaunchConfig_t cfg = split_config(g.ks, g.nunits, st, &at);
+      cfg = split_config(g.ks, g.nunits, st, at);
       LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_step_split_kernel, p));
     }
   }
