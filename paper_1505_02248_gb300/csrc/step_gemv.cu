@@ -15,72 +15,36 @@
 
 #include <cooperative_groups.h>
 
+#include "gemv_acc.cuh"
 #include "lem_internal.h"
 
 namespace lem {
 
 namespace {
 
-__device__ __forceinline__ void two_sum_d(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
-// Per-lane accumulators. FP64 rows: fused multiply-add. FP32 rows: each product split exactly
-// (FMA) and accumulated in float-float.
-struct AccD {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-};
-struct AccF {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float a, float b) {
-    const float p = __fmul_rn(a, b);
-    const float pe = fmaf(a, b, -p);
-    float s, e;
-    two_sum_d(hi, p, s, e);
-    hi = s;
-    lo = __fadd_rn(lo, __fadd_rn(e, pe));
-  }
-  // adds a partial sum already rounded to FP32
-  __device__ __forceinline__ void add1(float x) {
-    float s, e;
-    two_sum_d(hi, x, s, e);
-    hi = s;
-    lo = __fadd_rn(lo, e);
-  }
-};
-
-// Reduction over the 8 lanes of a row group (lanes 8g .. 8g + 7).
-__device__ __forceinline__ double group_reduce(AccD& a) {
-  for (int o = 4; o > 0; o >>= 1) a.s += __shfl_xor_sync(0xffffffffu, a.s, o);
-  return a.s;
-}
-__device__ __forceinline__ double group_reduce(AccF& a) {
-  for (int o = 4; o > 0; o >>= 1) {
-    const float oh = __shfl_xor_sync(0xffffffffu, a.hi, o);
-    const float ol = __shfl_xor_sync(0xffffffffu, a.lo, o);
-    float s, e;
-    two_sum_d(a.hi, oh, s, e);
-    a.hi = s;
-    a.lo = __fadd_rn(a.lo, __fadd_rn(ol, e));
-  }
-  return double(a.hi) + double(a.lo);
-}
-
 // Four propagator rows per warp, 8 lanes per row: y_i = sum_k P[i, k] w[k]. With vec (row
 // length a multiple of the vector width, rows 16-byte aligned) each lane streams its row in
 // 16-byte loads, four in flight; else scalar loads. Several rows in flight per warp keep the
-// load pipe busy through each row's reduction and owner update.
+// load pipe busy through each row's reduction and owner update. A launch may be chained to the
+// residual's: the blocks load their first chunks, then wait for it.
+// What bounds it: HBM, and how many blocks are resident to keep loads in flight (hence 40 registers
+// for FP32 rows); FP32 sums also took 60 % of the issue slots before they were packed; FP64 rows are
+// near the FP64 pipe's rate. 320^2 variable diffusion (308 MB
+// a step, its floor 45 us), a call of ten steps: 690 us; chained 674, the first 48 MB kept in L2 654,
+// packed sums, windows staged without divisions and owner values read before their row 578, first
+// chunks before the wait 564 to 573 (five blocks an SM 599, three chunks in flight 608). FP64 rows of
+// the same problem 1499 -> 1456 us, 101^2 with tiles of 12 212 -> 169. A Schroedinger line of 65536
+// (31 MB): 286, 270, 254, 205 us, its FP64 rows 822 -> 753.
 // CPLX: complex states (interleaved re, im) with real-embedded propagators
 // [[Re P, -Im P], [Im P, Re P]]: the window is staged as [re parts | im parts] (n_loc / 2 nodes
 // each, zero padded); each owner's Re and Im rows are read once, left halves only.
+constexpr int tiles_threads(int value, bool cplx) { return cplx && value == 4 ? 128 : 256; }
+constexpr int tiles_blocks(int value, bool cplx) { return cplx ? (value == 4 ? 8 : 4) : (value == 4 ? 6 : 5); }
 template <typename PT, bool CPLX>
-__global__ void __launch_bounds__(256) gemv_tiles_kernel(const PT* __restrict__ P, int64_t n_int, int64_t n_loc,
-                                                         const TileDesc* __restrict__ tiles,
-                                                         const double* __restrict__ src, double* __restrict__ u,
-                                                         int64_t ny, int64_t nx, int accumulate, int rsplit) {
+__global__ void __launch_bounds__(tiles_threads(sizeof(PT), CPLX), tiles_blocks(sizeof(PT), CPLX))
+    gemv_tiles_kernel(const PT* __restrict__ P, int64_t n_int, int64_t n_loc, const TileDesc* __restrict__ tiles,
+                      const double* __restrict__ src, double* __restrict__ u, int64_t ny, int64_t nx, int accumulate,
+                      int rsplit, int resident) {
   // the tile's window values, converted once to the propagator's precision
   extern __shared__ __align__(16) unsigned char wraw[];
   PT* w = reinterpret_cast<PT*>(wraw);
@@ -91,30 +55,57 @@ __global__ void __launch_bounds__(256) gemv_tiles_kernel(const PT* __restrict__ 
   const int wn = td.wext[0] * td.wext[1];  // window nodes
   const int hn = int(n_loc / 2);            // CPLX: padded window nodes
   const int wl = CPLX ? int(n_loc) : wn;    // staged window values
-  for (int k = threadIdx.x; k < wl; k += blockDim.x) {
-    const int node = CPLX ? k % hn : k, comp = CPLX ? k / hn : 0;
-    if (node >= wn) {
-      w[k] = PT(0);
-      continue;
-    }
-    const int a = node / td.wext[1], b = node % td.wext[1];
-    int64_t gy = int64_t(td.org[0]) + a, gx = int64_t(td.org[1]) + b;
-    gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
-    gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
-    w[k] = PT(CPLX ? src[2 * (gy * nx + gx) + comp] : src[gy * nx + gx]);
-  }
-  __syncthreads();
   const PT* Pt = P + int64_t(td.cls) * n_int * n_loc;
   const int ien = td.iext[0] * td.iext[1];  // owner nodes
   const int ie_all = ien;                   // owner nodes of this tile (CPLX: one group does both parts)
   const int rows_per = (ie_all + rsplit - 1) / rsplit;
   const int ib = part * rows_per, ie = min(ie_all, ib + rows_per);
+  constexpr int V = 16 / sizeof(PT);
+  const bool vec = (n_loc % V) == 0;  // (a row's end short of a whole chunk is masked, row_end)
+  const unsigned long long policy = l2_policy(td.cls < resident);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, nw = blockDim.x / 32;
   const int grp = lane / 8, gl = lane % 8;
-  constexpr int V = 16 / sizeof(PT);
+  // real rows: chunks j0 + gl + 8 k of a row; the first ones before the residual is waited for
   constexpr int U = 4;  // 16-byte loads in flight per lane
-  const bool vec = (n_loc % V) == 0 && (wl % V) == 0;
-  using Acc = typename std::conditional<sizeof(PT) == 8, AccD, AccF>::type;
+  const int nv = (wl + V - 1) / V;
+  int4 q[U];
+  auto load = [&](int row, int j0) {
+    const int4* r4 = reinterpret_cast<const int4*>(Pt + int64_t(row) * n_loc) + j0 + gl;
+    if (j0 + 8 * U <= nv) {
+#pragma unroll
+      for (int k = 0; k < U; ++k) q[k] = load_policy(r4 + 8 * k, policy);
+    } else {
+#pragma unroll
+      for (int k = 0; k < U; ++k) q[k] = j0 + 8 * k + gl < nv ? load_policy(r4 + 8 * k, policy) : make_int4(0, 0, 0, 0);
+    }
+  };
+  if (!CPLX && vec && ib + warp * 4 < ie) load(min(ib + warp * 4 + grp, ie - 1), 0);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // the window: node k = (a, b), then blockDim.x nodes further each time; zeros to a whole chunk
+  const int wx = td.wext[1], step_a = int(blockDim.x) / wx, step_b = int(blockDim.x) % wx;
+  for (int k = threadIdx.x, a = k / wx, b = k % wx; k < (CPLX ? hn : min((wn + V - 1) / V * V, int(n_loc)));
+       k += blockDim.x, a += step_a, b += step_b) {
+    if (b >= wx) {
+      b -= wx;
+      ++a;
+    }
+    if (k >= wn) {
+      w[k] = PT(0);
+      if (CPLX) w[hn + k] = PT(0);
+      continue;
+    }
+    int64_t gy = int64_t(td.org[0]) + a, gx = int64_t(td.org[1]) + b;
+    gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
+    gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
+    if (CPLX) {
+      const double2 v = *reinterpret_cast<const double2*>(src + 2 * (gy * nx + gx));
+      to_prec(v.x, w[k]);
+      to_prec(v.y, w[hn + k]);
+    } else {
+      to_prec(src[gy * nx + gx], w[k]);
+    }
+  }
+  __syncthreads();
   if constexpr (CPLX) {
     // complex: a row group per owner node o, reading its Re row (row o) and Im row (row
     // n_int / 2 + o) of the stored embedding, left halves only (the right halves repeat them):
@@ -124,9 +115,16 @@ __global__ void __launch_bounds__(256) gemv_tiles_kernel(const PT* __restrict__ 
     for (int o0 = ib + warp * 4; o0 < ie; o0 += nw * 4) {
       const int o = o0 + grp;
       const bool live = o < ie;
-      const PT* rre = Pt + int64_t(live ? o : 0) * n_loc;
-      const PT* rim = Pt + int64_t(live ? int(n_int / 2) + o : 0) * n_loc;
-      Acc are, aim;
+      const int oc = live ? o : ib;  // (groups past the last row read a row of the share, and drop it)
+      const PT* rre = Pt + int64_t(oc) * n_loc;
+      const PT* rim = Pt + int64_t(int(n_int / 2) + oc) * n_loc;
+      const int64_t p = int64_t(td.t0[0] + oc / td.iext[1]) * nx + td.t0[1] + oc % td.iext[1];
+      double br = 0.0, bi = 0.0;  // (read before the row, whose time hides theirs)
+      if (accumulate && gl == 0) {
+        br = u[2 * p];
+        bi = u[2 * p + 1];
+      }
+      typename std::conditional<sizeof(PT) == 8, AccCD, AccCF>::type acc;
       if (cvec) {
         // FP32 rows: four 16-byte loads per lane and row in flight, so a window of up to 128
         // nodes takes one round trip per row pair; FP64 rows are bound by the FP64 pipe.
@@ -138,57 +136,27 @@ __global__ void __launch_bounds__(256) gemv_tiles_kernel(const PT* __restrict__ 
           int4 qa[CU], qb[CU];
 #pragma unroll
           for (int k = 0; k < CU; ++k) {
-            const bool ok = live && j + 8 * k < nv;
-            qa[k] = ok ? __ldcs(a4 + j + 8 * k) : make_int4(0, 0, 0, 0);
-            qb[k] = ok ? __ldcs(b4 + j + 8 * k) : make_int4(0, 0, 0, 0);
+            const bool ok = j + 8 * k < nv;
+            qa[k] = ok ? load_policy(a4 + j + 8 * k, policy) : make_int4(0, 0, 0, 0);
+            qb[k] = ok ? load_policy(b4 + j + 8 * k, policy) : make_int4(0, 0, 0, 0);
           }
 #pragma unroll
           for (int k = 0; k < CU; ++k) {
             if (j + 8 * k >= nv) break;
-            const PT* pa = reinterpret_cast<const PT*>(&qa[k]);
-            const PT* pb = reinterpret_cast<const PT*>(&qb[k]);
             const int4 wr4 = *reinterpret_cast<const int4*>(w + (j + 8 * k) * V);
             const int4 wi4 = *reinterpret_cast<const int4*>(w + hl + (j + 8 * k) * V);
-            const PT* wr = reinterpret_cast<const PT*>(&wr4);
-            const PT* wi = reinterpret_cast<const PT*>(&wi4);
-            if constexpr (sizeof(PT) == 4) {
-              // FP32 rows: a chunk's eight products per part are summed by FMA in FP32 and the
-              // chunk sum enters the float-float accumulator (an exact product split for each of
-              // the four products an element takes part in would make the launch ALU-bound)
-              float sr = 0.0f, si = 0.0f;
-#pragma unroll
-              for (int h = 0; h < V; ++h) {
-                sr = fmaf(pa[h], wr[h], sr);
-                sr = fmaf(-pb[h], wi[h], sr);
-                si = fmaf(pb[h], wr[h], si);
-                si = fmaf(pa[h], wi[h], si);
-              }
-              are.add1(sr);
-              aim.add1(si);
-            } else {
-#pragma unroll
-              for (int h = 0; h < V; ++h) {
-                are.add(pa[h], wr[h]);
-                are.add(-pb[h], wi[h]);
-                aim.add(pb[h], wr[h]);
-                aim.add(pa[h], wi[h]);
-              }
-            }
+            acc.chunk(reinterpret_cast<const PT*>(&qa[k]), reinterpret_cast<const PT*>(&qb[k]),
+                      reinterpret_cast<const PT*>(&wr4), reinterpret_cast<const PT*>(&wi4));
           }
         }
-      } else if (live) {
-        for (int k = gl; k < hl; k += 8) {
-          are.add(rre[k], w[k]);
-          are.add(-rim[k], w[hl + k]);
-          aim.add(rim[k], w[k]);
-          aim.add(rre[k], w[hl + k]);
-        }
+      } else {
+        for (int k = gl; k < hl; k += 8) acc.add(rre[k], rim[k], w[k], w[hl + k]);
       }
-      const double yr = group_reduce(are), yi = group_reduce(aim);
+      double yr, yi;
+      group_reduce(acc, yr, yi);
       if (live && gl == 0) {
-        const int64_t p = int64_t(td.t0[0] + o / td.iext[1]) * nx + td.t0[1] + o % td.iext[1];
-        u[2 * p] = accumulate ? u[2 * p] + yr : yr;
-        u[2 * p + 1] = accumulate ? u[2 * p + 1] + yi : yi;
+        u[2 * p] = accumulate ? br + yr : yr;
+        u[2 * p + 1] = accumulate ? bi + yi : yi;
       }
     }
   } else {
@@ -196,37 +164,42 @@ __global__ void __launch_bounds__(256) gemv_tiles_kernel(const PT* __restrict__ 
     for (int i0 = ib + warp * 4; i0 < ie; i0 += nw * 4) {
       const int i = i0 + grp;
       const bool live = i < ie;
-      const PT* row = Pt + int64_t(live ? i : 0) * n_loc;
-      Acc acc;
+      const int ic = live ? i : ib;  // (groups past the last row read a row of the share, and drop it)
+      const int64_t p = int64_t(td.t0[0] + ic / td.iext[1]) * nx + td.t0[1] + ic % td.iext[1];
+      const double before = accumulate && gl == 0 ? u[p] : 0.0;  // (read before the row, whose time hides its)
+      typename std::conditional<sizeof(PT) == 8, AccD, AccF>::type acc;
       if (vec) {
-        const int nv = wl / V;
-        const int4* r4 = reinterpret_cast<const int4*>(row);
-        for (int j = gl; j < nv; j += 8 * U) {
-          int4 q[U];
-  #pragma unroll
-          for (int k = 0; k < U; ++k) q[k] = (live && j + 8 * k < nv) ? __ldcs(r4 + j + 8 * k) : make_int4(0, 0, 0, 0);
-  #pragma unroll
-          for (int k = 0; k < U; ++k) {
-            if (j + 8 * k >= nv) break;
-            const PT* pq = reinterpret_cast<const PT*>(&q[k]);
-            const int4 wq = *reinterpret_cast<const int4*>(w + (j + 8 * k) * V);  // same 16 bytes of w
-            const PT* pw = reinterpret_cast<const PT*>(&wq);
-  #pragma unroll
-            for (int h = 0; h < V; ++h) acc.add(pq[h], pw[h]);
+        const int4* w4 = reinterpret_cast<const int4*>(w);
+        for (int j0 = 0;;) {
+          if (j0 + 8 * U <= wl / V) {
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+              const int4 wq = w4[j0 + 8 * k + gl];
+              acc.chunk(reinterpret_cast<const PT*>(&q[k]), reinterpret_cast<const PT*>(&wq));
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+              const int j = j0 + 8 * k + gl;
+              if (j >= nv) break;
+              const int4 wq = w4[j];
+              row_end(q[k], Pt, wl - j * V);
+              acc.chunk(reinterpret_cast<const PT*>(&q[k]), reinterpret_cast<const PT*>(&wq));
+            }
           }
+          if ((j0 += 8 * U) >= nv) break;
+          load(ic, j0);
         }
-      } else if (live) {
+        if (i0 + nw * 4 < ie) load(min(i + nw * 4, ie - 1), 0);
+      } else {
+        const PT* row = Pt + int64_t(ic) * n_loc;
         for (int k = gl; k < wl; k += 8) acc.add(row[k], w[k]);
       }
       const double y = group_reduce(acc);
-      if (live && gl == 0) {
-        const int64_t p = int64_t(td.t0[0] + i / td.iext[1]) * nx + td.t0[1] + i % td.iext[1];
-        u[p] = accumulate ? u[p] + y : y;
-      }
+      if (live && gl == 0) u[p] = accumulate ? before + y : y;
     }
   }
 }
-
 
 // The defect of the third-order Rosenbrock step, times two: 2 dt (G(U) - G(u)) with
 // G(v) = F(v) - J(u_m) v. The linear parts cancel, so it is pointwise:
@@ -271,8 +244,7 @@ lem_status gemv_prepare_f32(lem_ctx* ctx) {
 // Jacobian refresh, one scheme stage).
 // A tile's owner rows are shared out over rsplit blocks (each stages the tile's window), so that a
 // handful of tiles still uses the device: the FP64 pipe does 2 multiply-adds per clock and SM, and
-// one block per tile of 64 x 96 took most of a step (1024 nodes, 16 tiles: 5.6 us a step; with 8
-// blocks of 8 rows a tile 4.2, of which the grid barrier is the larger part).
+// one block per tile of 64 x 96 took most of a step (16 tiles: 5.6 us a step).
 // SMEMP: one share of a tile per block, its propagator rows kept in shared memory for all steps.
 static int persist_threads(int rsplit) { return rsplit > 1 ? 128 : 256; }
 template <typename PT, bool SMEMP>
@@ -341,10 +313,11 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
         }
         w[k] = PT(v);
       }
+      if (threadIdx.x < 4 && wl + threadIdx.x < n_loc) w[wl + threadIdx.x] = PT(0);  // to a whole chunk
       __syncthreads();
       const PT* Pt = SMEMP ? Ps - int64_t(ib) * n_loc : P + int64_t(td.cls) * n_int * n_loc;
       constexpr int V = 16 / sizeof(PT);
-      const bool vec = (n_loc % V) == 0 && (wl % V) == 0;
+      const bool vec = (n_loc % V) == 0;
       for (int i0 = ib + warp * 4; i0 < ie; i0 += nw * 4) {
         const int i = i0 + grp;
         const bool live = i < ie;
@@ -355,11 +328,10 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
         if (live) {
           if (vec) {
             const int4* r4 = reinterpret_cast<const int4*>(row);
-            for (int j = gl; j < wl / V; j += 8) {
-              const int4 q = SMEMP ? r4[j] : __ldcs(r4 + j);
-              const PT* pq = reinterpret_cast<const PT*>(&q);
-#pragma unroll
-              for (int h = 0; h < V; ++h) acc.add(pq[h], w[j * V + h]);
+            for (int j = gl; j < (wl + V - 1) / V; j += 8) {
+              int4 q = SMEMP ? r4[j] : __ldcs(r4 + j);
+              row_end(q, row, wl - j * V);
+              acc.chunk(reinterpret_cast<const PT*>(&q), w + j * V);
             }
           } else {
             for (int k = gl; k < wl; k += 8) acc.add(row[k], w[k]);
@@ -456,7 +428,7 @@ lem_status step_gemv_multi(lem_ctx* ctx, double* d_u, int nsteps, bool f32, bool
 
 // Threads per GEMV block: 128 for the complex FP32 kernel (short rows, little work per block,
 // more blocks resident per SM), 256 otherwise.
-static int gemv_threads(const lem_ctx* ctx, bool f32) { return (ctx->cplx && f32) ? 128 : 256; }
+static int gemv_threads(const lem_ctx* ctx, bool f32) { return tiles_threads(f32 ? 4 : 8, ctx->cplx); }
 
 // Blocks per tile: about four waves of blocks (6 to 8 resident per SM), at least 32 owner rows
 // per block, each block's share a whole number of passes (a pass: 4 rows per warp), so that no
@@ -472,11 +444,22 @@ int gemv_row_split(const lem_ctx* ctx, int threads) {
   return std::max(1, (owners + rows - 1) / rows);
 }
 
+// Classes whose propagators are to stay in L2 from step to step: the first 48 MB (129 MB of L2 serve two
+// dies, and hold the state, the coefficients and what passes through as well). All others are read
+// as passing through. 320^2 variable diffusion (308 MB a step): none 674 us, 32 MB 659, 48 MB 654,
+// 64 MB 664 a call of ten steps; a Schroedinger line of 65536 (31 MB, all kept): 270 -> 254 us.
+static int resident_classes(const lem_ctx* ctx, bool f32) {
+  const int64_t bytes = ctx->n_int * ctx->n_loc * (f32 ? 4 : 8) / (ctx->cplx ? 2 : 1);
+  return int(std::min<int64_t>(48000000 / std::max<int64_t>(bytes, 1), int64_t(ctx->classes.size())));
+}
+
 // One LEM step by the batched GEMV: PHI reads the residual, EXP a copy of u^n.
 lem_status step_gemv(lem_ctx* ctx, double* d_u, bool f32) {
   cudaStream_t st = ctx->stream;
   const bool phi = ctx->desc.mode == LEM_MODE_PHI;
   const bool rb3 = ctx->desc.scheme == LEM_SCHEME_RB3 && ctx->desc.reaction;  // (linear: the defect is 0)
+  // (before the residual: the streamed apply reads propagators while the residual still runs)
+  if (f32 && ctx->p32_gen != ctx->build_gen) LEM_TRY(gemv_prepare_f32(ctx));
   if (rb3)
     LEM_CUDA_TRY(cudaMemcpyAsync(ctx->d_u0, d_u, sizeof(double) * ctx->npts, cudaMemcpyDeviceToDevice, st));
   const double* src;
@@ -488,34 +471,37 @@ lem_status step_gemv(lem_ctx* ctx, double* d_u, bool f32) {
                                  cudaMemcpyDeviceToDevice, st));
     src = ctx->d_r;
   }
-  if (f32 && ctx->p32_gen != ctx->build_gen) LEM_TRY(gemv_prepare_f32(ctx));
   const size_t smem = sizeof(double) * size_t(ctx->n_loc);
   const unsigned nt = unsigned(ctx->tiles.size());
   const int threads = gemv_threads(ctx, f32);
   const int rsplit = gemv_row_split(ctx, threads);
   cudaEvent_t stop;
   LEM_CUDA_TRY(ctx->timing_begin(&stop));
-  auto gemv = [&](const double* P64, const float* P32, const double* x) {
+  auto gemv = [&](const double* P64, const float* P32, const double* x, bool after_residual) -> lem_status {
     const int acc = phi ? 1 : 0;
-    if (ctx->cplx) {
-      if (f32)  // short rows, little work per block: 128 threads, more blocks resident per SM
-        gemv_tiles_kernel<float, true><<<nt * rsplit, threads, smem, st>>>(P32, ctx->n_int, ctx->n_loc, ctx->d_tiles, x,
-                                                                       d_u, ctx->ny, ctx->nx, acc, rsplit);
-      else
-        gemv_tiles_kernel<double, true><<<nt * rsplit, 256, smem, st>>>(P64, ctx->n_int, ctx->n_loc, ctx->d_tiles, x,
-                                                                        d_u, ctx->ny, ctx->nx, acc, rsplit);
-    } else if (f32) {
-      gemv_tiles_kernel<float, false><<<nt * rsplit, 256, smem, st>>>(P32, ctx->n_int, ctx->n_loc, ctx->d_tiles, x,
-                                                                      d_u, ctx->ny, ctx->nx, acc, rsplit);
-    } else {
-      gemv_tiles_kernel<double, false><<<nt * rsplit, 256, smem, st>>>(P64, ctx->n_int, ctx->n_loc, ctx->d_tiles, x,
-                                                                       d_u, ctx->ny, ctx->nx, acc, rsplit);
-    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(nt * rsplit);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = after_residual ? 1 : 0;  // (it waits for the residual before the windows only)
+    auto go = [&](auto kernel, auto P) -> lem_status {
+      LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, P, ctx->n_int, ctx->n_loc,
+                                      static_cast<const TileDesc*>(ctx->d_tiles), x, d_u, ctx->ny, ctx->nx,
+                                      acc, rsplit, resident_classes(ctx, f32)));
+      return LEM_OK;
+    };
+    if (f32) return ctx->cplx ? go(gemv_tiles_kernel<float, true>, P32) : go(gemv_tiles_kernel<float, false>, P32);
+    return ctx->cplx ? go(gemv_tiles_kernel<double, true>, P64) : go(gemv_tiles_kernel<double, false>, P64);
   };
-  gemv(ctx->d_P, ctx->d_P32, src);
+  LEM_TRY(gemv(ctx->d_P, ctx->d_P32, src, phi));
   if (rb3) {  // second stage: u^{n+1} = U + 2 phi_3(dt J_m) dt (G(U) - G(u^n)), window by window
     rb3_defect_kernel<<<1024, 256, 0, st>>>(d_u, ctx->d_u0, ctx->d_um, ctx->desc.dt, ctx->d_r, ctx->npts);
-    gemv(ctx->d_P3, ctx->d_P3_32, ctx->d_r);
+    LEM_TRY(gemv(ctx->d_P3, ctx->d_P3_32, ctx->d_r, false));
   }
   ctx->timing_end(stop);
   LEM_CUDA_TRY(cudaGetLastError());
@@ -538,7 +524,8 @@ lem_status step_gemv_scratch(lem_ctx* ctx, double* d_u, double* r) {
   const int rsplit = gemv_row_split(ctx, threads);
   const int acc = ctx->desc.mode == LEM_MODE_PHI ? 1 : 0;
   gemv_tiles_kernel<double, false><<<nt * rsplit, threads, smem, st>>>(ctx->d_P, ctx->n_int, ctx->n_loc, ctx->d_tiles,
-                                                                       r, d_u, ctx->ny, ctx->nx, acc, rsplit);
+                                                                       r, d_u, ctx->ny, ctx->nx, acc, rsplit,
+                                                                       resident_classes(ctx, false));
   LEM_CUDA_TRY(cudaGetLastError());
   return LEM_OK;
 }

@@ -99,6 +99,23 @@ def _run(shape, bc, tile, H, prec, steps, path, cplx=False, trunc=False, seed=0)
     ctx.close()
 
 
+SHAPES = [((130,), "dirichlet", (20,), (5,)), ((37, 41), "dirichlet", (9, 8), (3, 2)),
+          ((48, 70), "periodic", (16, 14), (6, 5)), ((1000,), "dirichlet", (64,), (33,))]
+
+
+@pytest.mark.parametrize("shape,bc,tile,H", SHAPES)
+@pytest.mark.parametrize("prec", ["fp64", "split_fast"])
+@pytest.mark.parametrize("steps", [1, 3])
+def test_per_tile_propagators(shape, bc, tile, H, prec, steps):
+    _run(shape, bc, tile, H, prec, steps, "f32_gemv" if prec == "split_fast" else "fp64_gemv", seed=steps)
+
+
+@pytest.mark.parametrize("n,tile,H", [(160, 20, 5), (405, 45, 13), (640, 80, 20)])
+@pytest.mark.parametrize("prec", ["fp64", "split_fast"])
+def test_complex_propagators(n, tile, H, prec):
+    _run((n,), "periodic", (tile,), (H,), prec, 2, "f32_gemv" if prec == "split_fast" else "fp64_gemv", cplx=True)
+
+
 @pytest.mark.parametrize("shape,bc,tile,H", [((130,), "dirichlet", (20,), (5,)), ((3000,), "dirichlet", (64,), (16,)),
                                              ((900,), "periodic", (45,), (11,)), ((31, 45), "dirichlet", (7, 9), (4, 4)),
                                              ((48, 96), "periodic", (24, 32), (4, 4))])
