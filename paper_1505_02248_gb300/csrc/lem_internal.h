@@ -181,8 +181,6 @@ lem_status split_from_ff(lem_ctx* ctx, const float* uh, const float* ul, double*
 void split_destroy(lem_ctx* ctx);
 lem_status split_check_error(lem_ctx* ctx);
 bool split_eligible(const lem_ctx* ctx);
-lem_status encode_f16_map(CUtensorMap* m, void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
-                          const cuuint32_t* box, const char* what, int swizzle_bytes = 128);
 // multi-problem split steps (one residual and one GEMM launch per step for a whole batch)
 struct SplitBatch;
 bool split_batch_eligible(lem_ctx* const* ctxs, int n);
