@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(tiles_threads(sizeof(PT), CPLX), tiles_blocks(
   // real rows: chunks j0 + gl + 8 k of a row; the first ones before the residual is waited for
   constexpr int U = 4;  // 16-byte loads in flight per lane
   const int nv = (wl + V - 1) / V;
+  const bool ragged = wl % V != 0;
   int4 q[U];
   auto load = [&](int row, int j0) {
     const int4* r4 = reinterpret_cast<const int4*>(Pt + int64_t(row) * n_loc) + j0 + gl;
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(tiles_threads(sizeof(PT), CPLX), tiles_blocks(
               const int j = j0 + 8 * k + gl;
               if (j >= nv) break;
               const int4 wq = w4[j];
-              row_end(q[k], Pt, wl - j * V);
+              if (ragged) row_end(q[k], Pt, wl - j * V);
               acc.chunk(reinterpret_cast<const PT*>(&q[k]), reinterpret_cast<const PT*>(&wq));
             }
           }
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
             const int4* r4 = reinterpret_cast<const int4*>(row);
             for (int j = gl; j < (wl + V - 1) / V; j += 8) {
               int4 q = SMEMP ? r4[j] : __ldcs(r4 + j);
-              row_end(q, row, wl - j * V);
+              if (wl % V != 0) row_end(q, row, wl - j * V);
               acc.chunk(reinterpret_cast<const PT*>(&q), w + j * V);
             }
           } else {
