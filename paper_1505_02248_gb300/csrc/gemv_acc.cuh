@@ -12,10 +12,11 @@ static __device__ __forceinline__ void two_sum_d(float a, float b, float& s, flo
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
-// A propagator's place in L2: kept (read again in the next step) or passing through.
+// A propagator's place in L2: of ordinary priority, so that it outlives what passes through and is there
+// in the next step, or passing through. (A priority above the ordinary would outlast the steps.)
 static __device__ __forceinline__ unsigned long long l2_policy(bool keep) {
   unsigned long long policy;
-  if (keep) asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(policy));
+  if (keep) asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
   else asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
   return policy;
 }
