@@ -57,10 +57,12 @@ typedef enum {
 
 typedef enum { LEM_BC_DIRICHLET0 = 0, LEM_BC_PERIODIC = 1 } lem_bc;
 typedef enum { LEM_MODE_PHI = 0, LEM_MODE_EXP = 1 } lem_mode;
-/* LEM_PREC_FP64: propagators, residual and apply in IEEE binary64, or closer to the exact sums:
- * where tiles share propagators (LEM_APPLY_FP64_GEMM) each output of the apply is an exact sum of
- * digit products of the FP64 operands on the tensor cores, rounded once (operands cut 2^-56 below
- * the largest value of their row or window).
+/* LEM_PREC_FP64: propagators, residual and apply in IEEE binary64. Where tiles share propagators
+ * (LEM_APPLY_FP64_GEMM) an output y = sum_k P_k u_k of the apply is a sum of digit products on the
+ * tensor cores (operands cut 2^-56 below the largest value of their row or window, products of digits
+ * from the eighth level on left out, one rounding) if sum |P_k| |u_k| is at least a quarter of a bound on
+ * max|P| max|u|, and FP64 multiply-adds if it is not: within 4.1 K 2^-53 sum |P_k| |u_k| of the
+ * exact sum of K terms either way, whatever the range of the values.
  * Propagators of the split tiers are built with tensor-core products (every Pade product,
  * squaring and elimination update an exact sum of FP16 slice products, about 2^-45 of the
  * operands' scale; the environment variable LEM_BUILD_PRODUCTS=fp64 forces FP64 products).

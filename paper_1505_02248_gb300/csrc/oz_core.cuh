@@ -10,8 +10,11 @@
 //   Fine    base 256 (|d| <= 128, 55 bits and a sign below 2^e_i). Levels 4..6 (at most 7 pairs)
 //           over 128 K, levels 0..3 (at most 4) over 256 K; 64-bit integer sums, so
 //             C_ij = 2^(e_i + f_j - 62) (hi 2^24 + lo)
-//           is exact but for the dropped levels (below 2^-58 of 2^(e_i + f_j) a term) and the one
-//           rounding to FP64: closer to the true sum than K FP64 multiply-adds.
+//           is exact but for the operands' cut (2^-56 of 2^e_i and of 2^f_j), the dropped levels and the
+//           one rounding to FP64. Level 7 is the largest that is dropped, six products of two
+//           digits: at most 2^-53.4 of 2^(e_i + f_j) a term, in the mean square 2^-56.3. That is an
+//           error by the largest value of a row and of a column, not by the terms of the sum: see
+//           kSmallSum for the sums that it does not suit.
 //   Coarse  base 128 (49 bits), stretches of 128 K, float-float sums of about 48 bits in the order
 //           of the levels: what the FP16 pieces of the split tiers resolve, and cheaper to drain.
 // The FP64 pipe (2 multiply-adds per clock and SM) does not take part.
@@ -55,6 +58,13 @@ constexpr int OUT_BYTES = EPI_WARPS * 32 * OUT_PITCH * 8;
 constexpr int SMEM = STAGES * STAGE + OUT_BYTES + 1024 + 256;
 constexpr uint64_t WAIT_NS = 2000000000ull;
 constexpr int SUM_PITCH = BM + 1;         // staged sums: column pitch in 16-byte (hi, lo) pairs
+// Fine sums |C_ij| below 2^-2 of 2^(e_i + f_j), |hi| below 2^36, are small: unless their terms are known
+// to be large (sum_k |A_ik| |B_kj| at least that), FP64 multiply-adds are closer to the true sum, and
+// the caller forms them so. The line is where the two errors cross. Root mean squares of digits
+// over multiply-adds on windows of the phi_1 and exponential propagators (K 96 .. 2304), by that sum
+// of magnitudes over 2^(e_i + f_j): in [1/16, 1/8) 3.2, [1/8, 1/4) 1.1 .. 1.5, [1/4, 1/2) 0.75 .. 1.3,
+// [1/2, 1) 0.36 .. 0.84, above 1 0.56 .. 0.03.
+constexpr int kSmallSum = 36;
 
 static_assert(STRETCH_LO % GROUP == 0 && GROUP < STAGES, "groups end stretches");
 static_assert(BN * SUM_PITCH * 16 <= STAGES * STAGE, "staged sums reuse the operand stages");
@@ -389,6 +399,10 @@ __device__ __forceinline__ void run(const Shared& sh, uint32_t tmem, Work& work,
   __syncthreads();
 }
 
+// Whether a fine sum is small (kSmallSum); levels 4..6 are below 2^22.
+__device__ __forceinline__ bool small_sum(long long hi) {
+  return unsigned(int(hi >> 32) + (1 << (kSmallSum - 32))) < (2u << (kSmallSum - 32));
+}
 // The usual finish: each thread's sums as doubles, passed through the warp's output chunk four
 // columns at a time, so that 4 lanes write 32 consecutive bytes of a row. Out:
 //   int scale(row, col)                  the element is its sums times 2^scale

@@ -4,12 +4,17 @@
 //   PHI:  r = dt F(u^n); the windows of r, cut into digits (gather and cut in one pass);
 //         y = P r|_M for 128 windows x 64 owner rows per CTA; u_D += y.
 //   EXP:  the windows of u^n, cut; u_D = P u|_M.
+//   Then, in either mode, the owners whose digit sums came out small (oz_small_kernel): a digit
+//   sum's error goes with the largest values of the window and of the owner row, so where the values
+//   that make up the sum lie far below those, it is formed again as FP64 multiply-adds. Each owner
+//   is within 4.1 K 2^-53 sum_k |P_k| |u_k| of its exact sum, as multiply-adds are within K 2^-53 of it; in the
+//   mean square the digits are the closer ones (oz::kSmallSum).
 //
 // GB300's FP64 pipe runs 1.1 TFLOP/s, its FP16 tensor cores 1900. The 1024^2 periodic problem
 // (1024 windows of 2304 nodes, 1024 x 2304 propagator) took 4.67 ms a step as one FP64 GEMM, at
-// the FP64 pipe's rate, and takes 0.134 ms here (products 104 us, window digits 20, residual 12, the
-// launches chained: 0.141 in a plain sequence); a walled 389 x 517 mesh with 16 classes, their GEMMs one
-// after another, 29.2 ms a step, and 0.103 ms here (0.109 unchained).
+// the FP64 pipe's rate, and takes 0.171 ms here (products 110 us, window digits 21, residual 12, small sums
+// 20 to 30; the launches chained); a walled 389 x 517 mesh with 16 classes, their GEMMs one
+// after another, 29.2 ms a step, and 0.113 ms here. Without the small sums' check it was 0.134 and 0.103 ms.
 //
 // Layout: windows are the rows of A (128 windows of one class form a block), owner rows of the
 // class's propagator the columns of B. The propagators are cut once per build. One launch covers
@@ -43,7 +48,8 @@ struct WinBlock {   // up to 128 windows of one class
   int32_t nkb;      // K blocks of 16 window nodes
   int64_t a_off;    // halves into the window digits
   int32_t e_off;    // scale exponents of its rows
-  int32_t pad;
+  int32_t f0;       // scale exponents of the class's owner rows
+  int64_t b0;       // halves into the propagator digits of the class
 };
 struct Unit {
   int32_t wb;       // window block
@@ -61,10 +67,38 @@ struct PropRows {   // 64 owner rows of one class
 __host__ __device__ __forceinline__ uint32_t div_inv(uint32_t d) { return d > 1 ? 0xFFFFFFFFu / d + 1u : 0u; }
 __device__ __forceinline__ int div_by(int k, uint32_t inv) { return inv ? int(__umulhi(uint32_t(k), inv)) : k; }
 
+// In place of a scale exponent: a row whose values are all zero (its products are 0).
+constexpr int kAllZero = 1 << 21;
+// Largest exponent field below which a row is formed in FP64: subnormal values are cut to 0.
+constexpr int kTiny = 64;
+
+// A row's scale exponent from the maximum of key_of over its values.
+__device__ __forceinline__ int key_of(double v) {  // exponent field, and whether it is not zero
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
+  return oz::exp_field(b) * 2 + ((b << 1) != 0 ? 1 : 0);
+}
+__device__ __forceinline__ int exp_of_key(int key) {
+  return key == 0 ? kAllZero : key < 2 * kTiny ? oz::kNonFinite : oz::scale_exp(key >> 1);
+}
+
+// Magnitudes of eight consecutive values in 8 bits, |x| 2^-e to the nearest 2^-8, from their digits
+// (N + kBias). Where a digit sum comes out small, the sum of these times the other operand's tells whether its
+// terms are large (a window that changes sign near the owner) or small (a window whose values lie
+// orders of magnitude apart).
+__device__ __forceinline__ uint2 magnitudes(const unsigned long long (&N)[8]) {
+  uint32_t w[2] = {0, 0};
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int n = int(N[u] >> 32) - int(oz::kBias >> 32);  // x 2^-e in units of 2^-23
+    w[u / 4] |= min((abs(n) + (1 << 14)) >> 15, 255) << (8 * (u % 4));
+  }
+  return make_uint2(w[0], w[1]);
+}
+
 // Window digits: a CTA cuts R windows of one block (8: one core-matrix row group, so the 16-byte
 // stores of 8 lanes fill 128 bytes; fewer where 8 a CTA would leave SMs idle). Its warps find each
 // window's largest exponent, then each thread cuts 8 consecutive nodes of one window. Bound by
-// the 14 bytes written per node and about 40 integer operations; the two reads of the window come
+// the 15 bytes written per node and about 40 integer operations; the two reads of the window come
 // from L2. (Eight windows per 256-thread CTA and 64-bit node arithmetic: 43 us for 1024 windows
 // of 2304 nodes.)
 constexpr int WIN_THREADS = 512;
@@ -73,13 +107,15 @@ __global__ void __launch_bounds__(WIN_THREADS) oz_windows_kernel(const double* _
                                                                  const TileDesc* __restrict__ tiles,
                                                                  const int32_t* __restrict__ order,
                                                                  const WinBlock* __restrict__ blocks, int wb0, int ny,
-                                                                 int nx, int* __restrict__ e, __half* __restrict__ out) {
+                                                                 int nx, int* __restrict__ e, __half* __restrict__ out,
+                                                                 uint8_t* __restrict__ mag, unsigned* __restrict__ nsmall) {
   constexpr int PER = oz::BM / R;  // CTAs per block
   const WinBlock b = blocks[wb0 + blockIdx.x / PER];
   const int r0 = (blockIdx.x % PER) * R;
   // (chained: the set-up of the multiplying kernel may begin under this one, this one's under the residual)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (blockIdx.x == 0 && threadIdx.x == 0) *nsmall = 0;
   if (r0 >= b.count) return;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   __shared__ int2 org[R];
@@ -110,16 +146,16 @@ __global__ void __launch_bounds__(WIN_THREADS) oz_windows_kernel(const double* _
 #pragma unroll 4
     for (int k = (warp % WPR) * 32 + lane; k < wn; k += 32 * WPR) {
       const int a = div_by(k, inv);
-      E = max(E, oz::exp_field(static_cast<unsigned long long>(__double_as_longlong(at(o, a, k - a * wx)))));
+      E = max(E, key_of(at(o, a, k - a * wx)));
     }
     for (int q = 16; q > 0; q >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, q));
     if (lane == 0) atomicMax(&ex[r], E);
   }
   __syncthreads();
   const int r = threadIdx.x % R;
-  const int sc = oz::scale_exp(ex[r]);
+  const int sc = exp_of_key(ex[r]);
   if (threadIdx.x < R) e[b.e_off + r0 + r] = sc;
-  const int er = sc == oz::kNonFinite ? 4096 : sc;  // (non-finite: every digit 0)
+  const int er = sc >= oz::kNonFinite ? 4096 : sc;  // (all zero, or formed in FP64: every digit 0)
   const int2 o = org[r];
   __half* dst0 = out + b.a_off;
   for (int k8 = (threadIdx.x / R) * 8; k8 < b.nkb * oz::KB; k8 += WIN_THREADS / R * 8) {
@@ -135,19 +171,14 @@ __global__ void __launch_bounds__(WIN_THREADS) oz_windows_kernel(const double* _
       }
     }
     oz::store_digits(dst0 + size_t(k8 / oz::KB) * oz::A_BLOCK + oz::tile_off(r0 + r, k8 % oz::KB), oz::A_SLICE, N);
+    *reinterpret_cast<uint2*>(mag + b.a_off / oz::S + size_t(r0 + r) * b.nkb * oz::KB + k8) = magnitudes(N);
   }
 }
 
-// Owner rows with at most SPARSE nonzero entries (selections, shifts) are formed as FP64
-// multiply-adds over those entries, in order: exact where the product with the whole row is,
-// whatever the range of the window's values, and cheaper. Their entries are kept with the digits.
-constexpr int SPARSE = 8;
-constexpr int kSparseRow = 1 << 21;  // in place of the scale exponent
-
-// Propagator digits, once per build: a CTA cuts 8 owner rows.
+// Propagator digits, once per build: a CTA cuts 8 owner rows. mid: where the row's largest entries lie.
 __global__ void __launch_bounds__(256) oz_prop_kernel(const double* __restrict__ P, int64_t n_int, int64_t n_loc,
                                                       const PropRows* __restrict__ rows, int* __restrict__ f,
-                                                      double* __restrict__ sv, int* __restrict__ sk,
+                                                      int* __restrict__ mid, uint8_t* __restrict__ mag,
                                                       __half* __restrict__ out) {
   const PropRows p = rows[blockIdx.x / 8];
   const int r0 = (blockIdx.x % 8) * 8;
@@ -155,32 +186,28 @@ __global__ void __launch_bounds__(256) oz_prop_kernel(const double* __restrict__
   __shared__ int ex[8];
   auto row = [&](int i) { return P + (int64_t(p.cls) * n_int + p.row0 + i) * n_loc; };
   {
-    int E = 0, cnt = 0;
-    const int fr = p.f_off + r0 + warp;
-    if (r0 + warp < p.rows)
-      for (int k0 = 0; k0 < p.cols; k0 += 32) {
-        const int k = k0 + lane;
-        const double v = k < p.cols ? row(r0 + warp)[k] : 0.0;
-        E = max(E, oz::exp_field(static_cast<unsigned long long>(__double_as_longlong(v))));
-        const unsigned nz = __ballot_sync(0xffffffffu, v != 0.0);
-        const int at = cnt + __popc(nz & ((1u << lane) - 1u));
-        if (v != 0.0 && at < SPARSE) {
-          sv[size_t(fr) * SPARSE + at] = v;
-          sk[size_t(fr) * SPARSE + at] = k;
-        }
-        cnt += __popc(nz);
-      }
+    const int fr = p.f_off + r0 + warp, cols = r0 + warp < p.rows ? p.cols : 0;
+    const double* P0 = row(r0 + warp);  // (not read past the last row)
+    int E = 0;
+    for (int k = lane; k < cols; k += 32) E = max(E, key_of(P0[k]));
     for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
-    if (lane < SPARSE && lane >= cnt) sk[size_t(fr) * SPARSE + lane] = -1;
+    int n = 0, at = 0;  // the entries of the largest exponent: their number, the sum of their places
+    for (int k = lane; k < cols; k += 32)
+      if (key_of(P0[k]) == E) {
+        ++n;
+        at += k;
+      }
+    n = __reduce_add_sync(0xffffffffu, n);
+    at = __reduce_add_sync(0xffffffffu, at);
     if (lane == 0) {
-      ex[warp] = oz::scale_exp(E);
-      f[fr] = ex[warp] != oz::kNonFinite && cnt > 0 && cnt <= SPARSE ? kSparseRow : ex[warp];
+      f[fr] = ex[warp] = exp_of_key(E);
+      mid[fr] = n ? at / n : 0;
     }
   }
   __syncthreads();
   const int r = threadIdx.x % 8;
   const bool live = r0 + r < p.rows;
-  const int er = ex[r] == oz::kNonFinite ? 4096 : ex[r];
+  const int er = ex[r] >= oz::kNonFinite ? 4096 : ex[r];
   for (int k8 = (threadIdx.x / 8) * 8; k8 < p.nkb * oz::KB; k8 += 256) {
     unsigned long long N[8];
 #pragma unroll
@@ -190,6 +217,7 @@ __global__ void __launch_bounds__(256) oz_prop_kernel(const double* __restrict__
     }
     oz::store_digits(out + p.b_off + size_t(k8 / oz::KB) * oz::B_BLOCK + oz::tile_off(r0 + r, k8 % oz::KB),
                      oz::B_SLICE, N);
+    *reinterpret_cast<uint2*>(mag + p.b_off / oz::S + size_t(r0 + r) * p.nkb * oz::KB + k8) = magnitudes(N);
   }
 }
 
@@ -202,103 +230,238 @@ struct StepParams {
   const __half* b;
   const int* e;
   const int* f;
-  const double* sv;    // entries of sparse owner rows
-  const int* sk;
-  const double* P;     // (rows with infinities or NaN are formed in FP64)
+  const int* mid;      // where the owner rows' largest entries lie
+  const uint8_t* amag; // magnitudes of windows and owner rows
+  const uint8_t* bmag;
+  const double* P;     // (elements formed in FP64)
   const double* src;
   double* u;
   int64_t n_int, n_loc, ny, nx;
   int unit0, nunits, ks, accumulate;
   int* err;
-};
-
-// The element of window `t` and owner row i in FP64, where an operand is not finite.
-__device__ __noinline__ double plain_dot(const StepParams& p, const TileDesc& t, int i) {
-  const double* row = p.P + (int64_t(t.cls) * p.n_int + i) * p.n_loc;
-  const int wn = t.wext[0] * t.wext[1];
-  double s = 0.0;
-  for (int k = 0; k < wn; ++k) {
-    int64_t gy = int64_t(t.org[0]) + k / t.wext[1], gx = int64_t(t.org[1]) + k % t.wext[1];
-    gy = gy < 0 ? gy + p.ny : (gy >= p.ny ? gy - p.ny : gy);
-    gx = gx < 0 ? gx + p.nx : (gx >= p.nx ? gx - p.nx : gx);
-    s = fma(row[k], p.src[gy * p.nx + gx], s);
-  }
-  return s;
-}
-
-// The same over the few entries of a sparse owner row.
-__device__ __noinline__ double sparse_dot(const StepParams& p, const TileDesc& t, int fr) {
-  double s = 0.0;
-  for (int q = 0; q < SPARSE; ++q) {
-    const int k = p.sk[size_t(fr) * SPARSE + q];
-    if (k < 0) break;
-    int64_t gy = int64_t(t.org[0]) + k / t.wext[1], gx = int64_t(t.org[1]) + k % t.wext[1];
-    gy = gy < 0 ? gy + p.ny : (gy >= p.ny ? gy - p.ny : gy);
-    gx = gx < 0 ? gx + p.nx : (gx >= p.nx ? gx - p.nx : gx);
-    s = fma(p.sv[size_t(fr) * SPARSE + q], p.src[gy * p.nx + gx], s);
-  }
-  return s;
-}
-
-// Where a unit's outputs go: window by window and owner by owner.
-struct StepUnit {
-  const StepParams& p;
-  Unit un;
-  WinBlock wb;
-  const int64_t* node0;  // first owner node and scale exponent of each window
-  const int* e;
-  const int* f;          // scale exponents of the 64 owner rows
-  int ix;                // owners per tile row
-  uint32_t inv;
-  // (rows and columns formed otherwise lie outside for the digit sums: formed() writes them)
-  __device__ int scale(int row, int col) const { return e[row] + f[col] - 62; }
-  __device__ double value(int, int, double v) const { return v; }
-  __device__ int64_t row_at(int row) const { return row < wb.count && e[row] != oz::kNonFinite ? node0[row] : -1; }
-  __device__ int64_t off(int col) const {
-    const int i = un.col0 + col, iy = div_by(i, inv);
-    return int64_t(iy) * p.nx + (i - iy * ix);
-  }
-  __device__ int64_t col_at(int col) const {
-    return col < un.ncol && f[col] != oz::kNonFinite && f[col] != kSparseRow ? off(col) : INT64_MIN / 2;
-  }
-  // Elements of non-finite windows, non-finite owner rows and sparse owner rows, by this warp:
-  // rows r0 .. r0 + nr - 1, columns c0 .. c0 + nc - 1.
-  __device__ void formed(int r0, int nr, int c0, int nc, int lane) const {
-    bool any = false;
-    for (int r = r0 + lane; r < r0 + nr; r += 32) any |= e[r] == oz::kNonFinite;
-    for (int c = c0 + lane; c < c0 + nc; c += 32) any |= f[c] == oz::kNonFinite || f[c] == kSparseRow;
-    if (!__any_sync(0xffffffffu, any)) return;
-    for (int q = lane; q < nr * nc; q += 32) {
-      const int row = r0 + q / nc, col = c0 + q % nc;
-      if (row >= wb.count || col >= un.ncol) continue;
-      const bool plain = e[row] == oz::kNonFinite || f[col] == oz::kNonFinite;
-      if (!plain && f[col] != kSparseRow) continue;
-      const TileDesc& t = p.tiles[p.order[wb.first + row]];
-      const double y = plain ? plain_dot(p, t, un.col0 + col) : sparse_dot(p, t, un.f_off + col);
-      const int64_t w = node0[row] + off(col);
-      store(w, y, load(w, row));
-    }
-  }
-  __device__ double load(int64_t w, int) const { return p.accumulate ? p.u[w] : 0.0; }
-  __device__ void store(int64_t w, double y, double old) const { p.u[w] = p.accumulate ? old + y : y; }
+  unsigned* nsmall;    // elements that oz_small_kernel looks at: their number,
+  uint2* small_at;     // window (block * 128 + row) and owner row (its place among the scale exponents; the top
+                       // bit: to be formed in any case),
+  double* small_old;   // and the owner's value before the step
 };
 
 // Per-unit tables of the epilogue.
 struct StepTables {
-  int64_t node0[oz::BM];
-  int e[oz::BM], f[oz::BN];
+  int64_t node0[oz::BM];              // first owner node of each window
+  int e[oz::BM], f[oz::BN];           // scale exponents of the windows, of the owner rows
+  uint32_t in[2], plain[2], zero[2];  // columns (32 a word): owner rows; formed in FP64; all zero
   int ix;
   __device__ void fill(const StepParams& p, const Unit& un, const WinBlock& wb, int t) {
+    if (t < 0) return;
     if (t < oz::BM) {
       const TileDesc& d = p.tiles[p.order[wb.first + min(t, wb.count - 1)]];
       node0[t] = int64_t(d.t0[0]) * p.nx + d.t0[1];
-      e[t] = p.e[wb.e_off + t];
+      e[t] = t < wb.count ? p.e[wb.e_off + t] : kAllZero;
       if (t == 0) ix = d.iext[1];
-    } else if (t < oz::BM + oz::BN) {
-      f[t - oz::BM] = p.f[un.f_off + t - oz::BM];
+    } else if (t < oz::BM + oz::BN) {  // (two whole warps)
+      const int c = t - oz::BM, v = p.f[un.f_off + c];
+      f[c] = v;
+      const uint32_t i = __ballot_sync(0xffffffffu, c < un.ncol);
+      const uint32_t q = __ballot_sync(0xffffffffu, v == oz::kNonFinite);
+      const uint32_t z = __ballot_sync(0xffffffffu, v == kAllZero);
+      if (c % 32 == 0) {
+        in[c / 32] = i;
+        plain[c / 32] = q;
+        zero[c / 32] = z;
+      }
     }
   }
 };
+
+// Where a unit's outputs go: window by window and owner by owner.
+struct StepUnit {
+  const StepParams& p;
+  const Unit& un;
+  const WinBlock& wb;
+  const StepTables& t;
+  uint32_t inv;          // owners per tile row
+  __device__ StepUnit(const StepParams& p_, const Unit& u_, const WinBlock& w_, const StepTables& t_)
+      : p(p_), un(u_), wb(w_), t(t_), inv(div_inv(uint32_t(t_.ix))) {}
+  __device__ int scale(int row, int col) const { return t.e[row] + t.f[col] - 62; }
+  __device__ double value(int, int, double v) const { return v; }
+  __device__ int64_t row_at(int row) const { return row < wb.count ? t.node0[row] : -1; }
+  __device__ int64_t col_at(int col) const {
+    const int i = un.col0 + col, iy = div_by(i, inv);
+    return col < un.ncol ? int64_t(iy) * p.nx + (i - iy * t.ix) : INT64_MIN / 2;
+  }
+  __device__ double load(int64_t w, int) const { return p.accumulate ? p.u[w] : 0.0; }
+  __device__ void store(int64_t w, double y, double old) const { p.u[w] = p.accumulate ? old + y : y; }
+  // Of columns 32 h .. 32 h + 31 of a row, those that oz_small_kernel forms in any case: windows or
+  // owner rows with infinities, NaN or values too small to cut.
+  __device__ uint32_t plain(int row, int h) const {
+    return row < wb.count ? (t.e[row] == oz::kNonFinite ? t.in[h] : t.plain[h] & t.in[h]) : 0u;
+  }
+  // And those that it looks at where their sums are small.
+  __device__ uint32_t checked(int row, int h) const {
+    return row < wb.count && t.e[row] != kAllZero ? t.in[h] & ~t.zero[h] : 0u;
+  }
+  // First of the places of this lane's `mine` elements on the list (the whole warp).
+  __device__ uint32_t places(int mine, int lane) const {
+    int upto = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+      const int v = __shfl_up_sync(0xffffffffu, upto, o);
+      if (lane >= o) upto += v;
+    }
+    unsigned base = 0;
+    if (lane == 31 && upto) base = atomicAdd(p.nsmall, unsigned(upto));
+    return __shfl_sync(0xffffffffu, base, 31) + uint32_t(upto - mine);
+  }
+  __device__ void list(uint32_t place, int row, int col, bool any_case, double old) const {
+    p.small_at[place] =
+        make_uint2(uint32_t(un.wb) * oz::BM + uint32_t(row), uint32_t(un.f_off + col) | (any_case ? 1u << 31 : 0u));
+    if (p.accumulate) p.small_old[place] = old;
+  }
+};
+
+// The elements that the digits may not give to FP64 accuracy: where the magnitudes of the owner row and of
+// the window make sum |P| |u| large, the digit sum stands; 512 nodes around the row's largest entries tell
+// as a rule, the others are looked at if they do not (eight lanes per element). Else
+// the element is formed as FP64 multiply-adds over the whole row, by a warp (an FP64 instruction takes 16 clk of the SM's
+// pipe: shared over the CTA, the sums across warps cost half as much again as the products).
+// A CTA takes elements from all over the list: those of a graded window follow one another there, and
+// are to be formed by many CTAs.
+// Of the elements of smooth fields 1 to 12 % come here (phi_1 of a residual, mu 50: 39 %), 0 to 0.2 % are
+// formed (mu 2, whose rows are narrow: 8 %). Bound by the latency of the loads (1024^2, 105 000 elements
+// of which 1000 to 1700 are formed: 39 us with cold caches, ncu), or by the FP64 pipe where many elements are formed: at
+// most what the step took before it used digits. Done in the epilogue of the products, the few
+// elements of one unit held up its CTA (four steps 2.9 ms instead of 0.69); a warp for 32 elements, one
+// after another, took 1.4 ms; 128 entries of the owner row in place of all magnitudes, too few for broad
+// rows, 1.3 ms.
+constexpr int SMALL_THREADS = 256;
+struct Formed {
+  int64_t row, to;   // the owner row in P, the owner in the state
+  double old;
+  int oy, ox, wx, wn;
+};
+__global__ void __launch_bounds__(SMALL_THREADS, 3) oz_small_kernel(const __grid_constant__ StepParams p) {
+  constexpr unsigned ALL = 0xffffffffu;
+  constexpr uint32_t LARGE = 1u << (16 - (38 - oz::kSmallSum));  // 2^-2 in units of 2^-16
+  constexpr int WARPS = SMALL_THREADS / 32;
+  __shared__ Formed todo[SMALL_THREADS];
+  __shared__ int ntodo;
+  const int warp = int(threadIdx.x) / 32, lane = int(threadIdx.x) % 32;
+  if (threadIdx.x == 0) ntodo = 0;
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int total = int(*p.nsmall), grid = int(gridDim.x);
+  const int ny = int(p.ny), nx = int(p.nx);
+  const uint4* ma = reinterpret_cast<const uint4*>(p.amag);
+  const uint4* mb = reinterpret_cast<const uint4*>(p.bmag);
+  for (int64_t first = blockIdx.x; first < total; first += int64_t(SMALL_THREADS) * grid) {
+    const int64_t place = first + int64_t(lane * WARPS + warp) * grid;  // (the warps fill evenly)
+    const bool valid = place < total;
+    const int q = valid ? int(place) : 0;
+    // this thread's element
+    uint2 at = make_uint2(0, 0);
+    int wfirst = 0, i = 0, nk = 0, mid = 0;
+    uint32_t oa = 0, ob = 0;  // its magnitudes, in 16 bytes
+    bool formed = false;
+    if (valid) {
+      at = p.small_at[q];
+      formed = at.y >> 31;
+      at.y &= 0x7fffffffu;
+      const WinBlock& wb = p.blocks[at.x / oz::BM];
+      wfirst = wb.first;
+      i = int(at.y) - wb.f0;
+      nk = formed ? 0 : wb.nkb;
+      oa = uint32_t(wb.a_off / (16 * oz::S)) + (at.x % oz::BM) * uint32_t(wb.nkb);
+      ob = uint32_t(wb.b0 / (16 * oz::S)) + uint32_t(i) * uint32_t(wb.nkb);
+      mid = max(min(p.mid[at.y] / 16 - 16, nk - 32), 0);
+    }
+    auto part = [&](uint32_t a, uint32_t b, int k, bool in) {
+      if (!in) return 0u;
+      const uint4 x = ma[a + k], y = mb[b + k];
+      return __dp4a(x.x, y.x, __dp4a(x.y, y.y, __dp4a(x.z, y.z, __dp4a(x.w, y.w, 0u))));
+    };
+    // eight lanes per element
+    const int g = lane / 8, sub = lane % 8;
+    uint32_t sum = 0;
+    const unsigned look = __ballot_sync(ALL, nk > 0);
+#pragma unroll 1
+    for (int e0 = 0; e0 < 32 && look >> e0; e0 += 8) {  // two elements a group
+      uint32_t s[2] = {0, 0};
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int e = e0 + 4 * r + g, m = __shfl_sync(ALL, mid, e) + sub, n = __shfl_sync(ALL, nk, e);
+        const uint32_t x = __shfl_sync(ALL, oa, e), y = __shfl_sync(ALL, ob, e);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) s[r] += part(x, y, m + 8 * h, m + 8 * h < n);
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s[r] += __shfl_xor_sync(ALL, s[r], o);
+        s[r] = __shfl_sync(ALL, s[r], (lane % 4) * 8);
+        if (lane / 4 == e0 / 4 + r) sum = s[r];
+      }
+    }
+    for (unsigned more = __ballot_sync(ALL, sum < LARGE && nk > 32); more;) {
+      int e = -1;  // this group's: the g-th of the next four
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j == g && more) e = __ffs(int(more)) - 1;
+        more &= more - 1;  // (0 stays 0)
+      }
+      const int l = max(e, 0), m = __shfl_sync(ALL, mid, l), nl = __shfl_sync(ALL, nk, l), n = e < 0 ? 0 : nl;
+      const uint32_t x = __shfl_sync(ALL, oa, l), y = __shfl_sync(ALL, ob, l);
+      uint32_t s = 0;
+#pragma unroll 6
+      for (int k = sub; k < n; k += 8) s += part(x, y, k, k < m || k >= m + 32);
+      __syncwarp();
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(ALL, s, o);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int to = __shfl_sync(ALL, e, 8 * j);
+        const uint32_t v = __shfl_sync(ALL, s, 8 * j);
+        if (lane == to) sum += v;
+      }
+    }
+    if (valid && (formed || sum < LARGE)) {
+      const TileDesc& t = p.tiles[p.order[wfirst + int(at.x % oz::BM)]];
+      const int iy = i / t.iext[1];
+      todo[atomicAdd(&ntodo, 1)] = Formed{(int64_t(t.cls) * p.n_int + i) * p.n_loc,
+                                          int64_t(t.t0[0] + iy) * p.nx + t.t0[1] + (i - iy * t.iext[1]),
+                                          p.accumulate ? p.small_old[q] : 0.0, t.org[0], t.org[1], t.wext[1],
+                                          t.wext[0] * t.wext[1]};
+    }
+    __syncthreads();
+    const int n = ntodo;
+    for (int d = warp; d < n; d += WARPS) {
+      const Formed f = todo[d];
+      const double* row = p.P + f.row;
+      const uint32_t inv = div_inv(uint32_t(f.wx));
+      double y = 0.0;
+      constexpr int U = 12;  // loads of each operand in flight
+      for (int k0 = lane; k0 < f.wn; k0 += 32 * U) {
+        double v[U], w[U];
+#pragma unroll
+        for (int h = 0; h < U; ++h) {
+          const int k = k0 + 32 * h, b = div_by(k, inv);
+          int gy = f.oy + b, gx = f.ox + (k - b * f.wx);
+          gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
+          gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
+          v[h] = k < f.wn ? row[k] : 0.0;
+          w[h] = k < f.wn ? p.src[uint32_t(gy) * uint32_t(nx) + uint32_t(gx)] : 0.0;
+        }
+#pragma unroll
+        for (int h = 0; h < U; ++h) y = fma(v[h], w[h], y);
+      }
+      for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(ALL, y, o);
+      if (lane == 0) p.u[f.to] = p.accumulate ? f.old + y : y;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) ntodo = 0;
+    __syncthreads();
+  }
+}
 
 // The units of one CTA, every gridDim.x-th: increments are added to the state (PHI) or the owners
 // stored (EXP).
@@ -320,10 +483,25 @@ struct StepWork {
   __device__ void finish(int k, int quarter, int half, int lane, double* out, const long long (&hi)[32],
                          const long long (&lo)[32]) {
     const Unit un = p.units[index(k)];
-    const StepTables& t = tab[k & 1];
-    StepUnit o{p, un, p.blocks[un.wb], t.node0, t.e, t.f, t.ix, div_inv(uint32_t(t.ix))};
+    const WinBlock wb = p.blocks[un.wb];
+    const StepUnit o(p, un, wb, tab[k & 1]);
+    const int row = 32 * quarter + lane;
+    uint32_t small = 0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) small |= oz::small_sum(hi[j]) ? 1u << j : 0u;
+    const uint32_t plain = o.plain(row, half);
+    small = (small & o.checked(row, half)) | plain;
+    if (__any_sync(0xffffffffu, small != 0)) {
+      uint32_t place = o.places(__popc(small), lane);
+      const int64_t at = o.row_at(row);
+#pragma unroll 4
+      for (; small; small &= small - 1) {
+        const int j = __ffs(int(small)) - 1, col = 32 * half + j;
+        o.list(place++, row, col, plain >> j & 1u, o.load(at + o.col_at(col), row));
+      }
+      __syncwarp();  // (before they are overwritten)
+    }
     oz::write_tile(o, quarter, half, lane, out, hi, lo);
-    o.formed(32 * quarter, 32, 32 * half, 32, lane);
   }
 };
 
@@ -375,16 +553,16 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_split_kernel(const __g
   cl.sync();
   const int lcw = 6 - (31 - __clz(ks)), cw = 1 << lcw, c0 = rank * cw;  // this CTA's columns
   if (!s_abort && c0 < un.ncol) {
-    const StepUnit o{p, un, wb, tab.node0, tab.e, tab.f, tab.ix, div_inv(uint32_t(tab.ix))};
+    const StepUnit o(p, un, wb, tab);
     constexpr int U = 4;  // elements per thread in flight
-    const int total = wb.count * cw;
-    for (int q0 = threadIdx.x; q0 < total; q0 += U * oz::THREADS) {
+    const int total = wb.count * cw, warp0 = int(threadIdx.x) / 32 * 32, lane = int(threadIdx.x) % 32;
+    for (int q0 = warp0; q0 < total; q0 += U * oz::THREADS) {  // (whole warps)
       int64_t where[U];
       double old[U];
       bool in[U];
 #pragma unroll
       for (int k = 0; k < U; ++k) {
-        const int q = q0 + k * oz::THREADS, row = min(q >> lcw, oz::BM - 1);
+        const int q = q0 + lane + k * oz::THREADS, row = min(q >> lcw, oz::BM - 1);
         const int64_t ra = o.row_at(row), ca = o.col_at(c0 + (q & (cw - 1)));
         in[k] = ra >= 0 && ca >= 0 && q < total;
         where[k] = ra + ca;
@@ -392,19 +570,23 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_split_kernel(const __g
       }
 #pragma unroll
       for (int k = 0; k < U; ++k) {
-        if (!in[k]) continue;
-        const int q = q0 + k * oz::THREADS, col = c0 + (q & (cw - 1)), row = q >> lcw;
+        const int q = q0 + lane + k * oz::THREADS, col = c0 + (q & (cw - 1)), row = min(q >> lcw, oz::BM - 1);
         longlong2 v = make_longlong2(0, 0);
-        for (int j = 0; j < ks; ++j) {
-          const longlong2 s = *cl.map_shared_rank(sums + col * oz::SUM_PITCH + row, j);
-          v.x += s.x;
-          v.y += s.y;
+        if (in[k])
+          for (int j = 0; j < ks; ++j) {
+            const longlong2 s = *cl.map_shared_rank(sums + col * oz::SUM_PITCH + row, j);
+            v.x += s.x;
+            v.y += s.y;
+          }
+        const uint32_t bit = 1u << (col % 32), plain = o.plain(row, col / 32) & bit;
+        const bool small = in[k] && (plain || (oz::small_sum(v.x) && (o.checked(row, col / 32) & bit)));
+        if (__any_sync(0xffffffffu, small)) {
+          const uint32_t place = o.places(small ? 1 : 0, lane);
+          if (small) o.list(place, row, col, plain != 0, old[k]);
         }
-        o.store(where[k], oz::sums_to_double(v.x, v.y, o.scale(row, col)), old[k]);
+        if (in[k]) o.store(where[k], oz::sums_to_double(v.x, v.y, o.scale(row, col)), old[k]);
       }
     }
-    // (ten warps: 128 / 8 rows for the first eight)
-    if (threadIdx.x < 256) o.formed(int(threadIdx.x) / 32 * 16, 16, c0, cw, int(threadIdx.x) % 32);
   }
   cl.sync();  // the sums stay until every CTA of the cluster has read them
   oz::release(tmem);
@@ -430,8 +612,13 @@ struct OzPlan {
   __half* d_b = nullptr;
   int* d_e = nullptr;
   int* d_f = nullptr;
-  double* d_sv = nullptr;
-  int* d_sk = nullptr;
+  int* d_mid = nullptr;
+  uint8_t* d_amag = nullptr;
+  uint8_t* d_bmag = nullptr;
+  unsigned* d_nsmall = nullptr;
+  uint2* d_small_at = nullptr;
+  double* d_small_old = nullptr;
+  int64_t max_owners = 0;      // of a group
   int* d_err = nullptr;
 };
 
@@ -447,14 +634,15 @@ void plan_oz(const lem_ctx* ctx, OzPlan* z) {
   };
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return nkb_of(a) > nkb_of(b); });
   OzPlan::Group g{0, 0, 0, 0, 1};
-  int64_t held = 0;
+  int64_t held = 0, owned = 0;
   int ge = 0;
   auto close = [&]() {
     if (g.nwb) z->groups.push_back(g);
     z->a_halves = std::max<size_t>(z->a_halves, size_t(held));
     z->ne = std::max(z->ne, ge);
+    z->max_owners = std::max(z->max_owners, owned);
     g = OzPlan::Group{int(z->blocks.size()), 0, int(z->units.size()), 0, 1};
-    held = 0;
+    held = owned = 0;
     ge = 0;
   };
   for (int c : order) {
@@ -472,8 +660,9 @@ void plan_oz(const lem_ctx* ctx, OzPlan* z) {
       const int64_t halves = int64_t(nkb) * oz::A_BLOCK;
       if (held && (held + halves) * 2 > kMaxWindowBytes) close();
       const int wb = int(z->blocks.size());
-      z->blocks.push_back(WinBlock{w, std::min(oz::BM, n1 - w), c, nkb, held, ge, 0});
+      z->blocks.push_back(WinBlock{w, std::min(oz::BM, n1 - w), c, nkb, held, ge, f0, b0});
       held += halves;
+      owned += int64_t(std::min(oz::BM, n1 - w)) * owners;
       ge += oz::BM;
       g.nwb++;
       for (int j = 0; j < ncb; ++j) {
@@ -544,7 +733,9 @@ void oz_destroy(lem_ctx* ctx) {
   if (!z) return;
   for (void* p : {static_cast<void*>(z->d_blocks), static_cast<void*>(z->d_units), static_cast<void*>(z->d_rows),
                   static_cast<void*>(z->d_a), static_cast<void*>(z->d_b), static_cast<void*>(z->d_e),
-                  static_cast<void*>(z->d_f), static_cast<void*>(z->d_sv), static_cast<void*>(z->d_sk),
+                  static_cast<void*>(z->d_f), static_cast<void*>(z->d_mid), static_cast<void*>(z->d_amag),
+                  static_cast<void*>(z->d_bmag), static_cast<void*>(z->d_nsmall),
+                  static_cast<void*>(z->d_small_at), static_cast<void*>(z->d_small_old),
                   static_cast<void*>(z->d_err)})
     if (p) cudaFreeAsync(p, ctx->stream);
   delete z;
@@ -568,8 +759,9 @@ lem_status oz_prepare(lem_ctx* ctx) {
   LEM_TRY(alloc(&z->d_b, z->b_halves));
   LEM_TRY(alloc(&z->d_e, size_t(z->ne)));
   LEM_TRY(alloc(&z->d_f, size_t(z->nf)));
-  LEM_TRY(alloc(&z->d_sv, size_t(z->nf) * SPARSE));
-  LEM_TRY(alloc(&z->d_sk, size_t(z->nf) * SPARSE));
+  LEM_TRY(alloc(&z->d_mid, size_t(z->nf)));
+  LEM_TRY(alloc(&z->d_bmag, z->b_halves / oz::S));
+  LEM_TRY(alloc(&z->d_nsmall, 1));
   LEM_TRY(alloc(&z->d_err, 1));
   cudaStream_t st = ctx->stream;
   LEM_CUDA_TRY(cudaMemcpyAsync(z->d_blocks, z->blocks.data(), sizeof(WinBlock) * z->blocks.size(),
@@ -586,7 +778,7 @@ lem_status oz_pack(lem_ctx* ctx) {
   OzPlan* z = ctx->oz;
   if (!z) return LEM_OK;
   oz_prop_kernel<<<unsigned(z->rows.size() * 8), 256, 0, ctx->stream>>>(ctx->d_P, ctx->n_int, ctx->n_loc, z->d_rows,
-                                                                        z->d_f, z->d_sv, z->d_sk, z->d_b);
+                                                                        z->d_f, z->d_mid, z->d_bmag, z->d_b);
   LEM_CUDA_TRY(cudaGetLastError());
   return LEM_OK;
 }
@@ -605,6 +797,11 @@ lem_status step_oz(lem_ctx* ctx, double* d_u) {
   OzPlan* z = ctx->oz;
   cudaStream_t st = ctx->stream;
   if (!z->d_a) {
+    if (!z->d_small_at)
+      LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&z->d_small_at), sizeof(uint2) * size_t(z->max_owners)));
+    if (!z->d_small_old && ctx->desc.mode == LEM_MODE_PHI)
+      LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&z->d_small_old), sizeof(double) * size_t(z->max_owners)));
+    if (!z->d_amag) LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&z->d_amag), z->a_halves / oz::S));
     LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&z->d_a), sizeof(__half) * z->a_halves));
     // rows past a block's last window are multiplied too (their sums are dropped)
     LEM_CUDA_TRY(cudaMemsetAsync(z->d_a, 0, sizeof(__half) * z->a_halves, st));
@@ -634,9 +831,10 @@ lem_status step_oz(lem_ctx* ctx, double* d_u) {
     LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, cut, src, static_cast<const TileDesc*>(ctx->d_tiles),
                                     static_cast<const int32_t*>(ctx->d_class_order),
                                     static_cast<const WinBlock*>(z->d_blocks), g.wb0, int(ctx->ny), int(ctx->nx), z->d_e,
-                                    z->d_a));
-    StepParams p{z->d_blocks, z->d_units, ctx->d_tiles, ctx->d_class_order, z->d_a, z->d_b, z->d_e, z->d_f, z->d_sv, z->d_sk, ctx->d_P,
-                 src, d_u, ctx->n_int, ctx->n_loc, ctx->ny, ctx->nx, g.unit0, g.nunits, g.ks, phi ? 1 : 0, z->d_err};
+                                    z->d_a, z->d_amag, z->d_nsmall));
+    StepParams p{z->d_blocks, z->d_units, ctx->d_tiles, ctx->d_class_order, z->d_a, z->d_b, z->d_e, z->d_f, z->d_mid, z->d_amag, z->d_bmag, ctx->d_P,
+                 src, d_u, ctx->n_int, ctx->n_loc, ctx->ny, ctx->nx, g.unit0, g.nunits, g.ks, phi ? 1 : 0, z->d_err, z->d_nsmall,
+                 z->d_small_at, z->d_small_old};
     if (g.ks == 1) {
       cfg.gridDim = dim3(unsigned(std::min(g.nunits, z->nsm)));
       cfg.blockDim = dim3(oz::THREADS);
@@ -646,6 +844,13 @@ lem_status step_oz(lem_ctx* ctx, double* d_u) {
       cfg = split_config(g.ks, g.nunits, st, at);
       LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_step_split_kernel, p));
     }
+    at[0] = chained();
+    cfg.gridDim = dim3(unsigned(3 * z->nsm));
+    cfg.blockDim = dim3(SMALL_THREADS);
+    cfg.dynamicSmemBytes = 0;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_small_kernel, p));
   }
   ctx->timing_end(stop);
   return LEM_OK;
