@@ -248,29 +248,22 @@ __global__ void lincomb_kernel(double* out, int n, int64_t ld, int ncols, Lin L)
 //   other rows:  (Pi G)[i, :] + Y_i (Pi G)[K, :],
 // one rank-kb product C = Y B + D with B the permuted pivot rows and D the permuted columns with
 // rows K taken as zero, on the tensor cores or (FP64 tier) as an FP64 product; one pivot at a time
-// every pivot read and wrote all of G.
-//
-// With the tensor cores, panels may be gathered GJ_SB columns at a time: a panel's product is applied to the other columns
-// of its group only (to those still to be eliminated and, being the tracker of the group's earlier
-// panels, to those already eliminated), after which the group's n x GJ_SB block is the tracker of
-// all its pivots, and one rank-GJ_SB product updates the columns behind the group. A tile of a
-// rank-64 product costs little less than one of a rank-256 product (its sums are converted and
-// written all the same): one product per panel took 11 ms of a build of 25 matrices of 784.
-constexpr int GJ_KB = 64, GJ_SB = 256;
+// every pivot read and wrote all of G. (One product of rank 256 for four panels saves a tenth of a build
+// of 25 matrices of 784, but rounds worse: 1.5 to 2.6 times the error of the propagators.)
+constexpr int GJ_KB = 64;
 
-// One pivot step of a panel at columns k0 - s0 .. of the group block Y (n x GJ_SB, its first column
-// standing for matrix column s0), for matrices too large for bgj_panel_kernel. In place: the
-// pivot column becomes the tracker column.
-__global__ void bgj_pivot_kernel(double* Y, int n, int c0, int k0, int c, int kb, int* piv, int* status) {
+// One pivot step of a panel at columns k0 .. of the matrix, copied to Y (n x GJ_KB), for matrices too large for
+// bgj_panel_kernel. In place: the pivot column becomes the tracker column.
+__global__ void bgj_pivot_kernel(double* Y, int n, int k0, int c, int kb, int* piv, int* status) {
   const int b = blockIdx.x;
-  double* M = Y + int64_t(b) * n * GJ_SB + c0;
+  double* M = Y + int64_t(b) * n * GJ_KB;
   const int r = k0 + c;
   __shared__ double sv[256];
   __shared__ int si[256];
   double best = -1.0;
   int bi = r;
   for (int i = r + threadIdx.x; i < n; i += blockDim.x) {
-    const double v = fabs(M[int64_t(i) * GJ_SB + c]);
+    const double v = fabs(M[int64_t(i) * GJ_KB + c]);
     if (v > best) { best = v; bi = i; }
   }
   sv[threadIdx.x] = best;
@@ -288,37 +281,37 @@ __global__ void bgj_pivot_kernel(double* Y, int n, int c0, int k0, int c, int kb
     __syncthreads();
   }
   const int p = si[0];
-  const double pv = M[int64_t(p) * GJ_SB + c];
+  const double pv = M[int64_t(p) * GJ_KB + c];
   __syncthreads();  // every thread holds pv before rows r / p are rewritten
   if (!(sv[0] > 0.0) || !isfinite(pv)) {
     if (threadIdx.x == 0) {
       atomicExch(status, int(LEM_ENUMERIC));
-      piv[b * GJ_SB + c0 + c] = r;  // no swap
+      piv[b * GJ_KB + c] = r;  // no swap
     }
     return;
   }
-  if (threadIdx.x == 0) piv[b * GJ_SB + c0 + c] = p;
+  if (threadIdx.x == 0) piv[b * GJ_KB + c] = p;
   const double inv = 1.0 / pv;
   for (int j = threadIdx.x; j < kb; j += blockDim.x) {
-    const double a = M[int64_t(r) * GJ_SB + j], q = M[int64_t(p) * GJ_SB + j];
-    if (p != r) M[int64_t(p) * GJ_SB + j] = a;
-    M[int64_t(r) * GJ_SB + j] = (j == c ? 1.0 : q) * inv;  // inject the unit column, then scale
+    const double a = M[int64_t(r) * GJ_KB + j], q = M[int64_t(p) * GJ_KB + j];
+    if (p != r) M[int64_t(p) * GJ_KB + j] = a;
+    M[int64_t(r) * GJ_KB + j] = (j == c ? 1.0 : q) * inv;  // inject the unit column, then scale
   }
 }
 
 // Eliminate panel column c from every row but the pivot row: 4 rows per block, thread t of a row
 // updates panel column t.
-__global__ void bgj_elim_kernel(double* Y, int n, int c0, int k0, int c, int kb) {
+__global__ void bgj_elim_kernel(double* Y, int n, int k0, int c, int kb) {
   const int b = blockIdx.y;
   const int i = blockIdx.x * 4 + threadIdx.x / 64, t = threadIdx.x % 64;
   const int r = k0 + c;
-  double* M = Y + int64_t(b) * n * GJ_SB + c0;
+  double* M = Y + int64_t(b) * n * GJ_KB;
   const bool live = i < n && i != r;
-  const double f = live ? M[int64_t(i) * GJ_SB + c] : 0.0;
+  const double f = live ? M[int64_t(i) * GJ_KB + c] : 0.0;
   __syncthreads();  // column c is read before it is overwritten
   if (!live || f == 0.0 || t >= kb) return;
-  double* m = M + int64_t(i) * GJ_SB + t;
-  *m = fma(-f, M[int64_t(r) * GJ_SB + t], t == c ? 0.0 : *m);
+  double* m = M + int64_t(i) * GJ_KB + t;
+  *m = fma(-f, M[int64_t(r) * GJ_KB + t], t == c ? 0.0 : *m);
 }
 
 // A whole panel in one launch, a cluster of CTAs per matrix, each holding a share of the panel's
@@ -345,11 +338,10 @@ struct PanelStep {
   double rrow[GJ_KB];  // row r
 };
 
-// src: the panel's columns (leading dimension lds, matrices ss apart); Y: where the tracker goes
-// (column c0 of the group block; may be src).
+// src: the panel's columns (leading dimension lds, matrices ss apart); Y: where the tracker goes.
 __global__ void __launch_bounds__(PANEL_THREADS) bgj_panel_kernel(const double* src, int64_t lds, int64_t ss, int n,
-                                                                  int c0, int k0, int kb, int csize, int rows_per,
-                                                                  double* Y, int* piv, int* status) {
+                                                                  int k0, int kb, int csize, int rows_per, double* Y,
+                                                                  int* piv, int* status) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ __align__(16) double psm[];
@@ -439,7 +431,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) bgj_panel_kernel(const double* 
     if (pval <= 0 || pval >= 0x7FF0000000000000ll) {  // zero or non-finite pivot (the same in every CTA)
       if (rank == 0) {
         if (tid == 0) atomicExch(status, int(LEM_ENUMERIC));
-        for (int q = c + tid; q < kb; q += PANEL_THREADS) piv[b * GJ_SB + c0 + q] = k0 + q;  // no more swaps
+        for (int q = c + tid; q < kb; q += PANEL_THREADS) piv[b * GJ_KB + q] = k0 + q;  // no more swaps
       }
       break;
     }
@@ -455,7 +447,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) bgj_panel_kernel(const double* 
         fzero[p - lo] = (__double_as_longlong(old) & 0x7FFFFFFFFFFFFFFFll) == 0;
       }
     }
-    if (rank == 0 && tid == 128) piv[b * GJ_SB + c0 + c] = p;
+    if (rank == 0 && tid == 128) piv[b * GJ_KB + c] = p;
     __syncthreads();
     if (j < kb) {
       const double pj = prow[j];
@@ -485,14 +477,14 @@ __global__ void __launch_bounds__(PANEL_THREADS) bgj_panel_kernel(const double* 
     __syncthreads();
   }
   cl.sync();  // no CTA leaves while another may write into its memory
-  double* Yb = Y + int64_t(b) * n * GJ_SB + c0;
+  double* Yb = Y + int64_t(b) * n * GJ_KB;
   for (int e = tid; e < cnt * GJ_KB; e += PANEL_THREADS) {
     const int i = e / GJ_KB, q = e % GJ_KB;
-    if (q < kb) Yb[int64_t(lo + i) * GJ_SB + q] = M[i * PANEL_PITCH + q];
+    if (q < kb) Yb[int64_t(lo + i) * GJ_KB + q] = M[i * PANEL_PITCH + q];
   }
 }
 
-static cudaError_t launch_panel(const double* src, int64_t lds, int64_t ss, int n, int c0, int k0, int kb, double* Y,
+static cudaError_t launch_panel(const double* src, int64_t lds, int64_t ss, int n, int k0, int kb, double* Y,
                                 int* piv, int* status, int nb, cudaStream_t st) {
   // 8 rows a CTA at least: panels of 64 rows took 167, 134 and 122 us on 2, 4 and 8 CTAs
   const int csize = std::min(PANEL_MAX_CLUSTER, (n + 7) / 8);
@@ -511,19 +503,19 @@ static cudaError_t launch_panel(const double* src, int64_t lds, int64_t ss, int 
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, bgj_panel_kernel, src, lds, ss, n, c0, k0, kb, csize, rows_per, Y, piv, status);
+  return cudaLaunchKernelEx(&cfg, bgj_panel_kernel, src, lds, ss, n, k0, kb, csize, rows_per, Y, piv, status);
 }
 
-// Row swaps k0 + c <-> piv[c], c < kb, in order, on columns [0, cols) of a matrix but [x0, x1).
+// Row swaps k0 + c <-> piv[c], c < kb, in order, on columns [0, cols) of a matrix.
 // rows (not null): the pivot rows k0 .. k0 + kb - 1 then move there (kb x cols), leaving zeros.
-__global__ void bgj_swap_kernel(double* M, int64_t ld, int64_t stride, int cols, int x0, int x1, int k0, int kb,
-                                const int* piv, double* rows) {
+__global__ void bgj_swap_kernel(double* M, int64_t ld, int64_t stride, int cols, int k0, int kb, const int* piv,
+                                double* rows) {
   const int b = blockIdx.y;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= cols || (j >= x0 && j < x1)) return;
+  if (j >= cols) return;
   double* m = M + int64_t(b) * stride + j;
   for (int c = 0; c < kb; ++c) {
-    const int p = piv[b * GJ_SB + c];
+    const int p = piv[b * GJ_KB + c];
     if (p == k0 + c) continue;
     const double a = m[int64_t(k0 + c) * ld];
     m[int64_t(k0 + c) * ld] = m[int64_t(p) * ld];
@@ -670,54 +662,35 @@ static lem_status mul_list(lem_ctx* ctx, TcGemm* tcg, int nbatch, const int* map
 }
 
 // Gauss-Jordan elimination of G = [Q | RHS] (nb matrices of n x gjcols): on exit the RHS
-// columns hold Q^{-1} RHS. Panels in FP64, the other columns by products (tcg: on tcgen05). The
-// split apply's propagators keep one product per panel: a group's product rounds otherwise, and
-// the FP16 pieces cut from the propagators would differ.
+// columns hold Q^{-1} RHS. Panels in FP64, the other columns by products (tcg: on tcgen05).
 static lem_status solve_gj(lem_ctx* ctx, TcGemm* tcg, double* G, int n, int gjcols, int nb, Scratch& ws) {
   cudaStream_t st = ctx->stream;
-  const int group = tcg && !ctx->split ? GJ_SB : GJ_KB;
   double *Y = nullptr, *rows = nullptr;
   int* piv = nullptr;
-  LEM_TRY(ws.get(&Y, size_t(nb) * n * GJ_SB));
-  LEM_TRY(ws.get(&piv, size_t(nb) * GJ_SB));
+  LEM_TRY(ws.get(&Y, size_t(nb) * n * GJ_KB));
+  LEM_TRY(ws.get(&piv, size_t(nb) * GJ_KB));
   // FP64 products write over their right factor: the pivot rows move out first
   if (!tcg) LEM_TRY(ws.get(&rows, size_t(nb) * GJ_KB * gjcols));
-  const int64_t sG = int64_t(n) * gjcols, sY = int64_t(n) * GJ_SB;
-  for (int s0 = 0; s0 < n; s0 += group) {  // a group of columns
-    const int sb = std::min(group, n - s0);
-    const bool one = sb <= GJ_KB && n <= PANEL_MAX_N;  // a single panel, read from G itself
-    if (!one) copy_cols_kernel<<<grid1(int64_t(n) * sb, nb), 256, 0, st>>>(Y, GJ_SB, 0, G, gjcols, s0, n, sb);
-    for (int c0 = 0; c0 < sb; c0 += GJ_KB) {
-      const int kb = std::min(GJ_KB, sb - c0), k0 = s0 + c0;
-      if (n <= PANEL_MAX_N) {
-        LEM_CUDA_TRY(one ? launch_panel(G + s0, gjcols, sG, n, c0, k0, kb, Y, piv, ctx->d_status, nb, st)
-                         : launch_panel(Y + c0, GJ_SB, sY, n, c0, k0, kb, Y, piv, ctx->d_status, nb, st));
-      } else {
-        for (int c = 0; c < kb; ++c) {
-          bgj_pivot_kernel<<<nb, 256, 0, st>>>(Y, n, c0, k0, c, kb, piv, ctx->d_status);
-          bgj_elim_kernel<<<dim3((n + 3) / 4, nb), 256, 0, st>>>(Y, n, c0, k0, c, kb);
-        }
+  const int64_t sG = int64_t(n) * gjcols, sY = int64_t(n) * GJ_KB;
+  for (int k0 = 0; k0 < n; k0 += GJ_KB) {  // a panel of columns
+    const int kb = std::min(GJ_KB, n - k0);
+    if (n <= PANEL_MAX_N) {
+      LEM_CUDA_TRY(launch_panel(G + k0, gjcols, sG, n, k0, kb, Y, piv, ctx->d_status, nb, st));
+    } else {
+      copy_cols_kernel<<<grid1(int64_t(n) * kb, nb), 256, 0, st>>>(Y, GJ_KB, 0, G, gjcols, k0, n, kb);
+      for (int c = 0; c < kb; ++c) {
+        bgj_pivot_kernel<<<nb, 256, 0, st>>>(Y, n, k0, c, kb, piv, ctx->d_status);
+        bgj_elim_kernel<<<dim3((n + 3) / 4, nb), 256, 0, st>>>(Y, n, k0, c, kb);
       }
-      if (kb == sb) continue;
-      // the group's other columns: C = Y_panel B + D with B the pivot rows, D without them
-      bgj_swap_kernel<<<dim3(1, nb), 256, 0, st>>>(Y, GJ_SB, sY, sb, c0, c0 + kb, k0, kb, piv + c0, nullptr);
-      LEM_CUDA_TRY(cudaGetLastError());
-      TcProduct pr[2];
-      int np = 0;
-      for (int side = 0; side < 2; ++side) {
-        double* T = Y + (side ? c0 + kb : 0);
-        const int cols = side ? sb - c0 - kb : c0;
-        if (cols > 0) pr[np++] = TcProduct{cols, T + int64_t(k0) * GJ_SB, GJ_SB, sY, T, GJ_SB, sY, T, GJ_SB, sY, nullptr};
-      }
-      LEM_TRY(mul_list(ctx, tcg, nb, nullptr, n, kb, Y + c0, GJ_SB, sY, pr, np, k0, k0 + kb));
     }
-    const int m_r = gjcols - (s0 + sb);
-    double* T = G + (s0 + sb);  // the columns behind the group
-    bgj_swap_kernel<<<dim3((m_r + 255) / 256, nb), 256, 0, st>>>(T, gjcols, sG, m_r, 0, 0, s0, sb, piv, rows);
+    // the columns behind the panel: C = Y B + D with B the pivot rows, D without them
+    const int m_r = gjcols - (k0 + kb);
+    double* T = G + (k0 + kb);
+    bgj_swap_kernel<<<dim3((m_r + 255) / 256, nb), 256, 0, st>>>(T, gjcols, sG, m_r, k0, kb, piv, rows);
     LEM_CUDA_TRY(cudaGetLastError());
-    const double* B = tcg ? T + int64_t(s0) * gjcols : rows;
-    const TcProduct pr{m_r, B, tcg ? gjcols : m_r, tcg ? sG : int64_t(sb) * m_r, T, gjcols, sG, T, gjcols, sG, nullptr};
-    LEM_TRY(mul_list(ctx, tcg, nb, nullptr, n, sb, Y, GJ_SB, sY, &pr, 1, s0, s0 + sb));
+    const double* B = tcg ? T + int64_t(k0) * gjcols : rows;
+    const TcProduct pr{m_r, B, tcg ? gjcols : m_r, tcg ? sG : int64_t(kb) * m_r, T, gjcols, sG, T, gjcols, sG, nullptr};
+    LEM_TRY(mul_list(ctx, tcg, nb, nullptr, n, kb, Y, GJ_KB, sY, &pr, 1, k0, k0 + kb));
   }
   LEM_CUDA_TRY(cudaGetLastError());
   return LEM_OK;
@@ -1124,7 +1097,7 @@ lem_status build_propagators_impl(lem_ctx* ctx, const double* d_state) {
   // batch size from a scratch budget of 8 GiB
   const int gjc = rb3 ? 5 * int(n) : ctx->desc.mode == LEM_MODE_PHI ? 3 * int(n) : 2 * int(n);
   const double per = double(nmat) * n * n * sizeof(double) +
-                     (ctx->build_tc ? double(tc_gemm_bytes(int(n), 1, gjc, ctx->desc.mode == LEM_MODE_PHI ? 4 : 2)) + sizeof(double) * n * GJ_SB : sizeof(double) * (double(n) * GJ_SB + double(gjc) * GJ_KB));
+                     (ctx->build_tc ? double(tc_gemm_bytes(int(n), 1, gjc, ctx->desc.mode == LEM_MODE_PHI ? 4 : 2)) + sizeof(double) * n * GJ_KB : sizeof(double) * (double(n) * GJ_KB + double(gjc) * GJ_KB));
   int64_t bmax = std::max<int64_t>(1, int64_t((8.0 * (1ull << 30)) / per));
   bmax = std::min<int64_t>(bmax, 65535);
   for (int64_t c0 = 0; c0 < nc; c0 += bmax) {

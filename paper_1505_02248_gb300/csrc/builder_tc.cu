@@ -228,12 +228,12 @@ inline int pad_to(int x, int m) { return (x + m - 1) / m * m; }
 struct Caps {
   size_t a, b, e, f;
 };
-// Room for products of np right factors of n x n, and for the rank-256 updates of an n x gjcols
+// Room for products of np right factors of n x n, and for the rank-64 updates of an n x gjcols
 // elimination (of rank n where n is less).
 Caps caps_for(int n, int nb, int gjcols, int np) {
   const size_t ka = pad_to(n, oz::KB) / oz::KB, ra = pad_to(n, oz::BM) / oz::BM, cb = pad_to(n, oz::BN) / oz::BN,
                cg = pad_to(std::max(gjcols, 1), oz::BN) / oz::BN;
-  return {size_t(nb) * ra * ka * oz::A_BLOCK, size_t(nb) * std::max(np * cb * ka, cg * std::min<size_t>(ka, 256 / oz::KB)) * oz::B_BLOCK,
+  return {size_t(nb) * ra * ka * oz::A_BLOCK, size_t(nb) * std::max(np * cb * ka, cg * std::min<size_t>(ka, 64 / oz::KB)) * oz::B_BLOCK,
           size_t(nb) * ra * oz::BM, size_t(nb) * std::max(np * cb, cg) * oz::BN};
 }
 

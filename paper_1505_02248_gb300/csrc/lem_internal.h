@@ -207,7 +207,7 @@ struct TcProduct {
   const double* diag;
 };
 // workspace for products of nb matrices of n x n with up to np right factors at once, and for
-// rank-256 updates of n x gjcols ones
+// rank-64 updates of n x gjcols ones
 size_t tc_gemm_bytes(int n, int nb, int gjcols, int np);
 lem_status tc_gemm_create(int n, int nb, int gjcols, int np, void* mem, cudaStream_t st, TcGemm** out);
 void tc_gemm_destroy(TcGemm* g);

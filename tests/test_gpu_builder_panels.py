@@ -1,0 +1,37 @@
+"""The solve of the propagator build, panel by panel (csrc/builder.cu, solve_gj)."""
+import numpy as np
+import pytest
+
+from paper_1505_02248_gb300 import lem as L
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1505_02248_gb300 import build as B
+    B.build()
+    L.load()
+
+
+@pytest.mark.parametrize("tile,H", [(8, 4), (16, 4), (16, 6)])
+def test_one_operator_is_built_alike_for_every_apply(tile, H):
+    """One operator for all windows (the tensor-core split apply) and the same coefficients node by node (a
+    propagator per tile, FP32 rows): the windows' matrices are the same, and so are the builds, bit for
+    bit: neither takes products that round worse."""
+    side = 4 * tile
+    coef = {"C": -46.0, "W": 14.0, "E": 10.0, "S": 12.0, "N": 10.0}
+    one = L.Lem((side, side), ("periodic",) * 2, coef, 1.0, (tile,) * 2, (H,) * 2, prec="split")
+    per = L.Lem((side, side), ("periodic",) * 2, {k: np.full(side * side, v) for k, v in coef.items()}, 1.0, (tile,) * 2,
+                (H,) * 2, prec="split_fast")
+    assert L.APPLY_PATHS[one.info()["apply_path"]] == "tc_split" and L.APPLY_PATHS[per.info()["apply_path"]] == "f32_gemv"
+    one.build()
+    per.build()
+    P = one.propagator(0)
+    for c in (0, 5, 15):
+        assert np.array_equal(per.propagator(c), P)
+    one.close()
+    per.close()
