@@ -25,15 +25,16 @@ lem_status cuda_fail(cudaError_t e, const char* what) {
 }
 
 // Host-side fault injection for tests: LEM_FAULT=alloc makes every device allocation of
-// a context fail with LEM_ENOMEM (no GPU fault is involved).
-static bool fault_alloc() {
+// a context fail with LEM_ENOMEM, LEM_FAULT=alloc=N those of exactly N bytes (no GPU fault is involved).
+bool fault_alloc(size_t bytes) {
   const char* f = std::getenv("LEM_FAULT");
-  return f && std::strcmp(f, "alloc") == 0;
+  if (!f || std::strncmp(f, "alloc", 5) != 0) return false;
+  return f[5] == '\0' || (f[5] == '=' && std::strtoull(f + 6, nullptr, 10) == bytes);
 }
 
 lem_status dev_alloc(lem_ctx* ctx, void** p, size_t bytes) {
   *p = nullptr;
-  if (fault_alloc()) return fail(LEM_ENOMEM, "device allocation refused (LEM_FAULT=alloc)");
+  if (fault_alloc(bytes)) return fail(LEM_ENOMEM, "device allocation refused (LEM_FAULT=alloc)");
   if (bytes == 0) bytes = 16;
   // stream-ordered: a context made or freed while other streams run (the server) must not
   // wait for the whole device, as cudaMalloc / cudaFree may

@@ -589,9 +589,8 @@ __global__ void copy_cols_kernel(double* dst, int64_t ldd, int dcol0, const doub
 // (refresh > 0) keeps one block of the size its builds took, up to kKeepBytes, and later batches
 // are laid out in it: taking and returning gigabytes at the stream-ordered pool cost 5 ms of a
 // 27 ms build, since the pool gives them back to the driver at every synchronisation. Otherwise
-// each piece comes from cudaMallocAsync and is freed after the build has synchronised its stream,
-// on the legacy stream: that waits for no non-blocking stream, where cudaFree would wait for the
-// whole device.
+// each piece comes from cudaMallocAsync and is freed in the order of the build's stream: a build that
+// fails half way leaves kernels in flight that still use it.
 constexpr size_t kKeepBytes = size_t(4) << 30;
 struct Scratch {
   lem_ctx* ctx;
@@ -607,6 +606,7 @@ struct Scratch {
       *p = static_cast<char*>(ctx->d_ws) + o;
       return LEM_OK;
     }
+    if (fault_alloc(bytes)) return fail(LEM_ENOMEM, "build scratch refused (LEM_FAULT=alloc)");
     LEM_CUDA_TRY(cudaMallocAsync(p, b, ctx->stream));
     own.push_back(*p);
     return LEM_OK;
@@ -614,9 +614,8 @@ struct Scratch {
   template <class T>
   lem_status get(T** p, size_t count) { return get(reinterpret_cast<void**>(p), sizeof(T) * count); }
   ~Scratch() {
-    for (void* p : own) cudaFreeAsync(p, 0);
+    for (void* p : own) cudaFreeAsync(p, ctx->stream);
     if (own.empty() || ctx->desc.refresh <= 0 || !ctx->desc.reaction || used > kKeepBytes) return;
-    // (the batch is over: its stream was synchronised, or the build failed and this context stays unbuilt)
     if (ctx->d_ws) cudaFreeAsync(ctx->d_ws, ctx->stream);
     ctx->device_bytes -= int64_t(ctx->ws_bytes);
     ctx->ws_bytes = 0;

@@ -231,6 +231,8 @@ __device__ __forceinline__ double abs_pow(double x, double e) {
 bool builder_uses_tc(int prec);
 // abi.cpp: take a built single-class propagator from a context with the same local operator
 lem_status adopt_propagators(lem_ctx* dst, lem_ctx* src, cudaEvent_t built);
+// whether tests want an allocation of that size to fail (abi.cpp)
+bool fault_alloc(size_t bytes);
 // allocation helper that tracks bytes
 lem_status dev_alloc(lem_ctx* ctx, void** p, size_t bytes);
 }  // namespace lem

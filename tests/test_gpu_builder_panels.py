@@ -35,3 +35,30 @@ def test_one_operator_is_built_alike_for_every_apply(tile, H):
         assert np.array_equal(per.propagator(c), P)
     one.close()
     per.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "split_fast"])
+def test_a_build_out_of_scratch_half_way(monkeypatch, prec):
+    """The elimination's scratch is refused when the products before it are already on their way: the build
+    reports it, and others, on another stream too, are not disturbed."""
+    coef = {"C": -2.0, "W": 1.0, "E": 1.0}
+    n = 700 + 2 * 40
+    make = lambda: L.Lem((2800,), ("periodic",), coef, 1.0, (700,), (40,), prec=prec,  # noqa: E731
+                         stream=torch.cuda.Stream().cuda_stream)
+    good = make()
+    good.build()
+    want = good.propagator(0)
+    for k in range(6):
+        bad, other = make(), make()
+        monkeypatch.setenv("LEM_FAULT", f"alloc={n * 64 * 8}")  # the panel's tracker
+        with pytest.raises(L.LemError) as e:
+            bad.build()
+        assert e.value.status == L.LEM_ENOMEM
+        monkeypatch.delenv("LEM_FAULT")
+        other.build()
+        assert np.array_equal(other.propagator(0), want)
+        bad.build()
+        assert np.array_equal(bad.propagator(0), want)
+        bad.close()
+        other.close()
+    good.close()
