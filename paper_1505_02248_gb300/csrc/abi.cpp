@@ -49,6 +49,14 @@ lem_status dev_alloc(lem_ctx* ctx, void** p, size_t bytes) {
   return LEM_OK;
 }
 
+cudaError_t allow_smem(const void* kernel, int device, size_t bytes, int reserved) {
+  int most = 0;
+  const cudaError_t e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+  if (e != cudaSuccess) return e;
+  if (bytes + size_t(reserved) > size_t(most)) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - reserved);
+}
+
 }  // namespace lem
 
 lem::Stencil lem_ctx::stencil() const {

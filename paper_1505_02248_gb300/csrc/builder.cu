@@ -490,8 +490,6 @@ static cudaError_t launch_panel(const double* src, int64_t lds, int64_t ss, int 
   const int csize = std::min(PANEL_MAX_CLUSTER, (n + 7) / 8);
   const int rows_per = (n + csize - 1) / csize;
   const size_t smem = 2 * sizeof(PanelStep) + sizeof(double) * (size_t(rows_per) * (PANEL_PITCH + 2) + GJ_KB);
-  cudaError_t e = cudaFuncSetAttribute(bgj_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(nb) * csize);
   cfg.blockDim = dim3(PANEL_THREADS);
@@ -670,6 +668,7 @@ static lem_status solve_gj(lem_ctx* ctx, TcGemm* tcg, double* G, int n, int gjco
   LEM_TRY(ws.get(&piv, size_t(nb) * GJ_KB));
   // FP64 products write over their right factor: the pivot rows move out first
   if (!tcg) LEM_TRY(ws.get(&rows, size_t(nb) * GJ_KB * gjcols));
+  LEM_CUDA_TRY(allow_smem(reinterpret_cast<const void*>(bgj_panel_kernel), ctx->device, 0, 1024));
   const int64_t sG = int64_t(n) * gjcols, sY = int64_t(n) * GJ_KB;
   for (int k0 = 0; k0 < n; k0 += GJ_KB) {  // a panel of columns
     const int kb = std::min(GJ_KB, n - k0);

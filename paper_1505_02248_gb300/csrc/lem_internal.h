@@ -233,6 +233,10 @@ bool builder_uses_tc(int prec);
 lem_status adopt_propagators(lem_ctx* dst, lem_ctx* src, cudaEvent_t built);
 // whether tests want an allocation of that size to fail (abi.cpp)
 bool fault_alloc(size_t bytes);
+// Lets `kernel` be launched on `device` with up to all of an SM's dynamic shared memory (less `reserved` bytes for
+// its static arrays); an error if `bytes` are more. The limit is the process's, not the context's: set to
+// one context's size it would refuse the launches of others, in this thread or another.
+cudaError_t allow_smem(const void* kernel, int device, size_t bytes, int reserved = 0);
 // allocation helper that tracks bytes
 lem_status dev_alloc(lem_ctx* ctx, void** p, size_t bytes);
 }  // namespace lem

@@ -1,4 +1,6 @@
 """The solve of the propagator build, panel by panel (csrc/builder.cu, solve_gj)."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -62,3 +64,38 @@ def test_a_build_out_of_scratch_half_way(monkeypatch, prec):
         bad.close()
         other.close()
     good.close()
+
+
+def test_builds_of_unlike_windows_in_threads():
+    """The panel kernel's shared memory follows the window: builds of large and small windows at once,
+    each on a stream of its own, do not disturb each other."""
+    coef = {"C": -2.0, "W": 1.0, "E": 1.0}
+    sizes = [(1000, 40), (200, 20), (216, 20), (280, 20)]  # windows of 1080, 240, 256 and 320 nodes
+    failed, want = [], []
+    ctxs = [L.Lem((4 * t,), ("periodic",), coef, 1.0, (t,), (h,), prec="split", stream=torch.cuda.Stream().cuda_stream)
+            for t, h in sizes]
+    for c in ctxs:
+        c.build()
+        want.append(c.propagator(0))
+    done = threading.Event()
+
+    def work(k, more):
+        try:
+            while more():
+                ctxs[k].build()
+            if not np.array_equal(ctxs[k].propagator(0), want[k]):
+                failed.append("other propagators")
+        except L.LemError as e:
+            failed.append(str(e))
+
+    left = iter([True] * 100 + [False])
+    small = [threading.Thread(target=work, args=(k, lambda: not done.is_set())) for k in (1, 2, 3)]
+    for t in small:
+        t.start()
+    work(0, lambda: next(left))
+    done.set()
+    for t in small:
+        t.join()
+    assert not failed
+    for c in ctxs:
+        c.close()
