@@ -506,7 +506,7 @@ lem_status band_prepare(lem_ctx* ctx) {
   if (b->cls.empty()) {
     LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&b->d_cls), sizeof(BandClass) * nc));
     LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&b->d_ext), sizeof(int) * 4 * nc));
-    LEM_CUDA_TRY(cudaFuncSetAttribute(band_extents_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    LEM_CUDA_TRY(allow_smem(reinterpret_cast<const void*>(band_extents_kernel), ctx->device, smem, 1024));
     b->cls.resize(nc);
     for (int k = 0; k < nc; ++k) {
       const ClassDesc& cd = ctx->classes[k];
@@ -572,13 +572,14 @@ lem_status band_prepare(lem_ctx* ctx) {
     // (pageable memory: the copy has left the vector when the call returns)
     LEM_CUDA_TRY(cudaMemcpyAsync(b->d_tiles, bt.data(), sizeof(BandTile) * bt.size(), cudaMemcpyHostToDevice, st));
   }
-  const int bytes = int(sizeof(double) * size_t(b->wmax + 4));
+  const size_t bytes = sizeof(double) * size_t(b->wmax + 4);
   if (bytes > 48 * 1024) {
-    LEM_CUDA_TRY(cudaFuncSetAttribute(gemv_band_row_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    LEM_CUDA_TRY(cudaFuncSetAttribute(gemv_band_row_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    auto allow = [&](auto* kernel) { return allow_smem(reinterpret_cast<const void*>(kernel), ctx->device, bytes); };
+    LEM_CUDA_TRY(allow(gemv_band_row_kernel<double>));
+    LEM_CUDA_TRY(allow(gemv_band_row_kernel<float>));
     for (int lpr : {2, 4, 8}) {
-      LEM_CUDA_TRY(cudaFuncSetAttribute(band_kernel_for<double>(lpr), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      LEM_CUDA_TRY(cudaFuncSetAttribute(band_kernel_for<float>(lpr), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+      LEM_CUDA_TRY(allow(band_kernel_for<double>(lpr)));
+      LEM_CUDA_TRY(allow(band_kernel_for<float>(lpr)));
     }
   }
   ctx->band_gen = ctx->build_gen;

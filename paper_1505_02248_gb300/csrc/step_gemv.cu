@@ -401,7 +401,7 @@ lem_status step_gemv_multi(lem_ctx* ctx, double* d_u, int nsteps, bool f32, bool
                          : reinterpret_cast<const void*>(gemv_persistent_kernel<double, true>);
   if (smemp) {  // every block must still be co-resident with the larger footprint
     int per_sm = 0, nsm = 0;
-    if (cudaFuncSetAttribute(fn_s, cudaFuncAttributeMaxDynamicSharedMemorySize, int(wbytes + pbytes)) != cudaSuccess ||
+    if (allow_smem(fn_s, ctx->device, wbytes + pbytes) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_s, persist_threads(rsplit), wbytes + pbytes) != cudaSuccess ||
         int64_t(per_sm) * nsm < blocks) {
@@ -533,17 +533,13 @@ lem_status step_gemv_scratch(lem_ctx* ctx, double* d_u, double* r) {
 }
 
 lem_status gemv_set_smem(lem_ctx* ctx) {
-  const int bytes = int(sizeof(double) * ctx->n_loc);
-  if (bytes > 48 * 1024) {
-    LEM_CUDA_TRY(cudaFuncSetAttribute(gemv_tiles_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      bytes));
-    LEM_CUDA_TRY(cudaFuncSetAttribute(gemv_tiles_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      bytes));
-    LEM_CUDA_TRY(cudaFuncSetAttribute(gemv_tiles_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      bytes));
-    LEM_CUDA_TRY(cudaFuncSetAttribute(gemv_tiles_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      bytes));
-  }
+  const size_t bytes = sizeof(double) * size_t(ctx->n_loc);
+  if (bytes > 48 * 1024)
+    for (const void* k : {reinterpret_cast<const void*>(gemv_tiles_kernel<float, false>),
+                          reinterpret_cast<const void*>(gemv_tiles_kernel<double, false>),
+                          reinterpret_cast<const void*>(gemv_tiles_kernel<float, true>),
+                          reinterpret_cast<const void*>(gemv_tiles_kernel<double, true>)})
+      LEM_CUDA_TRY(allow_smem(k, ctx->device, bytes));
   return LEM_OK;
 }
 
