@@ -252,6 +252,7 @@ struct Tile {
   const __half* a;  // the tile's first K block
   const __half* b;
   int nkb;
+  bool stall = false;  // test hook: its first stage is armed, but not all of its bytes are loaded
 };
 
 // Barrier among the epilogue warps.
@@ -289,7 +290,7 @@ __device__ __forceinline__ void run(const Shared& sh, uint32_t tmem, Work& work,
           uint8_t* st = sh.stage + q * STAGE;
           ptx::mbar_arrive_expect_tx(&sh.full[q], STAGE);
           ptx::bulk_load(st, t.a + size_t(kb) * A_BLOCK, A_BYTES, &sh.full[q]);
-          ptx::bulk_load(st + A_BYTES, t.b + size_t(kb) * B_BLOCK, B_BYTES, &sh.full[q]);
+          if (!t.stall || kb) ptx::bulk_load(st + A_BYTES, t.b + size_t(kb) * B_BLOCK, B_BYTES, &sh.full[q]);
           ++issued;
           if (++q == STAGES) {
             q = 0;

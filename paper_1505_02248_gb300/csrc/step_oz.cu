@@ -28,6 +28,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
+#include <cstring>
 #include <new>
 #include <string>
 #include <vector>
@@ -238,6 +240,7 @@ struct StepParams {
   double* u;
   int64_t n_int, n_loc, ny, nx;
   int unit0, nunits, ks, accumulate;
+  int fault;           // test hook (LEM_FAULT=timeout): the first CTA waits for bytes that never come
   int* err;
   unsigned* nsmall;    // elements that oz_small_kernel looks at: their number,
   uint2* small_at;     // window (block * 128 + row) and owner row (its place among the scale exponents; the top
@@ -473,7 +476,7 @@ struct StepWork {
   __device__ oz::Tile tile(int k) const {
     const Unit& un = p.units[index(k)];
     const WinBlock& wb = p.blocks[un.wb];
-    return {p.a + wb.a_off, p.b + un.b_off, wb.nkb};
+    return {p.a + wb.a_off, p.b + un.b_off, wb.nkb, p.fault && index(k) == 0};
   }
   __device__ void begin(int k) {
     const Unit& un = p.units[index(k)];
@@ -544,7 +547,8 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_split_kernel(const __g
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the window digits are written
   tab.fill(p, un, wb, int(threadIdx.x));
   const int k0 = wb.nkb * rank / ks, k1 = wb.nkb * (rank + 1) / ks;
-  SplitWork work{sh, {p.a + wb.a_off + size_t(k0) * oz::A_BLOCK, p.b + un.b_off + size_t(k0) * oz::B_BLOCK, k1 - k0}};
+  SplitWork work{sh, {p.a + wb.a_off + size_t(k0) * oz::A_BLOCK, p.b + un.b_off + size_t(k0) * oz::B_BLOCK, k1 - k0,
+                      p.fault && blockIdx.x == 0}};
   oz::run<oz::Fine>(sh, tmem, work, p.err, &s_abort);
   longlong2* sums = reinterpret_cast<longlong2*>(sh.stage);
   cg::cluster_group cl = cg::this_cluster();
@@ -552,7 +556,10 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_split_kernel(const __g
     for (int q = threadIdx.x; q < oz::BN * oz::SUM_PITCH; q += blockDim.x) sums[q] = make_longlong2(0, 0);
   cl.sync();
   const int lcw = 6 - (31 - __clz(ks)), cw = 1 << lcw, c0 = rank * cw;  // this CTA's columns
-  if (!s_abort && c0 < un.ncol) {
+  // a CTA that gave up has staged no sums: none of the cluster writes the unit
+  bool whole = true;
+  for (int j = 0; j < ks; ++j) whole = whole && !*cl.map_shared_rank(const_cast<int*>(&s_abort), j);
+  if (whole && c0 < un.ncol) {
     const StepUnit o(p, un, wb, tab);
     constexpr int U = 4;  // elements per thread in flight
     const int total = wb.count * cw, warp0 = int(threadIdx.x) / 32 * 32, lane = int(threadIdx.x) % 32;
@@ -619,6 +626,7 @@ struct OzPlan {
   uint2* d_small_at = nullptr;
   double* d_small_old = nullptr;
   int64_t max_owners = 0;      // of a group
+  int fault = 0;
   int* d_err = nullptr;
 };
 
@@ -763,6 +771,8 @@ lem_status oz_prepare(lem_ctx* ctx) {
   LEM_TRY(alloc(&z->d_bmag, z->b_halves / oz::S));
   LEM_TRY(alloc(&z->d_nsmall, 1));
   LEM_TRY(alloc(&z->d_err, 1));
+  const char* fault = std::getenv("LEM_FAULT");
+  z->fault = fault && std::strcmp(fault, "timeout") == 0 ? 1 : 0;
   cudaStream_t st = ctx->stream;
   LEM_CUDA_TRY(cudaMemcpyAsync(z->d_blocks, z->blocks.data(), sizeof(WinBlock) * z->blocks.size(),
                                cudaMemcpyHostToDevice, st));
@@ -833,7 +843,7 @@ lem_status step_oz(lem_ctx* ctx, double* d_u) {
                                     static_cast<const WinBlock*>(z->d_blocks), g.wb0, int(ctx->ny), int(ctx->nx), z->d_e,
                                     z->d_a, z->d_amag, z->d_nsmall));
     StepParams p{z->d_blocks, z->d_units, ctx->d_tiles, ctx->d_class_order, z->d_a, z->d_b, z->d_e, z->d_f, z->d_mid, z->d_amag, z->d_bmag, ctx->d_P,
-                 src, d_u, ctx->n_int, ctx->n_loc, ctx->ny, ctx->nx, g.unit0, g.nunits, g.ks, phi ? 1 : 0, z->d_err, z->d_nsmall,
+                 src, d_u, ctx->n_int, ctx->n_loc, ctx->ny, ctx->nx, g.unit0, g.nunits, g.ks, phi ? 1 : 0, z->fault, z->d_err, z->d_nsmall,
                  z->d_small_at, z->d_small_old};
     if (g.ks == 1) {
       cfg.gridDim = dim3(unsigned(std::min(g.nunits, z->nsm)));
