@@ -627,6 +627,7 @@ struct OzPlan {
   double* d_small_old = nullptr;
   int64_t max_owners = 0;      // of a group
   int fault = 0;
+  int64_t bytes = 0;           // device memory of the plan
   int* d_err = nullptr;
 };
 
@@ -746,8 +747,18 @@ void oz_destroy(lem_ctx* ctx) {
                   static_cast<void*>(z->d_small_at), static_cast<void*>(z->d_small_old),
                   static_cast<void*>(z->d_err)})
     if (p) cudaFreeAsync(p, ctx->stream);
+  ctx->device_bytes -= z->bytes;
   delete z;
   ctx->oz = nullptr;
+}
+
+// n elements of the plan's device memory at *p.
+template <class T>
+static lem_status take(lem_ctx* ctx, T** p, size_t n) {
+  const int64_t before = ctx->device_bytes;
+  const lem_status s = dev_alloc(ctx, reinterpret_cast<void**>(p), sizeof(T) * n);
+  ctx->oz->bytes += ctx->device_bytes - before;
+  return s;
 }
 
 // Plan and device memory of the tensor-core FP64 step (at lem_create).
@@ -760,17 +771,16 @@ lem_status oz_prepare(lem_ctx* ctx) {
   LEM_CUDA_TRY(cudaFuncSetAttribute(oz_step_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM));
   if (cudaDeviceGetAttribute(&z->nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || z->nsm < 1) z->nsm = 152;
   for (auto& g : z->groups) g.ks = pick_split(g, z, z->nsm);
-  auto alloc = [&](auto** p, size_t n) { return dev_alloc(ctx, reinterpret_cast<void**>(p), sizeof(**p) * n); };
-  LEM_TRY(alloc(&z->d_blocks, z->blocks.size()));
-  LEM_TRY(alloc(&z->d_units, z->units.size()));
-  LEM_TRY(alloc(&z->d_rows, z->rows.size()));
-  LEM_TRY(alloc(&z->d_b, z->b_halves));
-  LEM_TRY(alloc(&z->d_e, size_t(z->ne)));
-  LEM_TRY(alloc(&z->d_f, size_t(z->nf)));
-  LEM_TRY(alloc(&z->d_mid, size_t(z->nf)));
-  LEM_TRY(alloc(&z->d_bmag, z->b_halves / oz::S));
-  LEM_TRY(alloc(&z->d_nsmall, 1));
-  LEM_TRY(alloc(&z->d_err, 1));
+  LEM_TRY(take(ctx, &z->d_blocks, z->blocks.size()));
+  LEM_TRY(take(ctx, &z->d_units, z->units.size()));
+  LEM_TRY(take(ctx, &z->d_rows, z->rows.size()));
+  LEM_TRY(take(ctx, &z->d_b, z->b_halves));
+  LEM_TRY(take(ctx, &z->d_e, size_t(z->ne)));
+  LEM_TRY(take(ctx, &z->d_f, size_t(z->nf)));
+  LEM_TRY(take(ctx, &z->d_mid, size_t(z->nf)));
+  LEM_TRY(take(ctx, &z->d_bmag, z->b_halves / oz::S));
+  LEM_TRY(take(ctx, &z->d_nsmall, 1));
+  LEM_TRY(take(ctx, &z->d_err, 1));
   const char* fault = std::getenv("LEM_FAULT");
   z->fault = fault && std::strcmp(fault, "timeout") == 0 ? 1 : 0;
   cudaStream_t st = ctx->stream;
@@ -802,20 +812,31 @@ lem_status oz_check_error(lem_ctx* ctx) {
   return fail(LEM_ETIMEOUT, "FP64 tensor-core step gave up waiting on an mbarrier (code " + std::to_string(e) + ")");
 }
 
-// One FP64 step; the window digits are allocated at the first.
+// Window digits, and room for the list of small sums (at the first step).
+static lem_status oz_windows(lem_ctx* ctx) {
+  OzPlan* z = ctx->oz;
+  LEM_TRY(take(ctx, &z->d_small_at, size_t(z->max_owners)));
+  if (ctx->desc.mode == LEM_MODE_PHI) LEM_TRY(take(ctx, &z->d_small_old, size_t(z->max_owners)));
+  LEM_TRY(take(ctx, &z->d_amag, z->a_halves / oz::S));
+  LEM_TRY(take(ctx, &z->d_a, z->a_halves));
+  // rows past a block's last window are multiplied too (their sums are dropped)
+  LEM_CUDA_TRY(cudaMemsetAsync(z->d_a, 0, sizeof(__half) * z->a_halves, ctx->stream));
+  return LEM_OK;
+}
+
+// One FP64 step. Without room for the window digits the context goes over to the FP64 GEMM, as
+// lem_create does without room for those of the propagators.
 lem_status step_oz(lem_ctx* ctx, double* d_u) {
+  if (!ctx->oz->d_a) {
+    const lem_status s = oz_windows(ctx);
+    if (s == LEM_ENOMEM) {
+      oz_destroy(ctx);
+      return step_fp64(ctx, d_u);
+    }
+    LEM_TRY(s);
+  }
   OzPlan* z = ctx->oz;
   cudaStream_t st = ctx->stream;
-  if (!z->d_a) {
-    if (!z->d_small_at)
-      LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&z->d_small_at), sizeof(uint2) * size_t(z->max_owners)));
-    if (!z->d_small_old && ctx->desc.mode == LEM_MODE_PHI)
-      LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&z->d_small_old), sizeof(double) * size_t(z->max_owners)));
-    if (!z->d_amag) LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&z->d_amag), z->a_halves / oz::S));
-    LEM_TRY(dev_alloc(ctx, reinterpret_cast<void**>(&z->d_a), sizeof(__half) * z->a_halves));
-    // rows past a block's last window are multiplied too (their sums are dropped)
-    LEM_CUDA_TRY(cudaMemsetAsync(z->d_a, 0, sizeof(__half) * z->a_halves, st));
-  }
   const bool phi = ctx->desc.mode == LEM_MODE_PHI;
   const double* src = d_u;
   if (phi) {
