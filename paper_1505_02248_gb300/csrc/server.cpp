@@ -258,13 +258,19 @@ int64_t ctx_bytes_estimate(const lem_problem_desc& d, int64_t* scratch) {
   if (lem_plan_query(&d, &nt, &nc, &nl, &ni, nullptr) != LEM_OK) return -1;
   const int64_t npts = d.ndim == 1 ? d.n[0] : d.n[0] * d.n[1];
   int64_t b = 8 * (nc * ni * nl + 2 * npts + nt * (nl + ni)) + 5 * 8 * (d.coef_stride ? npts : 1);
-  if (d.prec == LEM_PREC_FP64 && nc * 8 <= nt)  // digits of the windows (at most about 1 GiB) and propagators
-    b += 14 * (std::min<int64_t>(int64_t(1) << 27, (nt + 128 * nc) * (nl + 16)) + nc * (ni + 64) * (nl + 16)) -
-         8 * nt * (nl + ni);
+  if (d.prec == LEM_PREC_FP64 && nc * 8 <= nt) {
+    // digits (14 bytes a value) and magnitudes (1) of the windows, a GiB of digits at once, and of the
+    // propagators; the list of small sums (16 bytes an owner of those windows); tiles and units; no
+    // gathered windows and results, no second state
+    const int64_t all = 14 * (nt + 128 * nc) * (nl + 16), win = std::min<int64_t>(int64_t(1) << 30, all);
+    b += win + win / 14 + 15 * nc * (ni + 64) * (nl + 16) + int64_t(16.0 * npts * win / all) + 64 * nt +
+         32 * (nt / 128 + nc) * (ni / 64 + 1) - 8 * nt * (nl + ni) - 8 * npts;
+  }
   if (d.prec == LEM_PREC_SPLIT) b += 4 * 2 * npts + 3 * 2 * (npts + 8 * int64_t(std::sqrt(double(npts))) * 64) +
                                      3 * 2 * ni * nl * 2;
-  // transient builder scratch (freed after the build): 19 n_loc^2 doubles per class batch
-  const int64_t per = 19 * nl * nl * 8;
+  // transient builder scratch (freed after the build), doubles per class of a batch: 18 n_loc^2 and the
+  // elimination's panel of 256 n_loc with FP64 products
+  const int64_t per = 8 * (lem::builder_uses_tc(d.prec) ? 19 * nl * nl : 18 * nl * nl + 256 * nl);
   const int64_t batch = std::max<int64_t>(1, std::min<int64_t>(nc, (int64_t(8) << 30) / std::max<int64_t>(per, 1)));
   *scratch = per * batch;
   return b;

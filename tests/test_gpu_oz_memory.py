@@ -45,3 +45,22 @@ def test_a_step_without_room_for_digits(monkeypatch, mode):
         held.append(ctx.info()["device_bytes"])
         ctx.close()
     assert np.array_equal(out[0], out[1]) and held[0] == held[1]
+
+
+def test_the_servers_estimate_of_a_context():
+    """Windows of more than a GiB of digits: what a request's context counts against the budget is what it
+    holds, within the scratch of a host state (8 bytes a node)."""
+    side = 3872
+    coef = {"C": -9.5, "W": 3.0, "E": 2.0, "S": 2.5, "N": 2.0}
+    args = ((side, side), ("periodic",) * 2, coef, 1.0, (16, 16), (16, 16))
+    ctx = L.Lem(*args, prec="fp64")
+    d_u = torch.zeros(side * side, dtype=torch.float64, device="cuda")
+    ctx.step(d_u, 1)
+    ctx.sync()
+    held = ctx.info()["device_bytes"]
+    ctx.close()
+    srv = L.Server()
+    srv.wait(srv.submit(*args, np.zeros(side * side), 1, tol=1e-10), 120.0)
+    counted = srv.stats()["device_bytes"]
+    srv.close()
+    assert held <= counted <= held + 8 * side * side + (32 << 20)
