@@ -39,6 +39,12 @@ lem_status dev_alloc(lem_ctx* ctx, void** p, size_t bytes) {
   // stream-ordered: a context made or freed while other streams run (the server) must not
   // wait for the whole device, as cudaMalloc / cudaFree may
   cudaError_t e = cudaMallocAsync(p, bytes, ctx->stream);
+  if (e == cudaErrorMemoryAllocation && ctx->d_ws) {  // the builder's kept scratch makes way
+    cudaGetLastError();
+    builder_release(ctx);
+    cudaStreamSynchronize(ctx->stream);
+    e = cudaMallocAsync(p, bytes, ctx->stream);
+  }
   if (e != cudaSuccess) {
     *p = nullptr;
     cudaGetLastError();
@@ -122,7 +128,7 @@ void free_ctx(lem_ctx* c) {
   cudaFreeAsync(c->d_Y, c->stream);
   cudaFreeAsync(c->d_state_tmp, c->stream);
   cudaFreeAsync(c->d_status, c->stream);
-  cudaFreeAsync(c->d_ws, c->stream);
+  builder_release(c);
   delete c;
 }
 

@@ -16,6 +16,7 @@
 // s = smallest integer >= 0 with ||Z||_1 / 2^s <= theta_13 from the exact 1-norm,
 // (V - U) R = (V + U) by Gauss-Jordan elimination with partial pivoting, then s squarings.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <numeric>
@@ -584,12 +585,14 @@ __global__ void copy_cols_kernel(double* dst, int64_t ldd, int dcol0, const doub
 }
 
 // Device scratch of one build batch, released when the batch is done. A context that rebuilds
-// (refresh > 0) keeps one block of the size its builds took, up to kKeepBytes, and later batches
-// are laid out in it: taking and returning gigabytes at the stream-ordered pool cost 5 ms of a
-// 27 ms build, since the pool gives them back to the driver at every synchronisation. Otherwise
+// (refresh > 0) keeps one block of the size its builds took, up to kKeepBytes and kKeepAll over all
+// contexts, and later batches are laid out in it: taking and returning gigabytes at the stream-ordered
+// pool cost 5 ms of a 27 ms build, since the pool gives them back to the driver at every synchronisation.
+// It is given back with the context, or when another allocation of the context finds no room. Otherwise
 // each piece comes from cudaMallocAsync and is freed in the order of the build's stream: a build that
 // fails half way leaves kernels in flight that still use it.
-constexpr size_t kKeepBytes = size_t(4) << 30;
+constexpr int64_t kKeepBytes = int64_t(4) << 30, kKeepAll = int64_t(16) << 30;
+std::atomic<int64_t> g_kept{0};
 struct Scratch {
   lem_ctx* ctx;
   size_t used = 0;
@@ -613,17 +616,32 @@ struct Scratch {
   lem_status get(T** p, size_t count) { return get(reinterpret_cast<void**>(p), sizeof(T) * count); }
   ~Scratch() {
     for (void* p : own) cudaFreeAsync(p, ctx->stream);
-    if (own.empty() || ctx->desc.refresh <= 0 || !ctx->desc.reaction || used > kKeepBytes) return;
-    if (ctx->d_ws) cudaFreeAsync(ctx->d_ws, ctx->stream);
-    ctx->device_bytes -= int64_t(ctx->ws_bytes);
-    ctx->ws_bytes = 0;
-    if (dev_alloc(ctx, &ctx->d_ws, used) == LEM_OK) ctx->ws_bytes = used;
+  }
+  // after a build that went well
+  void keep() {
+    if (own.empty() || ctx->desc.refresh <= 0 || !ctx->desc.reaction || int64_t(used) > kKeepBytes) return;
+    for (void* p : own) cudaFreeAsync(p, ctx->stream);
+    own.clear();
+    builder_release(ctx);
+    if (g_kept.fetch_add(int64_t(used)) + int64_t(used) > kKeepAll || dev_alloc(ctx, &ctx->d_ws, used) != LEM_OK)
+      g_kept -= int64_t(used);
+    else
+      ctx->ws_bytes = used;
   }
 };
 
 inline dim3 grid1(int64_t total, int by) { return dim3(unsigned((total + 255) / 256), by); }
 
 }  // namespace
+
+void builder_release(lem_ctx* ctx) {
+  if (!ctx->d_ws) return;
+  cudaFreeAsync(ctx->d_ws, ctx->stream);
+  ctx->d_ws = nullptr;
+  ctx->device_bytes -= int64_t(ctx->ws_bytes);
+  g_kept -= int64_t(ctx->ws_bytes);
+  ctx->ws_bytes = 0;
+}
 
 bool builder_uses_tc(int prec) {
   if (prec == LEM_PREC_FP64) return false;
@@ -850,6 +868,7 @@ static lem_status build_batch(lem_ctx* ctx, int c0, int nb, const double* d_stat
   LEM_CUDA_TRY(cudaStreamSynchronize(st));
   if (status != 0) return fail(LEM_ENUMERIC, "singular Pade denominator (V - U) in the propagator build");
   if (tc.g) LEM_TRY(tc_gemm_check(tc.g, st));
+  ws.keep();
   return LEM_OK;
 }
 
@@ -1074,6 +1093,7 @@ static lem_status build_batch_phi3(lem_ctx* ctx, int c0, int nb, const double* d
   LEM_CUDA_TRY(cudaStreamSynchronize(st));
   if (status != 0) return fail(LEM_ENUMERIC, "singular Pade denominator (V - U) in the propagator build");
   if (tc.g) LEM_TRY(tc_gemm_check(tc.g, st));
+  ws.keep();
   return LEM_OK;
 }
 

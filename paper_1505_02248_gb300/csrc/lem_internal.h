@@ -227,6 +227,8 @@ __device__ __forceinline__ double abs_pow(double x, double e) {
   return pow(a, e);
 }
 #endif
+// builder.cu: give back the scratch that a refreshing context keeps
+void builder_release(lem_ctx* ctx);
 // builder.cu: whether propagators of a precision tier are built with the tensor-core products
 bool builder_uses_tc(int prec);
 // abi.cpp: take a built single-class propagator from a context with the same local operator

@@ -99,3 +99,31 @@ def test_builds_of_unlike_windows_in_threads():
     assert not failed
     for c in ctxs:
         c.close()
+
+
+def test_scratch_kept_by_refreshing_contexts_is_bounded():
+    """Each keeps the scratch of its builds (about 3 GB here) while all of them together stay within 16 GiB;
+    what one gives back another may keep."""
+    side = 80
+    rng = np.random.default_rng(0)
+    h = 1.0 / (side + 1)
+    k = rng.uniform(0.5, 2.0) / h ** 2
+    coef = {"C": np.full(side * side, -4 * k), **{w: np.full(side * side, k) for w in "WESN"}}
+    u = torch.tensor(rng.standard_normal(side * side), device="cuda")
+    ctxs = [L.Lem((side, side), ("dirichlet",) * 2, coef, 2.0 / k, (16, 16), (6, 6), prec="split", reaction=True, refresh=1)
+            for _ in range(7)]
+    bare = [c.info()["device_bytes"] for c in ctxs]
+
+    def kept(c):
+        ctxs[c].build(u)
+        return ctxs[c].info()["device_bytes"] - bare[c]
+
+    held = [kept(c) for c in range(7)]
+    want = ctxs[0].propagator(3)
+    assert 1 << 30 < held[0] <= 4 << 30 and held[-1] == 0
+    assert sum(held) <= 16 << 30
+    ctxs[0].close()
+    assert kept(6) == held[1]
+    assert np.array_equal(ctxs[6].propagator(3), want) and np.array_equal(ctxs[5].propagator(3), want)
+    for c in ctxs[1:]:
+        c.close()
