@@ -507,7 +507,14 @@ void worker_loop(lem_server* s) {
           r = q.front();
         }
         const auto ta = Clock::now();
-        const bool admitted = try_admit(s, r, tier == 0 ? s->budget : s->budget - s->budget / 4);
+        // (the whole budget where nothing else runs or waits: a request that needs more than
+        // three quarters of it would wait for ever)
+        bool alone = s->active.empty();
+        {
+          std::lock_guard<std::mutex> lk(s->mu);
+          alone = alone && s->queue.empty();
+        }
+        const bool admitted = try_admit(s, r, tier == 0 || alone ? s->budget : s->budget - s->budget / 4);
         s->admit_s += std::chrono::duration<double>(Clock::now() - ta).count();
         if (!admitted) break;
         {
