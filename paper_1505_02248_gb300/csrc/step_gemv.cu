@@ -455,6 +455,24 @@ static int resident_classes(const lem_ctx* ctx, bool f32) {
   return int(std::min<int64_t>(32000000 / std::max<int64_t>(bytes, 1), int64_t(ctx->classes.size())));
 }
 
+// Shared memory a block for a chained launch of FP64 rows that fills less than a wave. Its blocks are
+// placed while the residual's still run, on whatever SM has room, and the SMs with most of them set the time
+// (the FP64 pipe's): no more of them fit an SM than an even spread puts there. 112^2 variable
+// diffusion, tiles of 16 (392 blocks), ten steps: 330 us placed anyhow, 293 without the chain, 254 so;
+// 128^2 (512 blocks) 386, 355, 339.
+static size_t spread_smem(unsigned blocks, int resident, size_t smem, int device) {
+  int nsm = 0, room = 0;
+  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || nsm < 1 ||
+      cudaDeviceGetAttribute(&room, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device) != cudaSuccess) {
+    cudaGetLastError();
+    return smem;
+  }
+  const int per = int((blocks + nsm - 1) / nsm);
+  if (per >= resident) return smem;
+  const size_t even = size_t(room / per - 1024) / 128 * 128 - 128;  // (1 KB a block is the system's)
+  return std::max(smem, even);
+}
+
 // One LEM step by the batched GEMV: PHI reads the residual, EXP a copy of u^n.
 lem_status step_gemv(lem_ctx* ctx, double* d_u, bool f32) {
   cudaStream_t st = ctx->stream;
@@ -484,7 +502,7 @@ lem_status step_gemv(lem_ctx* ctx, double* d_u, bool f32) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(nt * rsplit);
     cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = f32 || ctx->cplx ? smem : spread_smem(nt * rsplit, tiles_blocks(8, false), smem, ctx->device);
     cfg.stream = st;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -534,6 +552,7 @@ lem_status step_gemv_scratch(lem_ctx* ctx, double* d_u, double* r) {
 
 lem_status gemv_set_smem(lem_ctx* ctx) {
   const size_t bytes = sizeof(double) * size_t(ctx->n_loc);
+  LEM_CUDA_TRY(allow_smem(reinterpret_cast<const void*>(gemv_tiles_kernel<double, false>), ctx->device, 0));  // (spread_smem)
   if (bytes > 48 * 1024)
     for (const void* k : {reinterpret_cast<const void*>(gemv_tiles_kernel<float, false>),
                           reinterpret_cast<const void*>(gemv_tiles_kernel<double, false>),
