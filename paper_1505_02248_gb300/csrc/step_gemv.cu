@@ -248,8 +248,11 @@ lem_status gemv_prepare_f32(lem_ctx* ctx) {
 // one block per tile of 64 x 96 took most of a step (16 tiles: 5.6 us a step).
 // SMEMP: one share of a tile per block, its propagator rows kept in shared memory for all steps.
 static int persist_threads(int rsplit) { return rsplit > 1 ? 128 : 256; }
-template <typename PT, bool SMEMP>
-__global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restrict__ P, int64_t n_int, int64_t n_loc,
+// BLOCKS: how many an SM holds at least (its registers). Four leave the FP32 rows what they want; five
+// where the tiles then take a round less: a line of 120 000 nodes (1875 tiles), ten steps 272 us in four
+// rounds, 228 in three; 60 000 nodes (two rounds either way) 138 and 146.
+template <typename PT, bool SMEMP, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS) gemv_persistent_kernel(const PT* __restrict__ P, int64_t n_int, int64_t n_loc,
                                                               const TileDesc* __restrict__ tiles, int ntiles,
                                                               const double* __restrict__ coef, int64_t cstride,
                                                               int64_t ny, int64_t nx, int ndim, int pery, int perx,
@@ -267,14 +270,15 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
   PT* Ps = reinterpret_cast<PT*>(wraw + ((sizeof(double) * size_t(n_loc) + 15) & ~size_t(15)));
   // owner rows [*ib, *ie) of share `part` of a tile (shares are whole groups of 4 rows)
   auto share = [&](const TileDesc& td, int part, int* ib, int* ie) {
-    const int owners = td.iext[0] * td.iext[1], per = ((owners + rsplit - 1) / rsplit + 3) / 4 * 4;
+    const int owners = td.iext[0] * td.iext[1];
+    const int per = rsplit == 1 ? owners : ((owners + rsplit - 1) / rsplit + 3) / 4 * 4;
     *ib = min(owners, part * per);
     *ie = min(owners, *ib + per);
   };
   if (SMEMP) {
-    const TileDesc td = tiles[blockIdx.x / rsplit];
+    const TileDesc td = tiles[rsplit == 1 ? blockIdx.x : blockIdx.x / rsplit];
     int ib, ie;
-    share(td, blockIdx.x % rsplit, &ib, &ie);
+    share(td, rsplit == 1 ? 0 : blockIdx.x % rsplit, &ib, &ie);
     const PT* src_p = P + (int64_t(td.cls) * n_int + ib) * n_loc;
     for (int64_t e = threadIdx.x; e < (ie - ib) * n_loc; e += blockDim.x) Ps[e] = src_p[e];
     __syncthreads();
@@ -285,13 +289,13 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
   double* nxt = src;
   for (int step = 0; step < nsteps; ++step) {
     for (int t = blockIdx.x; t < ntiles * rsplit; t += gridDim.x) {
-      const TileDesc td = tiles[t / rsplit];
+      const TileDesc td = tiles[rsplit == 1 ? t : t / rsplit];
       const int wl = td.wext[0] * td.wext[1];
       int ib, ie;
-      share(td, t % rsplit, &ib, &ie);
+      share(td, rsplit == 1 ? 0 : t % rsplit, &ib, &ie);
       // the window's source from u^n: the residual dt A u^n at each window node (PHI), or u^n
       for (int k = threadIdx.x; k < wl; k += blockDim.x) {
-        const int a = k / td.wext[1], b = k % td.wext[1];
+        const int a = td.wext[0] == 1 ? 0 : k / td.wext[1], b = k - a * td.wext[1];
         int64_t gy = int64_t(td.org[0]) + a, gx = int64_t(td.org[1]) + b;
         gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
         gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
@@ -357,8 +361,8 @@ __global__ void __launch_bounds__(256) gemv_persistent_kernel(const PT* __restri
 }
 
 // Whether lem_step may run its steps in one persistent launch, and with how many blocks; *rsplit:
-// blocks per tile (at most one block per SM then, of 8 rows at least).
-static int persistent_blocks(lem_ctx* ctx, bool f32, int nsteps, int* rsplit) {
+// blocks per tile (at most one block per SM then, of 8 rows at least), *fn: the kernel.
+static int persistent_blocks(lem_ctx* ctx, bool f32, int nsteps, int* rsplit, const void** fn) {
   *rsplit = 1;
   const lem_problem_desc& d = ctx->desc;
   if (nsteps < 2 || d.reaction || d.scheme != LEM_SCHEME_EULER || ctx->cplx) return 0;
@@ -375,11 +379,24 @@ static int persistent_blocks(lem_ctx* ctx, bool f32, int nsteps, int* rsplit) {
   const int64_t nt = int64_t(ctx->tiles.size());
   *rsplit = int(std::max<int64_t>(1, std::min<int64_t>(nsm / nt, ctx->n_int / 8)));
   const int threads = persist_threads(*rsplit);
-  cudaError_t e = f32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemv_persistent_kernel<float, false>, threads, smem)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemv_persistent_kernel<double, false>, threads, smem);
-  if (e != cudaSuccess || per_sm < 1) {
-    cudaGetLastError();
-    return 0;
+  auto rounds = [&](const void* fn) {  // of the device, over the tiles; 0: not even one block an SM
+    per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess || per_sm < 1) {
+      cudaGetLastError();
+      return int64_t(0);
+    }
+    return (nt * *rsplit + int64_t(per_sm) * nsm - 1) / (int64_t(per_sm) * nsm);
+  };
+  *fn = f32 ? reinterpret_cast<const void*>(gemv_persistent_kernel<float, false, 4>)
+            : reinterpret_cast<const void*>(gemv_persistent_kernel<double, false, 4>);
+  const int64_t r4 = rounds(*fn);
+  if (r4 == 0) return 0;
+  if (f32 && r4 > 1) {
+    const int four = per_sm;
+    const void* five = reinterpret_cast<const void*>(gemv_persistent_kernel<float, false, 5>);
+    const int64_t r5 = rounds(five);
+    if (r5 > 0 && r5 < r4) *fn = five;
+    else per_sm = four;
   }
   return int(std::min<int64_t>(int64_t(per_sm) * nsm, nt * *rsplit));
 }
@@ -387,7 +404,8 @@ static int persistent_blocks(lem_ctx* ctx, bool f32, int nsteps, int* rsplit) {
 lem_status step_gemv_multi(lem_ctx* ctx, double* d_u, int nsteps, bool f32, bool* done) {
   *done = false;
   int rsplit = 1;
-  const int blocks = persistent_blocks(ctx, f32, nsteps, &rsplit);
+  const void* fn = nullptr;
+  const int blocks = persistent_blocks(ctx, f32, nsteps, &rsplit, &fn);
   if (blocks < 1) return LEM_OK;
   if (f32 && ctx->p32_gen != ctx->build_gen) LEM_TRY(gemv_prepare_f32(ctx));
   const lem_problem_desc& d = ctx->desc;
@@ -397,8 +415,8 @@ lem_status step_gemv_multi(lem_ctx* ctx, double* d_u, int nsteps, bool f32, bool
   const size_t pbytes = (f32 ? sizeof(float) : sizeof(double)) * rows * size_t(ctx->n_loc);
   bool smemp = int64_t(blocks) == int64_t(ctx->tiles.size()) * rsplit && wbytes + pbytes <= 200 * 1024 &&
                std::getenv("LEM_NO_SMEM_P") == nullptr;
-  const void* fn_s = f32 ? reinterpret_cast<const void*>(gemv_persistent_kernel<float, true>)
-                         : reinterpret_cast<const void*>(gemv_persistent_kernel<double, true>);
+  const void* fn_s = f32 ? reinterpret_cast<const void*>(gemv_persistent_kernel<float, true, 4>)
+                         : reinterpret_cast<const void*>(gemv_persistent_kernel<double, true, 4>);
   if (smemp) {  // every block must still be co-resident with the larger footprint
     int per_sm = 0, nsm = 0;
     if (allow_smem(fn_s, ctx->device, wbytes + pbytes) != cudaSuccess ||
@@ -410,9 +428,7 @@ lem_status step_gemv_multi(lem_ctx* ctx, double* d_u, int nsteps, bool f32, bool
     }
   }
   const size_t smem = smemp ? wbytes + pbytes : sizeof(double) * size_t(ctx->n_loc);
-  const void* fn = smemp ? fn_s
-                         : (f32 ? reinterpret_cast<const void*>(gemv_persistent_kernel<float, false>)
-                                : reinterpret_cast<const void*>(gemv_persistent_kernel<double, false>));
+  if (smemp) fn = fn_s;
   int ntiles = int(ctx->tiles.size()), ndim = d.ndim, pery = ctx->bcy == LEM_BC_PERIODIC,
       perx = ctx->bcx == LEM_BC_PERIODIC, phi = d.mode == LEM_MODE_PHI;
   int64_t n_int = ctx->n_int, n_loc = ctx->n_loc, cstride = d.coef_stride, ny = ctx->ny, nx = ctx->nx;
