@@ -4,7 +4,7 @@
 //   PHI:  r = dt F(u^n); the windows of r, cut into digits (gather and cut in one pass);
 //         y = P r|_M for 128 windows x 64 owner rows per CTA; u_D += y.
 //   EXP:  the windows of u^n, cut; u_D = P u|_M.
-//   Then, in either mode, the owners whose digit sums came out small (oz_small_kernel): a digit
+//   Then, in either mode, the owners whose digit sums came out small (settle_cta, oz_small_kernel): a digit
 //   sum's error goes with the largest values of the window and of the owner row, so where the values
 //   that make up the sum lie far below those, it is formed again as FP64 multiply-adds. Each owner
 //   is within 4.1 K 2^-53 sum_k |P_k| |u_k| of its exact sum, as multiply-adds are within K 2^-53 of it; in the
@@ -250,20 +250,28 @@ struct StepParams {
 
 // Per-unit tables of the epilogue.
 struct StepTables {
-  int64_t node0[oz::BM];              // first owner node of each window
+  int2 t0[oz::BM];                    // first owner node of each window
   int e[oz::BM], f[oz::BN];           // scale exponents of the windows, of the owner rows
+  int mid[oz::BN];                    // where the owner rows' largest entries lie
   uint32_t in[2], plain[2], zero[2];  // columns (32 a word): owner rows; formed in FP64; all zero
-  int ix;
+  int ix, wx, wn, oy, ox;             // owners and window nodes per row, window nodes, the owners' place in it
   __device__ void fill(const StepParams& p, const Unit& un, const WinBlock& wb, int t) {
     if (t < 0) return;
     if (t < oz::BM) {
       const TileDesc& d = p.tiles[p.order[wb.first + min(t, wb.count - 1)]];
-      node0[t] = int64_t(d.t0[0]) * p.nx + d.t0[1];
+      t0[t] = make_int2(d.t0[0], d.t0[1]);
       e[t] = t < wb.count ? p.e[wb.e_off + t] : kAllZero;
-      if (t == 0) ix = d.iext[1];
+      if (t == 0) {
+        ix = d.iext[1];
+        wx = d.wext[1];
+        wn = d.wext[0] * wx;
+        oy = d.iofs[0];
+        ox = d.iofs[1];
+      }
     } else if (t < oz::BM + oz::BN) {  // (two whole warps)
       const int c = t - oz::BM, v = p.f[un.f_off + c];
       f[c] = v;
+      mid[c] = p.mid[un.f_off + c];
       const uint32_t i = __ballot_sync(0xffffffffu, c < un.ncol);
       const uint32_t q = __ballot_sync(0xffffffffu, v == oz::kNonFinite);
       const uint32_t z = __ballot_sync(0xffffffffu, v == kAllZero);
@@ -287,7 +295,9 @@ struct StepUnit {
       : p(p_), un(u_), wb(w_), t(t_), inv(div_inv(uint32_t(t_.ix))) {}
   __device__ int scale(int row, int col) const { return t.e[row] + t.f[col] - 62; }
   __device__ double value(int, int, double v) const { return v; }
-  __device__ int64_t row_at(int row) const { return row < wb.count ? t.node0[row] : -1; }
+  __device__ int64_t row_at(int row) const {
+    return row < wb.count ? int64_t(t.t0[row].x) * p.nx + t.t0[row].y : -1;
+  }
   __device__ int64_t col_at(int col) const {
     const int i = un.col0 + col, iy = div_by(i, inv);
     return col < un.ncol ? int64_t(iy) * p.nx + (i - iy * t.ix) : INT64_MIN / 2;
@@ -303,8 +313,8 @@ struct StepUnit {
   __device__ uint32_t checked(int row, int h) const {
     return row < wb.count && t.e[row] != kAllZero ? t.in[h] & ~t.zero[h] : 0u;
   }
-  // First of the places of this lane's `mine` elements on the list (the whole warp).
-  __device__ uint32_t places(int mine, int lane) const {
+  // First of the places of this lane's `mine` elements on a list of `count` elements (the whole warp).
+  __device__ static uint32_t places(unsigned* count, int mine, int lane) {
     int upto = mine;
 #pragma unroll
     for (int o = 1; o < 32; o *= 2) {
@@ -312,7 +322,7 @@ struct StepUnit {
       if (lane >= o) upto += v;
     }
     unsigned base = 0;
-    if (lane == 31 && upto) base = atomicAdd(p.nsmall, unsigned(upto));
+    if (lane == 31 && upto) base = atomicAdd(count, unsigned(upto));
     return __shfl_sync(0xffffffffu, base, 31) + uint32_t(upto - mine);
   }
   __device__ void list(uint32_t place, int row, int col, bool any_case, double old) const {
@@ -327,15 +337,113 @@ struct StepUnit {
 // as a rule, the others are looked at if they do not (eight lanes per element). Else
 // the element is formed as FP64 multiply-adds over the whole row, by a warp (an FP64 instruction takes 16 clk of the SM's
 // pipe: shared over the CTA, the sums across warps cost half as much again as the products).
-// A CTA takes elements from all over the list: those of a graded window follow one another there, and
-// are to be formed by many CTAs.
+// The CTAs of a cluster that shares a unit hold few elements each: they list them in shared memory and look
+// at them behind the sums (settle_cta). 256^2, tiles of 16, ten steps 284 us, 327 by oz_small_kernel, whose launch and
+// chain of loads take 6 to 9 us a step. CTAs with whole units leave theirs to oz_small_kernel, by a list in
+// global memory, of which it takes elements from all over: those of a graded window follow one another
+// there, and in their own CTA they would hold up the step (1024^2, four steps 937 us instead of 685; a line of
+// 16 384 random values, ten steps, 1156 instead of 345).
 // Of the elements of smooth fields 1 to 12 % come here (phi_1 of a residual, mu 50: 39 %), 0 to 0.2 % are
-// formed (mu 2, whose rows are narrow: 8 %). Bound by the latency of the loads (1024^2, 105 000 elements
-// of which 1000 to 1700 are formed: 39 us with cold caches, ncu), or by the FP64 pipe where many elements are formed: at
-// most what the step took before it used digits. Done in the epilogue of the products, the few
-// elements of one unit held up its CTA (four steps 2.9 ms instead of 0.69); a warp for 32 elements, one
-// after another, took 1.4 ms; 128 entries of the owner row in place of all magnitudes, too few for broad
-// rows, 1.3 ms.
+// formed (mu 2, whose rows are narrow: 8 %). Bound by the latency of the loads, or by the FP64 pipe
+// where many elements are formed: at most what the step took before it used digits.
+constexpr unsigned ALL = 0xffffffffu;
+constexpr uint32_t LARGE = 1u << (16 - (38 - oz::kSmallSum));  // 2^-2 in units of 2^-16
+// Magnitudes k of the rows at a and b (in 16 bytes): their products, in units of 2^-16.
+__device__ __forceinline__ uint32_t magnitude_part(const StepParams& p, uint32_t a, uint32_t b, int k, bool in) {
+  if (!in) return 0u;
+  const uint4 x = reinterpret_cast<const uint4*>(p.amag)[a + k], y = reinterpret_cast<const uint4*>(p.bmag)[b + k];
+  return __dp4a(x.x, y.x, __dp4a(x.y, y.y, __dp4a(x.z, y.z, __dp4a(x.w, y.w, 0u))));
+}
+__device__ __forceinline__ uint32_t sum_of_eight(uint32_t s) {  // over lanes 8 g .. 8 g + 7
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(ALL, s, o);
+  return s;
+}
+// sum |P| |u| of eight lanes' element, as far as they have to look: nk 16-node parts, the 32 from mid on first.
+__device__ __forceinline__ uint32_t magnitude_sum(const StepParams& p, uint32_t a, uint32_t b, int nk, int mid) {
+  const int sub = int(threadIdx.x) % 8;
+  uint32_t s = 0;
+#pragma unroll
+  for (int h = 0; h < 4; ++h) s += magnitude_part(p, a, b, mid + sub + 8 * h, mid + sub + 8 * h < nk);
+  s = sum_of_eight(s);
+  const bool more = s < LARGE && nk > 32;
+  if (!__any_sync(ALL, more)) return s;
+  uint32_t r = 0;
+  if (more) {
+#pragma unroll 6
+    for (int k = sub; k < nk; k += 8) r += magnitude_part(p, a, b, k, k < mid || k >= mid + 32);
+  }
+  __syncwarp();
+  return s + sum_of_eight(r);
+}
+__device__ __forceinline__ int middle(int mid, int nk) { return max(min(mid / 16 - 16, nk - 32), 0); }
+// The element of an owner row and the window at (oy, ox), wn nodes, wx a row, by a warp.
+__device__ __forceinline__ double form(const StepParams& p, const double* row, int oy, int ox, int wx, int wn) {
+  const int lane = int(threadIdx.x) % 32, ny = int(p.ny), nx = int(p.nx);
+  const uint32_t inv = div_inv(uint32_t(wx));
+  double y = 0.0;
+  constexpr int U = 12;  // loads of each operand in flight
+  for (int k0 = lane; k0 < wn; k0 += 32 * U) {
+    double v[U], w[U];
+#pragma unroll
+    for (int h = 0; h < U; ++h) {
+      const int k = k0 + 32 * h, b = div_by(k, inv);
+      int gy = oy + b, gx = ox + (k - b * wx);
+      gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
+      gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
+      v[h] = k < wn ? row[k] : 0.0;
+      w[h] = k < wn ? p.src[uint32_t(gy) * uint32_t(nx) + uint32_t(gx)] : 0.0;
+    }
+#pragma unroll
+    for (int h = 0; h < U; ++h) y = fma(v[h], w[h], y);
+  }
+  for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(ALL, y, o);
+  return y;
+}
+
+// A CTA's own list, in shared memory.
+struct SmallList {
+  double* old;      // the owner's value before the step
+  uint16_t* at;     // column * 128 + row; bit 13: to be formed in any case
+  uint16_t* todo;   // entries to be formed
+  unsigned* count;  // entries; [1]: to be formed
+  static constexpr size_t kBytes = 12;  // an entry
+  __device__ SmallList(uint8_t* mem, int room, unsigned* n)
+      : old(reinterpret_cast<double*>(mem)),
+        at(reinterpret_cast<uint16_t*>(old + room)),
+        todo(at + room),
+        count(n) {}
+  __device__ void put(uint32_t place, int row, int col, bool any_case, double before) const {
+    old[place] = before;
+    at[place] = uint16_t(col * oz::BM + row) | uint16_t(any_case ? 1 << 13 : 0);
+  }
+};
+// Every thread of the CTA calls it, the unit's digit sums written.
+__device__ __forceinline__ void settle_cta(const StepUnit& o, const SmallList& l) {
+  __syncthreads();
+  const int n = int(l.count[0]);
+  if (n == 0) return;
+  const int warp = int(threadIdx.x) / 32, lane = int(threadIdx.x) % 32, warps = int(blockDim.x) / 32;
+  const uint32_t a0 = uint32_t(o.wb.a_off / (16 * oz::S)), b0 = uint32_t(o.wb.b0 / (16 * oz::S));
+  for (int i0 = warp * 4; i0 < n; i0 += warps * 4) {
+    const int i = i0 + lane / 8, at = i < n ? l.at[i] : 0;
+    const int row = at % oz::BM, col = at / oz::BM % oz::BN;
+    const bool any_case = at >> 13;
+    const int nk = i < n && !any_case ? o.wb.nkb : 0;
+    const uint32_t s = magnitude_sum(o.p, a0 + uint32_t(row * o.wb.nkb), b0 + uint32_t(o.un.col0 + col) * uint32_t(o.wb.nkb),
+                                     nk, middle(o.t.mid[col], nk));
+    if (lane % 8 == 0 && i < n && s < LARGE) l.todo[atomicAdd(l.count + 1, 1u)] = uint16_t(i);
+  }
+  __syncthreads();
+  const int m = int(l.count[1]);
+  for (int d = warp; d < m; d += warps) {
+    const int i = l.todo[d], at = l.at[i], row = at % oz::BM, col = at / oz::BM % oz::BN;
+    const double y = form(o.p, o.p.P + (int64_t(o.wb.cls) * o.p.n_int + o.un.col0 + col) * o.p.n_loc,
+                          o.t.t0[row].x - o.t.oy, o.t.t0[row].y - o.t.ox, o.t.wx, o.t.wn);
+    if (lane == 0) o.store(o.row_at(row) + o.col_at(col), y, l.old[i]);
+  }
+}
+
 constexpr int SMALL_THREADS = 256;
 struct Formed {
   int64_t row, to;   // the owner row in P, the owner in the state
@@ -343,8 +451,6 @@ struct Formed {
   int oy, ox, wx, wn;
 };
 __global__ void __launch_bounds__(SMALL_THREADS, 3) oz_small_kernel(const __grid_constant__ StepParams p) {
-  constexpr unsigned ALL = 0xffffffffu;
-  constexpr uint32_t LARGE = 1u << (16 - (38 - oz::kSmallSum));  // 2^-2 in units of 2^-16
   constexpr int WARPS = SMALL_THREADS / 32;
   __shared__ Formed todo[SMALL_THREADS];
   __shared__ int ntodo;
@@ -354,9 +460,6 @@ __global__ void __launch_bounds__(SMALL_THREADS, 3) oz_small_kernel(const __grid
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int total = int(*p.nsmall), grid = int(gridDim.x);
-  const int ny = int(p.ny), nx = int(p.nx);
-  const uint4* ma = reinterpret_cast<const uint4*>(p.amag);
-  const uint4* mb = reinterpret_cast<const uint4*>(p.bmag);
   for (int64_t first = blockIdx.x; first < total; first += int64_t(SMALL_THREADS) * grid) {
     const int64_t place = first + int64_t(lane * WARPS + warp) * grid;  // (the warps fill evenly)
     const bool valid = place < total;
@@ -376,13 +479,8 @@ __global__ void __launch_bounds__(SMALL_THREADS, 3) oz_small_kernel(const __grid
       nk = formed ? 0 : wb.nkb;
       oa = uint32_t(wb.a_off / (16 * oz::S)) + (at.x % oz::BM) * uint32_t(wb.nkb);
       ob = uint32_t(wb.b0 / (16 * oz::S)) + uint32_t(i) * uint32_t(wb.nkb);
-      mid = max(min(p.mid[at.y] / 16 - 16, nk - 32), 0);
+      mid = middle(p.mid[at.y], nk);
     }
-    auto part = [&](uint32_t a, uint32_t b, int k, bool in) {
-      if (!in) return 0u;
-      const uint4 x = ma[a + k], y = mb[b + k];
-      return __dp4a(x.x, y.x, __dp4a(x.y, y.y, __dp4a(x.z, y.z, __dp4a(x.w, y.w, 0u))));
-    };
     // eight lanes per element
     const int g = lane / 8, sub = lane % 8;
     uint32_t sum = 0;
@@ -395,12 +493,11 @@ __global__ void __launch_bounds__(SMALL_THREADS, 3) oz_small_kernel(const __grid
         const int e = e0 + 4 * r + g, m = __shfl_sync(ALL, mid, e) + sub, n = __shfl_sync(ALL, nk, e);
         const uint32_t x = __shfl_sync(ALL, oa, e), y = __shfl_sync(ALL, ob, e);
 #pragma unroll
-        for (int h = 0; h < 4; ++h) s[r] += part(x, y, m + 8 * h, m + 8 * h < n);
+        for (int h = 0; h < 4; ++h) s[r] += magnitude_part(p, x, y, m + 8 * h, m + 8 * h < n);
       }
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) s[r] += __shfl_xor_sync(ALL, s[r], o);
+        s[r] = sum_of_eight(s[r]);
         s[r] = __shfl_sync(ALL, s[r], (lane % 4) * 8);
         if (lane / 4 == e0 / 4 + r) sum = s[r];
       }
@@ -416,10 +513,9 @@ __global__ void __launch_bounds__(SMALL_THREADS, 3) oz_small_kernel(const __grid
       const uint32_t x = __shfl_sync(ALL, oa, l), y = __shfl_sync(ALL, ob, l);
       uint32_t s = 0;
 #pragma unroll 6
-      for (int k = sub; k < n; k += 8) s += part(x, y, k, k < m || k >= m + 32);
+      for (int k = sub; k < n; k += 8) s += magnitude_part(p, x, y, k, k < m || k >= m + 32);
       __syncwarp();
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(ALL, s, o);
+      s = sum_of_eight(s);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int to = __shfl_sync(ALL, e, 8 * j);
@@ -439,25 +535,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 3) oz_small_kernel(const __grid
     const int n = ntodo;
     for (int d = warp; d < n; d += WARPS) {
       const Formed f = todo[d];
-      const double* row = p.P + f.row;
-      const uint32_t inv = div_inv(uint32_t(f.wx));
-      double y = 0.0;
-      constexpr int U = 12;  // loads of each operand in flight
-      for (int k0 = lane; k0 < f.wn; k0 += 32 * U) {
-        double v[U], w[U];
-#pragma unroll
-        for (int h = 0; h < U; ++h) {
-          const int k = k0 + 32 * h, b = div_by(k, inv);
-          int gy = f.oy + b, gx = f.ox + (k - b * f.wx);
-          gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
-          gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
-          v[h] = k < f.wn ? row[k] : 0.0;
-          w[h] = k < f.wn ? p.src[uint32_t(gy) * uint32_t(nx) + uint32_t(gx)] : 0.0;
-        }
-#pragma unroll
-        for (int h = 0; h < U; ++h) y = fma(v[h], w[h], y);
-      }
-      for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(ALL, y, o);
+      const double y = form(p, p.P + f.row, f.oy, f.ox, f.wx, f.wn);
       if (lane == 0) p.u[f.to] = p.accumulate ? f.old + y : y;
     }
     __syncthreads();
@@ -495,7 +573,7 @@ struct StepWork {
     const uint32_t plain = o.plain(row, half);
     small = (small & o.checked(row, half)) | plain;
     if (__any_sync(0xffffffffu, small != 0)) {
-      uint32_t place = o.places(__popc(small), lane);
+      uint32_t place = o.places(p.nsmall, __popc(small), lane);
       const int64_t at = o.row_at(row);
 #pragma unroll 4
       for (; small; small &= small - 1) {
@@ -539,7 +617,12 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_split_kernel(const __g
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ volatile int s_abort;
   __shared__ StepTables tab;
+  __shared__ unsigned s_count[2];
+  constexpr size_t SUMS = sizeof(longlong2) * oz::BN * oz::SUM_PITCH;
+  static_assert(SUMS % 8 == 0 && SUMS + SmallList::kBytes * oz::BM * oz::BN / 2 <= size_t(oz::STAGES) * oz::STAGE,
+                "the list of half the columns fits behind the sums");
   const oz::Shared sh = oz::carve(smem_raw);
+  if (threadIdx.x < 2) s_count[threadIdx.x] = 0;
   const int ks = p.ks, rank = int(blockIdx.x) % ks;
   const Unit un = p.units[p.unit0 + int(blockIdx.x) / ks];
   const WinBlock wb = p.blocks[un.wb];
@@ -561,6 +644,7 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_split_kernel(const __g
   for (int j = 0; j < ks; ++j) whole = whole && !*cl.map_shared_rank(const_cast<int*>(&s_abort), j);
   if (whole && c0 < un.ncol) {
     const StepUnit o(p, un, wb, tab);
+    const SmallList own(sh.stage + SUMS, oz::BM * oz::BN / 2, s_count);
     constexpr int U = 4;  // elements per thread in flight
     const int total = wb.count * cw, warp0 = int(threadIdx.x) / 32 * 32, lane = int(threadIdx.x) % 32;
     for (int q0 = warp0; q0 < total; q0 += U * oz::THREADS) {  // (whole warps)
@@ -588,12 +672,13 @@ __global__ void __launch_bounds__(oz::THREADS, 1) oz_step_split_kernel(const __g
         const uint32_t bit = 1u << (col % 32), plain = o.plain(row, col / 32) & bit;
         const bool small = in[k] && (plain || (oz::small_sum(v.x) && (o.checked(row, col / 32) & bit)));
         if (__any_sync(0xffffffffu, small)) {
-          const uint32_t place = o.places(small ? 1 : 0, lane);
-          if (small) o.list(place, row, col, plain != 0, old[k]);
+          const uint32_t place = o.places(own.count, small ? 1 : 0, lane);
+          if (small) own.put(place, row, col, plain != 0, old[k]);
         }
         if (in[k]) o.store(where[k], oz::sums_to_double(v.x, v.y, o.scale(row, col)), old[k]);
       }
     }
+    settle_cta(o, own);
   }
   cl.sync();  // the sums stay until every CTA of the cluster has read them
   oz::release(tmem);
@@ -607,7 +692,10 @@ struct OzPlan {
   std::vector<WinBlock> blocks;
   std::vector<Unit> units;
   std::vector<PropRows> rows;
-  struct Group { int wb0, nwb, unit0, nunits, ks; };
+  struct Group {
+    int wb0, nwb, unit0, nunits, ks;
+    int64_t owners;
+  };
   std::vector<Group> groups;   // window blocks whose digits are held together
   int nsm = 152;
   size_t a_halves = 0, b_halves = 0;
@@ -625,7 +713,7 @@ struct OzPlan {
   unsigned* d_nsmall = nullptr;
   uint2* d_small_at = nullptr;
   double* d_small_old = nullptr;
-  int64_t max_owners = 0;      // of a group
+  int64_t max_owners = 0;      // of a group whose units are not shared
   int fault = 0;
   int64_t bytes = 0;           // device memory of the plan
   int* d_err = nullptr;
@@ -642,16 +730,15 @@ void plan_oz(const lem_ctx* ctx, OzPlan* z) {
     return (ctx->classes[c].wext[0] * ctx->classes[c].wext[1] + oz::KB - 1) / oz::KB;
   };
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return nkb_of(a) > nkb_of(b); });
-  OzPlan::Group g{0, 0, 0, 0, 1};
-  int64_t held = 0, owned = 0;
+  OzPlan::Group g{0, 0, 0, 0, 1, 0};
+  int64_t held = 0;
   int ge = 0;
   auto close = [&]() {
     if (g.nwb) z->groups.push_back(g);
     z->a_halves = std::max<size_t>(z->a_halves, size_t(held));
     z->ne = std::max(z->ne, ge);
-    z->max_owners = std::max(z->max_owners, owned);
-    g = OzPlan::Group{int(z->blocks.size()), 0, int(z->units.size()), 0, 1};
-    held = owned = 0;
+    g = OzPlan::Group{int(z->blocks.size()), 0, int(z->units.size()), 0, 1, 0};
+    held = 0;
     ge = 0;
   };
   for (int c : order) {
@@ -671,7 +758,7 @@ void plan_oz(const lem_ctx* ctx, OzPlan* z) {
       const int wb = int(z->blocks.size());
       z->blocks.push_back(WinBlock{w, std::min(oz::BM, n1 - w), c, nkb, held, ge, f0, b0});
       held += halves;
-      owned += int64_t(std::min(oz::BM, n1 - w)) * owners;
+      g.owners += int64_t(std::min(oz::BM, n1 - w)) * owners;
       ge += oz::BM;
       g.nwb++;
       for (int j = 0; j < ncb; ++j) {
@@ -770,7 +857,10 @@ lem_status oz_prepare(lem_ctx* ctx) {
   LEM_CUDA_TRY(cudaFuncSetAttribute(oz_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM));
   LEM_CUDA_TRY(cudaFuncSetAttribute(oz_step_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM));
   if (cudaDeviceGetAttribute(&z->nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || z->nsm < 1) z->nsm = 152;
-  for (auto& g : z->groups) g.ks = pick_split(g, z, z->nsm);
+  for (auto& g : z->groups) {
+    g.ks = pick_split(g, z, z->nsm);
+    if (g.ks == 1) z->max_owners = std::max(z->max_owners, g.owners);
+  }
   LEM_TRY(take(ctx, &z->d_blocks, z->blocks.size()));
   LEM_TRY(take(ctx, &z->d_units, z->units.size()));
   LEM_TRY(take(ctx, &z->d_rows, z->rows.size()));
@@ -815,8 +905,8 @@ lem_status oz_check_error(lem_ctx* ctx) {
 // Window digits, and room for the list of small sums (at the first step).
 static lem_status oz_windows(lem_ctx* ctx) {
   OzPlan* z = ctx->oz;
-  LEM_TRY(take(ctx, &z->d_small_at, size_t(z->max_owners)));
-  if (ctx->desc.mode == LEM_MODE_PHI) LEM_TRY(take(ctx, &z->d_small_old, size_t(z->max_owners)));
+  if (z->max_owners) LEM_TRY(take(ctx, &z->d_small_at, size_t(z->max_owners)));
+  if (z->max_owners && ctx->desc.mode == LEM_MODE_PHI) LEM_TRY(take(ctx, &z->d_small_old, size_t(z->max_owners)));
   LEM_TRY(take(ctx, &z->d_amag, z->a_halves / oz::S));
   LEM_TRY(take(ctx, &z->d_a, z->a_halves));
   // rows past a block's last window are multiplied too (their sums are dropped)
@@ -875,6 +965,7 @@ lem_status step_oz(lem_ctx* ctx, double* d_u) {
       cfg = split_config(g.ks, g.nunits, st, at);
       LEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_step_split_kernel, p));
     }
+    if (g.ks > 1) continue;
     at[0] = chained();
     cfg.gridDim = dim3(unsigned(3 * z->nsm));
     cfg.blockDim = dim3(SMALL_THREADS);
