@@ -127,3 +127,21 @@ def test_scratch_kept_by_refreshing_contexts_is_bounded():
     assert np.array_equal(ctxs[6].propagator(3), want) and np.array_equal(ctxs[5].propagator(3), want)
     for c in ctxs[1:]:
         c.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "split_fast"])
+def test_windows_beyond_the_panel_kernel(prec):
+    """Windows of more than 2880 nodes, whose panels do not fit a cluster's shared memory, are eliminated
+    column by column: one window that is the line, against the sine modes of its Laplacian. The bar is that
+    of the other builder tests, 1e-11 of max|P|."""
+    n, mu = 2901, 2.0  # (the last panel is ragged)
+    ctx = L.Lem((n,), ("dirichlet",), {"C": -2 * mu, "W": mu, "E": mu}, 1.0, (n,), (0,), prec=prec)
+    assert ctx.info()["n_loc"] == n
+    ctx.build()
+    P = ctx.propagator(0)
+    ctx.close()
+    j = np.arange(1, n + 1)
+    lam = -4 * mu * np.sin(np.pi * j / (2 * (n + 1))) ** 2
+    S = np.sin(np.pi * np.outer(j, j) / (n + 1))
+    want = (S * (np.expm1(lam) / lam)) @ S * (2 / (n + 1))
+    assert np.abs(P - want).max() <= 1e-11 * np.abs(want).max()
