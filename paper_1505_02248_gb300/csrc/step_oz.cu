@@ -893,12 +893,14 @@ lem_status oz_pack(lem_ctx* ctx) {
   return LEM_OK;
 }
 
+// (on the context's stream: a plain copy would wait for whatever runs on the legacy stream)
 lem_status oz_check_error(lem_ctx* ctx) {
   if (!ctx->oz) return LEM_OK;
   int e = 0;
-  LEM_CUDA_TRY(cudaMemcpy(&e, ctx->oz->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  LEM_CUDA_TRY(cudaMemcpyAsync(&e, ctx->oz->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  LEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
   if (e == 0) return LEM_OK;
-  cudaMemset(ctx->oz->d_err, 0, sizeof(int));
+  cudaMemsetAsync(ctx->oz->d_err, 0, sizeof(int), ctx->stream);
   return fail(LEM_ETIMEOUT, "FP64 tensor-core step gave up waiting on an mbarrier (code " + std::to_string(e) + ")");
 }
 

@@ -1619,9 +1619,10 @@ lem_status split_check_error(lem_ctx* ctx) {
   LEM_TRY(oz_check_error(ctx));
   if (!ctx->split) return LEM_OK;
   int e = 0;
-  LEM_CUDA_TRY(cudaMemcpy(&e, ctx->split->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  LEM_CUDA_TRY(cudaMemcpyAsync(&e, ctx->split->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  LEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
   if (e != 0) {
-    cudaMemset(ctx->split->d_err, 0, sizeof(int));
+    cudaMemsetAsync(ctx->split->d_err, 0, sizeof(int), ctx->stream);
     if (e == ERR_NUMERIC) return fail(LEM_ENUMERIC, "split path: propagator rows too heavy for an exact integer product");
     return fail(LEM_ETIMEOUT, "tensor-core kernel gave up waiting on an mbarrier (code " + std::to_string(e) + ")");
   }

@@ -1,5 +1,7 @@
-"""Contexts of unlike windows in one process: the shared memory that one's kernels take does not bound
-the other's."""
+"""Contexts beside others in one process: the shared memory that one's kernels take does not bound the other's, and
+a context on a stream of its own does not wait for work on the legacy stream."""
+import time
+
 import numpy as np
 import pytest
 
@@ -52,3 +54,25 @@ def test_a_second_context_with_smaller_windows(tol):
     check(large, (80, 90))
     large.close()
     small.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "split"])
+def test_sync_waits_for_the_contexts_stream_only(prec):
+    st = torch.cuda.Stream()
+    coef = {"C": -46.0, "W": 14.0, "E": 10.0, "S": 12.0, "N": 10.0}
+    ctx = L.Lem((64, 64), ("periodic",) * 2, coef, 0.1, (8, 8), (4, 4), prec=prec, stream=st.cuda_stream)
+    assert L.APPLY_PATHS[ctx.info()["apply_path"]] == ("fp64_gemm" if prec == "fp64" else "tc_split")
+    ctx.build()
+    u = torch.ones(64 * 64, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    ctx.step(u, 1)
+    ctx.sync()
+    torch.cuda._sleep(2_000_000_000)  # about a second on the legacy stream
+    t0 = time.perf_counter()
+    ctx.step(u, 1)
+    ctx.sync()
+    took = time.perf_counter() - t0
+    torch.cuda.synchronize()
+    whole = time.perf_counter() - t0
+    assert whole > 0.5 and took < 0.5 * whole
+    ctx.close()
