@@ -953,9 +953,9 @@ def main():
                    "prec": a.prec, "apply_path": path, "l2": "256 MiB write between timed steps",
                    "parallelism": f"replicas x{world}", "build_ms": round(build_ms, 1)},
         # split: max|r| pass (which also converts FP64 -> float-float), (residual + GEMM) per LEM
-        # step, float-float -> FP64; FP64: residual, window digits, products per LEM step
+        # step, float-float -> FP64; FP64: residual, window digits, products, small sums per LEM step
         "gpu_launches": a.steps * ((2 + 2 * a.inner) if path == "tc_split" else
-                                   a.inner * (2 if "gemv" in path else 3)),
+                                   a.inner * (2 if "gemv" in path else 4)),
     }
     if gemm_launches:
         avg_ms = gemm_ms / gemm_launches
@@ -972,7 +972,7 @@ def main():
         else:
             flops = 28 * flops1  # FP16 digit products per FP64 product
             fp64_peak = fp64_dgemm_tflops(dev)
-            line["roofline"] = {"kernel": "oz_windows_kernel and oz_step_kernel (FP64 step, tcgen05 kind::f16)",
+            line["roofline"] = {"kernel": "oz_windows_kernel, oz_step_kernel and oz_small_kernel (FP64 step, tcgen05 kind::f16)",
                                 "bound": "tensor", "achieved": flops / (avg_ms * 1e-3) / 1e12, "peak": tflops_peak,
                                 "unit": "TFLOP/s", "frac": flops / (avg_ms * 1e-3) / 1e12 / tflops_peak, "traffic": None,
                                 "avg_launch_us": avg_ms * 1e3, "launches": gemm_launches,

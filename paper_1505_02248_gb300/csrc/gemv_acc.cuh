@@ -1,4 +1,4 @@
-// Accumulators of the batched GEMVs (step_gemv.cu).
+// Accumulators and loads of the batched GEMVs (step_gemv.cu) and of the truncated apply (step_band.cu).
 #pragma once
 #include <cuda_runtime.h>
 

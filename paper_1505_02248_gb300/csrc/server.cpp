@@ -15,7 +15,7 @@
 // kMaxFp64Active of them run and the budget keeps a quarter free for the split tier. Streams
 // of split-tier contexts have the device's highest priority and FP64-tier ones its lowest,
 // and FP64-tier chunks are issued only while the split tier has nothing on the GPU (or one
-// every kFp64GapMs), so long FP64 kernels do not hold back the quick tier.
+// every kFp64GapMs), so that an FP64 step, which takes every SM whole, does not hold back the quick tier.
 //
 // A split-tier request keeps its state in float-float on the device from admission to
 // completion, with the residual scale carried from chunk to chunk, so its result is the same
@@ -526,8 +526,8 @@ void worker_loop(lem_server* s) {
       }
     }
     // issue and retire chunks. FP64-tier steps are issued only while no split-tier request
-    // has work on the GPU or waits for admission (a long FP64 kernel holds SMs that the
-    // tensor-core kernels need whole), or at most every kFp64GapMs when the split tier never
+    // has work on the GPU or waits for admission (an FP64 step holds whole SMs, as the split
+    // tier's kernels do: 0.02 to 0.2 ms each), or at most every kFp64GapMs when the split tier never
     // pauses, so that the FP64 tier still advances.
     bool quick_busy = false;
     {
@@ -558,8 +558,8 @@ void worker_loop(lem_server* s) {
                           r->cc->stream);
           r->state = RS::CopyBack;
         } else {
-          // FP64-tier requests advance one step per chunk: their steps are long, and shorter
-          // chunks interleave better with the split tier
+          // FP64-tier requests advance one step per chunk: shorter chunks interleave better with the
+          // split tier (set when a step took milliseconds on the FP64 pipe)
           const int chunk = std::min(r->remaining, r->fp64_tier ? 1 : kChunk);
           const auto ti = Clock::now();
           lem_status st = LEM_OK;

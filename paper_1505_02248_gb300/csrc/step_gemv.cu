@@ -34,7 +34,7 @@ namespace {
 // packed sums, windows staged without divisions and owner values read before their row 578, first
 // chunks before the wait 564 to 573 (five blocks an SM 599, three chunks in flight 608). FP64 rows of
 // the same problem 1499 -> 1456 us, 101^2 with tiles of 12 212 -> 169. A Schroedinger line of 65536
-// (31 MB): 286, 270, 254, 206 us, its FP64 rows 822 -> 753.
+// (63 MB): 286, 270, 254, 206 us, its FP64 rows 822 -> 753.
 // CPLX: complex states (interleaved re, im) with real-embedded propagators
 // [[Re P, -Im P], [Im P, Re P]]: the window is staged as [re parts | im parts] (n_loc / 2 nodes
 // each, zero padded); each owner's Re and Im rows are read once, left halves only.
@@ -465,7 +465,7 @@ int gemv_row_split(const lem_ctx* ctx, int threads) {
 // dies, and hold the state, the coefficients and what passes through as well). All others are read
 // as passing through. A call of ten steps on 320^2 variable diffusion (308 MB a step): 32 MB 571.6 us,
 // 48 MB 572.5, 80 MB 586 (before sums were packed: none 674, 32 MB 659); a Schroedinger line of 65536
-// (31 MB, all kept): 206 us, with room for 80 MB 218 (before: none 270, kept 254).
+// (63 MB, 416 of 820 classes kept): 206 us, with room for all of it 218 (before: none 270, kept 254).
 static int resident_classes(const lem_ctx* ctx, bool f32) {
   const int64_t bytes = ctx->n_int * ctx->n_loc * (f32 ? 4 : 8) / (ctx->cplx ? 2 : 1);
   return int(std::min<int64_t>(32000000 / std::max<int64_t>(bytes, 1), int64_t(ctx->classes.size())));
