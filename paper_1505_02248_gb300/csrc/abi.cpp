@@ -177,6 +177,13 @@ lem_status adopt_propagators(lem_ctx* dst, lem_ctx* src, cudaEvent_t built) {
   LEM_CUDA_TRY(cudaStreamWaitEvent(dst->stream, built, 0));
   LEM_CUDA_TRY(cudaMemcpyAsync(dst->d_P, src->d_P, sizeof(double) * dst->n_int * dst->n_loc,
                                cudaMemcpyDeviceToDevice, dst->stream));
+  // what src's stream frees or rewrites later comes after the copy
+  cudaEvent_t copied;
+  LEM_CUDA_TRY(cudaEventCreateWithFlags(&copied, cudaEventDisableTiming));
+  cudaError_t e = cudaEventRecord(copied, dst->stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(src->stream, copied, 0);
+  cudaEventDestroy(copied);
+  LEM_CUDA_TRY(e);
   LEM_TRY(oz_pack(dst));
   dst->squarings = src->squarings;
   dst->built = true;
