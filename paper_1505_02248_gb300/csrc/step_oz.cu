@@ -32,6 +32,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "lem_internal.h"
@@ -335,8 +336,7 @@ struct StepUnit {
 // The elements that the digits may not give to FP64 accuracy: where the magnitudes of the owner row and of
 // the window make sum |P| |u| large, the digit sum stands; 512 nodes around the row's largest entries tell
 // as a rule, the others are looked at if they do not (eight lanes per element). Else
-// the element is formed as FP64 multiply-adds over the whole row, by a warp (an FP64 instruction takes 16 clk of the SM's
-// pipe: shared over the CTA, the sums across warps cost half as much again as the products).
+// the element is formed as FP64 multiply-adds over the whole row.
 // The CTAs of a cluster that shares a unit hold few elements each: they list them in shared memory and look
 // at them behind the sums (settle_cta). 256^2, tiles of 16, ten steps 284 us, 327 by oz_small_kernel, whose launch and
 // chain of loads take 6 to 9 us a step. CTAs with whole units leave theirs to oz_small_kernel, by a list in
@@ -345,7 +345,8 @@ struct StepUnit {
 // 16 384 random values, ten steps, 1156 instead of 345).
 // Of the elements of smooth fields 1 to 12 % come here (phi_1 of a residual, mu 50: 39 %), 0 to 0.2 % are
 // formed (mu 2, whose rows are narrow: 8 %). Bound by the latency of the loads, or by the FP64 pipe
-// where many elements are formed: at most what the step took before it used digits.
+// where many elements are formed: a step all of whose elements are takes about what it took before it
+// used digits (0.9 to 1.1 of it).
 constexpr unsigned ALL = 0xffffffffu;
 constexpr uint32_t LARGE = 1u << (16 - (38 - oz::kSmallSum));  // 2^-2 in units of 2^-16
 // Magnitudes k of the rows at a and b (in 16 bytes): their products, in units of 2^-16.
@@ -377,17 +378,19 @@ __device__ __forceinline__ uint32_t magnitude_sum(const StepParams& p, uint32_t 
   return s + sum_of_eight(r);
 }
 __device__ __forceinline__ int middle(int mid, int nk) { return max(min(mid / 16 - 16, nk - 32), 0); }
-// The element of an owner row and the window at (oy, ox), wn nodes, wx a row, by a warp.
+// The element of an owner row and the window at (oy, ox), wn nodes, wx a row, by LANES lanes of a warp
+// (every lane of the warp calls it; wn 0: no element).
+template <int LANES>
 __device__ __forceinline__ double form(const StepParams& p, const double* row, int oy, int ox, int wx, int wn) {
-  const int lane = int(threadIdx.x) % 32, ny = int(p.ny), nx = int(p.nx);
+  const int lane = int(threadIdx.x) % LANES, ny = int(p.ny), nx = int(p.nx);
   const uint32_t inv = div_inv(uint32_t(wx));
   double y = 0.0;
   constexpr int U = 12;  // loads of each operand in flight
-  for (int k0 = lane; k0 < wn; k0 += 32 * U) {
+  for (int k0 = lane; k0 < wn; k0 += LANES * U) {
     double v[U], w[U];
 #pragma unroll
     for (int h = 0; h < U; ++h) {
-      const int k = k0 + 32 * h, b = div_by(k, inv);
+      const int k = k0 + LANES * h, b = div_by(k, inv);
       int gy = oy + b, gx = ox + (k - b * wx);
       gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
       gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
@@ -397,8 +400,19 @@ __device__ __forceinline__ double form(const StepParams& p, const double* row, i
 #pragma unroll
     for (int h = 0; h < U; ++h) y = fma(v[h], w[h], y);
   }
-  for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(ALL, y, o);
+  __syncwarp();
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) y += __shfl_xor_sync(ALL, y, o);
   return y;
+}
+// Calls f with the lanes per element, a constant: eight where `each`, the elements a warp has to form, are more
+// than two, so that the sums across lanes (16 clk each of the SM's FP64 pipe, as every FP64 instruction) are
+// a small part; a whole warp where they are few and their latency counts. All of a bump's elements, one step:
+// 512^2, tiles of 8, 465 -> 332 us (307 with the FP64 GEMM), tiles of 16 1240 -> 827 (846), of 32 2235 -> 2094 (2413).
+template <class F>
+__device__ __forceinline__ void with_lanes(int each, F f) {
+  if (each > 2) f(std::integral_constant<int, 8>());
+  else f(std::integral_constant<int, 32>());
 }
 
 // A CTA's own list, in shared memory.
@@ -436,12 +450,16 @@ __device__ __forceinline__ void settle_cta(const StepUnit& o, const SmallList& l
   }
   __syncthreads();
   const int m = int(l.count[1]);
-  for (int d = warp; d < m; d += warps) {
-    const int i = l.todo[d], at = l.at[i], row = at % oz::BM, col = at / oz::BM % oz::BN;
-    const double y = form(o.p, o.p.P + (int64_t(o.wb.cls) * o.p.n_int + o.un.col0 + col) * o.p.n_loc,
-                          o.t.t0[row].x - o.t.oy, o.t.t0[row].y - o.t.ox, o.t.wx, o.t.wn);
-    if (lane == 0) o.store(o.row_at(row) + o.col_at(col), y, l.old[i]);
-  }
+  with_lanes((m + warps - 1) / warps, [&](auto lanes) {
+    constexpr int L = decltype(lanes)::value;
+    for (int d0 = warp * (32 / L); d0 < m; d0 += warps * (32 / L)) {
+      const int d = d0 + lane / L;
+      const int i = l.todo[min(d, m - 1)], at = l.at[i], row = at % oz::BM, col = at / oz::BM % oz::BN;
+      const double y = form<L>(o.p, o.p.P + (int64_t(o.wb.cls) * o.p.n_int + o.un.col0 + col) * o.p.n_loc,
+                               o.t.t0[row].x - o.t.oy, o.t.t0[row].y - o.t.ox, o.t.wx, d < m ? o.t.wn : 0);
+      if (d < m && lane % L == 0) o.store(o.row_at(row) + o.col_at(col), y, l.old[i]);
+    }
+  });
 }
 
 constexpr int SMALL_THREADS = 256;
@@ -533,11 +551,15 @@ __global__ void __launch_bounds__(SMALL_THREADS, 3) oz_small_kernel(const __grid
     }
     __syncthreads();
     const int n = ntodo;
-    for (int d = warp; d < n; d += WARPS) {
-      const Formed f = todo[d];
-      const double y = form(p, p.P + f.row, f.oy, f.ox, f.wx, f.wn);
-      if (lane == 0) p.u[f.to] = p.accumulate ? f.old + y : y;
-    }
+    with_lanes((n + WARPS - 1) / WARPS, [&](auto lanes) {
+      constexpr int L = decltype(lanes)::value;
+      for (int d0 = warp * (32 / L); d0 < n; d0 += WARPS * (32 / L)) {
+        const int d = d0 + lane / L;
+        const Formed f = todo[min(d, n - 1)];
+        const double y = form<L>(p, p.P + f.row, f.oy, f.ox, f.wx, d < n ? f.wn : 0);
+        if (d < n && lane % L == 0) p.u[f.to] = p.accumulate ? f.old + y : y;
+      }
+    });
     __syncthreads();
     if (threadIdx.x == 0) ntodo = 0;
     __syncthreads();
